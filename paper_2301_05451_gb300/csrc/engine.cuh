@@ -23,15 +23,17 @@ constexpr int kSpecFwdRegBits = 2;
 constexpr int kSpecRevRegBits = 2;
 // tiled programs specialised to the circuit: their passes stream the state
 // through HBM, and wide register passes mean fewer shared-memory round trips
-// (the 20-qubit ladder: 4/4 bits 4715 evals/s against 4536 at 4/3 and 4407
-// at 3/3, GB300)
+// (the 20-qubit ladder, 64 rows: 6.22 ms at 4/4 bits, 6.60 at 3/4, 6.83 at
+// 4/3, 7.18 at 3/3; a third CTA per SM at 80 / 85 registers gained nothing
+// forward and cost 20 % in reverse)
 constexpr int kTiledSpecFwdRegBits = 4;
 constexpr int kTiledSpecRevRegBits = 4;
-// Gradient slots at most per reverse register pass (its accumulators live in
-// registers beside the pass's amplitudes; the 20-qubit ladder's reverse
-// passes spilled registers with 20 and more)
+// Gradient slots at most per reverse register pass of a specialised program
+// (its accumulators live in registers beside the pass's amplitudes: 64 + 16 of
+// the 128 that two CTAs of 256 threads leave a thread; at 8 the 20-qubit
+// ladder needs half as many passes again).  The generic kernels keep none.
 #ifndef TDQ_REV_PASS_SLOTS
-#define TDQ_REV_PASS_SLOTS 8
+#define TDQ_REV_PASS_SLOTS 16
 #endif
 constexpr int kRevPassSlots = TDQ_REV_PASS_SLOTS;
 
@@ -57,8 +59,10 @@ struct DOp {
 static_assert(sizeof(DOp) == 16, "DOp layout");
 
 // Bank-conflict-free shared-memory index of tile element x (8-byte
-// elements): the low 4 bits are XORed with bits 4..7.  A bijection.
-__device__ __forceinline__ uint32_t swz(uint32_t x) { return x ^ ((x >> 4) & 15u); }
+// elements): the low 4 bits are XORed with bits 4..7 and 8..11.  A linear
+// bijection; a half-warp whose lanes differ in four bits of different
+// residues mod 4 reads 16 different slots.
+__device__ __forceinline__ uint32_t swz(uint32_t x) { return x ^ ((x >> 4) & 15u) ^ ((x >> 8) & 15u); }
 
 // Gate tensor of op o for one row: forward matrix (diagonal gates keep their
 // two phases in m00 / m11), and for U3 dU3/dtheta.
@@ -541,6 +545,8 @@ __device__ __forceinline__ void adj_group(c2* psi, c2* lam, const RegPass& rp, c
 }
 
 // Asynchronous 8-byte global -> shared copy (cp.async, completed in groups).
+// A host compiler (the kernels' CPU check) copies at once.
+#if defined(__CUDACC__) || defined(__CUDACC_RTC__)
 __device__ __forceinline__ void cp_async8(c2* dst_smem, const c2* src_gmem) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst_smem);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src_gmem) : "memory");
@@ -549,6 +555,12 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 // Wait until at most N of this thread's committed groups are still in flight.
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+#else
+inline void cp_async8(c2* dst_smem, const c2* src_gmem) { *dst_smem = *src_gmem; }
+inline void cp_async_commit() {}
+template <int N>
+inline void cp_async_wait() {}
+#endif
 
 // Warp-reduced gradient share v, added by lane 0 to entry `index` of its
 // warp's own row (length `stride`) of partial sums: no atomics, each warp
@@ -566,25 +578,31 @@ __device__ __forceinline__ void grad_share(float* gpart, int stride, int index, 
 // low); lanes with the low 5 - log2 K bits clear add it to entry idx[j] of
 // their warp's row (length stride) of partial sums.  K - 1 + (5 - log2 K)
 // shuffles instead of 5 K.
+// (Written as template recursion: in the largest kernels a loop over v was
+// unrolled too late for v to leave local memory.)
+template <int K, int H, int J>
+__device__ __forceinline__ void grad_exchange(float (&v)[K], bool up, int o) {
+  if constexpr (J < H) {
+    const float send = up ? v[J] : v[J + H];
+    const float keep = up ? v[J + H] : v[J];
+    v[J] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    grad_exchange<K, H, J + 1>(v, up, o);
+  }
+}
+template <int K, int H, int O>
+__device__ __forceinline__ void grad_butterfly(float (&v)[K], int lane) {
+  if constexpr (O > 0) {
+    if constexpr (H > 0) grad_exchange<K, H, 0>(v, (lane & O) != 0, O);
+    else v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
+    grad_butterfly<K, H / 2, O / 2>(v, lane);
+  }
+}
 template <int K>
 __device__ __forceinline__ void grad_share_multi(float* gpart, int stride, const int* idx, float (&v)[K]) {
   static_assert(K >= 1 && K <= 32 && (K & (K - 1)) == 0, "K: a power of two up to 32");
   const int lane = threadIdx.x & 31;
   constexpr int LK = K == 1 ? 0 : K == 2 ? 1 : K == 4 ? 2 : K == 8 ? 3 : K == 16 ? 4 : 5;
-#pragma unroll
-  for (int st = 0; st < LK; st++) {
-    const int o = 16 >> st;
-    const int h = K >> (st + 1);  // values after this exchange
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int j = 0; j < h; j++) {
-      const float send = up ? v[j] : v[j + h];
-      const float keep = up ? v[j + h] : v[j];
-      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-  }
-#pragma unroll
-  for (int o = 16 >> LK; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  grad_butterfly<K, K / 2, 16>(v, lane);
   constexpr int low = 5 - LK;
   if ((lane & ((1 << low) - 1)) == 0) gpart[(threadIdx.x >> 5) * stride + idx[lane >> low]] += v[0];
 }
@@ -613,5 +631,193 @@ __device__ __forceinline__ OpMat build_recipe(const SweepArgs& a, const SweepOp*
   }
   return om;
 }
+
+// ------------------------------------------------------ programs in a linear frame
+// Gates of the specialised programs (lin_program.h) on a register group.
+// Member j of the group is the amplitude at y0 ^ (the pass's vector j); a
+// gate's two members are j and j ^ MJ, and the logical bit of member j is
+// parity(FR & j) xor a sign word's top bit that the group shares.
+//
+// Rotations are applied without their common factor, two fused multiply-adds
+// per pair instead of four products: for |cos| >= |sin| the pair becomes
+// (a0 - t a1, a1 + t a0) with t = sin / cos and the factor cos is left to the
+// pass's scale; else (u a0 - a1, u a1 + a0) with u = cos / sin and factor sin.
+// |t|, |u| <= 1, so a pass grows the amplitudes by at most sqrt(2) per gate.
+// What bounds the tiled kernels is issue slots and latency at 16 warps per SM
+// (ncu, 20-qubit ladder: issue 52 % forward, 45 % reverse, FMA pipe 31-36 %,
+// DRAM 41 % of its rate).  Against one fused 2 x 2 product per qubit forward
+// and one op per gate in reverse, with CNOTs as register moves: 20-qubit
+// ladder, 64 rows, value and gradient 12.74 -> 6.17 ms (tile passes 8 -> 6);
+// its 481 shifted circuits 26.3 -> 13.0 ms; 16 qubits of random gates, 24
+// rows, 611 -> 223 us; state vectors of 20 qubits, 16 rows, 1024 -> 644 us.
+
+__device__ __forceinline__ float sx(float v, uint32_t sign) { return __uint_as_float(__float_as_uint(v) ^ sign); }
+
+__host__ __device__ constexpr int cpar(int v) { return ((v >> 3) ^ (v >> 2) ^ (v >> 1) ^ v) & 1; }
+
+// sin x and cos x as unevaluated sums hi + lo of two floats, correct to about
+// 2^-28: the coefficients' errors are the same for every amplitude, so they,
+// not the rounding of single amplitudes, decide the error of an expectation.
+// x is reduced by multiples of pi/2 in double (a handful of FP64
+// instructions); the remainder's Taylor series (to r^9 / r^10, |r| <= pi/4)
+// runs in float with its leading terms kept as two floats.
+struct SinCos {
+  float s, sl, c, cl;
+};
+__device__ __forceinline__ SinCos sincos2(float x) {
+  const double y = (double)x;
+  const double k = rint(y * 0.63661977236758134308);
+  if (fabs(y) > 1e5) {  // rare: the reduction below needs a small multiple
+    double s, c;
+    sincos(y, &s, &c);
+    SinCos r = {(float)s, 0.f, (float)c, 0.f};
+    r.sl = (float)(s - (double)r.s);
+    r.cl = (float)(c - (double)r.c);
+    return r;
+  }
+  const double rd = fma(k, -1.57079632679489661923, y);
+  const float r = (float)rd, rl = (float)(rd - (double)r);
+  const float p = r * r, pl = fmaf(r, r, -p) + 2.f * r * rl;
+  // sin = r + (rl + r^3 (-1/6 + p/120 - p^2/5040 + p^3/362880))
+  const float sp = fmaf(p, fmaf(p, fmaf(p, 2.7557319e-6f, -1.98412698e-4f), 8.33333333e-3f), -0.166666667f);
+  const float sx0 = fmaf(r * p, sp, rl);
+  const float s0 = r + sx0, s1 = sx0 - (s0 - r);
+  // cos = 1 - p/2 + (-pl/2 + p^2 (1/24 - p/720 + p^2/40320 - p^3/3628800))
+  const float cp = fmaf(p, fmaf(p, fmaf(p, -2.75573192e-7f, 2.48015873e-5f), -1.38888889e-3f), 4.16666667e-2f);
+  const float c00 = fmaf(-0.5f, p, 1.f), c01 = fmaf(-0.5f, p, 1.f - c00);
+  const float cx0 = fmaf(p * p, cp, fmaf(-0.5f, pl, c01));
+  const float c0 = c00 + cx0, c1 = cx0 - (c0 - c00);
+  const int q = (int)k & 3;
+  SinCos o;
+  o.s = (q & 1) ? c0 : s0;
+  o.sl = (q & 1) ? c1 : s1;
+  o.c = (q & 1) ? s0 : c0;
+  o.cl = (q & 1) ? s1 : c1;
+  if (q & 2) { o.s = -o.s; o.sl = -o.sl; }
+  if (q == 1 || q == 2) { o.c = -o.c; o.cl = -o.cl; }
+  return o;
+}
+
+// Table row of a rotation: {t or u, left-out factor (two floats), u form ? ~0 : 0}.
+__device__ __forceinline__ float4 rot_coef(float ang) {
+  SinCos r = sincos2(0.5f * ang);
+  const bool u = fabsf(r.s) > fabsf(r.c);
+  if (u) r = {r.c, r.cl, r.s, r.sl};
+  const float t = r.s / r.c;  // (s + sl) / (c + cl), rounded once
+  const float e = (fmaf(-t, r.c, r.s) + fmaf(-t, r.cl, r.sl)) / r.c;
+  return make_float4(t + e, r.c, r.cl, __uint_as_float(u ? 0xffffffffu : 0u));
+}
+
+__device__ __forceinline__ float coef_angle(const SweepArgs& a, const SweepOp* ops, int code, int64_t b, int k,
+                                            int* bad) {
+  const int gi = code >> 2, j = code & 3;
+  float v = op_angle(ops[gi], j, a.params, a.pstride, a.inputs, a.F, b, bad);
+  if (k > 0) {
+    const int e = (k - 1) >> 1;
+    if (a.ps_gate[e] == gi && a.ps_ang[e] == j) v += ((k - 1) & 1) ? -kHalfPiF : kHalfPiF;
+  }
+  return v;
+}
+
+// Gate-tensor table of a specialised program, built by the whole CTA for row
+// b (shift copy k); rows r0.. of the recipes go to mats[0..nrec).  Rotations:
+// see rot_coef.  Phases: {cos a/2, sin a/2, cos a, sin a}.  Scale of a
+// register pass: {Re S, Im S, 1 / |S|, 0}, S the product of its gates'
+// left-out factors, multiplied out in double (an exact program's RX in the u
+// form leaves -i sin; its phase does not reach expectations).  The caller
+// synchronises afterwards.
+__device__ __forceinline__ void build_coefs(const SweepArgs& a, const SweepOp* ops, const int* rec_ptr,
+                                            const int* rec_ops, int r0, int nrec, float4* mats, int64_t b, int k,
+                                            int* bad) {
+  for (int r = threadIdx.x; r < nrec; r += blockDim.x) {
+    const int e0 = rec_ptr[r0 + r], type = rec_ops[e0] & 255;
+    if (type != C_ROT && type != C_PHASE) continue;
+    const float v = coef_angle(a, ops, rec_ops[e0 + 1], b, k, bad);
+    if (type == C_ROT) {
+      mats[r] = rot_coef(v);
+    } else {
+      const SinCos h = sincos2(0.5f * v), f = sincos2(v);
+      mats[r] = make_float4(h.c, h.s, f.c, f.s);
+    }
+  }
+  __syncthreads();
+  for (int r = threadIdx.x; r < nrec; r += blockDim.x) {
+    const int e0 = rec_ptr[r0 + r], e1 = rec_ptr[r0 + r + 1], type = rec_ops[e0] & 255;
+    if (type == C_ROT || type == C_PHASE) continue;
+    const int nh = rec_ops[e0] >> 8;  // factors 1 / sqrt 2
+    double S = (nh & 1) ? 0.70710678118654752440 : 1.0;
+    for (int i = nh >> 1; i > 0; i--) S *= 0.5;
+    int turns = 0;  // factors -i
+    for (int e = e0 + 1; e < e1; e++) {
+      const float4 q = mats[rec_ops[e] >> 1];
+      S *= (double)q.y + (double)q.z;
+      turns += (rec_ops[e] & 1) && __float_as_uint(q.w) != 0u ? 1 : 0;
+    }
+    c2 z = {(float)S, 0.f};
+    if (type == C_NORM_EXACT) z = quarter_turns(z, -turns & 3);
+    mats[r] = make_float4(z.x, z.y, (float)(1.0 / fabs(S)), 0.f);
+  }
+}
+
+// The generated code names every member (no register arrays: in the largest
+// programs their indices became constants too late for them to leave local
+// memory) and calls these on one pair at a time.
+__device__ __forceinline__ void ry_t(c2& a0, c2& a1, float2 t, float2 nt) {
+  const float2 x0 = v2(a0), x1 = v2(a1);
+  a0 = c2v(fma2(nt, x1, x0));
+  a1 = c2v(fma2(t, x0, x1));
+}
+__device__ __forceinline__ void ry_u(c2& a0, c2& a1, float u) {
+  const c2 x0 = a0, x1 = a1;
+  a0 = {fmaf(u, x0.x, -x1.x), fmaf(u, x0.y, -x1.y)};
+  a1 = {fmaf(u, x1.x, x0.x), fmaf(u, x1.y, x0.y)};
+}
+// RX: (a0 - i t a1, a1 - i t a0), or (a1 + i u a0, a0 + i u a1) with factor -i sin.
+__device__ __forceinline__ void rx_t(c2& a0, c2& a1, float t) {
+  const c2 x0 = a0, x1 = a1;
+  a0 = {fmaf(t, x1.y, x0.x), fmaf(-t, x1.x, x0.y)};
+  a1 = {fmaf(t, x0.y, x1.x), fmaf(-t, x0.x, x1.y)};
+}
+__device__ __forceinline__ void rx_u(c2& a0, c2& a1, float u) {
+  const c2 x0 = a0, x1 = a1;
+  a0 = {fmaf(-u, x0.y, x1.x), fmaf(u, x0.x, x1.y)};
+  a1 = {fmaf(-u, x1.y, x0.x), fmaf(u, x1.x, x0.y)};
+}
+// H without its factor 1 / sqrt 2: (a0 + a1, a0 - a1), s = +-1 swaps the roles.
+__device__ __forceinline__ void h_pair(c2& a0, c2& a1, float2 s, float2 ns) {
+  const float2 x0 = v2(a0), x1 = v2(a1);
+  a0 = c2v(fma2(s, x0, x1));
+  a1 = c2v(fma2(ns, x1, x0));
+}
+// Im <lambda| Y |psi> of a pair is Re(conj l1 p0) - Re(conj l0 p1): the two
+// sums, packed.
+__device__ __forceinline__ void dot_y(c2 p0, c2 p1, c2 l0, c2 l1, float2& gp, float2& gn) {
+  gp = fma2(v2(l1), v2(p0), gp);
+  gn = fma2(v2(l0), v2(p1), gn);
+}
+// Im <lambda| X |psi> of a pair, as the difference of two sums.
+__device__ __forceinline__ void dot_x(c2 p0, c2 p1, c2 l0, c2 l1, float& gp, float& gn) {
+  gp = fmaf(l1.x, p0.y, fmaf(l0.x, p1.y, gp));
+  gn = fmaf(l1.y, p0.x, fmaf(l0.y, p1.x, gn));
+}
+
+// g += v, now: left to itself the compiler moves a share's last sums to the
+// end of the pass and keeps their operands in registers until then (up to 10
+// times the share's own; the ladder's reverse kernels spilled 30 to 3700 bytes).
+__device__ __forceinline__ void lin_share(float& g, float v) {
+  g += v;
+#if defined(__CUDACC__) || defined(__CUDACC_RTC__)
+  asm volatile("" : "+f"(g));
+#endif
+}
+
+// acc += Im(conj(l) p)
+__device__ __forceinline__ float lin_im(c2 l, c2 p, float acc) { return fmaf(-l.y, p.x, fmaf(l.x, p.y, acc)); }
+
+__device__ __forceinline__ void lin_mul(c2& a, c2 m) {
+  a = {fmaf(-a.y, m.y, a.x * m.x), fmaf(a.y, m.x, a.x * m.y)};
+}
+__device__ __forceinline__ void lin_scale(c2& a, float s) { a = c2v(mul2(bc2(s), v2(a))); }
+__device__ __forceinline__ void lin_neg(c2& a, uint32_t sign) { a = {sx(a.x, sign), sx(a.y, sign)}; }
 
 }  // namespace tdq

@@ -55,7 +55,7 @@ struct TileShared {
   c2* lam;
   c2* psi2;     // second buffers (double-buffered loads), or NULL
   c2* lam2;
-  OpMat* mats;  // [recipes of the pass]
+  OpMat* mats;  // [recipes of the pass] (specialised programs: float4 rows)
   DOp* dops;    // [decoded ops of the pass]
   double* red;
   double* vsum;         // [n_groups]
@@ -64,16 +64,16 @@ struct TileShared {
   int8_t* loc;
 };
 
-// layout: psi[2^k] x npsi | lambda[2^k] x nlam | mats[nrec] | dops[ndops] | red[32] |
+// layout: psi[2^k] x npsi | lambda[2^k] x nlam | gate tensors[mbytes] | dops[ndops] | red[32] |
 //         vsum[ng] | gpart[gbytes] | off[2^(k-L)] | loc[32]
-__host__ __device__ __forceinline__ size_t k1_smem_bytes(int k, int L, int npsi, int nlam, int nrec, int ndops,
+__host__ __device__ __forceinline__ size_t k1_smem_bytes(int k, int L, int npsi, int nlam, int mbytes, int ndops,
                                                         int ng, int gbytes) {
-  return (size_t)(1 << k) * sizeof(c2) * (npsi + nlam) + sizeof(OpMat) * nrec + sizeof(DOp) * ndops +
+  return (size_t)(1 << k) * sizeof(c2) * (npsi + nlam) + (size_t)mbytes + sizeof(DOp) * ndops +
          (32 + (size_t)ng) * sizeof(double) + (((size_t)gbytes + 7) & ~(size_t)7) + sizeof(int) * (1 << (k - L)) +
          32 + 16;
 }
 
-__device__ __forceinline__ TileShared carve(unsigned char* raw, int k, int L, int npsi, int nlam, int nrec,
+__device__ __forceinline__ TileShared carve(unsigned char* raw, int k, int L, int npsi, int nlam, int mbytes,
                                             int ndops, int ng, int gbytes) {
   TileShared s;
   const int nloc = 1 << k;
@@ -85,7 +85,7 @@ __device__ __forceinline__ TileShared carve(unsigned char* raw, int k, int L, in
   s.lam2 = nlam > 1 ? p + nloc : nullptr;
   p += nlam * nloc;
   s.mats = reinterpret_cast<OpMat*>(p);
-  s.dops = reinterpret_cast<DOp*>(s.mats + nrec);
+  s.dops = reinterpret_cast<DOp*>(reinterpret_cast<unsigned char*>(p) + mbytes);
   s.red = reinterpret_cast<double*>(s.dops + ndops);
   s.vsum = s.red + 32;
   s.gpart = reinterpret_cast<unsigned char*>(s.vsum + ng);
@@ -106,16 +106,26 @@ __device__ __forceinline__ float obs_weight(const SweepArgs& a, int g, uint32_t 
   return diag_weight(a.terms, a.group_ptr[g], a.group_ptr[g + 1], x);
 }
 
+// Bytes of a pass's gate tensors.
+template <class Prog>
+__device__ __forceinline__ int k1_mat_bytes(const TiledDev& t) {
+  return t.nrec * (int)(Prog::kSpecialised ? sizeof(float4) : sizeof(OpMat));
+}
+
 // Per-CTA set-up: offsets, local bits, this row's gate tensors (K0), the
 // decoded ops (interpreted programs) and zeroed partial sums.
+template <class Prog>
 __device__ __forceinline__ void k1_setup(const SweepArgs& a, const TiledDev& t, const TileShared& s, int64_t b,
                                          int kk, int* bad) {
   const int noff = 1 << (t.k - t.L);
   for (int i = threadIdx.x; i < noff; i += blockDim.x) s.off[i] = t.off[i];
   if (threadIdx.x < 32) s.loc[threadIdx.x] = t.loc[threadIdx.x];
-  // shifted gates are numbered in pass order (tiled_compile)
-  for (int i = threadIdx.x; i < t.nrec; i += blockDim.x)
-    s.mats[i] = build_recipe(a, t.ops, t.rec_ptr, t.rec_ops, t.rec0 + i, b, kk, bad);
+  // (interpreted programs: shifted gates are numbered in pass order, tiled_compile)
+  if constexpr (Prog::kSpecialised)
+    build_coefs(a, t.ops, t.rec_ptr, t.rec_ops, t.rec0, t.nrec, reinterpret_cast<float4*>(s.mats), b, kk, bad);
+  else
+    for (int i = threadIdx.x; i < t.nrec; i += blockDim.x)
+      s.mats[i] = build_recipe(a, t.ops, t.rec_ptr, t.rec_ops, t.rec0 + i, b, kk, bad);
   for (int i = threadIdx.x; i < t.ndops; i += blockDim.x) s.dops[i] = t.dops[i];
   for (int i = threadIdx.x; i < t.gbytes / 4; i += blockDim.x) reinterpret_cast<float*>(s.gpart)[i] = 0.f;
   for (int g = threadIdx.x; g < a.n_groups; g += blockDim.x) s.vsum[g] = 0.0;
@@ -124,6 +134,14 @@ __device__ __forceinline__ void k1_setup(const SweepArgs& a, const TiledDev& t, 
 
 // Gate program decoded at run time; gradient shares in FP64 per (recipe, angle).
 struct InterpTile {
+  static constexpr bool kSpecialised = false;
+  static constexpr bool kFirst = false, kSecond = false;
+  __device__ __forceinline__ static bool in_first(uint32_t) { return true; }
+  // f(shared-memory slot, global index) for this thread's elements of a tile
+  template <int NT, class F>
+  __device__ __forceinline__ static void every(const TiledDev& t, const TileShared& s, uint32_t base, F&& f) {
+    for (uint32_t j = threadIdx.x; j < (1u << t.k); j += blockDim.x) f(swz(j), gidx(s, base, j, t.L));
+  }
   __device__ __forceinline__ static void forward(const TiledDev& t, const TileShared& s, uint32_t base) {
     const int ngroups = 1 << (t.k - kFwdRegBits);
     for (int i = 0; i < t.nfp; i++) {
@@ -158,8 +176,17 @@ struct InterpTile {
 
 // Starts the asynchronous load of tile `base` of state g into buffer buf
 // (one commit group per thread).
-__device__ __forceinline__ void k1_issue(c2* buf, const c2* g, const TileShared& s, uint32_t base, int k, int L) {
-  for (uint32_t j = threadIdx.x; j < (1u << k); j += blockDim.x) cp_async8(&buf[swz(j)], &g[gidx(s, base, j, L)]);
+// sparse: only the elements on the first pass's space; the others are zero.
+template <int NT, class Prog>
+__device__ __forceinline__ void k1_issue(c2* buf, const c2* g, const TiledDev& t, const TileShared& s, uint32_t base,
+                                         bool sparse = false) {
+  if (Prog::kSecond && sparse)
+    Prog::template every<NT>(t, s, base, [&](uint32_t j, uint32_t x) {
+      if (Prog::in_first(x)) cp_async8(&buf[j], &g[x]);
+      else buf[j] = {0.f, 0.f};
+    });
+  else
+    Prog::template every<NT>(t, s, base, [&](uint32_t j, uint32_t x) { cp_async8(&buf[j], &g[x]); });
 }
 
 // The (row, tile) units of this CTA: a contiguous range of the row-major
@@ -186,12 +213,21 @@ __device__ __forceinline__ void k1_for_segments(const TiledDev& t, F&& f) {
 // and run this pass's reverse sweep at once (psi and lambda then written).
 // Tiles after the first of a row segment are read while the previous one is
 // being computed (two shared-memory buffers).
-template <bool FIRST, bool LAST, bool GRAD, class Prog>
+// NT: threads per CTA (specialised programs).
+//
+// From |0...0> the state after the first pass is zero outside the pass's tile
+// at base 0 (the space V0).  Specialised programs use that at both ends: the
+// first pass only visits that tile (the launch has one tile per row); the
+// second pass (Prog::kSecond) takes every element outside V0 as zero instead
+// of reading it, and its reverse sweep keeps psi and lambda only on V0, all
+// that the first pass's reverse sweep visits (its gradient shares are
+// products with psi, zero elsewhere).  On the 20-qubit ladder (64 rows) the
+// first pass went from 116 to 27 us forward and from 2.9 ms to 82 us in reverse.
+template <int NT, bool FIRST, bool LAST, bool GRAD, class Prog>
 __device__ __forceinline__ void k1_forward_body(const SweepArgs& a, const TiledDev& t, int store) {
   extern __shared__ __align__(16) unsigned char raw[];
-  const TileShared s = carve(raw, t.k, t.L, (FIRST || !t.dbl) ? 1 : 2, (GRAD && LAST) ? 1 : 0, t.nrec, t.ndops,
-                             a.n_groups, t.gbytes);
-  const uint32_t nloc = 1u << t.k;
+  const TileShared s = carve(raw, t.k, t.L, (FIRST || !t.dbl) ? 1 : 2, (GRAD && LAST) ? 1 : 0, k1_mat_bytes<Prog>(t),
+                             t.ndops, a.n_groups, t.gbytes);
   const uint32_t dim = 1u << t.n;
   const uint32_t other = (dim - 1u) & ~t.smask;
   k1_for_segments(t, [&](int lr, int tile0, int tile1) {
@@ -199,107 +235,104 @@ __device__ __forceinline__ void k1_forward_body(const SweepArgs& a, const TiledD
     const int64_t b = row / a.ps_copies;
     const int kk = row % a.ps_copies;
     int bad = 0;
-    k1_setup(a, t, s, b, kk, &bad);
+    k1_setup<Prog>(a, t, s, b, kk, &bad);
     if (bad) atomicOr(a.status, 1 << TDQ_ERR_NONFINITE);
     c2* gpsi = t.psi + (size_t)lr * dim;
     c2* glam = GRAD ? t.lam + (size_t)lr * dim : nullptr;
     if (!FIRST && t.dbl && tile0 < tile1) {
-      k1_issue(s.psi, gpsi, s, deposit((uint32_t)tile0, other), t.k, t.L);
+      k1_issue<NT, Prog>(s.psi, gpsi, t, s, deposit((uint32_t)tile0, other), !a.init);
       cp_async_commit();
     }
     for (int tile = tile0, it = 0; tile < tile1; tile++, it++) {
       const uint32_t base = deposit((uint32_t)tile, other);
       TileShared sc = s;
-      if (FIRST && !a.init && base != 0u) {
+      // this thread's elements: f(shared-memory slot, global index)
+      auto every = [&](auto&& f) { Prog::template every<NT>(t, s, base, f); };
+      if (FIRST && !Prog::kSpecialised && !a.init && base != 0u) {
         // from |0...0>, the pass's gates mix amplitudes within a tile only,
         // so every tile but the one at base 0 stays zero: write it out as
         // zeros (psi, and lambda = O psi = 0 when the reverse sweep is fused)
         // without its gates; nothing in shared memory is touched
         if (store || (LAST && GRAD))
-          for (uint32_t j = threadIdx.x; j < nloc; j += blockDim.x) {
-            const uint32_t x = gidx(s, base, j, t.L);
+          every([&](uint32_t, uint32_t x) {
             gpsi[x] = {0.f, 0.f};
             if (LAST && GRAD) glam[x] = {0.f, 0.f};
-          }
+          });
         continue;
       }
       if (FIRST) {
         if (a.init) {
           const c2* p0 = a.init + b * a.init_stride;
-          for (uint32_t j = threadIdx.x; j < nloc; j += blockDim.x) sc.psi[swz(j)] = p0[gidx(s, base, j, t.L)];
+          every([&](uint32_t j, uint32_t x) { sc.psi[j] = quarter_turns(p0[x], a.quarter); });
         } else {
-          for (uint32_t j = threadIdx.x; j < nloc; j += blockDim.x)
-            sc.psi[swz(j)] = {(base == 0u && j == 0u) ? 1.f : 0.f, 0.f};
+          every([&](uint32_t j, uint32_t x) { sc.psi[j] = quarter_turns({x == 0u ? 1.f : 0.f, 0.f}, a.quarter); });
         }
       } else if (t.dbl) {
         sc.psi = (it & 1) ? s.psi2 : s.psi;
         if (tile + 1 < tile1) {  // the buffer of the previous tile is free (barrier at the loop end)
-          k1_issue((it & 1) ? s.psi : s.psi2, gpsi, s, deposit((uint32_t)(tile + 1), other), t.k, t.L);
+          k1_issue<NT, Prog>((it & 1) ? s.psi : s.psi2, gpsi, t, s, deposit((uint32_t)(tile + 1), other), !a.init);
           cp_async_commit();
           cp_async_wait<1>();
         } else {
           cp_async_wait<0>();
         }
       } else {  // one buffer: load, then compute
-        k1_issue(s.psi, gpsi, s, base, t.k, t.L);
+        k1_issue<NT, Prog>(s.psi, gpsi, t, s, base, !a.init);
         cp_async_commit();
         cp_async_wait<0>();
       }
       __syncthreads();
       Prog::forward(t, sc, base);
+      auto store_both = [&] {  // nothing reads them after the first pass's reverse sweep
+        if (FIRST && Prog::kSpecialised) return;
+        every([&](uint32_t j, uint32_t x) {
+          if (Prog::kSecond && !a.init && !Prog::in_first(x)) return;
+          gpsi[x] = sc.psi[j];
+          glam[x] = sc.lam[j];
+        });
+      };
       if (LAST && GRAD && a.output == TDQ_OUT_EXPVAL && a.n_groups == 1) {
         // one output group: its diagonal weight d(x) gives both the value
         // (sum |psi|^2 d) and lambda = w d psi in one pass over the tile
         const float w = a.gw ? (float)a.gw[b] : 1.f;
         float acc = 0.f;
-        for (uint32_t j = threadIdx.x; j < nloc; j += blockDim.x) {
-          const float d = obs_weight(a, 0, gidx(s, base, j, t.L));
-          const c2 v = sc.psi[swz(j)];
+        every([&](uint32_t j, uint32_t x) {
+          const float d = obs_weight(a, 0, x);
+          const c2 v = sc.psi[j];
           acc += (v.x * v.x + v.y * v.y) * d;
-          sc.lam[swz(j)] = {w * d * v.x, w * d * v.y};
-        }
+          sc.lam[j] = {w * d * v.x, w * d * v.y};
+        });
         acc = warp_sum_f(acc);
         if ((threadIdx.x & 31) == 0) atomicAdd(&s.vsum[0], (double)acc);
         __syncthreads();
         Prog::reverse(t, sc, base);
-        for (uint32_t j = threadIdx.x; j < nloc; j += blockDim.x) {
-          const uint32_t x = gidx(s, base, j, t.L);
-          gpsi[x] = sc.psi[swz(j)];
-          glam[x] = sc.lam[swz(j)];
-        }
+        store_both();
       } else if (LAST && a.output == TDQ_OUT_EXPVAL) {
         for (int g = 0; g < a.n_groups; g++) {
           float acc = 0.f;
-          for (uint32_t j = threadIdx.x; j < nloc; j += blockDim.x) {
-            const c2 v = sc.psi[swz(j)];
-            acc += (v.x * v.x + v.y * v.y) * obs_weight(a, g, gidx(s, base, j, t.L));
-          }
+          every([&](uint32_t j, uint32_t x) {
+            const c2 v = sc.psi[j];
+            acc += (v.x * v.x + v.y * v.y) * obs_weight(a, g, x);
+          });
           acc = warp_sum_f(acc);
           if ((threadIdx.x & 31) == 0) atomicAdd(&s.vsum[g], (double)acc);
         }
         if (GRAD) {
-          for (uint32_t j = threadIdx.x; j < nloc; j += blockDim.x) {
-            const uint32_t x = gidx(s, base, j, t.L);
+          every([&](uint32_t j, uint32_t x) {
             float d = 0.f;
             for (int g = 0; g < a.n_groups; g++) {
               const float w = a.gw ? (float)a.gw[b * a.n_groups + g] : 1.f;
               d += w * obs_weight(a, g, x);
             }
-            const c2 v = sc.psi[swz(j)];
-            sc.lam[swz(j)] = {d * v.x, d * v.y};
-          }
+            const c2 v = sc.psi[j];
+            sc.lam[j] = {d * v.x, d * v.y};
+          });
           __syncthreads();
           Prog::reverse(t, sc, base);
-          for (uint32_t j = threadIdx.x; j < nloc; j += blockDim.x) {
-            const uint32_t x = gidx(s, base, j, t.L);
-            gpsi[x] = sc.psi[swz(j)];
-            glam[x] = sc.lam[swz(j)];
-          }
+          store_both();
         }
       }
-      if (!(LAST && GRAD) && store) {
-        for (uint32_t j = threadIdx.x; j < nloc; j += blockDim.x) gpsi[gidx(s, base, j, t.L)] = sc.psi[swz(j)];
-      }
+      if (!(LAST && GRAD) && store) every([&](uint32_t j, uint32_t x) { gpsi[x] = sc.psi[j]; });
       __syncthreads();
     }
     if (LAST && a.output == TDQ_OUT_EXPVAL) {
@@ -313,27 +346,27 @@ __device__ __forceinline__ void k1_forward_body(const SweepArgs& a, const TiledD
 
 // Reverse pass over the tiles of one pass (passes before the last); psi and
 // lambda of the next tile are read while the current one is computed.
-template <class Prog>
+template <int NT, class Prog>
 __device__ __forceinline__ void k1_reverse_body(const SweepArgs& a, const TiledDev& t) {
   extern __shared__ __align__(16) unsigned char raw[];
   const int nb = t.dbl ? 2 : 1;
-  const TileShared s = carve(raw, t.k, t.L, nb, nb, t.nrec, t.ndops, a.n_groups, t.gbytes);
-  const uint32_t nloc = 1u << t.k;
+  const TileShared s = carve(raw, t.k, t.L, nb, nb, k1_mat_bytes<Prog>(t), t.ndops, a.n_groups, t.gbytes);
   const uint32_t dim = 1u << t.n;
   const uint32_t other = (dim - 1u) & ~t.smask;
   k1_for_segments(t, [&](int lr, int tile0, int tile1) {
     const int row = t.row0 + lr;
     const int64_t b = row / a.ps_copies;
     int bad = 0;
-    k1_setup(a, t, s, b, 0, &bad);
+    k1_setup<Prog>(a, t, s, b, 0, &bad);
     c2* gpsi = t.psi + (size_t)lr * dim;
     c2* glam = t.lam + (size_t)lr * dim;
-    if (t.dbl && tile0 < tile1) {
-      const uint32_t base0 = deposit((uint32_t)tile0, other);
-      k1_issue(s.psi, gpsi, s, base0, t.k, t.L);
-      k1_issue(s.lam, glam, s, base0, t.k, t.L);
+    auto issue = [&](c2* psi, c2* lam, int tile) {
+      const uint32_t base = deposit((uint32_t)tile, other);
+      k1_issue<NT, Prog>(psi, gpsi, t, s, base);
+      k1_issue<NT, Prog>(lam, glam, t, s, base);
       cp_async_commit();
-    }
+    };
+    if (t.dbl && tile0 < tile1) issue(s.psi, s.lam, tile0);
     for (int tile = tile0, it = 0; tile < tile1; tile++, it++) {
       const uint32_t base = deposit((uint32_t)tile, other);
       TileShared sc = s;
@@ -341,27 +374,23 @@ __device__ __forceinline__ void k1_reverse_body(const SweepArgs& a, const TiledD
         sc.psi = (it & 1) ? s.psi2 : s.psi;
         sc.lam = (it & 1) ? s.lam2 : s.lam;
         if (tile + 1 < tile1) {
-          const uint32_t nxt = deposit((uint32_t)(tile + 1), other);
-          k1_issue((it & 1) ? s.psi : s.psi2, gpsi, s, nxt, t.k, t.L);
-          k1_issue((it & 1) ? s.lam : s.lam2, glam, s, nxt, t.k, t.L);
-          cp_async_commit();
+          issue((it & 1) ? s.psi : s.psi2, (it & 1) ? s.lam : s.lam2, tile + 1);
           cp_async_wait<1>();
         } else {
           cp_async_wait<0>();
         }
       } else {  // one buffer per state: load, then compute
-        k1_issue(s.psi, gpsi, s, base, t.k, t.L);
-        k1_issue(s.lam, glam, s, base, t.k, t.L);
-        cp_async_commit();
+        issue(s.psi, s.lam, tile);
         cp_async_wait<0>();
       }
       __syncthreads();
       Prog::reverse(t, sc, base);
-      for (uint32_t j = threadIdx.x; j < nloc; j += blockDim.x) {
-        const uint32_t x = gidx(s, base, j, t.L);
-        gpsi[x] = sc.psi[swz(j)];
-        glam[x] = sc.lam[swz(j)];
-      }
+      if (!Prog::kFirst)
+        Prog::template every<NT>(t, s, base, [&](uint32_t j, uint32_t x) {
+          if (Prog::kSecond && !a.init && !Prog::in_first(x)) return;
+          gpsi[x] = sc.psi[j];
+          glam[x] = sc.lam[j];
+        });
       __syncthreads();
     }
     Prog::flush(a, t, s, lr);

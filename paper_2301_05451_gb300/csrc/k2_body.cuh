@@ -16,6 +16,7 @@ namespace tdq {
 // FP64 shared-memory sums, one per parameter column.
 struct InterpProg {
   static constexpr bool kSpecialised = false;
+  using Mat = OpMat;
   const RegPass* passes;
   int npf, npb;
   const DOp* dops;  // in shared memory
@@ -58,7 +59,8 @@ __device__ __forceinline__ void k2_body(const SweepArgs& a, Prog prog, const DOp
   const int dim = 1 << a.n;
   c2* psi = reinterpret_cast<c2*>(smem_raw);
   c2* lam = psi + dim;
-  OpMat* mats = reinterpret_cast<OpMat*>(psi + (GRAD ? 2 : 1) * dim);
+  using Mat = typename Prog::Mat;
+  Mat* mats = reinterpret_cast<Mat*>(psi + (GRAD ? 2 : 1) * dim);
   DOp* dops = reinterpret_cast<DOp*>(mats + nrec);
   unsigned char* gbase = reinterpret_cast<unsigned char*>(dops + ndops);
   const size_t gbytes = GRAD ? k2_grad_bytes(Prog::kSpecialised, a.P, blockDim.x) : 0;
@@ -74,14 +76,17 @@ __device__ __forceinline__ void k2_body(const SweepArgs& a, Prog prog, const DOp
   __syncthreads();
   // K0: this row's gate tensors (fused products for the forward program)
   int bad = 0;
-  for (int i = tid; i < nrec; i += nt) mats[i] = build_recipe(a, a.ops, rec_ptr, rec_ops, i, b, k, &bad);
+  if constexpr (Prog::kSpecialised)
+    build_coefs(a, a.ops, rec_ptr, rec_ops, 0, nrec, mats, b, k, &bad);
+  else
+    for (int i = tid; i < nrec; i += nt) mats[i] = build_recipe(a, a.ops, rec_ptr, rec_ops, i, b, k, &bad);
   for (int i = tid; i < ndops; i += nt) dops[i] = gdops[i];
   if (bad) atomicOr(sbad, 1);
   if (a.init) {
     const c2* p0 = a.init + b * a.init_stride;
-    for (int x = tid; x < dim; x += nt) psi[swz(x)] = p0[x];
+    for (int x = tid; x < dim; x += nt) psi[swz(x)] = quarter_turns(p0[x], a.quarter);
   } else {
-    for (int x = tid; x < dim; x += nt) psi[swz(x)] = {x == 0 ? 1.f : 0.f, 0.f};
+    for (int x = tid; x < dim; x += nt) psi[swz(x)] = quarter_turns({x == 0 ? 1.f : 0.f, 0.f}, a.quarter);
   }
   if (GRAD) {
     if (Prog::kSpecialised)
@@ -124,13 +129,13 @@ __device__ __forceinline__ void k2_body(const SweepArgs& a, Prog prog, const DOp
     }
   } else if (k == 0 && a.output == TDQ_OUT_STATE) {
     for (int x = tid; x < dim; x += nt) {
-      const c2 v = psi[swz(x)];
+      const c2 v = psi[swz(lin_index(a, (uint32_t)x))];
       a.values[(b * dim + x) * 2] = v.x;
       a.values[(b * dim + x) * 2 + 1] = v.y;
     }
   } else if (k == 0 && a.output == TDQ_OUT_PROBS) {
     for (int x = tid; x < dim; x += nt) {
-      const c2 v = psi[swz(x)];
+      const c2 v = psi[swz(lin_index(a, (uint32_t)x))];
       a.values[b * dim + x] = (double)v.x * v.x + (double)v.y * v.y;
     }
   }

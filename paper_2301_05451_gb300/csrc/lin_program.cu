@@ -1,0 +1,269 @@
+// Scheduling of gate programs in a linear frame (see lin_program.h).
+#include "lin_program.h"
+
+#include <algorithm>
+
+namespace tdq {
+
+void LinSpace::add(uint32_t m) {
+  m = reduce(m);
+  int p = 31;
+  while (!((m >> p) & 1u)) p--;
+  for (uint32_t& w : v)
+    if ((w >> p) & 1u) w ^= m;
+  v.push_back(m);
+  pivot.push_back(p);
+}
+
+std::vector<LinOp> lin_ops(const std::vector<SweepOp>& ops, int n, LinMap* map) {
+  LinMap& A = *map;
+  A.n = n;
+  A.row.assign(n, 0);
+  A.col.assign(n, 0);
+  A.b = 0;
+  A.quarter = 0;
+  for (int q = 0; q < n; q++) A.row[q] = A.col[q] = 1u << q;
+  std::vector<LinOp> out;
+  auto put = [&](LinKind kind, int q, int op, int ang, int slot, bool p) {
+    LinOp o{};
+    o.kind = kind;
+    o.m = kind == L_RY || kind == L_RX || kind == L_H ? A.col[q] : 0u;
+    o.f = A.row[q];
+    o.b = (uint8_t)((A.b >> q) & 1u);
+    o.p = p;
+    o.op = op;
+    o.ang = ang;
+    o.slot = slot;
+    out.push_back(o);
+  };
+  for (int i = 0; i < (int)ops.size(); i++) {
+    const SweepOp& g = ops[i];
+    switch (g.kind) {
+      case K_CNOT:
+        A.row[g.p1] ^= A.row[g.p0];
+        A.b ^= ((A.b >> g.p0) & 1u) << g.p1;
+        A.col[g.p0] ^= A.col[g.p1];
+        break;
+      case K_X: A.b ^= 1u << g.p0; break;
+      case K_Y:  // Y = i X Z
+        put(L_SIGN, g.p0, -1, 0, -1, false);
+        A.b ^= 1u << g.p0;
+        A.quarter = (A.quarter + 1) & 3;
+        break;
+      case K_Z: put(L_SIGN, g.p0, -1, 0, -1, false); break;
+      case K_H: put(L_H, g.p0, -1, 0, -1, false); break;
+      case K_RX: put(L_RX, g.p0, i, 0, g.slot[0], false); break;
+      case K_RY: put(L_RY, g.p0, i, 0, g.slot[0], false); break;
+      case K_RZ: put(L_PHASE, g.p0, i, 0, g.slot[0], false); break;
+      case K_U3:
+        put(L_PHASE, g.p0, i, 2, g.slot[2], true);
+        put(L_RY, g.p0, i, 0, g.slot[0], false);
+        put(L_PHASE, g.p0, i, 1, g.slot[1], true);
+        break;
+      case K_RZZ:  // a phase by the parity of the two bits
+        put(L_PHASE, g.p0, i, 0, g.slot[0], false);
+        out.back().f ^= A.row[g.p1];
+        out.back().b ^= (uint8_t)((A.b >> g.p1) & 1u);
+        break;
+      default:  // K_CZ
+        put(L_CZ, g.p0, -1, 0, -1, false);
+        out.back().f2 = A.row[g.p1];
+        out.back().b2 = (uint8_t)((A.b >> g.p1) & 1u);
+    }
+  }
+  return out;
+}
+
+// Pauli products (x mask, z parity) that generate an op; at most two.
+static int generators(const LinOp& o, uint32_t (&x)[2], uint32_t (&z)[2]) {
+  switch (o.kind) {
+    case L_RY: x[0] = o.m; z[0] = o.f; return 1;
+    case L_RX: x[0] = o.m; z[0] = 0; return 1;
+    case L_H: x[0] = o.m; z[0] = 0; x[1] = 0; z[1] = o.f; return 2;
+    case L_CZ: x[0] = x[1] = 0; z[0] = o.f; z[1] = o.f2; return 2;
+    default: x[0] = 0; z[0] = o.f; return 1;
+  }
+}
+
+bool lin_commute(const LinOp& a, const LinOp& b) {
+  uint32_t ax[2], az[2], bx[2], bz[2];
+  const int na = generators(a, ax, az), nb = generators(b, bx, bz);
+  for (int i = 0; i < na; i++)
+    for (int j = 0; j < nb; j++)
+      if (parity32(ax[i] & bz[j]) ^ parity32(az[i] & bx[j])) return false;
+  return true;
+}
+
+namespace {
+
+// Takes ops of `todo` (program order) whose masks fit a space of at most dim
+// vectors grown from `space`; an op may pass earlier ones left behind that it
+// commutes with.  mask(o): the op's mask in the space's coordinates.
+// max_slots > 0 caps the gradient slots taken (the first op always fits).
+template <class Mask>
+void take(const std::vector<LinOp>& ops, std::vector<int>& todo, int dim, LinSpace& space, int max_slots, Mask mask,
+          std::vector<int>* taken) {
+  std::vector<int> left;
+  int ns = 0;
+  for (int o : todo) {
+    bool ok = true;
+    for (size_t i = 0; i < left.size() && ok; i++) ok = lin_commute(ops[o], ops[left[i]]);
+    const int s = ops[o].slot >= 0 ? 1 : 0;
+    if (ok && max_slots > 0 && !taken->empty() && ns + s > max_slots) ok = false;
+    if (ok && ops[o].m) {
+      const uint32_t m = mask(ops[o].m);
+      if (space.reduce(m)) {
+        if ((int)space.v.size() < dim) space.add(m);
+        else ok = false;
+      }
+    }
+    if (ok) {
+      taken->push_back(o);
+      ns += s;
+    } else {
+      left.push_back(o);
+    }
+  }
+  todo.swap(left);
+}
+
+// Register passes over the tile's ops.  A pass's group index bits are sent to
+// the local bits outside U's pivots so that 16 consecutive groups read 16
+// different shared-memory slots (see swz: local bit p moves slot bit p mod 4
+// for p < 12), as far as the free bits allow.
+std::vector<LinReg> reg_passes(const std::vector<LinOp>& ops, const LinTile& t, const LinSpace& V, int mreg,
+                               int max_slots) {
+  std::vector<LinReg> out;
+  const int M = std::min(mreg, t.k);
+  auto local = [&](uint32_t m) {  // coordinates of m in the tile's basis
+    uint32_t l = 0;
+    for (int i = 0; i < t.k; i++)
+      if ((m >> V.pivot[i]) & 1u) l |= 1u << i;
+    return l;
+  };
+  std::vector<int> todo = t.ops;
+  while (!todo.empty()) {
+    LinReg r;
+    r.M = M;
+    LinSpace U;
+    take(ops, todo, M, U, max_slots, local, &r.ops);
+    for (int l = 0; l < t.k && (int)U.v.size() < M; l++)
+      if (U.reduce(1u << l)) U.add(1u << l);
+    // order by pivot; the pivots are free to choose: prefer those that leave
+    // every slot bit a local bit outside them
+    for (int i = 0; i < M; i++) r.u[i] = U.v[i];
+    uint32_t piv = U.pivots();
+    int best = -1;
+    std::vector<int> choice(M), pick(M);
+    // all pivot sets (one local bit per basis vector, re-reduced) are tried
+    // greedily: move a pivot to another set bit of its vector when that frees
+    // a slot bit no free local bit reaches
+    auto reach = [&](uint32_t p) {
+      int c = 0;
+      for (int b = 0; b < 4; b++) {
+        bool any = false;
+        for (int l = b; l < std::min(t.k, 12); l += 4) any = any || !((p >> l) & 1u);
+        c += any ? 1 : 0;
+      }
+      return c;
+    };
+    best = reach(piv);
+    for (int round = 0; round < M && best < 4; round++)
+      for (int i = 0; i < M && best < 4; i++)
+        for (int l = 0; l < t.k; l++) {
+          if (!((U.v[i] >> l) & 1u) || l == U.pivot[i]) continue;
+          const uint32_t p2 = (piv & ~(1u << U.pivot[i])) | (1u << l);
+          if (reach(p2) <= best) continue;
+          for (int j = 0; j < M; j++)
+            if (j != i && ((U.v[j] >> l) & 1u)) U.v[j] ^= U.v[i];
+          U.pivot[i] = l;
+          piv = p2;
+          best = reach(p2);
+          break;
+        }
+    for (int i = 0; i < M; i++) r.u[i] = U.v[i];
+    std::vector<int> free_pos;
+    for (int l = 0; l < t.k; l++)
+      if (!((piv >> l) & 1u)) free_pos.push_back(l);
+    // the first four group bits: free local bits of different slot bits
+    std::vector<char> used(free_pos.size(), 0);
+    uint32_t slots = 0;
+    for (size_t i = 0; i < free_pos.size() && r.grp_pos.size() < 4; i++)
+      if (free_pos[i] < 12 && !((slots >> (free_pos[i] & 3)) & 1u)) {
+        slots |= 1u << (free_pos[i] & 3);
+        used[i] = 1;
+        r.grp_pos.push_back(free_pos[i]);
+      }
+    for (size_t i = 0; i < free_pos.size(); i++)
+      if (!used[i]) r.grp_pos.push_back(free_pos[i]);
+    out.push_back(r);
+  }
+  return out;
+}
+
+}  // namespace
+
+LinProgram lin_program(const std::vector<SweepOp>& gates, int n, int k, int L, int mf, int mr, bool adj, bool exact) {
+  LinProgram P;
+  P.n = n;
+  P.exact = exact;
+  P.ops = lin_ops(gates, n, &P.map);
+  P.coef.assign(P.ops.size(), -1);
+  std::vector<int> todo;
+  for (int i = 0; i < (int)P.ops.size(); i++) todo.push_back(i);
+  do {
+    LinTile t;
+    t.k = k;
+    LinSpace V;
+    for (int i = 0; i < L; i++) V.add(1u << i);
+    // a tile pass keeps at most kTileSlots gradient accumulators in shared memory
+    constexpr int kTileSlots = 512;
+    take(P.ops, todo, k, V, kTileSlots, [](uint32_t m) { return m; }, &t.ops);
+    for (int p = 0; p < n && (int)V.v.size() < k; p++)
+      if (V.reduce(1u << p)) V.add(1u << p);
+    // local bits in the order of their pivots (the L lowest first)
+    std::vector<int> order(k);
+    for (int i = 0; i < k; i++) order[i] = i;
+    std::sort(order.begin(), order.end(), [&](int a, int b) { return V.pivot[a] < V.pivot[b]; });
+    LinSpace W;
+    for (int i : order) {
+      W.v.push_back(V.v[i]);
+      W.pivot.push_back(V.pivot[i]);
+    }
+    t.v = W.v;
+    t.pivots = W.pivots();
+    t.fwd = reg_passes(P.ops, t, W, mf, 0);
+    if (adj) t.rev = reg_passes(P.ops, t, W, mr, kRevPassSlots);
+    // the gate-tensor table: one row per angle, one per register pass with
+    // unscaled gates
+    auto row = [&](int type) {
+      t.rec_ops.push_back(type);
+      return (int)t.rec_ptr.size() - 1;
+    };
+    for (int o : t.ops) {
+      const LinOp& g = P.ops[o];
+      if (g.kind != L_RY && g.kind != L_RX && g.kind != L_PHASE) continue;
+      P.coef[o] = row(g.kind == L_PHASE ? C_PHASE : C_ROT);
+      t.rec_ops.push_back(4 * g.op + g.ang);
+      t.rec_ptr.push_back((int)t.rec_ops.size());
+    }
+    for (std::vector<LinReg>* rs : {&t.fwd, &t.rev})
+      for (LinReg& r : *rs) {
+        int nh = 0, nd = 0;
+        for (int o : r.ops) {
+          nh += P.ops[o].kind == L_H ? 1 : 0;
+          nd += P.ops[o].m ? 1 : 0;
+        }
+        if (!nd) continue;
+        r.norm = row((exact ? C_NORM_EXACT : C_NORM) + (nh << 8));
+        for (int o : r.ops)
+          if (P.ops[o].kind == L_RY || P.ops[o].kind == L_RX)
+            t.rec_ops.push_back(2 * P.coef[o] + (P.ops[o].kind == L_RX ? 1 : 0));
+        t.rec_ptr.push_back((int)t.rec_ops.size());
+      }
+    P.tiles.push_back(t);
+  } while (!todo.empty());
+  return P;
+}
+
+}  // namespace tdq

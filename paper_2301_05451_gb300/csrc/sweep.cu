@@ -196,6 +196,8 @@ struct SweepExec final : tdq_exec {
   int* d_slot_ang = nullptr;
   double* d_ps_F = nullptr;
   RegPass* d_passes = nullptr;
+  uint32_t* d_lin = nullptr;  // whole-state specialised programs: SweepArgs::lin
+  int quarter = 0;
   float* d_odiag = nullptr;  // observable diagonal per group [ng][2^n] (whole state; tiled when small)
   DOp* d_dops = nullptr;
   int* d_rec_ptr = nullptr;
@@ -220,6 +222,7 @@ struct SweepExec final : tdq_exec {
     cudaFree(d_ps_F);
     cudaFree(d_passes);
     cudaFree(d_odiag);
+    cudaFree(d_lin);
     cudaFree(d_dops);
     cudaFree(d_rec_ptr);
     cudaFree(d_rec_ops);
@@ -246,6 +249,8 @@ struct SweepExec final : tdq_exec {
     a.values = values; a.gw = gw; a.grads = grads; a.P = P; a.status = d_status;
     a.ps_copies = copies; a.ps_gate = d_ps_gate; a.ps_ang = d_ps_ang; a.ps_F = d_ps_F;
     a.odiag = d_odiag;
+    a.lin = d_lin;
+    a.quarter = quarter;
     a.init = init;
     a.init_stride = init_stride;
     last_launches = 0;
@@ -479,27 +484,25 @@ static double out_bytes_row(int output, int n, int A, int ng) {
 // the program).
 static int k2_threads(int n, int M) { return std::max(32, std::min(256, (1 << n) >> M)); }
 
-// Source of the specialised whole-state kernel of circuit c (adjoint: with
-// the reverse program).
-static void k2_program(const tdq_circuit* c, bool adj, int fb, int rb, Program& prog, int* npf, int* npb,
-                       bool peel) {
+// The whole-state program of circuit c in a linear frame (adj: with its
+// reverse passes; peel: without the Clifford tail, for expectation outputs,
+// which do not need the global phase either).
+static LinProgram k2_program(const tdq_circuit* c, bool adj, int fb, int rb, bool peel) {
   std::vector<int> psg, psa;
   const std::vector<int> tail = peel ? clifford_tail(c) : std::vector<int>();
-  const std::vector<SweepOp> ops = sweep_ops(c, &psg, &psa, &tail);
-  int8_t loc[32];
-  for (int p = 0; p < 32; p++) loc[p] = (int8_t)(p < c->n ? p : -1);
-  build_program(ops, 0, (int)ops.size(), loc, c->n, true, 0, fb, prog);
-  *npf = (int)prog.passes.size();
-  if (adj) build_program(ops, 0, (int)ops.size(), loc, c->n, false, 0, rb, prog);
-  *npb = (int)prog.passes.size() - *npf;
+  return lin_program(sweep_ops(c, &psg, &psa, &tail), c->n, c->n, 0, fb, rb, adj, !peel);
 }
 
-static std::string k2_source(const tdq_circuit* c, bool adj, int fb, int rb, Program& prog, int* npf, int* npb,
-                             bool peel) {
-  k2_program(c, adj, fb, rb, prog, npf, npb, peel);
-  const int M = std::min(fb, c->n);
-  return k2_specialised_source(prog, *npf, *npb, M, std::min(rb, c->n), k2_threads(c->n, M),
-                               c->n_params, c->n, "tdq_k2_specialised");
+// Observable terms and amplitude requests in the frame of a linear program:
+// the parity of x over a term's bits is a parity of y, up to a sign.
+static void terms_to_frame(const LinMap& map, std::vector<TermDev>& terms) {
+  for (TermDev& t : terms) {
+    uint32_t m = 0;
+    for (int q = 0; q < map.n; q++)
+      if ((t.pmask_lo >> q) & 1u) m ^= map.row[q];
+    if (__builtin_popcount(t.pmask_lo & map.b) & 1) t.coeff = -t.coeff;
+    t.pmask_lo = m;
+  }
 }
 
 // Part of a multi-circuit launch: the circuit's tables only (its program is
@@ -590,9 +593,7 @@ static tdq_status compile_sweep_impl(const tdq_circuit* c, const tdq_compile_opt
   }
   tdq_status s;
   if ((s = upload(&e->d_ops, ops)) != TDQ_OK) return bail(s);
-  if ((s = upload(&e->d_terms, terms)) != TDQ_OK) return bail(s);
   if ((s = upload(&e->d_group_ptr, gptr)) != TDQ_OK) return bail(s);
-  if ((s = upload(&e->d_amp, amp)) != TDQ_OK) return bail(s);
   if (cudaMalloc(&e->d_status, sizeof(int)) != cudaSuccess) return bail(fail(TDQ_ERR_OOM, "status word"));
   cudaMemset(e->d_status, 0, sizeof(int));
 
@@ -635,102 +636,99 @@ static tdq_status compile_sweep_impl(const tdq_circuit* c, const tdq_compile_opt
   e->smem_path = c->n <= smem_max_n;
   e->flops_row = sweep_flops(c, adj, tail);
   if (o->grad == TDQ_GRAD_PARAM_SHIFT) e->flops_row *= e->copies;
+  // the generic kernels' program, and the specialised one in a linear frame;
+  // terms and amplitudes follow whichever runs
   Program prog;
-  if (e->smem_path) {
-    int8_t loc[32];
-    for (int p = 0; p < 32; p++) loc[p] = (int8_t)(p < c->n ? p : -1);
-    build_program(ops, 0, (int)ops.size(), loc, c->n, true, 0, fb, prog);
-    e->npf = (int)prog.passes.size();
-    if (adj) build_program(ops, 0, (int)ops.size(), loc, c->n, false, 0, rb, prog);
-    e->npb = (int)prog.passes.size() - e->npf;
-    e->ndops = (int)prog.dops.size();
-    e->nrec = (int)prog.rec_ptr.size() - 1;
-    const size_t dim = (size_t)1 << c->n;
-    e->smem_bytes = dim * sizeof(c2) * (adj ? 2 : 1) + sizeof(OpMat) * e->nrec + sizeof(DOp) * e->ndops +
-                    (adj ? sizeof(double) * e->P : 0) + 32 * sizeof(double) + 16;
-    if (e->smem_bytes > 227 * 1024) e->smem_path = false;
-  }
-  if (hook && !e->smem_path)
-    return bail(fail(TDQ_ERR_UNSUPPORTED, "tdq_compile_multi: a circuit's state does not fit one CTA's shared memory"));
+  LinProgram lin;
+  const bool exact = o->output == TDQ_OUT_STATE || o->output == TDQ_OUT_AMPLITUDE;
+  const size_t dim = (size_t)1 << c->n;
+  bool spec = !o->interpret;
   if (e->smem_path) {
     e->M = std::min(fb, c->n);
     e->threads = hook ? hook->threads : (threads_override > 0 ? threads_override : k2_threads(c->n, e->M));
-    if ((s = upload(&e->d_passes, prog.passes)) != TDQ_OK) return bail(s);
-    if (e->output == TDQ_OUT_EXPVAL) {  // D_g[x] = sum_{t in g} c_t (-1)^{popc(x & mask_t)}
-      const size_t dim = (size_t)1 << c->n;
-      std::vector<float> od((size_t)e->ng * dim);
-      for (int g = 0; g < e->ng; g++)
-        for (size_t x = 0; x < dim; x++) {
-          double d = 0.0;
-          for (int t = gptr[g]; t < gptr[g + 1]; t++)
-            d += (__builtin_popcount((unsigned)x & terms[t].pmask_lo) & 1) ? -(double)terms[t].coeff : (double)terms[t].coeff;
-          od[(size_t)g * dim + x] = (float)d;
-        }
-      if ((s = upload(&e->d_odiag, od)) != TDQ_OK) return bail(s);
-    }
-    if ((s = upload(&e->d_dops, prog.dops)) != TDQ_OK) return bail(s);
-    if ((s = upload(&e->d_rec_ptr, prog.rec_ptr)) != TDQ_OK) return bail(s);
-    if ((s = upload(&e->d_rec_ops, prog.rec_ops)) != TDQ_OK) return bail(s);
-    cudaError_t ce = cudaSuccess;
-    if (!o->interpret) {
-      // specialised program: no decoded ops in shared memory; per-warp FP32
-      // gradient rows instead of FP64 sums
-      const size_t dim = (size_t)1 << c->n;
+    // specialised: the state(s), the gate-tensor rows, per-warp FP32 gradient rows
+    size_t sb = 0;
+    if (spec) {
+      lin = lin_program(ops, c->n, c->n, 0, fb, rb, adj, exact);
+      e->nrec = (int)lin.tiles[0].rec_ptr.size() - 1;
       const size_t gb = adj ? k2_grad_bytes(true, e->P, e->threads) : 0;
-      const size_t sb = dim * sizeof(c2) * (adj ? 2 : 1) + sizeof(OpMat) * e->nrec + ((gb + 7) & ~(size_t)7) +
-                        32 * sizeof(double) + 16;
-      if (hook) {  // compiled later with the other circuits of the launch
-        if (sb > 227 * 1024)
-          return bail(fail(TDQ_ERR_UNSUPPORTED, "tdq_compile_multi: a circuit's program does not fit shared memory"));
-        e->smem_bytes = sb;
-        e->kclass = 2;
-        e->bytes_row = 4.0 * e->P + 4.0 * e->F + out_bytes_row(e->output, c->n, e->A, e->ng) + (adj ? 4.0 * e->P : 0);
-        *out = e;
-        return ok();
-      }
-      if (sb <= 227 * 1024) {
-        const std::string src = k2_specialised_source(prog, e->npf, e->npb, e->M, std::min(rb, c->n),
-                                                      e->threads, e->P, c->n, "tdq_k2_specialised");
-        if ((s = jit_kernel(src, "tdq_k2_specialised", &e->spec_kernel)) != TDQ_OK) return bail(s);
-        e->smem_bytes = sb;
-        ce = cudaFuncSetAttribute(e->spec_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb);
-        if (ce != cudaSuccess)
-          return bail(fail(TDQ_ERR_CUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(ce)));
-      }
+      sb = dim * sizeof(c2) * (adj ? 2 : 1) + sizeof(float4) * e->nrec + ((gb + 7) & ~(size_t)7) + 32 * sizeof(double) + 16;
+      if (sb > 227 * 1024) spec = false;
+      else e->smem_bytes = sb;
     }
-    if (!e->spec_kernel && (fb != kFwdRegBits || rb != kRevRegBits)) {
-      // the specialised program did not fit: the generic kernels' program
-      if (o->fwd_reg_bits || o->rev_reg_bits)
-        return bail(fail(TDQ_ERR_UNSUPPORTED, "tdq_compile_sweep: register bits need a specialised program"));
-      prog = Program{};
+    if (!spec) {
+      if (hook)
+        return bail(fail(TDQ_ERR_UNSUPPORTED, "tdq_compile_multi: a circuit's program does not fit shared memory"));
+      // the generic program: decoded ops in shared memory, FP64 gradient sums
+      const int gf = o->interpret ? fb : kFwdRegBits, gr = o->interpret ? rb : kRevRegBits;
       int8_t loc[32];
       for (int p = 0; p < 32; p++) loc[p] = (int8_t)(p < c->n ? p : -1);
-      build_program(ops, 0, (int)ops.size(), loc, c->n, true, 0, kFwdRegBits, prog);
+      build_program(ops, 0, (int)ops.size(), loc, c->n, true, 0, gf, prog);
       e->npf = (int)prog.passes.size();
-      if (adj) build_program(ops, 0, (int)ops.size(), loc, c->n, false, 0, kRevRegBits, prog);
+      if (adj) build_program(ops, 0, (int)ops.size(), loc, c->n, false, 0, gr, prog);
       e->npb = (int)prog.passes.size() - e->npf;
       e->ndops = (int)prog.dops.size();
       e->nrec = (int)prog.rec_ptr.size() - 1;
-      e->M = std::min(kFwdRegBits, c->n);
-      e->threads = k2_threads(c->n, e->M);
-      const size_t dim = (size_t)1 << c->n;
+      e->M = std::min(gf, c->n);
       e->smem_bytes = dim * sizeof(c2) * (adj ? 2 : 1) + sizeof(OpMat) * e->nrec + sizeof(DOp) * e->ndops +
                       (adj ? sizeof(double) * e->P : 0) + 32 * sizeof(double) + 16;
-      cudaFree(e->d_passes);
-      cudaFree(e->d_dops);
-      cudaFree(e->d_rec_ptr);
-      cudaFree(e->d_rec_ops);
-      e->d_passes = nullptr;
-      e->d_dops = nullptr;
-      e->d_rec_ptr = e->d_rec_ops = nullptr;
+      if (e->smem_bytes > 227 * 1024) e->smem_path = false;
+      else if (!o->interpret && (o->fwd_reg_bits || o->rev_reg_bits))
+        return bail(fail(TDQ_ERR_UNSUPPORTED, "tdq_compile_sweep: register bits need a specialised program"));
+      // the generic kernel's launch bound caps its CTA size
+      e->threads = std::min(k2_threads(c->n, e->M), kK2GenericThreads);
+    }
+  }
+  if (!e->smem_path && !o->interpret) {  // the tiled program (its launch shape follows in tiled_compile)
+    spec = true;
+    if ((s = tiled_lin_plan(e->tiled, c, ops, e->B * e->copies, adj, o->tile_qubits, fb1, rb1, exact, lin)) != TDQ_OK)
+      return bail(s);
+  }
+  if (spec) {
+    terms_to_frame(lin.map, terms);
+    for (uint32_t& x : amp) x = lin.map.to_y(x);
+  }
+  if ((s = upload(&e->d_terms, terms)) != TDQ_OK) return bail(s);
+  if ((s = upload(&e->d_amp, amp)) != TDQ_OK) return bail(s);
+  if (hook && !e->smem_path)
+    return bail(fail(TDQ_ERR_UNSUPPORTED, "tdq_compile_multi: a circuit's state does not fit one CTA's shared memory"));
+  // D_g[y] = sum_{t in g} c_t (-1)^{popc(y & mask_t)}: whole states always;
+  // tiled sweeps while the tables stay small enough to live in L2 (at most 64
+  // MiB), read by the last tile pass instead of evaluating every term
+  if (e->output == TDQ_OUT_EXPVAL && (e->smem_path || std::ldexp((double)e->ng * 4.0, c->n) <= 64.0 * 1024 * 1024)) {
+    std::vector<float> od((size_t)e->ng * dim);
+    for (int g = 0; g < e->ng; g++)
+      for (size_t x = 0; x < dim; x++) {
+        double d = 0.0;
+        for (int t = gptr[g]; t < gptr[g + 1]; t++)
+          d += (__builtin_popcount((unsigned)x & terms[t].pmask_lo) & 1) ? -(double)terms[t].coeff : (double)terms[t].coeff;
+        od[(size_t)g * dim + x] = (float)d;
+      }
+    if ((s = upload(&e->d_odiag, od)) != TDQ_OK) return bail(s);
+  }
+  if (e->smem_path) {
+    cudaError_t ce = cudaSuccess;
+    e->kclass = 2;
+    // compulsory HBM bytes per row: parameters, inputs, outputs, gradients
+    e->bytes_row = 4.0 * e->P + 4.0 * e->F + out_bytes_row(e->output, c->n, e->A, e->ng) + (adj ? 4.0 * e->P : 0);
+    if ((s = upload(&e->d_rec_ptr, spec ? lin.tiles[0].rec_ptr : prog.rec_ptr)) != TDQ_OK) return bail(s);
+    if ((s = upload(&e->d_rec_ops, spec ? lin.tiles[0].rec_ops : prog.rec_ops)) != TDQ_OK) return bail(s);
+    if (spec) {
+      std::vector<uint32_t> map = lin.map.col;
+      map.push_back(lin.map.to_y(0));
+      if ((s = upload(&e->d_lin, map)) != TDQ_OK) return bail(s);
+      e->quarter = exact ? lin.map.quarter : 0;
+      if (hook) {  // compiled later with the other circuits of the launch
+        *out = e;
+        return ok();
+      }
+      const std::string src = k2_specialised_source(lin, adj, e->threads, e->P, "tdq_k2_specialised");
+      if ((s = jit_kernel(src, "tdq_k2_specialised", &e->spec_kernel)) != TDQ_OK) return bail(s);
+      ce = cudaFuncSetAttribute(e->spec_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e->smem_bytes);
+    } else {
       if ((s = upload(&e->d_passes, prog.passes)) != TDQ_OK) return bail(s);
       if ((s = upload(&e->d_dops, prog.dops)) != TDQ_OK) return bail(s);
-      if ((s = upload(&e->d_rec_ptr, prog.rec_ptr)) != TDQ_OK) return bail(s);
-      if ((s = upload(&e->d_rec_ops, prog.rec_ops)) != TDQ_OK) return bail(s);
     }
-    // the generic kernel's launch bound caps its CTA size (the specialised
-    // kernel is compiled for e->threads)
-    if (!e->spec_kernel) e->threads = std::min(e->threads, kK2GenericThreads);
 #define TDQ_SETSM(MF, MB, GG) ce = cudaFuncSetAttribute(k2_sweep_smem<MF, MB, GG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e->smem_bytes)
     if (e->spec_kernel) {
     } else if (e->M >= 4) { if (adj) TDQ_SETSM(4, 3, true); else TDQ_SETSM(4, 3, false); }
@@ -739,28 +737,9 @@ static tdq_status compile_sweep_impl(const tdq_circuit* c, const tdq_compile_opt
     else { if (adj) TDQ_SETSM(1, 1, true); else TDQ_SETSM(1, 1, false); }
 #undef TDQ_SETSM
     if (ce != cudaSuccess) return bail(fail(TDQ_ERR_CUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(ce)));
-    e->kclass = 2;
-    // compulsory HBM bytes per row: parameters, inputs, outputs, gradients
-    e->bytes_row = 4.0 * e->P + 4.0 * e->F + out_bytes_row(e->output, c->n, e->A, e->ng) + (adj ? 4.0 * e->P : 0);
   }
   if (!e->smem_path) {
-    // the observable's diagonal per output group, read by the last tile pass
-    // instead of evaluating every term per amplitude: kept while the tables
-    // stay small enough to live in L2 (at most 64 MiB)
-    if (e->output == TDQ_OUT_EXPVAL && (std::ldexp((double)e->ng * 4.0, c->n) <= 64.0 * 1024 * 1024)) {
-      const size_t dim = (size_t)1 << c->n;
-      std::vector<float> od((size_t)e->ng * dim);
-      for (int g = 0; g < e->ng; g++)
-        for (size_t x = 0; x < dim; x++) {
-          double d = 0.0;
-          for (int t = gptr[g]; t < gptr[g + 1]; t++)
-            d += (__builtin_popcount((unsigned)x & terms[t].pmask_lo) & 1) ? -(double)terms[t].coeff
-                                                                          : (double)terms[t].coeff;
-          od[(size_t)g * dim + x] = (float)d;
-        }
-      if ((s = upload(&e->d_odiag, od)) != TDQ_OK) return bail(s);
-    }
-    s = tiled_compile(e->tiled, c, ops, ps_gate, e->B * e->copies, adj, o->tile_qubits, o->interpret != 0, fb1, rb1,
+    s = tiled_compile(e->tiled, c, ops, ps_gate, e->B * e->copies, adj, o->tile_qubits, spec ? &lin : nullptr, fb1, rb1,
                       &e->bytes_row);
     if (s != TDQ_OK) return bail(s);
     // outputs: the state read back from HBM and written out as values
@@ -870,12 +849,12 @@ static tdq_status sweep_autotune(const tdq_circuit* c, const tdq_compile_opts* o
       pool.emplace_back([&, k] {
         try {
           if (cudaSetDevice(o->device) != cudaSuccess) return;
-          Program prog;
-          int npf = 0, npb = 0;
-          k2_program(c, adj, k.bits, k.bits, prog, &npf, &npb, o->output == TDQ_OUT_EXPVAL);
-          const std::string src = k2_specialised_source(prog, npf, npb, std::min(k.bits, c->n),
-                                                        std::min(k.bits, c->n), k.threads, c->n_params, c->n,
-                                                        "tdq_k2_specialised");
+          std::vector<int> psg, psa;
+          const std::vector<int> tail = o->output == TDQ_OUT_EXPVAL ? clifford_tail(c) : std::vector<int>();
+          const bool exact = o->output == TDQ_OUT_STATE || o->output == TDQ_OUT_AMPLITUDE;
+          const std::string src = k2_specialised_source(
+              lin_program(sweep_ops(c, &psg, &psa, &tail), c->n, c->n, 0, k.bits, k.bits, adj, exact), adj, k.threads,
+              c->n_params, "tdq_k2_specialised");
           const void* kern = nullptr;
           jit_kernel(src, "tdq_k2_specialised", &kern);  // failures surface again in the build below
         } catch (...) {  // (the build below reports it)
@@ -933,20 +912,20 @@ extern "C" tdq_status tdq_sweep_source(const tdq_circuit* c, int grad, int tile_
   std::string src;
   if (tile_qubits == 0) {
     if (c->n > 14) return fail(TDQ_ERR_UNSUPPORTED, "tdq_sweep_source: more than 14 qubits in one CTA");
-    Program prog;
-    int npf = 0, npb = 0;
-    src = k2_source(c, adj, kSpecFwdRegBits, kSpecRevRegBits, prog, &npf, &npb, c->n_groups > 0);
+    src = k2_specialised_source(k2_program(c, adj, kSpecFwdRegBits, kSpecRevRegBits, c->n_groups > 0), adj,
+                                k2_threads(c->n, std::min(kSpecFwdRegBits, c->n)), c->n_params, "tdq_k2_specialised");
   } else {
     if (c->n > 30) return fail(TDQ_ERR_UNSUPPORTED, "tdq_sweep_source: more than 30 qubits");
     std::vector<int> psg, psa;
     const std::vector<int> tail = c->n_groups > 0 ? clifford_tail(c) : std::vector<int>();
     const std::vector<SweepOp> ops = sweep_ops(c, &psg, &psa, &tail);
     TiledSweep t;
-    TiledHost h;
-    tdq_status s = tiled_plan(t, c, ops, psg, 1, adj, tile_qubits, kTiledSpecFwdRegBits, kTiledSpecRevRegBits, h);
+    LinProgram lin;
+    tdq_status s = tiled_lin_plan(t, c, ops, 1, adj, tile_qubits, kTiledSpecFwdRegBits, kTiledSpecRevRegBits,
+                                  c->n_groups == 0, lin);
     if (s != TDQ_OK) return s;
     std::vector<int> nacc;
-    src = k1_specialised_source(t, h.prog, std::max(32, std::min(256, 1 << (t.k - kTiledSpecFwdRegBits))),
+    src = k1_specialised_source(t, lin, std::max(32, std::min(256, 1 << (t.k - kTiledSpecFwdRegBits))),
                                 std::max(32, std::min(256, 1 << (t.k - kTiledSpecRevRegBits))), &nacc);
   }
   *len = src.size() + 1;
@@ -1101,12 +1080,11 @@ static int multi_maxrreg(int threads) { return std::min(255, 65536 / threads); }
 // autotuner, so that they share one compilation.
 static std::vector<std::string> multi_modules(const tdq_circuit* const* cs, int nc, bool adj, int threads, int fb,
                                               int rb) {
-  std::vector<Program> progs(nc);
+  std::vector<LinProgram> progs(nc);
   std::vector<K2Part> parts;
   for (int c = 0; c < nc; c++) {
-    int npf = 0, npb = 0;
-    k2_program(cs[c], adj, fb, rb, progs[c], &npf, &npb, true);
-    parts.push_back({&progs[c], npf, npb, std::min(fb, cs[c]->n), std::min(rb, cs[c]->n), cs[c]->n_params, cs[c]->n});
+    progs[c] = k2_program(cs[c], adj, fb, rb, true);
+    parts.push_back({&progs[c], cs[c]->n_params});
   }
   return k2_multi_modules(parts, adj, threads, "tdq_k2_multi");
 }
@@ -1160,6 +1138,7 @@ static tdq_status multi_build(const tdq_circuit* const* cs, const int* batch, in
     a.P = x->P; a.status = e->d_status;
     a.ps_copies = x->copies; a.ps_gate = x->d_ps_gate; a.ps_ang = x->d_ps_ang; a.ps_F = x->d_ps_F;
     a.odiag = x->d_odiag;
+    a.lin = x->d_lin;
     m.rec_ptr = x->d_rec_ptr;
     m.rec_ops = x->d_rec_ops;
     m.nrec = x->nrec;

@@ -186,7 +186,30 @@ struct SweepArgs {
   // initial state of row b: init + b * init_stride (NULL: |0...0>)
   const c2* init;
   int64_t init_stride;
+  // programs in a linear frame: entry y of the state holds the basis index x
+  // with y = XOR of lin[q] over the bits q of x, XOR lin[n] (NULL: y = x);
+  // quarter: the state carries i^-quarter
+  const uint32_t* lin;
+  int quarter;
 };
+
+// Rows of the gate-tensor table of a specialised program (build_coef).
+enum : int { C_ROT = 0, C_PHASE = 1, C_NORM = 2, C_NORM_EXACT = 3 };
+
+// Place in the state buffer of basis index x.
+__device__ __forceinline__ uint32_t lin_index(const SweepArgs& a, uint32_t x) {
+  if (!a.lin) return x;
+  uint32_t y = a.lin[a.n];
+  for (int q = 0; q < a.n; q++) y ^= (0u - ((x >> q) & 1u)) & a.lin[q];
+  return y;
+}
+
+// i^q a
+__device__ __forceinline__ c2 quarter_turns(c2 a, int q) {
+  if (q & 1) a = {-a.y, a.x};
+  if (q & 2) a = {-a.x, -a.y};
+  return a;
+}
 
 // One circuit of a multi-circuit launch: its sweep arguments with the
 // per-call pointers left NULL, its gate-tensor recipes, and the offsets

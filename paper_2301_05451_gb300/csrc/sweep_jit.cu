@@ -21,154 +21,555 @@ namespace tdq {
 
 namespace {
 
-// Index bits of one register pass: the group base inserts zeros at the
-// pass's tile bits; member j of a group sits at base ^ off(j) (disjoint bits).
-struct PassBits {
-  int m;
-  int lb[4];
-  uint32_t off(int j) const {
-    uint32_t o = 0;
-    for (int i = 0; i < m; i++)
-      if ((j >> i) & 1) o |= 1u << lb[i];
-    return o;
+uint32_t swz_host(uint32_t x) { return x ^ ((x >> 4) & 15u) ^ ((x >> 8) & 15u); }
+
+// A sign known at compile time up to group-dependent words: the XOR of the
+// words w<i> (top bit) and a constant.
+struct Sign {
+  bool c = false;
+  std::vector<int> w;
+  void flip(const Sign& o) {
+    c ^= o.c;
+    for (int i : o.w) {
+      auto it = std::find(w.begin(), w.end(), i);
+      if (it == w.end()) w.push_back(i);
+      else w.erase(it);
+    }
+  }
+  bool constant() const { return w.empty(); }
+  bool zero() const { return w.empty() && !c; }
+  std::string str() const {
+    std::string s;
+    for (int i : w) s += (s.empty() ? "w" : " ^ w") + std::to_string(i);
+    if (c) s += s.empty() ? "0x80000000u" : " ^ 0x80000000u";
+    return s.empty() ? "0u" : s;
   }
 };
 
-uint32_t swz_host(uint32_t x) { return x ^ ((x >> 4) & 15u); }
-
-PassBits pass_bits(const RegPass& rp) {
-  PassBits b{};
-  b.m = rp.m;
-  for (int i = 0; i < 4; i++) b.lb[i] = rp.lb[i];
-  return b;
-}
-
-// "gb" computed from the group index, then the swizzled base "sb".
-void emit_group_base(std::ostringstream& s, const PassBits& pb) {
-  s << "    uint32_t gb = (uint32_t)grp;\n";
-  for (int i = 0; i < pb.m; i++) s << "    gb = insert0(gb, " << pb.lb[i] << ");\n";
-  s << "    const uint32_t sb = swz(gb);\n";
-}
-
-// Loads (store = false) or stores the group's amplitudes; swz is linear over
-// XOR and the offsets share no bit with gb, so swz(gb | off) = sb ^ swz(off).
-void emit_move(std::ostringstream& s, const PassBits& pb, const char* arr, const char* reg, bool store) {
-  for (int j = 0; j < (1 << pb.m); j++) {
-    const uint32_t so = swz_host(pb.off(j));
-    if (store)
-      s << "    " << arr << "[sb ^ " << so << "u] = " << reg << "[" << j << "];\n";
-    else
-      s << "    " << reg << "[" << j << "] = " << arr << "[sb ^ " << so << "u];\n";
-  }
-}
-
-// Value of a bit that is not a register bit: a tile bit of the group base
-// (l >= 0), else global position p of the tile's base index.
-std::string fixed_bit(int l, int p) {
-  std::ostringstream s;
-  if (l >= 0) s << "((gb >> " << l << ") & 1u)";
-  else s << "((base >> " << p << ") & 1u)";
-  return s.str();
-}
-
-bool dense_kind(int k) {
-  return k == K_FUSED || k == K_RX || k == K_RY || k == K_U3 || k == K_H || k == K_X || k == K_Y;
-}
-
-// Forward absorption of one decoded op into the register array `a` (M
-// register bits).
-void emit_fwd_op(std::ostringstream& s, const DOp& d, int M, const char* a) {
-  const int k = d.kind;
-  s << "    {  // kind " << k << "\n";
-  if (dense_kind(k)) {
-    s << "      reg_pair<" << M << ", " << (int)d.r0 << ">(" << a << ", mats[" << d.mat << "].m);\n";
-  } else if (k == K_CNOT) {  // control p0, target p1 (a register bit)
-    if (d.r0 >= 0)
-      s << "      swap_ctrl<" << M << ", " << (int)d.r1 << ", " << (int)d.r0 << ">(" << a << ");\n";
-    else
-      s << "      if (" << fixed_bit(d.l0, d.p0) << ") swap_ctrl<" << M << ", " << (int)d.r1 << ", -1>(" << a << ");\n";
-  } else if (k == K_CZ) {
-    if (d.r0 >= 0 && d.r1 >= 0)
-      s << "      neg_and<" << M << ", " << (int)d.r0 << ", " << (int)d.r1 << ">(" << a << ");\n";
-    else if (d.r0 >= 0 || d.r1 >= 0) {
-      const int r = d.r0 >= 0 ? d.r0 : d.r1, l = d.r0 >= 0 ? d.l1 : d.l0, pp = d.r0 >= 0 ? d.p1 : d.p0;
-      s << "      if (" << fixed_bit(l, pp) << ") neg_and<" << M << ", " << r << ", " << r << ">(" << a << ");\n";
-    } else {
-      s << "      if (" << fixed_bit(d.l0, d.p0) << " & " << fixed_bit(d.l1, d.p1) << ")\n"
-        << "        for (int j = 0; j < " << (1 << M) << "; j++) " << a << "[j] = {-" << a << "[j].x, -" << a
-        << "[j].y};\n";
+// Writes one register pass: the group loop, its loads, gates and stores.
+// Diagonal gates are gathered into blocks (an op may pass others it commutes
+// with): a block multiplies every class of members that its parities tell
+// apart by one product of phases.  The part of the phases that a whole group
+// shares, and the scale that the unscaled rotations left out, are one factor
+// per group, merged into the pass's largest block.  Signs (Z, CZ with one
+// register bit) wait as a frame: a later gate on the bit flips its
+// off-diagonal sign, a phase block absorbs them.
+class PassWriter {
+ public:
+  PassWriter(std::ostringstream& s, const LinProgram& P, const LinTile& t, const LinReg& r, bool rev)
+      : s_(s), P_(P), t_(t), r_(r), rev_(rev), N_(1 << r.M) {
+    for (int pos : r.grp_pos) varying_ |= t.v[pos];
+    const uint32_t all = P.n >= 32 ? ~0u : (1u << P.n) - 1u;
+    varying_ |= all & ~t.pivots;
+    for (int i = 0; i < r.M; i++) {
+      gu_[i] = 0;
+      for (int l = 0; l < t.k; l++)
+        if ((r.u[i] >> l) & 1u) gu_[i] ^= t.v[l];
     }
-  } else {  // diagonal phases: RZ / Z (one bit), RZZ (parity of two bits)
-    const bool two = k == K_RZZ;
-    s << "      c2 d0 = mats[" << d.mat << "].m.m00, d1 = mats[" << d.mat << "].m.m11;\n";
-    std::string fx;
-    if (d.r0 < 0) fx = fixed_bit(d.l0, d.p0);
-    if (two && d.r1 < 0) fx = fx.empty() ? fixed_bit(d.l1, d.p1) : "(" + fx + " ^ " + fixed_bit(d.l1, d.p1) + ")";
-    if (!fx.empty()) s << "      if (" << fx << ") { const c2 t = d0; d0 = d1; d1 = t; }\n";
-    s << "      diag_par<" << M << ", " << (int)d.r0 << ", " << (two ? (int)d.r1 : -1) << ">(" << a
-      << ", d0, d1);\n";
   }
-  s << "    }\n";
-}
 
-// Reverse step of one op on p[], l[]: gradient shares into gs<i> variables.
-void emit_rev_op(std::ostringstream& s, const DOp& d, int M, const std::vector<int>& gvar) {
-  const int k = d.kind;
-  s << "    {  // kind " << k << "\n";
-  auto add = [&](int j, const char* expr) {
-    if (j < d.nang && d.slot[j] >= 0 && gvar[j] >= 0)
-      s << "      gs" << gvar[j] / 32 << "[" << gvar[j] % 32 << "] += " << expr << ";\n";
+  // share(o): where the gradient share of op o goes ("" if nowhere)
+  template <class Share>
+  void write(int nthreads, const std::string& y0, const std::vector<const char*>& arrays,
+             const std::vector<const char*>& regs, Share share) {
+    const int groups = 1 << (t_.k - r_.M);
+    s_ << "  for (int grp = threadIdx.x; grp < " << groups << "; grp += " << nthreads << ") {\n";
+    s_ << "    const uint32_t gb = " << spread() << ";\n    const uint32_t sb = swz(gb);\n    const uint32_t y0 = " << y0
+       << ";\n    (void)y0;\n";
+    regs_ = regs;
+    for (size_t i = 0; i < arrays.size(); i++) move(arrays[i], regs[i], false);
+    plan();
+    prelude();
+    for (size_t i = 0; i < items_.size(); i++) {
+      const std::vector<int>& it = items_[i];
+      if (P_.ops[it[0]].kind == L_PHASE) block(it, (int)i == merge_, share);
+      else gate(it[0], share);
+    }
+    if (merge_ < 0 && group_factor_) {
+      const char* f = complex_factor_ ? "lin_mul" : "lin_scale";
+      for (const char* g : regs)
+        for (int j = 0; j < N_; j++) s_ << "    " << f << "(" << g << j << ", " << (complex_factor_ ? "G" : "G.x") << ");\n";
+    }
+    for (const Frame& f : frame_) flush(f);
+    frame_.clear();
+    for (size_t i = 0; i < arrays.size(); i++) move(arrays[i], regs[i], true);
+    s_ << "  }\n";
+  }
+
+ private:
+  struct Frame {
+    int fr;
+    Sign sign;
   };
-  if (k == K_CNOT || k == K_CZ) {  // self-inverse: the forward action on both states
-    s << "    }\n";
-    emit_fwd_op(s, d, M, "p");
-    emit_fwd_op(s, d, M, "l");
-    return;
-  } else if (!dense_kind(k)) {  // RZ / Z / RZZ
-    const bool two = k == K_RZZ;
-    s << "      c2 d0 = mats[" << d.mat << "].m.m00, d1 = mats[" << d.mat << "].m.m11;\n"
-      << "      d0.y = -d0.y; d1.y = -d1.y;\n";
-    std::string fx;
-    if (d.r0 < 0) fx = fixed_bit(d.l0, d.p0);
-    if (two && d.r1 < 0) fx = fx.empty() ? fixed_bit(d.l1, d.p1) : "(" + fx + " ^ " + fixed_bit(d.l1, d.p1) + ")";
-    if (!fx.empty()) s << "      const bool fx = " << fx << ";\n      if (fx) { const c2 t = d0; d0 = d1; d1 = t; }\n";
-    s << "      float acc = 0.f;\n"
-      << "      diag_par_adj<" << M << ", " << (int)d.r0 << ", " << (two ? (int)d.r1 : -1)
-      << ">(p, l, d0, d1, acc);\n";
-    add(0, fx.empty() ? "acc" : "(fx ? -acc : acc)");
-  } else {
-    s << "      float g[3] = {0.f, 0.f, 0.f};\n"
-      << "      reg_adj_1q<" << M << ", " << (int)d.r0 << ">(p, l, " << k << ", mats[" << d.mat << "], g);\n";
-    add(0, "g[0]");
-    add(1, "g[1]");
-    add(2, "g[2]");
+
+  // local index of the group's first member: group bit i at local bit grp_pos[i]
+  std::string spread() const {
+    std::ostringstream e;
+    const int n = (int)r_.grp_pos.size();
+    if (n == 0) return "0u * (uint32_t)grp";
+    for (int i = 0; i < n;) {
+      int j = i + 1;
+      while (j < n && r_.grp_pos[j] == r_.grp_pos[i] + (j - i)) j++;
+      const uint32_t mask = ((1u << (j - i)) - 1u) << i;
+      const int sh = r_.grp_pos[i] - i;
+      e << (i ? " | " : "") << "(((uint32_t)grp & " << mask << "u) " << (sh >= 0 ? "<< " : ">> ") << (sh >= 0 ? sh : -sh)
+        << ")";
+      i = j;
+    }
+    return e.str();
   }
-  s << "    }\n";
+
+  uint32_t member(int j) const {  // local index of member j from the group's first
+    uint32_t l = 0;
+    for (int i = 0; i < r_.M; i++)
+      if ((j >> i) & 1) l ^= r_.u[i];
+    return l;
+  }
+
+  void move(const char* arr, const char* reg, bool store) {
+    for (int j = 0; j < N_; j++) {
+      const uint32_t so = swz_host(member(j));
+      if (store) s_ << "    " << arr << "[sb ^ " << so << "u] = " << reg << j << ";\n";
+      else s_ << "    c2 " << reg << j << " = " << arr << "[sb ^ " << so << "u];\n";
+    }
+  }
+
+  // the op's parity over the members: bit i the parity of f on vector i
+  int reg_parity(uint32_t f) const {
+    int fr = 0;
+    for (int i = 0; i < r_.M; i++) fr |= parity32(f & gu_[i]) << i;
+    return fr;
+  }
+  int reg_mask(uint32_t m) const {  // members j, j ^ mask pair up under m
+    for (int j = 1; j < N_; j++) {
+      uint32_t g = 0;
+      for (int i = 0; i < r_.M; i++)
+        if ((j >> i) & 1) g ^= gu_[i];
+      if (g == m) return j;
+    }
+    return 0;
+  }
+  // the part of the parity that the group shares
+  Sign group_sign(uint32_t f, int b) {
+    Sign g;
+    g.c = b != 0;
+    bool moves = (f & ~t_.pivots & (P_.n >= 32 ? ~0u : (1u << P_.n) - 1u)) != 0;
+    for (int pos : r_.grp_pos) moves = moves || parity32(f & t_.v[pos]);
+    if (!moves) return g;
+    const uint32_t m = f & varying_;
+    auto it = words_.find(m);
+    if (it == words_.end()) {
+      it = words_.emplace(m, (int)words_.size()).first;
+      s_ << "    const uint32_t w" << it->second << " = ";
+      if ((m & (m - 1u)) == 0) {
+        int p = 0;
+        while (!((m >> p) & 1u)) p++;
+        s_ << "(y0 << " << 31 - p << ") & 0x80000000u;\n";
+      } else {
+        s_ << "(uint32_t)__popc(y0 & " << m << "u) << 31;\n";
+      }
+    }
+    g.w.push_back(it->second);
+    return g;
+  }
+
+  // order of execution: gates as early as they commute ahead, phases gathered
+  void plan() {
+    std::vector<int> todo = r_.ops;
+    if (rev_) std::reverse(todo.begin(), todo.end());
+    items_.clear();
+    while (!todo.empty()) {
+      int pick = -1;
+      for (size_t i = 0; i < todo.size() && pick < 0; i++) {
+        if (P_.ops[todo[i]].kind == L_PHASE) continue;
+        bool ok = true;
+        for (size_t j = 0; j < i && ok; j++) ok = lin_commute(P_.ops[todo[i]], P_.ops[todo[j]]);
+        if (ok) pick = (int)i;
+      }
+      if (pick >= 0) {
+        items_.push_back({todo[pick]});
+        todo.erase(todo.begin() + pick);
+        continue;
+      }
+      std::vector<int> blk, left;
+      for (int o : todo) {
+        bool ok = P_.ops[o].kind == L_PHASE;
+        for (size_t j = 0; j < left.size() && ok; j++) ok = lin_commute(P_.ops[o], P_.ops[left[j]]);
+        (ok ? blk : left).push_back(o);
+      }
+      items_.push_back(blk);
+      todo.swap(left);
+    }
+  }
+
+  std::string mat(int o) const { return "mats[" + std::to_string(P_.coef[o]) + "]"; }
+
+  // sign words of every op, the group factor G (scale, shared phases, shared
+  // signs) and the block it is merged into
+  void prelude() {
+    complex_factor_ = false;
+    bool signs = false;
+    std::vector<std::string> phase, flips;
+    for (int o : r_.ops) {
+      const LinOp& g = P_.ops[o];
+      const Sign a = group_sign(g.f, g.b);
+      if (g.kind == L_PHASE) {
+        // e^{-+i a/2} by the shared sign (conjugate in reverse); constant
+        // ones are a global phase, kept for exact programs only
+        Sign sg = a;
+        sg.c = sg.c == rev_;  // forward, sign 0: (cos, -sin)
+        if (!a.constant() || P_.exact)
+          phase.push_back("    { const float4 q = " + mat(o) + "; G = cmul(G, {q.x, sx(q.y, " + sg.str() + ")}); }\n");
+        if (g.p && P_.exact) phase.push_back("    { const float4 q = " + mat(o) + "; G = cmul(G, {q.x, q.y}); }\n");
+      } else if (g.kind == L_CZ) {
+        const Sign b = group_sign(g.f2, g.b2);
+        if (!a.zero() && !b.zero() && (P_.exact || !a.constant() || !b.constant())) {
+          flips.push_back("    gs ^= (" + a.str() + ") & (" + b.str() + ");\n");
+          signs = true;
+        }
+      } else if (g.kind == L_SIGN) {
+        if (!a.zero() && (P_.exact || !a.constant())) {
+          flips.push_back("    gs ^= " + a.str() + ";\n");
+          signs = true;
+        }
+      }
+    }
+    // unscaled rotations of the u form leave their sign to the group factor;
+    // their words need the frame at that point, so it is walked here first
+    std::vector<Frame> fr;
+    for (const std::vector<int>& it : items_) {
+      const LinOp& g = P_.ops[it[0]];
+      if (g.kind == L_PHASE) {
+        std::vector<int> basis;
+        std::vector<int> frs;
+        for (int o : it) frs.push_back(reg_parity(P_.ops[o].f));
+        absorb(frs, fr, nullptr);
+        continue;
+      }
+      if (!g.m) {
+        add_frames(g, fr);
+        continue;
+      }
+      const int mj = reg_mask(g.m);
+      if (g.kind == L_H) {
+        drop_hit(fr, mj, nullptr);
+        continue;
+      }
+      Sign sg = frame_sign(fr, mj);
+      if (g.kind == L_RY) sg.flip(group_sign(g.f, g.b));
+      if (!sg.zero() && (P_.exact || !sg.constant())) {
+        flips.push_back("    gs ^= __float_as_uint(" + mat(it[0]) + ".w) & (" + sg.str() + ");\n");
+        signs = true;
+      }
+    }
+    merge_ = -1;
+    size_t big = 0;
+    group_factor_ = r_.norm >= 0 || !phase.empty() || signs;
+    if (group_factor_)
+      for (size_t i = 0; i < items_.size(); i++)
+        if (P_.ops[items_[i][0]].kind == L_PHASE && items_[i].size() > big) {
+          big = items_[i].size();
+          merge_ = (int)i;
+        }
+    complex_factor_ = !phase.empty() || P_.exact;
+    if (!group_factor_) return;
+    if (r_.norm >= 0) s_ << "    const float4 nrm = mats[" << r_.norm << "];\n";
+    s_ << "    uint32_t gs = 0u;\n";
+    for (const std::string& f : flips) s_ << f;
+    s_ << "    c2 G = {sx(" << (r_.norm >= 0 ? "nrm.x" : "1.f") << ", gs), "
+       << (r_.norm >= 0 && P_.exact ? "sx(nrm.y, gs)" : "0.f") << "};\n";
+    for (const std::string& f : phase) s_ << f;
+    if (rev_ && r_.norm >= 0) s_ << "    float sc = 1.f;\n";
+  }
+
+  Sign frame_sign(const std::vector<Frame>& fr, int mj) const {
+    Sign s;
+    for (const Frame& f : fr)
+      if (cpar(f.fr & mj)) s.flip(f.sign);
+    return s;
+  }
+
+  static void push_frame(std::vector<Frame>& fr, int bits, const Sign& sign) {
+    if (!bits || sign.zero()) return;
+    for (size_t i = 0; i < fr.size(); i++)
+      if (fr[i].fr == bits) {
+        fr[i].sign.flip(sign);
+        if (fr[i].sign.zero()) fr.erase(fr.begin() + i);
+        return;
+      }
+    fr.push_back({bits, sign});
+  }
+
+  // the frame signs of CZ and SIGN ops (their member-wise product of two
+  // register parities is applied by gate())
+  void add_frames(const LinOp& g, std::vector<Frame>& fr) {
+    const int f0 = reg_parity(g.f);
+    Sign one;
+    one.c = true;
+    if (g.kind == L_SIGN) {
+      push_frame(fr, f0, one);
+      return;
+    }
+    const int f1 = reg_parity(g.f2);
+    push_frame(fr, f0, group_sign(g.f2, g.b2));
+    push_frame(fr, f1, group_sign(g.f, g.b));
+  }
+
+  template <class Emit>
+  static void drop_frames(std::vector<Frame>& fr, const std::vector<char>& drop, Emit emit) {
+    std::vector<Frame> keep;
+    for (size_t i = 0; i < fr.size(); i++) {
+      if (drop[i]) emit(fr[i]);
+      else keep.push_back(fr[i]);
+    }
+    fr.swap(keep);
+  }
+
+  // frames that anticommute with a pairing mask, taken out (applied if `self`)
+  void drop_hit(std::vector<Frame>& fr, int mj, PassWriter* self) {
+    std::vector<char> d;
+    for (const Frame& f : fr) d.push_back((char)cpar(f.fr & mj));
+    drop_frames(fr, d, [&](const Frame& f) {
+      if (self) self->flush(f);
+    });
+  }
+
+  // frames in the span of a block's parities, taken out into `out`
+  static void absorb(const std::vector<int>& frs, std::vector<Frame>& fr, std::vector<Frame>* out) {
+    std::vector<int> basis;
+    for (int f : frs)
+      if (f) add_basis(basis, f);
+    std::vector<char> d;
+    for (const Frame& f : fr) d.push_back((char)(combo(basis, f.fr) >= 0));
+    drop_frames(fr, d, [&](const Frame& f) {
+      if (out) out->push_back(f);
+    });
+  }
+
+  static bool add_basis(std::vector<int>& basis, int f) {
+    if (combo(basis, f) >= 0) return false;
+    basis.push_back(f);
+    return true;
+  }
+  // f as an XOR of basis vectors (bit i: vector i), or -1
+  static int combo(const std::vector<int>& basis, int f) {
+    for (int c = 0; c < (1 << basis.size()); c++) {
+      int x = 0;
+      for (size_t i = 0; i < basis.size(); i++)
+        if ((c >> i) & 1) x ^= basis[i];
+      if (x == f) return c;
+    }
+    return -1;
+  }
+
+  void flush(const Frame& f) {
+    for (const char* g : regs_)
+      for (int j = 0; j < N_; j++)
+        if (cpar(f.fr & j)) s_ << "    lin_neg(" << g << j << ", " << f.sign.str() << ");\n";
+  }
+
+  template <class Share>
+  void gate(int o, Share share) {
+    const LinOp& g = P_.ops[o];
+    if (!g.m) {
+      if (g.kind == L_CZ) {
+        const int f0 = reg_parity(g.f), f1 = reg_parity(g.f2);
+        for (const char* a : regs_)
+          for (int j = 0; j < N_; j++)
+            if (cpar(f0 & j) && cpar(f1 & j)) s_ << "    lin_neg(" << a << j << ", 0x80000000u);\n";
+      }
+      add_frames(g, frame_);
+      return;
+    }
+    const int mj = reg_mask(g.m), fr = reg_parity(g.f);
+    if (g.kind == L_H) {
+      drop_hit(frame_, mj, this);
+      s_ << "    {\n    const float2 hs = bc2(sx(1.f, " << group_sign(g.f, g.b).str() << ")), hn = bc2(-hs.x);\n";
+      for (const char* a : regs_)
+        pairs(mj, fr, [&](int j, int k) { s_ << "    h_pair(" << a << j << ", " << a << k << ", hs, hn);\n"; });
+      s_ << "    }\n";
+      if (rev_ && r_.norm >= 0) s_ << "    sc *= 0.70710678118654752f;\n";
+      return;
+    }
+    Sign sg = frame_sign(frame_, mj);
+    if (g.kind == L_RY) sg.flip(group_sign(g.f, g.b));
+    s_ << "    {\n    const float4 q = " << mat(o) << ";\n";
+    const std::string dst = rev_ ? share(o) : "";
+    const bool ry = g.kind == L_RY;
+    if (!dst.empty()) {
+      const char* type = ry ? "float2" : "float";
+      const char* zero = ry ? "make_float2(0.f, 0.f)" : "0.f";
+      s_ << "    " << type << " gp = " << zero << ", gn = " << zero << ";\n";
+      pairs(mj, ry ? fr : mj & -mj, [&](int j, int k) {
+        s_ << "    dot_" << (ry ? "y" : "x") << "(p" << j << ", p" << k << ", l" << j << ", l" << k << ", gp, gn);\n";
+      });
+      s_ << "    lin_share(" << dst << ", sx(sc * sc * (" << (ry ? "(gp.x + gp.y) - (gn.x + gn.y)" : "gp - gn") << "), " << sg.str()
+         << "));\n";
+    }
+    if (rev_) {
+      Sign inv;
+      inv.c = true;
+      sg.flip(inv);
+    }
+    s_ << "    const float v = sx(q.x, " << sg.str() << ");\n    if (__float_as_uint(q.w) == 0u) {\n";
+    if (ry) s_ << "    const float2 t = bc2(v), nt = bc2(-v);\n";
+    for (const char* a : regs_)
+      pairs(mj, ry ? fr : mj & -mj, [&](int j, int k) {
+        s_ << "    " << (ry ? "ry_t(" : "rx_t(") << a << j << ", " << a << k << (ry ? ", t, nt);\n" : ", v);\n");
+      });
+    s_ << "    } else {\n";
+    for (const char* a : regs_)
+      pairs(mj, ry ? fr : mj & -mj, [&](int j, int k) {
+        s_ << "    " << (ry ? "ry_u(" : "rx_u(") << a << j << ", " << a << k << ", v);\n";
+      });
+    s_ << "    }\n";
+    if (rev_ && r_.norm >= 0) s_ << "    sc *= q.y;\n";
+    s_ << "    }\n";
+  }
+
+  // f(j, j ^ mj) over the members of even parity fr
+  template <class F>
+  void pairs(int mj, int fr, F f) {
+    for (int j = 0; j < N_; j++)
+      if (!cpar(fr & j)) f(j, j ^ mj);
+  }
+
+  // a block of phases (see the class comment); merge: G multiplies every member
+  template <class Share>
+  void block(const std::vector<int>& ops, bool merge, Share share) {
+    s_ << "    {\n";
+    // gradient shares: Im(conj(l) p) summed per class of up to three parities
+    std::vector<int> withg;
+    if (rev_)
+      for (int o : ops)
+        if (!share(o).empty()) withg.push_back(o);
+    for (size_t c0 = 0; c0 < withg.size(); c0 += 3) {
+      const size_t c1 = std::min(withg.size(), c0 + 3);
+      std::vector<int> basis;
+      for (size_t i = c0; i < c1; i++)
+        if (int f = reg_parity(P_.ops[withg[i]].f)) add_basis(basis, f);
+      const int nc = 1 << basis.size();
+      s_ << "    {\n";
+      for (int c = 0; c < nc; c++) s_ << (c ? ", v" : "    float v") << c << " = 0.f";
+      s_ << ";\n";
+      for (int j = 0; j < N_; j++) {
+        int cls = 0;
+        for (size_t i = 0; i < basis.size(); i++) cls |= cpar(basis[i] & j) << i;
+        s_ << "    v" << cls << " = lin_im(l" << j << ", p" << j << ", v" << cls << ");\n";
+      }
+      for (size_t i = c0; i < c1; i++) {
+        const LinOp& g = P_.ops[withg[i]];
+        const int cm = combo(basis, reg_parity(g.f));
+        s_ << "    lin_share(" << share(withg[i]) << ", sx(" << (r_.norm >= 0 ? "sc * sc * (" : "(");
+        for (int c = 0; c < nc; c++) s_ << (cpar(cm & c) ? " - " : c ? " + " : "") << "v" << c;
+        s_ << "), " << group_sign(g.f, g.b).str() << "));\n";
+      }
+      s_ << "    }\n";
+    }
+    // phases per register parity, in class space
+    std::vector<int> frs, basis;
+    for (int o : ops) frs.push_back(reg_parity(P_.ops[o].f));
+    std::vector<Frame> signs;
+    absorb(frs, frame_, &signs);
+    for (int f : frs)
+      if (f) add_basis(basis, f);
+    struct Elem {
+      int cm;
+      std::string name;  // phase, or ""
+      Sign sign;
+    };
+    std::vector<Elem> el;
+    for (size_t i = 0; i < ops.size(); i++) {
+      if (!frs[i]) continue;  // shared by the group: in G
+      const LinOp& g = P_.ops[ops[i]];
+      Sign sg = group_sign(g.f, g.b);
+      if (rev_) sg.c = !sg.c;
+      const std::string nm = "h" + std::to_string(i);
+      s_ << "    const c2 " << nm << " = {" << mat(ops[i]) << ".z, sx(" << mat(ops[i]) << ".w, " << sg.str() << ")};\n";
+      el.push_back({combo(basis, frs[i]), nm, Sign()});
+    }
+    for (const Frame& f : signs) el.push_back({combo(basis, f.fr), "", f.sign});
+    int tmp = 0;
+    classes(basis, el, 0, 0, merge ? "G" : "", &tmp, merge);
+    if (merge && rev_ && r_.norm >= 0) s_ << "    sc *= nrm.z;\n";
+    s_ << "    }\n";
+  }
+
+  template <class Elem>
+  void classes(const std::vector<int>& basis, const std::vector<Elem>& el, size_t i, int cls, std::string ph, int* tmp,
+               bool merge) {
+    if (i < basis.size()) {
+      classes(basis, el, i + 1, cls, ph, tmp, merge);
+      for (const Elem& e : el)
+        if (e.cm == (1 << i) && !e.name.empty()) ph = times(ph, e.name, tmp);
+      classes(basis, el, i + 1, cls | (1 << i), ph, tmp, merge);
+      return;
+    }
+    Sign sg;
+    for (const Elem& e : el) {
+      if (!cpar(e.cm & cls)) continue;
+      if (e.name.empty()) sg.flip(e.sign);
+      else if (e.cm & (e.cm - 1)) ph = times(ph, e.name, tmp);
+    }
+    if (!ph.empty() && !sg.zero()) {
+      const std::string nm = "t" + std::to_string((*tmp)++);
+      s_ << "    c2 " << nm << " = " << ph << ";\n    lin_neg(" << nm << ", " << sg.str() << ");\n";
+      ph = nm;
+    }
+    for (const char* g : regs_)
+      for (int j = 0; j < N_; j++) {
+        int c = 0;
+        for (size_t b = 0; b < basis.size(); b++) c |= cpar(basis[b] & j) << b;
+        if (c != cls) continue;
+        if (!ph.empty()) s_ << "    lin_mul(" << g << j << ", " << ph << ");\n";
+        else if (!sg.zero()) s_ << "    lin_neg(" << g << j << ", " << sg.str() << ");\n";
+      }
+  }
+
+  std::string times(const std::string& a, const std::string& b, int* tmp) {
+    if (a.empty()) return b;
+    const std::string nm = "t" + std::to_string((*tmp)++);
+    s_ << "    const c2 " << nm << " = cmul(" << a << ", " << b << ");\n";
+    return nm;
+  }
+
+  std::ostringstream& s_;
+  const LinProgram& P_;
+  const LinTile& t_;
+  const LinReg& r_;
+  const bool rev_;
+  const int N_;
+  uint32_t gu_[4];        // the pass's vectors as index masks
+  uint32_t varying_ = 0;  // index bits that the group base can have
+  std::map<uint32_t, int> words_;
+  std::vector<std::vector<int>> items_;
+  std::vector<Frame> frame_;
+  std::vector<const char*> regs_;
+  bool group_factor_ = false, complex_factor_ = false;
+  int merge_ = -1;
+};
+
+// The index of a group's first member: its tile's base XOR its local index
+// through the tile's vectors (whole states: the local index).
+std::string group_index(const LinProgram& P, const LinTile& t, int L) {
+  if (t.k == P.n) return "gb";
+  const std::string low = std::to_string((1u << L) - 1u);
+  return "base ^ (gb & " + low + "u) ^ (uint32_t)s.off[gb >> " + std::to_string(L) + "]";
 }
 
-// One forward register pass as a group loop over the tile (or state) in
-// `st` of 2^k amplitudes; ops [op0 + rp.op_begin, op0 + rp.op_end) of dops.
-void emit_fwd_pass(std::ostringstream& s, const RegPass& rp, const std::vector<DOp>& dops, int op0, int k,
-                   const char* st) {
-  const PassBits pb = pass_bits(rp);
-  s << "  for (int grp = threadIdx.x; grp < " << (1 << (k - pb.m)) << "; grp += blockDim.x) {\n";
-  emit_group_base(s, pb);
-  s << "    c2 a[" << (1 << pb.m) << "];\n";
-  emit_move(s, pb, st, "a", false);
-  for (int o = rp.op_begin; o < rp.op_end; o++) emit_fwd_op(s, dops[op0 + o], pb.m, "a");
-  emit_move(s, pb, st, "a", true);
+void emit_fwd_pass(std::ostringstream& s, const LinProgram& P, const LinTile& t, const LinReg& r, int L, int nthreads) {
+  s << "  {\n";
+  PassWriter(s, P, t, r, false).write(nthreads, group_index(P, t, L), {"psi"}, {"a"}, [](int) { return std::string(); });
   s << "  }\n  __syncthreads();\n";
 }
 
 // One reverse register pass: gradient shares go to accumulator index
-// acc_index(op, angle) of the per-warp rows gpart[warp * stride + index],
-// reduced over the warp for up to 32 accumulators at once (grad_share_multi;
-// their index tables are declared into `decl`).
+// acc_index(op) of the per-warp rows gpart[warp * stride + index], reduced
+// over the warp for up to 32 accumulators at once (grad_share_multi; their
+// index tables are declared into `decl`).
 template <class F>
-void emit_rev_pass(std::ostringstream& s, std::ostringstream& decl, int* uid, const RegPass& rp,
-                   const std::vector<DOp>& dops, int op0, int k, const char* sp, const char* sl, int stride,
-                   F acc_index) {
-  const PassBits pb = pass_bits(rp);
+void emit_rev_pass(std::ostringstream& s, std::ostringstream& decl, int* uid, const LinProgram& P, const LinTile& t,
+                   const LinReg& r, int L, int nthreads, int stride, F acc_index) {
   // The pass's gradient shares, summed per accumulator index in registers
   // gs<chunk>[position] (a chunk holds at most 32 distinct indices; shares of
   // gates that use one parameter add into one register), then reduced over
@@ -178,118 +579,87 @@ void emit_rev_pass(std::ostringstream& s, std::ostringstream& decl, int* uid, co
   // the same old value and one addition would be lost.  A chunk of g indices
   // is padded to K = 2^ceil(log2 g) with indices the chunk does not use (the
   // padding lanes add zero there); if fewer than K - g are free, it is cut
-  // into power-of-two chunks instead.  gv holds 32 * chunk + position.
-  std::vector<std::vector<int>> gv(rp.op_end - rp.op_begin, std::vector<int>(3, -1));
-  std::vector<std::vector<int>> chunks;  // accumulator indices, by position
-  std::vector<int> open_idx;             // distinct indices of the chunk being filled
-  std::vector<std::pair<std::pair<int, int>, int>> open_sh;  // ((op, angle), position in open_idx)
-  auto close_chunk = [&] {
-    int g = (int)open_idx.size();
-    int at = 0;
-    while (g > 0) {
-      int kk = 1;
-      while (kk < g) kk <<= 1;
-      if (kk - g > stride - g) kk >>= 1;  // too few free indices: the largest power of two below g
-      const int take = std::min(kk, g);
-      const int c = (int)chunks.size();
-      chunks.emplace_back(open_idx.begin() + at, open_idx.begin() + at + take);
-      for (const auto& sh : open_sh)
-        if (sh.second >= at && sh.second < at + take) gv[sh.first.first][sh.first.second] = 32 * c + sh.second - at;
-      at += take;
-      g -= take;
+  // into power-of-two chunks instead.
+  std::vector<int> distinct;
+  for (int o : r.ops)
+    if (P.ops[o].slot >= 0) {
+      const int idx = acc_index(o);
+      if (std::find(distinct.begin(), distinct.end(), idx) == distinct.end()) distinct.push_back(idx);
     }
-    open_idx.clear();
-    open_sh.clear();
-  };
-  for (int o = rp.op_begin; o < rp.op_end; o++) {
-    const DOp& d = dops[op0 + o];
-    for (int j = 0; j < d.nang && j < 3; j++)
-      if (d.slot[j] >= 0) {
-        const int idx = acc_index(op0 + o, j);
-        auto it = std::find(open_idx.begin(), open_idx.end(), idx);
-        if (it == open_idx.end() && open_idx.size() == 32) {
-          close_chunk();
-          it = open_idx.end();
-        }
-        if (it == open_idx.end()) {
-          open_idx.push_back(idx);
-          it = open_idx.end() - 1;
-        }
-        open_sh.push_back({{o - rp.op_begin, j}, (int)(it - open_idx.begin())});
-      }
-  }
-  close_chunk();
-  std::vector<int> chunk_k;  // padded size of each chunk
-  for (auto& ch : chunks) {
+  std::vector<std::vector<int>> chunks;
+  std::map<int, std::pair<int, int>> place;  // accumulator index -> chunk, position
+  for (size_t at = 0; at < distinct.size();) {
+    const int g = (int)std::min<size_t>(32, distinct.size() - at);
     int kk = 1;
-    while (kk < (int)ch.size()) kk <<= 1;
-    chunk_k.push_back(kk);
+    while (kk < g) kk <<= 1;
+    if (kk > stride) kk >>= 1;  // too few free indices: the largest power of two below g
+    const int take = std::min(kk, g);
+    for (int i = 0; i < take; i++) place[distinct[at + i]] = {(int)chunks.size(), i};
+    chunks.emplace_back(distinct.begin() + at, distinct.begin() + at + take);
+    std::vector<int>& ch = chunks.back();
     // padding: the lowest accumulator indices the chunk does not use
     for (int cand = 0; (int)ch.size() < kk && cand < stride; cand++)
       if (std::find(ch.begin(), ch.end(), cand) == ch.end()) ch.push_back(cand);
+    at += take;
   }
   s << "  {\n";
-  for (size_t c = 0; c < chunk_k.size(); c++) {
-    s << "  float gs" << c << "[" << chunk_k[c] << "] = {";
-    for (int j = 0; j < chunk_k[c]; j++) s << (j ? ", " : "") << "0.f";
+  for (size_t c = 0; c < chunks.size(); c++) {
+    s << "  float gs" << c << "[" << chunks[c].size() << "] = {";
+    for (size_t j = 0; j < chunks[c].size(); j++) s << (j ? ", " : "") << "0.f";
     s << "};\n";
   }
-  s << "  for (int grp = threadIdx.x; grp < " << (1 << (k - pb.m)) << "; grp += blockDim.x) {\n";
-  emit_group_base(s, pb);
-  s << "    c2 p[" << (1 << pb.m) << "], l[" << (1 << pb.m) << "];\n";
-  emit_move(s, pb, sp, "p", false);
-  emit_move(s, pb, sl, "l", false);
-  for (int o = rp.op_end - 1; o >= rp.op_begin; o--) emit_rev_op(s, dops[op0 + o], pb.m, gv[o - rp.op_begin]);
-  emit_move(s, pb, sp, "p", true);
-  emit_move(s, pb, sl, "l", true);
-  s << "  }\n";
-  for (size_t c = 0; c < chunk_k.size(); c++) {
+  PassWriter(s, P, t, r, true)
+      .write(nthreads, group_index(P, t, L), {"psi", "lam"}, {"p", "l"}, [&](int o) {
+        if (P.ops[o].slot < 0) return std::string();
+        const auto& at = place.at(acc_index(o));
+        return "gs" + std::to_string(at.first) + "[" + std::to_string(at.second) + "]";
+      });
+  for (size_t c = 0; c < chunks.size(); c++) {
     const int id = (*uid)++;
-    decl << "__constant__ int tdq_gi_" << id << "[" << chunk_k[c] << "] = {";
-    for (int j = 0; j < chunk_k[c]; j++) decl << (j ? ", " : "") << chunks[c][j];
+    decl << "__constant__ int tdq_gi_" << id << "[" << chunks[c].size() << "] = {";
+    for (size_t j = 0; j < chunks[c].size(); j++) decl << (j ? ", " : "") << chunks[c][j];
     decl << "};\n";
-    s << "  grad_share_multi<" << chunk_k[c] << ">(gpart, " << stride << ", tdq_gi_" << id << ", gs" << c << ");\n";
+    s << "  grad_share_multi<" << chunks[c].size() << ">(gpart, " << stride << ", tdq_gi_" << id << ", gs" << c << ");\n";
   }
   s << "  __syncthreads();\n  }\n";
 }
 
 }  // namespace
 
-// The program struct `sname` of one circuit (forward passes [0, npf), reverse
-// passes [npf, npf + npb)); constant tables go to decl, numbered from *uid.
-static void k2_prog_struct(std::ostringstream& s, std::ostringstream& decl, int* uid, const Program& prog, int npf,
-                           int npb, int P, int n, const std::string& sname) {
+// The program struct `sname` of one circuit; constant tables go to decl,
+// numbered from *uid.
+static void k2_prog_struct(std::ostringstream& s, std::ostringstream& decl, int* uid, const LinProgram& P, int nparams,
+                           int nthreads, bool grad, const std::string& sname) {
+  const LinTile& t = P.tiles[0];
   s << "struct " << sname << " {\n"
-    << "  static constexpr bool kSpecialised = true;\n  const DOp* dops;\n";
-  s << "  template <int MF>\n  __device__ __forceinline__ void forward(c2* psi, const OpMat* mats, int) const {\n"
-    << "  const uint32_t base = 0u;\n";
-  for (int pi = 0; pi < npf; pi++) {
+    << "  static constexpr bool kSpecialised = true;\n  using Mat = float4;\n  const DOp* dops;\n";
+  s << "  template <int MF>\n  __device__ __forceinline__ void forward(c2* psi, const float4* mats, int) const {\n";
+  for (size_t pi = 0; pi < t.fwd.size(); pi++) {
     s << "  // forward pass " << pi << "\n";
-    emit_fwd_pass(s, prog.passes[pi], prog.dops, 0, n, "psi");
+    emit_fwd_pass(s, P, t, t.fwd[pi], 0, nthreads);
   }
   s << "  }\n";
-  s << "  template <int MB>\n  __device__ __forceinline__ void reverse(c2* psi, c2* lam, const OpMat* mats, int, "
-       "double*, float* gpart) const {\n  const uint32_t base = 0u;\n";
-  for (int pi = npf + npb - 1; pi >= npf; pi--) {
-    s << "  // reverse pass " << pi << "\n";
-    emit_rev_pass(s, decl, uid, prog.passes[pi], prog.dops, 0, n, "psi", "lam", P,
-                  [&](int o, int j) { return (int)prog.dops[o].slot[j]; });
-  }
+  s << "  template <int MB>\n  __device__ __forceinline__ void reverse(c2* psi, c2* lam, const float4* mats, int, "
+       "double*, float* gpart) const {\n";
+  if (grad)
+    for (int pi = (int)t.rev.size() - 1; pi >= 0; pi--) {
+      s << "  // reverse pass " << pi << "\n";
+      emit_rev_pass(s, decl, uid, P, t, t.rev[pi], 0, nthreads, nparams, [&](int o) { return P.ops[o].slot; });
+    }
   s << "  }\n};\n";
 }
 
-std::string k2_specialised_source(const Program& prog, int npf, int npb, int mf, int mb, int nthreads,
-                                  int P, int n, const char* name) {
+std::string k2_specialised_source(const LinProgram& prog, bool grad, int nthreads, int nparams, const char* name) {
   std::ostringstream s, decl;
   int uid = 0;
-  k2_prog_struct(s, decl, &uid, prog, npf, npb, P, n, "SpecProg");
+  k2_prog_struct(s, decl, &uid, prog, nparams, nthreads, grad, "SpecProg");
   s << "}  // namespace tdq\n";
   std::ostringstream out;
   out << "#include \"k2_body.cuh\"\nnamespace tdq {\n" << decl.str() << s.str();
   const int minb = nthreads >= 256 ? 2 : 1;
   out << "extern \"C\" __global__ void __launch_bounds__(" << nthreads << ", " << minb << ") " << name
     << "(tdq::SweepArgs a, const tdq::DOp* gdops, int ndops, const int* rec_ptr, const int* rec_ops, int nrec) {\n"
-    << "  tdq::k2_body<" << mf << ", " << mb << ", " << (npb > 0 ? "true" : "false")
+    << "  tdq::k2_body<0, 0, " << (grad ? "true" : "false")
     << ", tdq::SpecProg>(a, tdq::SpecProg{nullptr}, gdops, 0, rec_ptr, rec_ops, nrec, blockIdx.x);\n}\n";
   return out.str();
 }
@@ -300,14 +670,13 @@ std::vector<std::string> k2_multi_modules(const std::vector<K2Part>& parts, bool
   int uid = 0;  // constant tables numbered across modules: their names stay unique at link time
   for (size_t c = 0; c < parts.size(); c++) {
     std::ostringstream s, decl;
-    k2_prog_struct(s, decl, &uid, *parts[c].prog, parts[c].npf, parts[c].npb, parts[c].P, parts[c].n,
-                   "SpecProg_" + std::to_string(c));
+    k2_prog_struct(s, decl, &uid, *parts[c].prog, parts[c].P, nthreads, grad, "SpecProg_" + std::to_string(c));
     std::ostringstream out;
     out << "#include \"k2_body.cuh\"\nnamespace tdq {\n" << decl.str() << s.str() << "}  // namespace tdq\n";
     // the circuit's row body: a function of its own, linked to the launch module
     out << "__device__ __noinline__ void tdq_multi_row_" << c
-        << "(const tdq::SweepArgs& a, const tdq::MultiCirc& m, int r) {\n  tdq::k2_body<" << parts[c].mf << ", "
-        << parts[c].mb << ", " << (grad ? "true" : "false") << ", tdq::SpecProg_" << c << ">(a, tdq::SpecProg_"
+        << "(const tdq::SweepArgs& a, const tdq::MultiCirc& m, int r) {\n  tdq::k2_body<0, 0, "
+        << (grad ? "true" : "false") << ", tdq::SpecProg_" << c << ">(a, tdq::SpecProg_"
         << c << "{nullptr}, nullptr, 0, m.rec_ptr, m.rec_ops, m.nrec, r);\n}\n";
     mods.push_back(out.str());
   }
@@ -342,43 +711,74 @@ std::vector<std::string> k2_multi_modules(const std::vector<K2Part>& parts, bool
   return mods;
 }
 
-std::string k1_specialised_source(const TiledSweep& t, const Program& prog, int nthreads, int nthreads_r,
+// every(f): f(shared-memory slot, global index) for this thread's elements of
+// a tile.  A thread's local indices are tid + NT i: the part of both indices
+// that tid gives is computed once per tile, the rest are constants.
+static void emit_every(std::ostringstream& s, const LinTile& t, int L) {
+  s << "  template <int NT, class F>\n  __device__ __forceinline__ static void every(const TiledDev&, const TileShared& s, "
+       "uint32_t base, F&& f) {\n"
+    << "    constexpr uint32_t v[" << t.k << "] = {";
+  for (int i = 0; i < t.k; i++) s << (i ? ", " : "") << t.v[i] << "u";
+  s << "};\n    if (NT > " << (1 << t.k) << " && threadIdx.x >= " << (1 << t.k) << ") return;\n"
+    << "    const uint32_t y = base ^ (threadIdx.x & " << (1u << L) - 1u << "u) ^ (uint32_t)s.off[threadIdx.x >> " << L
+    << "], z = swz(threadIdx.x);\n"
+    << "#pragma unroll\n    for (uint32_t i = 0; i < " << (1 << t.k) << "u; i += NT) {\n"
+    << "      uint32_t x = 0;\n#pragma unroll\n      for (int q = 0; q < " << t.k
+    << "; q++) x ^= ((i >> q) & 1u) ? v[q] : 0u;\n"
+    << "      f(z ^ swz(i), y ^ x);\n    }\n  }\n";
+}
+
+// in_first(x): whether index x lies in the first pass's space (the remainder
+// of x by the space's basis is zero).
+static void emit_in_first(std::ostringstream& s, const LinTile& t, int n) {
+  const uint32_t out = (n >= 32 ? ~0u : (1u << n) - 1u) & ~t.pivots;
+  s << "  __device__ __forceinline__ static bool in_first(uint32_t x) {\n    uint32_t r = x & " << out << "u;\n";
+  for (uint32_t v : t.v) {
+    if (!(v & out)) continue;
+    int p = 0;
+    while (!((v & t.pivots) >> p & 1u)) p++;
+    s << "    if ((x >> " << p << ") & 1u) r ^= " << (v & out) << "u;\n";
+  }
+  s << "    return r == 0u;\n  }\n";
+}
+
+std::string k1_specialised_source(const TiledSweep& t, const LinProgram& prog, int nthreads, int nthreads_r,
                                   std::vector<int>* nacc) {
   std::ostringstream s, decl;
   int uid = 0;
-  const int np = (int)t.passes.size();
+  const int np = (int)prog.tiles.size();
   nacc->assign(np, 0);
   for (int p = 0; p < np; p++) {
-    const int d0 = t.dop_begin[p];
-    // gradient accumulators of the pass: one per (reverse op, angle) with a slot
-    std::map<std::pair<int, int>, int> acc;
+    const LinTile& tile = prog.tiles[p];
+    // gradient accumulators of the pass: one per angle with a slot
+    std::map<int, int> acc;
     std::vector<int> slots;
     if (t.adj)
-      for (int q = t.bp_begin[p]; q < t.bp_end[p]; q++)
-        for (int o = prog.passes[q].op_begin; o < prog.passes[q].op_end; o++) {
-          const DOp& d = prog.dops[d0 + o];
-          for (int j = 0; j < d.nang && j < 3; j++)
-            if (d.slot[j] >= 0) {
-              acc[{d0 + o, j}] = (int)slots.size();
-              slots.push_back(d.slot[j]);
-            }
+      for (int o : tile.ops)
+        if (prog.ops[o].slot >= 0) {
+          acc[o] = (int)slots.size();
+          slots.push_back(prog.ops[o].slot);
         }
     (*nacc)[p] = (int)slots.size();
     const int na = std::max(1, (int)slots.size());
     s << "__constant__ int tdq_slots_" << p << "[" << na << "] = {";
     for (int i = 0; i < na; i++) s << (i ? ", " : "") << (i < (int)slots.size() ? slots[i] : 0);
     s << "};\n";
-    s << "struct TilePass" << p << " {\n";
+    s << "struct TilePass" << p << " {\n  static constexpr bool kSpecialised = true, kFirst = "
+      << (p == 0 ? "true" : "false") << ", kSecond = " << (p == 1 ? "true" : "false") << ";\n";
+    emit_in_first(s, prog.tiles[0], t.n);
+    emit_every(s, tile, t.L);
     s << "  __device__ __forceinline__ static void forward(const TiledDev&, const TileShared& s, uint32_t base) {\n"
-      << "  c2* psi = s.psi;\n  const OpMat* mats = s.mats;\n";
-    for (int q = t.fp_begin[p]; q < t.fp_end[p]; q++) emit_fwd_pass(s, prog.passes[q], prog.dops, d0, t.k, "psi");
+      << "  c2* psi = s.psi;\n  const float4* mats = reinterpret_cast<const float4*>(s.mats);\n";
+    for (const LinReg& r : tile.fwd) emit_fwd_pass(s, prog, tile, r, t.L, nthreads);
     s << "  }\n";
     s << "  __device__ __forceinline__ static void reverse(const TiledDev&, const TileShared& s, uint32_t base) {\n"
-      << "  c2* psi = s.psi;\n  c2* lam = s.lam;\n  const OpMat* mats = s.mats;\n"
+      << "  c2* psi = s.psi;\n  c2* lam = s.lam;\n  const float4* mats = reinterpret_cast<const float4*>(s.mats);\n"
       << "  float* gpart = reinterpret_cast<float*>(s.gpart);\n";
-    for (int q = t.bp_end[p] - 1; q >= t.bp_begin[p]; q--)
-      emit_rev_pass(s, decl, &uid, prog.passes[q], prog.dops, d0, t.k, "psi", "lam", na,
-                    [&](int o, int j) { return acc.at({o, j}); });
+    // (the fused last pass runs its reverse program with the forward kernel's threads)
+    for (int q = (int)tile.rev.size() - 1; q >= 0; q--)
+      emit_rev_pass(s, decl, &uid, prog, tile, tile.rev[q], t.L, p == np - 1 ? nthreads : nthreads_r, na,
+                    [&](int o) { return acc.at(o); });
     s << "  }\n";
     s << "  __device__ __forceinline__ static void flush(const SweepArgs& a, const TiledDev& t, const TileShared& s, "
          "int lr) {\n"
@@ -395,13 +795,14 @@ std::string k1_specialised_source(const TiledSweep& t, const Program& prog, int 
   for (int p = 0; p < np; p++) {
     const bool f = p == 0, l = p == np - 1;
     out << "extern \"C\" __global__ void __launch_bounds__(" << nthreads << ", " << minb << ") tdq_k1f_" << p
-      << "(tdq::SweepArgs a, tdq::TiledDev t, int store) {\n  tdq::k1_forward_body<" << (f ? "true" : "false") << ", "
-      << (l ? "true" : "false") << ", " << ((l && t.adj) ? "true" : "false") << ", tdq::TilePass" << p
+      << "(tdq::SweepArgs a, tdq::TiledDev t, int store) {\n  tdq::k1_forward_body<" << nthreads << ", "
+      << (f ? "true" : "false") << ", " << (l ? "true" : "false") << ", " << ((l && t.adj) ? "true" : "false")
+      << ", tdq::TilePass" << p
       << ">(a, t, store);\n}\n";
     if (t.adj && !l)
       out << "extern \"C\" __global__ void __launch_bounds__(" << nthreads_r << ", " << (nthreads_r <= 256 ? 2 : 1)
           << ") tdq_k1r_" << p
-        << "(tdq::SweepArgs a, tdq::TiledDev t) {\n  tdq::k1_reverse_body<tdq::TilePass" << p << ">(a, t);\n}\n";
+        << "(tdq::SweepArgs a, tdq::TiledDev t) {\n  tdq::k1_reverse_body<" << nthreads_r << ", tdq::TilePass" << p << ">(a, t);\n}\n";
   }
   return out.str();
 }

@@ -1,27 +1,27 @@
-// Specialised sweep programs: the register passes of one circuit written out
-// as straight-line device code (every gate kind, register bit and table row a
-// compile-time constant), compiled at run time for the device in use.
+// Specialised sweep programs: the register passes of one circuit (in a linear
+// frame of the basis index, lin_program.h) written out as straight-line device
+// code -- every gate kind, pairing and table row a compile-time constant --,
+// compiled at run time for the device in use.
 #pragma once
 
 #include <string>
 #include <vector>
 
+#include "lin_program.h"
 #include "sweep_tiled.cuh"
 #include "tdq_internal.h"
 
 namespace tdq {
 
-// Source of a K2 kernel named `name` for the program `prog` of an n-qubit
-// state: forward passes [0, npf), reverse passes [npf, npf + npb) (npb = 0:
-// no gradients).  mf / mb register bits, nthreads threads per CTA, P gradient
-// columns.
-std::string k2_specialised_source(const Program& prog, int npf, int npb, int mf, int mb, int nthreads,
-                                  int P, int n, const char* name);
+// Source of a K2 kernel named `name` for the whole-state program `prog` (one
+// tile; grad: with its reverse passes).  nthreads threads per CTA, nparams
+// gradient columns.
+std::string k2_specialised_source(const LinProgram& prog, bool grad, int nthreads, int nparams, const char* name);
 
 // One circuit of a multi-circuit whole-state kernel.
 struct K2Part {
-  const Program* prog;
-  int npf, npb, mf, mb, P, n;
+  const LinProgram* prog;
+  int P;
 };
 
 // Modules of a persistent kernel `name` over several circuits: module 0 is the
@@ -41,7 +41,7 @@ constexpr const char* kModuleMark = "// ==== tdq module ";
 // tdq_k1f_<p> (forward; the last one also runs its reverse sweep with
 // gradients) and tdq_k1r_<p> (reverse, passes before the last).  nacc[p]:
 // gradient accumulators of pass p (per-warp FP32 rows in shared memory).
-std::string k1_specialised_source(const TiledSweep& t, const Program& prog, int nthreads, int nthreads_r,
+std::string k1_specialised_source(const TiledSweep& t, const LinProgram& prog, int nthreads, int nthreads_r,
                                   std::vector<int>* nacc);
 
 // Compiles `src` for the current device and returns the kernel `name` (a

@@ -16,10 +16,10 @@ namespace {
 
 template <bool FIRST, bool LAST, bool GRAD>
 __global__ void __launch_bounds__(256) k1_forward(SweepArgs a, TiledDev t, int store) {
-  k1_forward_body<FIRST, LAST, GRAD, InterpTile>(a, t, store);
+  k1_forward_body<256, FIRST, LAST, GRAD, InterpTile>(a, t, store);
 }
 
-__global__ void __launch_bounds__(256) k1_reverse(SweepArgs a, TiledDev t) { k1_reverse_body<InterpTile>(a, t); }
+__global__ void __launch_bounds__(256) k1_reverse(SweepArgs a, TiledDev t) { k1_reverse_body<256, InterpTile>(a, t); }
 
 // Copy out the chunk's values, F for the shift rule, gradients, amplitudes.
 __global__ void k1_finalize(SweepArgs a, TiledDev t, int nrows, int grad_adj) {
@@ -52,14 +52,25 @@ __global__ void k1_finalize(SweepArgs a, TiledDev t, int nrows, int grad_adj) {
 
 // The chunk's final states as the output: the whole state (TDQ_OUT_STATE) or
 // the probabilities (TDQ_OUT_PROBS) of every row, grid-stride over (row, x).
-__global__ void k1_state_out(SweepArgs a, TiledDev t, int nrows) {
+// Basis index x sits at place y(x), linear over its bits: tables of y over
+// the bits 0..7, 8..15, 16..23 and 24..29 give it with four reads.
+__global__ void __launch_bounds__(256) k1_state_out(SweepArgs a, TiledDev t, int nrows) {
+  __shared__ uint32_t tab[4][256];
+  for (int q = 0; q < 4; q++) {
+    uint32_t y = 0;
+    for (int i = 0; i < 8; i++)
+      if (((threadIdx.x >> i) & 1u) && 8 * q + i < t.n) y ^= a.lin ? a.lin[8 * q + i] : 1u << (8 * q + i);
+    tab[q][threadIdx.x] = y ^ (q == 0 && a.lin ? a.lin[t.n] : 0u);
+  }
+  __syncthreads();
   const int64_t dim = (int64_t)1 << t.n, tot = dim * nrows;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < tot; i += (int64_t)gridDim.x * blockDim.x) {
-    const int lr = (int)(i / dim);
+    const int lr = (int)(i >> t.n);
     const int row = t.row0 + lr;
     if (row % a.ps_copies) continue;
     const int64_t b = row / a.ps_copies, x = i - (int64_t)lr * dim;
-    const c2 v = t.psi[i];
+    const uint32_t y = tab[0][x & 255] ^ tab[1][(x >> 8) & 255] ^ tab[2][(x >> 16) & 255] ^ tab[3][(x >> 24) & 255];
+    const c2 v = t.psi[(size_t)lr * dim + y];
     if (a.output == TDQ_OUT_STATE) {
       a.values[(b * dim + x) * 2] = v.x;
       a.values[(b * dim + x) * 2 + 1] = v.y;
@@ -86,6 +97,8 @@ void tiled_free(TiledSweep& t) {
   cudaFree(t.d_dops);
   cudaFree(t.d_rec_ptr);
   cudaFree(t.d_rec_ops);
+  cudaFree(t.d_lin);
+  t.d_lin = nullptr;
   t.d_ps_gate_pass = nullptr;
   t.d_rpass = nullptr;
   t.d_dops = nullptr;
@@ -239,12 +252,62 @@ tdq_status tiled_plan(TiledSweep& t, const tdq_circuit* c, const std::vector<Swe
   return TDQ_OK;
 }
 
+tdq_status tiled_lin_plan(TiledSweep& t, const tdq_circuit* c, const std::vector<SweepOp>& ops, int rows, bool adj,
+                          int tile_qubits, int fb, int rb, bool exact, LinProgram& prog) {
+  t.fb = fb;
+  t.rb = rb;
+  t.n = c->n;
+  const int kq = tile_qubits > 0 ? tile_qubits : 12;
+  if (kq < 5 || kq > 13) return fail(TDQ_ERR_ARG, "tile_qubits must be in 5..13");
+  t.k = std::min(t.n, kq);
+  t.L = std::min(4, t.k);
+  t.adj = adj;
+  t.rows = rows;
+  t.P = c->n_params;
+  t.ng = c->n_groups;
+  if (t.ng > 1024) return fail(TDQ_ERR_UNSUPPORTED, "tiled sweep: more than 1024 output groups");
+  prog = lin_program(ops, t.n, t.k, t.L, fb, rb, adj, exact);
+  t.passes.clear();
+  t.max_rec = 0;
+  t.max_dops = 0;
+  int r0 = 0;
+  for (const LinTile& tile : prog.tiles) {
+    t.passes.push_back({tile.pivots, 0, 0});
+    const int nr = (int)tile.rec_ptr.size() - 1;
+    t.rec_begin.push_back(r0);
+    t.rec_end.push_back(r0 += nr);
+    t.max_rec = std::max(t.max_rec, nr);
+    for (std::vector<int>* v : {&t.fp_begin, &t.fp_end, &t.bp_begin, &t.bp_end, &t.bo_begin, &t.bo_end, &t.dop_begin,
+                                &t.dop_end})
+      v->push_back(0);
+  }
+  return TDQ_OK;
+}
+
 tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<SweepOp>& ops,
-                         const std::vector<int>& ps_gate, int rows, bool adj, int tile_qubits, bool interpret,
+                         const std::vector<int>& ps_gate, int rows, bool adj, int tile_qubits, const LinProgram* lin,
                          int fb, int rb, double* bytes_row) {
   TiledHost h;
-  tdq_status s0 = tiled_plan(t, c, ops, ps_gate, rows, adj, tile_qubits, fb, rb, h);
-  if (s0 != TDQ_OK) return s0;
+  if (!lin) {
+    tdq_status s0 = tiled_plan(t, c, ops, ps_gate, rows, adj, tile_qubits, fb, rb, h);
+    if (s0 != TDQ_OK) return s0;
+  } else {  // ops in circuit order; every pass's index offsets and table rows
+    h.pops = ops;
+    h.psp = ps_gate;
+    for (const LinTile& tile : lin->tiles) {
+      for (int j = 0; j < (1 << (t.k - t.L)); j++) {
+        uint32_t o = 0;
+        for (int i = 0; i < t.k - t.L; i++)
+          if ((j >> i) & 1) o ^= tile.v[t.L + i];
+        h.offs.push_back((int)o);
+      }
+      for (int p = 0; p < 32; p++) h.locs.push_back(-1);
+      const int e0 = (int)h.prog.rec_ops.size();
+      for (size_t r = 1; r < tile.rec_ptr.size(); r++) h.prog.rec_ptr.push_back(e0 + tile.rec_ptr[r]);
+      h.prog.rec_ops.insert(h.prog.rec_ops.end(), tile.rec_ops.begin(), tile.rec_ops.end());
+    }
+  }
+  const bool interpret = lin == nullptr;
   const int n = c->n;
   const std::vector<SweepOp>& pops = h.pops;
   const std::vector<int>& offs = h.offs;
@@ -252,12 +315,19 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
   const Program& prog = h.prog;
   const std::vector<int>& psp = h.psp;
   auto up = [](void** d, const void* h, size_t bytes) -> tdq_status {
+    if (bytes == 0) return TDQ_OK;
     if (cudaMalloc(d, bytes) != cudaSuccess) return fail(TDQ_ERR_OOM, "tiled sweep: cudaMalloc");
     if (cudaMemcpy(*d, h, bytes, cudaMemcpyHostToDevice) != cudaSuccess)
       return fail(TDQ_ERR_CUDA, "tiled sweep: cudaMemcpy");
     return TDQ_OK;
   };
   tdq_status s;
+  if (lin) {
+    std::vector<uint32_t> map = lin->map.col;
+    map.push_back(lin->map.to_y(0));
+    if ((s = up((void**)&t.d_lin, map.data(), sizeof(uint32_t) * map.size())) != TDQ_OK) return s;
+    t.quarter = lin->exact ? lin->map.quarter : 0;
+  }
   if ((s = up((void**)&t.d_ops, pops.data(), sizeof(SweepOp) * pops.size())) != TDQ_OK) return s;
   if ((s = up((void**)&t.d_off, offs.data(), sizeof(int) * offs.size())) != TDQ_OK) return s;
   if ((s = up((void**)&t.d_loc, locs.data(), locs.size())) != TDQ_OK) return s;
@@ -295,7 +365,7 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
   if (!interpret) {
     // every tile pass as straight-line code; one compilation for all passes
     std::vector<int> nacc;
-    src = k1_specialised_source(t, prog, t.nthreads, t.nthreads_r, &nacc);
+    src = k1_specialised_source(t, *lin, t.nthreads, t.nthreads_r, &nacc);
     const int nw = std::max(t.nthreads, t.nthreads_r) / 32;
     for (int p = 0; p < np; p++) {
       t.spec_gbytes.push_back(4 * nw * std::max(1, nacc[p]));
@@ -310,12 +380,13 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
   // kernels hold psi and lambda in one buffer each: two CTAs of 256 threads
   // per SM then interleave one CTA's tile loads with the other's compute,
   // which measured faster than one double-buffered CTA of 512 threads.
+  const int mbytes = t.max_rec * (int)(interpret ? sizeof(OpMat) : sizeof(float4));
   auto sizes = [&](int nb) {
     t.smem_f.assign(np, 0);
     for (int p = 0; p < np; p++)
-      t.smem_f[p] = k1_smem_bytes(t.k, t.L, p == 0 ? 1 : nb, (adj && p == np - 1) ? 1 : 0, t.max_rec, ndops_sm,
+      t.smem_f[p] = k1_smem_bytes(t.k, t.L, p == 0 ? 1 : nb, (adj && p == np - 1) ? 1 : 0, mbytes, ndops_sm,
                                   t.ng, gmax);
-    t.smem_r = adj ? k1_smem_bytes(t.k, t.L, 1, 1, t.max_rec, ndops_sm, t.ng, gmax) : 0;
+    t.smem_r = adj ? k1_smem_bytes(t.k, t.L, 1, 1, mbytes, ndops_sm, t.ng, gmax) : 0;
     size_t m = t.smem_r;
     for (size_t v : t.smem_f) m = std::max(m, v);
     return m;
@@ -395,11 +466,20 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
   const double dim = std::ldexp(1.0, n);
   const double obs = c->n_groups > 0 ? (3.0 + 2.0 * (double)c->terms.size()) * dim : 0.0;
   std::vector<double> fw(np, 0.0), dots(np, 0.0);
-  for (int p = 0; p < np; p++)
+  for (int p = 0; p < np; p++) {
     for (int o = t.passes[p].op_begin; o < t.passes[p].op_end; o++) {
       fw[p] += gate_fwd_flops(pops[o].kind, dim);
       dots[p] += gate_dot_flops(pops[o].kind, dim);
     }
+    if (lin)
+      for (int o : lin->tiles[p].ops) {
+        const LinOp& g = lin->ops[o];
+        if (g.p) continue;  // a factor of a U3, counted with its RY
+        const int kind = g.kind == L_SIGN ? K_Z : g.kind == L_CZ ? K_CZ : g.kind == L_H ? K_H : ops[g.op].kind;
+        fw[p] += gate_fwd_flops(kind, dim);
+        dots[p] += gate_dot_flops(kind, dim);
+      }
+  }
   t.unit_flops.clear();
   t.unit_bytes.clear();
   t.unit_kind.clear();
@@ -443,6 +523,8 @@ tdq_status tiled_execute(TiledSweep& t, const SweepArgs& a0, int grad, cudaStrea
                          int* launches) {
   SweepArgs a = a0;
   if (a.ps_copies > 1) a.ps_gate = t.d_ps_gate_pass;
+  a.lin = t.d_lin;
+  a.quarter = t.quarter;
   const bool adj = grad == TDQ_GRAD_ADJOINT;
   const int np = (int)t.passes.size();
   const int ntiles = 1 << (t.n - t.k);
@@ -454,8 +536,12 @@ tdq_status tiled_execute(TiledSweep& t, const SweepArgs& a0, int grad, cudaStrea
       return fail(TDQ_ERR_CUDA, "tiled sweep: memset");
     // one wave per kernel: as many CTAs as fit on the GPU at once, each
     // with an equal share of the chunk's (row, tile) units
-    const int64_t total = (int64_t)nr * ntiles;
-    auto grid_for = [&](int slots, TiledDev& dd) {
+    // (specialised programs from |0...0>: the first pass's one tile at base 0,
+    // see k1_forward_body; a lone pass still writes a state output's zeros)
+    const bool lone = !a.init && !t.kf.empty() && (np > 1 || a.output == TDQ_OUT_EXPVAL);
+    auto grid_for = [&](int slots, TiledDev& dd, int p) {
+      dd.ntiles = p == 0 && lone ? 1 : ntiles;
+      const int64_t total = (int64_t)nr * dd.ntiles;
       const int64_t n0 = std::max<int64_t>(1, std::min<int64_t>(total, slots));
       const int64_t upc = (total + n0 - 1) / n0;
       dd.tiles_per_cta = (int)upc;
@@ -470,7 +556,6 @@ tdq_status tiled_execute(TiledSweep& t, const SweepArgs& a0, int grad, cudaStrea
     d.n = t.n;
     d.k = t.k;
     d.L = t.L;
-    d.ntiles = ntiles;
     d.row0 = row0;
     d.nrows = nr;
     d.dbl = t.dbl;
@@ -484,7 +569,7 @@ tdq_status tiled_execute(TiledSweep& t, const SweepArgs& a0, int grad, cudaStrea
       d.op_end = t.passes[p].op_end;
       set_pass(t, d, p);
       const bool f = p == 0, l = p == np - 1;
-      const dim3 grid = grid_for(t.slots_f[p], d);
+      const dim3 grid = grid_for(t.slots_f[p], d, p);
       const bool rec = !t.ev.empty() && row0 == 0;
       if (rec) cudaEventRecord(t.ev[2 * p], st);
       if (!t.kf.empty()) {
@@ -514,7 +599,7 @@ tdq_status tiled_execute(TiledSweep& t, const SweepArgs& a0, int grad, cudaStrea
         d.op_begin = t.passes[p].op_begin;
         d.op_end = t.passes[p].op_end;
         set_pass(t, d, p);
-        const dim3 grid = grid_for(t.slots_r, d);
+        const dim3 grid = grid_for(t.slots_r, d, p);
         d.dbl = 0;  // reverse kernels: one buffer per state (see tiled_compile)
         const int u = np + (np - 2 - p);  // launch unit of this reverse pass
         const bool rec = !t.ev.empty() && row0 == 0;
@@ -534,7 +619,7 @@ tdq_status tiled_execute(TiledSweep& t, const SweepArgs& a0, int grad, cudaStrea
     (*launches)++;
     if (a.output == TDQ_OUT_STATE || a.output == TDQ_OUT_PROBS) {
       const int64_t tot = (int64_t)nr << t.n;
-      k1_state_out<<<(unsigned)std::min<int64_t>((tot + 255) / 256, 8192), 256, 0, st>>>(a, d, nr);
+      k1_state_out<<<(unsigned)std::min<int64_t>((tot + 255) / 256, 2432), 256, 0, st>>>(a, d, nr);
       (*launches)++;
     }
     cudaError_t e = cudaGetLastError();

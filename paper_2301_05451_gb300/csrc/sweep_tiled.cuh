@@ -7,6 +7,8 @@
 // one HBM read and write of the state per pass instead of one per gate.
 // Gates acting on bits outside S are still absorbed when those bits are
 // constant on the tile: diagonal gates (RZ, Z, CZ, RZZ) and CNOT controls.
+// Programs specialised to the circuit run in a linear frame of the index
+// (lin_program.h): S is then a k-dimensional subspace and CNOTs are free.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -14,6 +16,7 @@
 #include <vector>
 
 #include "engine.cuh"
+#include "lin_program.h"
 #include "sweep_common.cuh"
 #include "tdq_internal.h"
 
@@ -40,7 +43,7 @@ inline double gate_dot_flops(int kind, double dim) {
 }
 
 struct TiledPass {
-  uint32_t smask;  // bit positions held in the tile
+  uint32_t smask;  // bit positions held in the tile (linear frame: its pivots)
   int op_begin, op_end;
 };
 
@@ -73,6 +76,8 @@ struct TiledSweep {
   // shared-memory bytes of each pass's gradient rows
   std::vector<const void*> kf, kr;
   std::vector<int> spec_gbytes;
+  uint32_t* d_lin = nullptr;             // specialised programs: place of a basis index (SweepArgs::lin)
+  int quarter = 0;
   int nthreads = 256, nthreads_r = 256;  // forward / reverse kernels
   std::vector<size_t> smem_f;            // per forward kernel
   size_t smem_r = 0;
@@ -123,8 +128,13 @@ tdq_status tiled_plan(TiledSweep& t, const tdq_circuit* c, const std::vector<Swe
                       const std::vector<int>& ps_gate, int rows, bool adj, int tile_qubits, int fb, int rb,
                       TiledHost& h);
 
+// A tiled plan in a linear frame: t's pass masks and launch shape, and the program.
+tdq_status tiled_lin_plan(TiledSweep& t, const tdq_circuit* c, const std::vector<SweepOp>& ops, int rows, bool adj,
+                          int tile_qubits, int fb, int rb, bool exact, LinProgram& prog);
+
+// lin: the program of tiled_lin_plan, or NULL for the generic kernels
 tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<SweepOp>& ops,
-                         const std::vector<int>& ps_gate, int rows, bool adj, int tile_qubits, bool interpret,
+                         const std::vector<int>& ps_gate, int rows, bool adj, int tile_qubits, const LinProgram* lin,
                          int fb, int rb, double* bytes_row);
 tdq_status tiled_execute(TiledSweep& t, const SweepArgs& a, int grad, cudaStream_t st,
                          int* launches);
