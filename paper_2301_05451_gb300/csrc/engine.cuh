@@ -19,8 +19,13 @@ constexpr int kMaxRegBits = 4;
 // and tiled programs, and whole-state programs specialised to a circuit
 constexpr int kFwdRegBits = 4;
 constexpr int kRevRegBits = 3;
-constexpr int kSpecFwdRegBits = 2;
-constexpr int kSpecRevRegBits = 2;
+// Whole-state programs specialised to a circuit: narrow passes while a few
+// hundred groups are all a pass has (their straight-line code is shorter, and
+// fetching it is what a small state waits for: 9 qubits, 1001 rows, values,
+// 32 us at 2 bits, 36 at 3; 6 qubits, value and gradient, 17.9 against 19.7),
+// 3 bits from 11 qubits (12 qubits, 256 rows, value and gradient: 86 us at 3/3
+// bits, 100 at 2/2, 85 at 4/4, which has twice the code).
+__host__ __device__ constexpr int spec_reg_bits(int n) { return n >= 11 ? 3 : 2; }
 // tiled programs specialised to the circuit: their passes stream the state
 // through HBM, and wide register passes mean fewer shared-memory round trips
 // (the 20-qubit ladder, 64 rows: 6.22 ms at 4/4 bits, 6.60 at 3/4, 6.83 at
@@ -28,6 +33,11 @@ constexpr int kSpecRevRegBits = 2;
 // forward and cost 20 % in reverse)
 constexpr int kTiledSpecFwdRegBits = 4;
 constexpr int kTiledSpecRevRegBits = 4;
+// Reverse passes of a tiled program with at most this many tiles per SM in a
+// launch take 3 bits: each SM then runs the code once or twice, and fetching
+// it decides (17-qubit ladder, 5 rows, 1.05 tiles per SM: 214 us at 3 bits, 248
+// at 4; 16 qubits, 24 rows, 2.5 tiles per SM: 224 against 218).
+constexpr int kTiledFewTiles = 2;
 // Gradient slots at most per reverse register pass of a specialised program
 // (its accumulators live in registers beside the pass's amplitudes: 64 + 16 of
 // the 128 that two CTAs of 256 threads leave a thread; at 8 the 20-qubit
@@ -544,6 +554,19 @@ __device__ __forceinline__ void adj_group(c2* psi, c2* lam, const RegPass& rp, c
   }
 }
 
+// Chained launches: the kernel may be dispatched while the one before it in
+// the stream is finishing.  What it does before chain_wait must not read what
+// that kernel writes, nor may it write anything.
+#if defined(__CUDACC__) || defined(__CUDACC_RTC__)
+__device__ __forceinline__ void chain_dispatch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+#else
+inline void chain_dispatch() {}
+inline void chain_wait() {}
+inline void prefetch_l2(const void*) {}
+#endif
+
 // Asynchronous 8-byte global -> shared copy (cp.async, completed in groups).
 // A host compiler (the kernels' CPU check) copies at once.
 #if defined(__CUDACC__) || defined(__CUDACC_RTC__)
@@ -639,17 +662,25 @@ __device__ __forceinline__ OpMat build_recipe(const SweepArgs& a, const SweepOp*
 // parity(FR & j) xor a sign word's top bit that the group shares.
 //
 // Rotations are applied without their common factor, two fused multiply-adds
-// per pair instead of four products: for |cos| >= |sin| the pair becomes
-// (a0 - t a1, a1 + t a0) with t = sin / cos and the factor cos is left to the
-// pass's scale; else (u a0 - a1, u a1 + a0) with u = cos / sin and factor sin.
-// |t|, |u| <= 1, so a pass grows the amplitudes by at most sqrt(2) per gate.
+// per pair instead of four products: the pair becomes (a0 - t a1, a1 + t a0)
+// with t = sin / cos of the half angle, and the factor cos is left to the
+// pass's scale.  Past 45 degrees the rotation by 90 is split off, which is a
+// Pauli product: it is not applied, but kept as the row's frame (the state in
+// memory is the true one up to it), where it flips the signs of later gates'
+// angles -- known once per row, in build_coefs -- and moves the index at which
+// the observable is read.  So |t| <= 1, a pass grows the amplitudes by at most
+// sqrt(2) per gate, and every gate has one form.  Programs that return
+// amplitudes (exact) need the frame's phase too; they keep a second form
+// instead, (u a0 - a1, u a1 + a0) with u = cos / sin and factor sin.
 // What bounds the tiled kernels is issue slots and latency at 16 warps per SM
 // (ncu, 20-qubit ladder: issue 52 % forward, 45 % reverse, FMA pipe 31-36 %,
 // DRAM 41 % of its rate).  Against one fused 2 x 2 product per qubit forward
 // and one op per gate in reverse, with CNOTs as register moves: 20-qubit
-// ladder, 64 rows, value and gradient 12.74 -> 6.17 ms (tile passes 8 -> 6);
-// its 481 shifted circuits 26.3 -> 13.0 ms; 16 qubits of random gates, 24
-// rows, 611 -> 223 us; state vectors of 20 qubits, 16 rows, 1024 -> 644 us.
+// ladder, 64 rows, value and gradient 12.74 -> 6.17 ms (tile passes 8 -> 6),
+// 5.5 with one form per rotation (a second one behind a branch had a third of
+// the code); its 481 shifted circuits 26.3 -> 13.0 -> 11.3 ms; 16 qubits of
+// random gates, 24 rows, 611 -> 223 us; state vectors of 20 qubits, 16 rows,
+// 1024 -> 644 -> 590 us.
 
 __device__ __forceinline__ float sx(float v, uint32_t sign) { return __uint_as_float(__float_as_uint(v) ^ sign); }
 
@@ -658,25 +689,35 @@ __host__ __device__ constexpr int cpar(int v) { return ((v >> 3) ^ (v >> 2) ^ (v
 // sin x and cos x as unevaluated sums hi + lo of two floats, correct to about
 // 2^-28: the coefficients' errors are the same for every amplitude, so they,
 // not the rounding of single amplitudes, decide the error of an expectation.
-// x is reduced by multiples of pi/2 in double (a handful of FP64
-// instructions); the remainder's Taylor series (to r^9 / r^10, |r| <= pi/4)
-// runs in float with its leading terms kept as two floats.
+// x is reduced by multiples of pi/2 (Cody and Waite: the constant in pieces of
+// 8 and 11 bits and a rest, so that the products are exact); the remainder's
+// Taylor series (to r^9 / r^10, |r| <= pi/4) has its leading terms as two
+// floats.  All in float: FP64 runs at a 64th of the rate, and the tables of
+// 1001 nine-qubit rows alone would take 4 us of it.
 struct SinCos {
   float s, sl, c, cl;
+  bool u;  // the nearest multiple of pi/2 is odd: |sin| >= |cos|
 };
+// rare: angles too large for the reduction (or not finite)
+static __device__ __noinline__ SinCos sincos2_far(float x) {
+  double s, c;
+  sincos((double)x, &s, &c);
+  SinCos r = {(float)s, 0.f, (float)c, 0.f, fabs(s) > fabs(c)};
+  r.sl = (float)(s - (double)r.s);
+  r.cl = (float)(c - (double)r.c);
+  return r;
+}
+__device__ __forceinline__ bool reducible(float x) { return fabsf(x) <= 6000.f; }
+__device__ __forceinline__ float quadrant(float x) { return rintf(x * 0.636619772f); }
+
 __device__ __forceinline__ SinCos sincos2(float x) {
-  const double y = (double)x;
-  const double k = rint(y * 0.63661977236758134308);
-  if (fabs(y) > 1e5) {  // rare: the reduction below needs a small multiple
-    double s, c;
-    sincos(y, &s, &c);
-    SinCos r = {(float)s, 0.f, (float)c, 0.f};
-    r.sl = (float)(s - (double)r.s);
-    r.cl = (float)(c - (double)r.c);
-    return r;
-  }
-  const double rd = fma(k, -1.57079632679489661923, y);
-  const float r = (float)rd, rl = (float)(rd - (double)r);
+  if (!reducible(x)) return sincos2_far(x);
+  const float k = quadrant(x);
+  const float r1 = fmaf(-k, 1.5703125f, x), t = k * 4.83751297e-4f;
+  const float r2 = r1 - t, tb = r2 - r1;
+  const float re = (r1 - (r2 - tb)) - (t + tb);  // r1 - t = r2 + re
+  const float rc = fmaf(-k, 7.54979013e-8f, re);
+  const float r = r2 + rc, rl = rc - (r - r2);
   const float p = r * r, pl = fmaf(r, r, -p) + 2.f * r * rl;
   // sin = r + (rl + r^3 (-1/6 + p/120 - p^2/5040 + p^3/362880))
   const float sp = fmaf(p, fmaf(p, fmaf(p, 2.7557319e-6f, -1.98412698e-4f), 8.33333333e-3f), -0.166666667f);
@@ -689,6 +730,7 @@ __device__ __forceinline__ SinCos sincos2(float x) {
   const float c0 = c00 + cx0, c1 = cx0 - (c0 - c00);
   const int q = (int)k & 3;
   SinCos o;
+  o.u = (q & 1) != 0;
   o.s = (q & 1) ? c0 : s0;
   o.sl = (q & 1) ? c1 : s1;
   o.c = (q & 1) ? s0 : c0;
@@ -697,65 +739,122 @@ __device__ __forceinline__ SinCos sincos2(float x) {
   if (q == 1 || q == 2) { o.c = -o.c; o.cl = -o.cl; }
   return o;
 }
-
-// Table row of a rotation: {t or u, left-out factor (two floats), u form ? ~0 : 0}.
-__device__ __forceinline__ float4 rot_coef(float ang) {
-  SinCos r = sincos2(0.5f * ang);
-  const bool u = fabsf(r.s) > fabsf(r.c);
-  if (u) r = {r.c, r.cl, r.s, r.sl};
-  const float t = r.s / r.c;  // (s + sl) / (c + cl), rounded once
-  const float e = (fmaf(-t, r.c, r.s) + fmaf(-t, r.cl, r.sl)) / r.c;
-  return make_float4(t + e, r.c, r.cl, __uint_as_float(u ? 0xffffffffu : 0u));
+// sincos2's u alone.
+__device__ __forceinline__ bool past_45(float x) {
+  return reducible(x) ? ((int)quadrant(x) & 1) != 0 : sincos2_far(x).u;
 }
 
-__device__ __forceinline__ float coef_angle(const SweepArgs& a, const SweepOp* ops, int code, int64_t b, int k,
-                                            int* bad) {
-  const int gi = code >> 2, j = code & 3;
-  float v = op_angle(ops[gi], j, a.params, a.pstride, a.inputs, a.F, b, bad);
+// Table row of a rotation: {t or cos / sin, left-out factor (two floats),
+// second form ? ~0 : 0}.
+__device__ __forceinline__ float4 rot_coef(float ang) {
+  SinCos r = sincos2(0.5f * ang);
+  if (r.u) r = {r.c, r.cl, r.s, r.sl, true};
+  const float t = r.s / r.c;  // (s + sl) / (c + cl), rounded once
+  const float e = (fmaf(-t, r.c, r.s) + fmaf(-t, r.cl, r.sl)) / r.c;
+  return make_float4(t + e, r.c, r.cl, __uint_as_float(r.u ? 0xffffffffu : 0u));
+}
+
+__device__ __forceinline__ float coef_angle(const SweepArgs& a, const CoefRec& q, int64_t b, int k, int* bad) {
+  float v;
+  if (q.src >= 0) v = a.params[b * a.pstride + q.src];
+  else if (q.src == -1) v = q.fixed;
+  else v = a.inputs[b * a.F + (-2 - q.src)];
+  if (!isfinite(v)) *bad = 1;
   if (k > 0) {
     const int e = (k - 1) >> 1;
-    if (a.ps_gate[e] == gi && a.ps_ang[e] == j) v += ((k - 1) & 1) ? -kHalfPiF : kHalfPiF;
+    if (4 * a.ps_gate[e] + a.ps_ang[e] == q.code) v += ((k - 1) & 1) ? -kHalfPiF : kHalfPiF;
   }
   return v;
 }
 
-// Gate-tensor table of a specialised program, built by the whole CTA for row
-// b (shift copy k); rows r0.. of the recipes go to mats[0..nrec).  Rotations:
-// see rot_coef.  Phases: {cos a/2, sin a/2, cos a, sin a}.  Scale of a
-// register pass: {Re S, Im S, 1 / |S|, 0}, S the product of its gates'
-// left-out factors, multiplied out in double (an exact program's RX in the u
-// form leaves -i sin; its phase does not reach expectations).  The caller
-// synchronises afterwards.
-__device__ __forceinline__ void build_coefs(const SweepArgs& a, const SweepOp* ops, const int* rec_ptr,
-                                            const int* rec_ops, int r0, int nrec, float4* mats, int64_t b, int k,
+// Gate-tensor table of a specialised program: mats[nrec], then for programs
+// with a frame every row's sign bit sig[nrec], the rotations past 45 degrees as
+// a bit set, and the index part of the frame at the program's end.
+__host__ __device__ __forceinline__ int coef_words(int nrec, int nrot) { return nrot ? nrec + (nrot + 31) / 32 + 1 : 0; }
+__host__ __device__ __forceinline__ int coef_bytes(int nrec, int nrot) {
+  return 16 * nrec + ((4 * coef_words(nrec, nrot) + 15) & ~15);
+}
+__device__ __forceinline__ uint32_t coef_frame(const float4* mats, int nrec, int nrot) {
+  return nrot ? reinterpret_cast<const uint32_t*>(mats + nrec)[coef_words(nrec, nrot) - 1] : 0u;
+}
+
+// Builds the table, by the whole CTA, for row b (shift copy k): records r0..
+// of a.coef to mats[0..nrec).  Rotations: see rot_coef, with a frame {t,
+// factor, factor, sign bit}, t with the frame's sign.  Phases: {cos a/2, sin
+// a/2, cos a, sin a}, a with the frame's sign.  Scale of a register pass: {Re
+// S, Im S, 1 / |S|, 0}, S the product of its gates' left-out factors in two
+// floats (an exact program's RX in the second form leaves -i sin; its phase
+// does not reach expectations).  The caller synchronises afterwards.  Small
+// states wait for this: records hold what a row needs (two dependent reads,
+// record and parameter), and signs and scales follow one barrier.
+__device__ __forceinline__ void build_coefs(const SweepArgs& a, int r0, int nrec, float4* mats, int64_t b, int k,
                                             int* bad) {
+  const CoefRec* rec = a.coef + r0;
+  uint32_t* sig = reinterpret_cast<uint32_t*>(mats + nrec);
+  uint32_t* past = sig + nrec;
+  const int words = (a.nrot + 31) / 32;
+  for (int j0 = (int)(threadIdx.x & ~31u); j0 < a.nrot; j0 += blockDim.x) {
+    const int j = j0 + (int)(threadIdx.x & 31u);
+    const bool u = j < a.nrot && past_45(0.5f * coef_angle(a, a.rot[j], b, k, bad));
+    const uint32_t bits = __ballot_sync(0xffffffffu, u);
+    if ((threadIdx.x & 31u) == 0) past[j0 >> 5] = bits;
+  }
   for (int r = threadIdx.x; r < nrec; r += blockDim.x) {
-    const int e0 = rec_ptr[r0 + r], type = rec_ops[e0] & 255;
-    if (type != C_ROT && type != C_PHASE) continue;
-    const float v = coef_angle(a, ops, rec_ops[e0 + 1], b, k, bad);
-    if (type == C_ROT) {
-      mats[r] = rot_coef(v);
-    } else {
+    const CoefRec q = rec[r];
+    if (q.type == C_ROT) {
+      mats[r] = rot_coef(coef_angle(a, q, b, k, bad));
+    } else if (q.type == C_PHASE) {
+      const float v = coef_angle(a, q, b, k, bad);
       const SinCos h = sincos2(0.5f * v), f = sincos2(v);
       mats[r] = make_float4(h.c, h.s, f.c, f.s);
     }
   }
   __syncthreads();
   for (int r = threadIdx.x; r < nrec; r += blockDim.x) {
-    const int e0 = rec_ptr[r0 + r], e1 = rec_ptr[r0 + r + 1], type = rec_ops[e0] & 255;
-    if (type == C_ROT || type == C_PHASE) continue;
-    const int nh = rec_ops[e0] >> 8;  // factors 1 / sqrt 2
-    double S = (nh & 1) ? 0.70710678118654752440 : 1.0;
-    for (int i = nh >> 1; i > 0; i--) S *= 0.5;
-    int turns = 0;  // factors -i
-    for (int e = e0 + 1; e < e1; e++) {
-      const float4 q = mats[rec_ops[e] >> 1];
-      S *= (double)q.y + (double)q.z;
-      turns += (rec_ops[e] & 1) && __float_as_uint(q.w) != 0u ? 1 : 0;
+    const CoefRec q = rec[r];
+    if (q.type == C_ROT || q.type == C_PHASE) {
+      if (!a.nrot) continue;
+      int flips = 0;
+      for (int w = 0; w < words; w++) flips += __popc(past[w] & a.rot_flips[(size_t)(r0 + r) * words + w]);
+      const uint32_t sign = (uint32_t)flips << 31;
+      sig[r] = sign;
+      float4 m = mats[r];
+      if (q.type == C_ROT) {  // past 45 degrees: the rotation by 90 less, t = -cos / sin
+        mats[r].x = sx(m.x, sign ^ (__float_as_uint(m.w) & 0x80000000u));
+        mats[r].w = __uint_as_float(sign);
+      } else {
+        mats[r].y = sx(m.y, sign);
+        mats[r].w = sx(m.w, sign);
+      }
+      continue;
     }
-    c2 z = {(float)S, 0.f};
-    if (type == C_NORM_EXACT) z = quarter_turns(z, -turns & 3);
-    mats[r] = make_float4(z.x, z.y, (float)(1.0 / fabs(S)), 0.f);
+    const int nh = q.type >> 8;  // factors 1 / sqrt 2 = 0.70710678 + 1.21e-8
+    float S = (nh & 1) ? 0.70710678f : 1.f, Sl = (nh & 1) ? 1.21016175e-8f : 0.f;
+    for (int i = nh >> 1; i > 0; i--) {
+      S *= 0.5f;
+      Sl *= 0.5f;
+    }
+    int turns = 0;  // factors -i
+    for (int e = 0; e < q.src; e++) {
+      const int code = a.norm[q.code + e];
+      const float4& m = mats[code >> 1];  // (y, z: not touched above)
+      const float y = m.y, z = m.z, p = S * y;
+      Sl = fmaf(S, y, -p) + fmaf(S, z, Sl * y);
+      S = p + Sl;
+      Sl -= S - p;
+      if ((code & 1) && !a.nrot) turns += __float_as_uint(m.w) != 0u ? 1 : 0;
+    }
+    c2 z = {S, 0.f};
+    if ((q.type & 255) == C_NORM_EXACT) z = quarter_turns(z, -turns & 3);
+    mats[r] = make_float4(z.x, z.y, 1.f / fabsf(S), 0.f);
+  }
+  if (a.nrot && threadIdx.x < 32) {  // the index part of the frame at the end
+    uint32_t m = 0;
+    for (int j = threadIdx.x; j < a.nrot; j += 32)
+      if ((past[j >> 5] >> (j & 31)) & 1u) m ^= a.rot_x[j];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m ^= __shfl_xor_sync(0xffffffffu, m, o);
+    if (threadIdx.x == 0) past[words] = m;
   }
 }
 

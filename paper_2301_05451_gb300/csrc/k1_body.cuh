@@ -39,7 +39,7 @@ struct TiledDev {
   int row0;
   int nrows;           // rows of the chunk: units are (row, tile), row-major
   int gbytes;          // shared-memory bytes of the gradient partial sums
-  int dbl;             // 1: two tile buffers per state (loads overlap compute)
+  int dbl;             // 1: two tile buffers in the forward kernels (loads overlap compute)
 };
 
 // Spread the bits of t over the positions of mask (lowest first).
@@ -53,8 +53,7 @@ __device__ __forceinline__ uint32_t deposit(uint32_t t, uint32_t mask) {
 struct TileShared {
   c2* psi;
   c2* lam;
-  c2* psi2;     // second buffers (double-buffered loads), or NULL
-  c2* lam2;
+  c2* psi2;     // second state buffer (double-buffered loads), or NULL
   OpMat* mats;  // [recipes of the pass] (specialised programs: float4 rows)
   DOp* dops;    // [decoded ops of the pass]
   double* red;
@@ -73,16 +72,19 @@ __host__ __device__ __forceinline__ size_t k1_smem_bytes(int k, int L, int npsi,
          32 + 16;
 }
 
+// Specialised programs have the tile's size and buffers as constants (kK tile
+// bits, kBuffers state buffers of the forward kernels), so that lambda and
+// the second buffer are immediate offsets.
+template <class Prog>
 __device__ __forceinline__ TileShared carve(unsigned char* raw, int k, int L, int npsi, int nlam, int mbytes,
                                             int ndops, int ng, int gbytes) {
   TileShared s;
-  const int nloc = 1 << k;
+  const int nloc = 1 << (Prog::kSpecialised ? Prog::kK : k);
   c2* p = reinterpret_cast<c2*>(raw);
   s.psi = p;
   s.psi2 = npsi > 1 ? p + nloc : nullptr;
   p += npsi * nloc;
   s.lam = nlam > 0 ? p : nullptr;
-  s.lam2 = nlam > 1 ? p + nloc : nullptr;
   p += nlam * nloc;
   s.mats = reinterpret_cast<OpMat*>(p);
   s.dops = reinterpret_cast<DOp*>(reinterpret_cast<unsigned char*>(p) + mbytes);
@@ -95,21 +97,22 @@ __device__ __forceinline__ TileShared carve(unsigned char* raw, int k, int L, in
 }
 
 __device__ __forceinline__ uint32_t gidx(const TileShared& s, uint32_t base, uint32_t j, int L) {
-  return base + (uint32_t)s.off[j >> L] + (j & ((1u << L) - 1u));
+  return base ^ (uint32_t)s.off[j >> L] ^ (j & ((1u << L) - 1u));
 }
 
 // Diagonal weight of output group g at basis index x: from the table of
 // every group's diagonal when the compile made one (read through L2, the
 // same for every row), else from the group's Z-product terms.
+template <class Prog>
 __device__ __forceinline__ float obs_weight(const SweepArgs& a, int g, uint32_t x) {
-  if (a.odiag) return a.odiag[((size_t)g << a.n) + x];
+  if (Prog::kDiag || a.odiag) return a.odiag[((size_t)g << a.n) + x];
   return diag_weight(a.terms, a.group_ptr[g], a.group_ptr[g + 1], x);
 }
 
 // Bytes of a pass's gate tensors.
 template <class Prog>
-__device__ __forceinline__ int k1_mat_bytes(const TiledDev& t) {
-  return t.nrec * (int)(Prog::kSpecialised ? sizeof(float4) : sizeof(OpMat));
+__device__ __forceinline__ int k1_mat_bytes(const SweepArgs& a, const TiledDev& t) {
+  return Prog::kSpecialised ? coef_bytes(t.nrec, a.nrot) : t.nrec * (int)sizeof(OpMat);
 }
 
 // Per-CTA set-up: offsets, local bits, this row's gate tensors (K0), the
@@ -122,7 +125,7 @@ __device__ __forceinline__ void k1_setup(const SweepArgs& a, const TiledDev& t, 
   if (threadIdx.x < 32) s.loc[threadIdx.x] = t.loc[threadIdx.x];
   // (interpreted programs: shifted gates are numbered in pass order, tiled_compile)
   if constexpr (Prog::kSpecialised)
-    build_coefs(a, t.ops, t.rec_ptr, t.rec_ops, t.rec0, t.nrec, reinterpret_cast<float4*>(s.mats), b, kk, bad);
+    build_coefs(a, t.rec0, t.nrec, reinterpret_cast<float4*>(s.mats), b, kk, bad);
   else
     for (int i = threadIdx.x; i < t.nrec; i += blockDim.x)
       s.mats[i] = build_recipe(a, t.ops, t.rec_ptr, t.rec_ops, t.rec0 + i, b, kk, bad);
@@ -135,29 +138,31 @@ __device__ __forceinline__ void k1_setup(const SweepArgs& a, const TiledDev& t, 
 // Gate program decoded at run time; gradient shares in FP64 per (recipe, angle).
 struct InterpTile {
   static constexpr bool kSpecialised = false;
-  static constexpr bool kFirst = false, kSecond = false;
+  static constexpr bool kFirst = false, kSecond = false, kDiag = false;
+  static constexpr int kK = 0, kN = 30, kBuffers = 0, kGroups = 0;
   __device__ __forceinline__ static bool in_first(uint32_t) { return true; }
   // f(shared-memory slot, global index) for this thread's elements of a tile
   template <int NT, class F>
   __device__ __forceinline__ static void every(const TiledDev& t, const TileShared& s, uint32_t base, F&& f) {
     for (uint32_t j = threadIdx.x; j < (1u << t.k); j += blockDim.x) f(swz(j), gidx(s, base, j, t.L));
   }
-  __device__ __forceinline__ static void forward(const TiledDev& t, const TileShared& s, uint32_t base) {
+  // buf: offset of the state buffer in use
+  __device__ __forceinline__ static void forward(const TiledDev& t, const TileShared& s, uint32_t base, uint32_t buf) {
     const int ngroups = 1 << (t.k - kFwdRegBits);
     for (int i = 0; i < t.nfp; i++) {
       const RegPass rp = t.fp[i];
       for (int grp = threadIdx.x; grp < ngroups; grp += blockDim.x)
-        fwd_group<kFwdRegBits>(s.psi, rp, s.dops, s.mats, base, (uint32_t)grp);
+        fwd_group<kFwdRegBits>(s.psi + buf, rp, s.dops, s.mats, base, (uint32_t)grp);
       __syncthreads();
     }
   }
-  __device__ __forceinline__ static void reverse(const TiledDev& t, const TileShared& s, uint32_t base) {
+  __device__ __forceinline__ static void reverse(const TiledDev& t, const TileShared& s, uint32_t base, uint32_t buf) {
     const int ngroups = 1 << (t.k - kRevRegBits);
     double* gp = reinterpret_cast<double*>(s.gpart);
     for (int i = t.nbp - 1; i >= 0; i--) {
       const RegPass rp = t.bp[i];
       for (int g0 = 0; g0 < ngroups; g0 += blockDim.x)
-        adj_group<kRevRegBits, false>(s.psi, s.lam, rp, s.dops, s.mats, base, (uint32_t)(g0 + threadIdx.x),
+        adj_group<kRevRegBits, false>(s.psi + buf, s.lam, rp, s.dops, s.mats, base, (uint32_t)(g0 + threadIdx.x),
                                          g0 + (int)threadIdx.x < ngroups, gp);
       __syncthreads();
     }
@@ -174,19 +179,27 @@ struct InterpTile {
   }
 };
 
+// Element x of a state in HBM (a 32-bit byte offset where the state is small
+// enough for one).
+template <class Prog>
+__device__ __forceinline__ c2* elem(c2* g, uint32_t x) {
+  if (Prog::kSpecialised && Prog::kN <= 29) return reinterpret_cast<c2*>(reinterpret_cast<unsigned char*>(g) + (x << 3));
+  return g + x;
+}
+
 // Starts the asynchronous load of tile `base` of state g into buffer buf
 // (one commit group per thread).
 // sparse: only the elements on the first pass's space; the others are zero.
 template <int NT, class Prog>
-__device__ __forceinline__ void k1_issue(c2* buf, const c2* g, const TiledDev& t, const TileShared& s, uint32_t base,
+__device__ __forceinline__ void k1_issue(c2* buf, c2* g, const TiledDev& t, const TileShared& s, uint32_t base,
                                          bool sparse = false) {
   if (Prog::kSecond && sparse)
     Prog::template every<NT>(t, s, base, [&](uint32_t j, uint32_t x) {
-      if (Prog::in_first(x)) cp_async8(&buf[j], &g[x]);
+      if (Prog::in_first(x)) cp_async8(&buf[j], elem<Prog>(g, x));
       else buf[j] = {0.f, 0.f};
     });
   else
-    Prog::template every<NT>(t, s, base, [&](uint32_t j, uint32_t x) { cp_async8(&buf[j], &g[x]); });
+    Prog::template every<NT>(t, s, base, [&](uint32_t j, uint32_t x) { cp_async8(&buf[j], elem<Prog>(g, x)); });
 }
 
 // The (row, tile) units of this CTA: a contiguous range of the row-major
@@ -226,26 +239,41 @@ __device__ __forceinline__ void k1_for_segments(const TiledDev& t, F&& f) {
 template <int NT, bool FIRST, bool LAST, bool GRAD, class Prog>
 __device__ __forceinline__ void k1_forward_body(const SweepArgs& a, const TiledDev& t, int store) {
   extern __shared__ __align__(16) unsigned char raw[];
-  const TileShared s = carve(raw, t.k, t.L, (FIRST || !t.dbl) ? 1 : 2, (GRAD && LAST) ? 1 : 0, k1_mat_bytes<Prog>(t),
-                             t.ndops, a.n_groups, t.gbytes);
+  const int nbuf = FIRST ? 1 : Prog::kSpecialised ? Prog::kBuffers : (t.dbl ? 2 : 1);
+  const TileShared s = carve<Prog>(raw, t.k, t.L, nbuf, (GRAD && LAST) ? 1 : 0, k1_mat_bytes<Prog>(a, t), t.ndops,
+                                   a.n_groups, t.gbytes);
   const uint32_t dim = 1u << t.n;
   const uint32_t other = (dim - 1u) & ~t.smask;
+  // the gate tensors and tables are built while the kernel before finishes
+  // (the first kernel of an execution is launched unchained): 17-qubit ladder,
+  // 5 rows, 7 passes of 15 to 50 us, 215 -> 143 us; 16 qubits, 24 rows, 218 -> 168
+  chain_dispatch();
+  bool waited = false;
   k1_for_segments(t, [&](int lr, int tile0, int tile1) {
     const int row = t.row0 + lr;
     const int64_t b = row / a.ps_copies;
     const int kk = row % a.ps_copies;
     int bad = 0;
     k1_setup<Prog>(a, t, s, b, kk, &bad);
+    if (!waited) chain_wait();
+    waited = true;
     if (bad) atomicOr(a.status, 1 << TDQ_ERR_NONFINITE);
     c2* gpsi = t.psi + (size_t)lr * dim;
     c2* glam = GRAD ? t.lam + (size_t)lr * dim : nullptr;
-    if (!FIRST && t.dbl && tile0 < tile1) {
+    // index part of the row's frame: the observable of y is read at y ^ mu
+    uint32_t mu = 0u;
+    if constexpr (Prog::kSpecialised && LAST) {
+      mu = coef_frame(reinterpret_cast<const float4*>(s.mats), t.nrec, a.nrot);
+      if (a.row_frame && threadIdx.x == 0) a.row_frame[lr] = mu;
+    }
+    if (!FIRST && nbuf == 2 && tile0 < tile1) {
       k1_issue<NT, Prog>(s.psi, gpsi, t, s, deposit((uint32_t)tile0, other), !a.init);
       cp_async_commit();
     }
     for (int tile = tile0, it = 0; tile < tile1; tile++, it++) {
       const uint32_t base = deposit((uint32_t)tile, other);
-      TileShared sc = s;
+      // offset of the state buffer in use
+      const uint32_t buf = !FIRST && nbuf == 2 && (it & 1) ? (uint32_t)(s.psi2 - s.psi) : 0u;
       // this thread's elements: f(shared-memory slot, global index)
       auto every = [&](auto&& f) { Prog::template every<NT>(t, s, base, f); };
       if (FIRST && !Prog::kSpecialised && !a.init && base != 0u) {
@@ -263,12 +291,11 @@ __device__ __forceinline__ void k1_forward_body(const SweepArgs& a, const TiledD
       if (FIRST) {
         if (a.init) {
           const c2* p0 = a.init + b * a.init_stride;
-          every([&](uint32_t j, uint32_t x) { sc.psi[j] = quarter_turns(p0[x], a.quarter); });
+          every([&](uint32_t j, uint32_t x) { s.psi[j] = quarter_turns(p0[x], a.quarter); });
         } else {
-          every([&](uint32_t j, uint32_t x) { sc.psi[j] = quarter_turns({x == 0u ? 1.f : 0.f, 0.f}, a.quarter); });
+          every([&](uint32_t j, uint32_t x) { s.psi[j] = quarter_turns({x == 0u ? 1.f : 0.f, 0.f}, a.quarter); });
         }
-      } else if (t.dbl) {
-        sc.psi = (it & 1) ? s.psi2 : s.psi;
+      } else if (nbuf == 2) {
         if (tile + 1 < tile1) {  // the buffer of the previous tile is free (barrier at the loop end)
           k1_issue<NT, Prog>((it & 1) ? s.psi : s.psi2, gpsi, t, s, deposit((uint32_t)(tile + 1), other), !a.init);
           cp_async_commit();
@@ -282,57 +309,39 @@ __device__ __forceinline__ void k1_forward_body(const SweepArgs& a, const TiledD
         cp_async_wait<0>();
       }
       __syncthreads();
-      Prog::forward(t, sc, base);
-      auto store_both = [&] {  // nothing reads them after the first pass's reverse sweep
-        if (FIRST && Prog::kSpecialised) return;
-        every([&](uint32_t j, uint32_t x) {
-          if (Prog::kSecond && !a.init && !Prog::in_first(x)) return;
-          gpsi[x] = sc.psi[j];
-          glam[x] = sc.lam[j];
-        });
-      };
-      if (LAST && GRAD && a.output == TDQ_OUT_EXPVAL && a.n_groups == 1) {
-        // one output group: its diagonal weight d(x) gives both the value
-        // (sum |psi|^2 d) and lambda = w d psi in one pass over the tile
-        const float w = a.gw ? (float)a.gw[b] : 1.f;
-        float acc = 0.f;
-        every([&](uint32_t j, uint32_t x) {
-          const float d = obs_weight(a, 0, x);
-          const c2 v = sc.psi[j];
-          acc += (v.x * v.x + v.y * v.y) * d;
-          sc.lam[j] = {w * d * v.x, w * d * v.y};
-        });
-        acc = warp_sum_f(acc);
-        if ((threadIdx.x & 31) == 0) atomicAdd(&s.vsum[0], (double)acc);
-        __syncthreads();
-        Prog::reverse(t, sc, base);
-        store_both();
-      } else if (LAST && a.output == TDQ_OUT_EXPVAL) {
-        for (int g = 0; g < a.n_groups; g++) {
+      Prog::forward(t, s, base, buf);
+      if (LAST && a.output == TDQ_OUT_EXPVAL) {
+        // the observable's diagonal gives the values (sum |psi|^2 d) and, with
+        // gradients, lambda = sum_g w_g d_g psi (a thread's own elements: no
+        // barrier between the groups)
+        const int ng = Prog::kGroups == 1 ? 1 : a.n_groups;
+        for (int g = 0; g < ng; g++) {
           float acc = 0.f;
+          const float w = GRAD && a.gw ? (float)a.gw[b * ng + g] : 1.f;
           every([&](uint32_t j, uint32_t x) {
-            const c2 v = sc.psi[j];
-            acc += (v.x * v.x + v.y * v.y) * obs_weight(a, g, x);
+            const c2 v = s.psi[j ^ buf];
+            const float d = obs_weight<Prog>(a, g, x ^ mu);
+            acc += (v.x * v.x + v.y * v.y) * d;
+            if (GRAD) {
+              const c2 l = g ? s.lam[j] : c2{0.f, 0.f};
+              s.lam[j] = {fmaf(w * d, v.x, l.x), fmaf(w * d, v.y, l.y)};
+            }
           });
           acc = warp_sum_f(acc);
           if ((threadIdx.x & 31) == 0) atomicAdd(&s.vsum[g], (double)acc);
         }
         if (GRAD) {
-          every([&](uint32_t j, uint32_t x) {
-            float d = 0.f;
-            for (int g = 0; g < a.n_groups; g++) {
-              const float w = a.gw ? (float)a.gw[b * a.n_groups + g] : 1.f;
-              d += w * obs_weight(a, g, x);
-            }
-            const c2 v = sc.psi[j];
-            sc.lam[j] = {d * v.x, d * v.y};
-          });
           __syncthreads();
-          Prog::reverse(t, sc, base);
-          store_both();
+          Prog::reverse(t, s, base, buf);
+          if (!(FIRST && Prog::kSpecialised))  // nothing reads them after the first pass's reverse sweep
+            every([&](uint32_t j, uint32_t x) {
+              if (Prog::kSecond && !a.init && !Prog::in_first(x)) return;
+              *elem<Prog>(gpsi, x) = s.psi[j ^ buf];
+              *elem<Prog>(glam, x) = s.lam[j];
+            });
         }
       }
-      if (!(LAST && GRAD) && store) every([&](uint32_t j, uint32_t x) { gpsi[x] = sc.psi[j]; });
+      if (!(LAST && GRAD) && store) every([&](uint32_t j, uint32_t x) { *elem<Prog>(gpsi, x) = s.psi[j ^ buf]; });
       __syncthreads();
     }
     if (LAST && a.output == TDQ_OUT_EXPVAL) {
@@ -344,52 +353,51 @@ __device__ __forceinline__ void k1_forward_body(const SweepArgs& a, const TiledD
   });
 }
 
-// Reverse pass over the tiles of one pass (passes before the last); psi and
-// lambda of the next tile are read while the current one is computed.
+// Reverse pass over the tiles of one pass (passes before the last), one
+// buffer per state: two CTAs per SM overlap one's loads with the other's
+// compute.
 template <int NT, class Prog>
 __device__ __forceinline__ void k1_reverse_body(const SweepArgs& a, const TiledDev& t) {
   extern __shared__ __align__(16) unsigned char raw[];
-  const int nb = t.dbl ? 2 : 1;
-  const TileShared s = carve(raw, t.k, t.L, nb, nb, k1_mat_bytes<Prog>(t), t.ndops, a.n_groups, t.gbytes);
+  const TileShared s = carve<Prog>(raw, t.k, t.L, 1, 1, k1_mat_bytes<Prog>(a, t), t.ndops, a.n_groups, t.gbytes);
   const uint32_t dim = 1u << t.n;
   const uint32_t other = (dim - 1u) & ~t.smask;
+  chain_dispatch();
+  bool waited = false;
   k1_for_segments(t, [&](int lr, int tile0, int tile1) {
     const int row = t.row0 + lr;
     const int64_t b = row / a.ps_copies;
     int bad = 0;
     k1_setup<Prog>(a, t, s, b, 0, &bad);
+    if (!waited) chain_wait();
+    waited = true;
     c2* gpsi = t.psi + (size_t)lr * dim;
     c2* glam = t.lam + (size_t)lr * dim;
-    auto issue = [&](c2* psi, c2* lam, int tile) {
+    for (int tile = tile0; tile < tile1; tile++) {
       const uint32_t base = deposit((uint32_t)tile, other);
-      k1_issue<NT, Prog>(psi, gpsi, t, s, base);
-      k1_issue<NT, Prog>(lam, glam, t, s, base);
+      Prog::template every<NT>(t, s, base, [&](uint32_t j, uint32_t x) {
+        cp_async8(&s.psi[j], elem<Prog>(gpsi, x));
+        cp_async8(&s.lam[j], elem<Prog>(glam, x));
+      });
       cp_async_commit();
-    };
-    if (t.dbl && tile0 < tile1) issue(s.psi, s.lam, tile0);
-    for (int tile = tile0, it = 0; tile < tile1; tile++, it++) {
-      const uint32_t base = deposit((uint32_t)tile, other);
-      TileShared sc = s;
-      if (t.dbl) {
-        sc.psi = (it & 1) ? s.psi2 : s.psi;
-        sc.lam = (it & 1) ? s.lam2 : s.lam;
-        if (tile + 1 < tile1) {
-          issue((it & 1) ? s.psi : s.psi2, (it & 1) ? s.lam : s.lam2, tile + 1);
-          cp_async_wait<1>();
-        } else {
-          cp_async_wait<0>();
+      // the next tile's lines on their way to L2 meanwhile (a thread per
+      // 128-byte run of 16 amplitudes)
+      if (tile + 1 < tile1) {
+        const uint32_t next = deposit((uint32_t)(tile + 1), other);
+        for (uint32_t r = threadIdx.x; r < (1u << (t.k - t.L)); r += blockDim.x) {
+          const uint32_t x = gidx(s, next, r << t.L, t.L);
+          prefetch_l2(gpsi + x);
+          prefetch_l2(glam + x);
         }
-      } else {  // one buffer per state: load, then compute
-        issue(s.psi, s.lam, tile);
-        cp_async_wait<0>();
       }
+      cp_async_wait<0>();
       __syncthreads();
-      Prog::reverse(t, sc, base);
+      Prog::reverse(t, s, base, 0u);
       if (!Prog::kFirst)
         Prog::template every<NT>(t, s, base, [&](uint32_t j, uint32_t x) {
           if (Prog::kSecond && !a.init && !Prog::in_first(x)) return;
-          gpsi[x] = sc.psi[j];
-          glam[x] = sc.lam[j];
+          *elem<Prog>(gpsi, x) = s.psi[j];
+          *elem<Prog>(glam, x) = s.lam[j];
         });
       __syncthreads();
     }

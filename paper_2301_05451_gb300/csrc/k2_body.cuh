@@ -51,7 +51,7 @@ __host__ __device__ constexpr size_t k2_grad_bytes(bool specialised, int P, int 
 }
 
 // Row r of the batch (with parameter shift: sample r / copies, copy r % copies).
-// layout: psi[dim] | lambda[dim] (GRAD) | mats[nrec] | dops[ndops] | grad accumulators | red[32] | bad
+// layout: psi[dim] | lambda[dim] (GRAD) | mats[nrec] (specialised: coef_bytes) | dops[ndops] | grad accumulators | red[32] | bad
 template <int MF, int MB, bool GRAD, class Prog>
 __device__ __forceinline__ void k2_body(const SweepArgs& a, Prog prog, const DOp* gdops, int ndops,
                                         const int* rec_ptr, const int* rec_ops, int nrec, int r) {
@@ -61,7 +61,8 @@ __device__ __forceinline__ void k2_body(const SweepArgs& a, Prog prog, const DOp
   c2* lam = psi + dim;
   using Mat = typename Prog::Mat;
   Mat* mats = reinterpret_cast<Mat*>(psi + (GRAD ? 2 : 1) * dim);
-  DOp* dops = reinterpret_cast<DOp*>(mats + nrec);
+  DOp* dops = reinterpret_cast<DOp*>(reinterpret_cast<unsigned char*>(mats) +
+                                     (Prog::kSpecialised ? coef_bytes(nrec, a.nrot) : (int)sizeof(Mat) * nrec));
   unsigned char* gbase = reinterpret_cast<unsigned char*>(dops + ndops);
   const size_t gbytes = GRAD ? k2_grad_bytes(Prog::kSpecialised, a.P, blockDim.x) : 0;
   double* gacc = reinterpret_cast<double*>(gbase);
@@ -77,7 +78,7 @@ __device__ __forceinline__ void k2_body(const SweepArgs& a, Prog prog, const DOp
   // K0: this row's gate tensors (fused products for the forward program)
   int bad = 0;
   if constexpr (Prog::kSpecialised)
-    build_coefs(a, a.ops, rec_ptr, rec_ops, 0, nrec, mats, b, k, &bad);
+    build_coefs(a, 0, nrec, mats, b, k, &bad);
   else
     for (int i = tid; i < nrec; i += nt) mats[i] = build_recipe(a, a.ops, rec_ptr, rec_ops, i, b, k, &bad);
   for (int i = tid; i < ndops; i += nt) dops[i] = gdops[i];
@@ -98,6 +99,9 @@ __device__ __forceinline__ void k2_body(const SweepArgs& a, Prog prog, const DOp
   __syncthreads();
   prog.template forward<MF>(psi, mats, dim);
 
+  // index part of the row's frame: basis place y sits at y ^ mu
+  uint32_t mu = 0u;
+  if constexpr (Prog::kSpecialised) mu = coef_frame(mats, nrec, a.nrot);
   // observable epilogue (K6) / amplitude, state or probability read-out
   double Fval = 0.0;
   if (a.output == TDQ_OUT_EXPVAL) {
@@ -108,12 +112,12 @@ __device__ __forceinline__ void k2_body(const SweepArgs& a, Prog prog, const DOp
         const float* D = a.odiag + (size_t)g * dim;
         for (int x = tid; x < dim; x += nt) {
           const c2 v = psi[swz(x)];
-          acc += (v.x * v.x + v.y * v.y) * D[x];
+          acc += (v.x * v.x + v.y * v.y) * D[(uint32_t)x ^ mu];
         }
       } else {
         for (int x = tid; x < dim; x += nt) {
           const c2 v = psi[swz(x)];
-          acc += (v.x * v.x + v.y * v.y) * diag_weight(a.terms, t0, t1, (uint32_t)x);
+          acc += (v.x * v.x + v.y * v.y) * diag_weight(a.terms, t0, t1, (uint32_t)x ^ mu);
         }
       }
       const double tot = block_sum((double)acc, red);
@@ -135,7 +139,7 @@ __device__ __forceinline__ void k2_body(const SweepArgs& a, Prog prog, const DOp
     }
   } else if (k == 0 && a.output == TDQ_OUT_PROBS) {
     for (int x = tid; x < dim; x += nt) {
-      const c2 v = psi[swz(lin_index(a, (uint32_t)x))];
+      const c2 v = psi[swz(lin_index(a, (uint32_t)x) ^ mu)];
       a.values[b * dim + x] = (double)v.x * v.x + (double)v.y * v.y;
     }
   }
@@ -147,8 +151,8 @@ __device__ __forceinline__ void k2_body(const SweepArgs& a, Prog prog, const DOp
       float d = 0.f;
       for (int g = 0; g < a.n_groups; g++) {
         const float w = a.gw ? (float)a.gw[b * a.n_groups + g] : 1.f;
-        d += w * (a.odiag ? a.odiag[(size_t)g * dim + x]
-                          : diag_weight(a.terms, a.group_ptr[g], a.group_ptr[g + 1], (uint32_t)x));
+        d += w * (a.odiag ? a.odiag[(size_t)g * dim + ((uint32_t)x ^ mu)]
+                          : diag_weight(a.terms, a.group_ptr[g], a.group_ptr[g + 1], (uint32_t)x ^ mu));
       }
       const c2 v = psi[swz(x)];
       lam[swz(x)] = {d * v.x, d * v.y};

@@ -201,6 +201,49 @@ std::vector<LinReg> reg_passes(const std::vector<LinOp>& ops, const LinTile& t, 
   return out;
 }
 
+CoefRec angle_record(const std::vector<SweepOp>& gates, const LinOp& g) {
+  const SweepOp& op = gates[g.op];
+  return {op.src[g.ang], op.fixed[g.ang], 4 * g.op + g.ang, g.kind == L_PHASE ? C_PHASE : C_ROT};
+}
+
+// The rows' sign flips and the final index part: the Pauli product of every
+// rotation, carried through the ops after it (CZ and H change it, the others
+// commute or flip sign with it).
+void frame_tables(const std::vector<SweepOp>& gates, LinProgram& P) {
+  std::vector<int> rots;
+  for (int i = 0; i < (int)P.ops.size(); i++)
+    if (P.ops[i].kind == L_RY || P.ops[i].kind == L_RX) {
+      rots.push_back(i);
+      P.rot.push_back(angle_record(gates, P.ops[i]));
+    }
+  const int words = ((int)rots.size() + 31) / 32;
+  std::vector<int> tile_of(P.ops.size(), -1);
+  for (int t = 0; t < (int)P.tiles.size(); t++) {
+    P.tiles[t].flips.assign(P.tiles[t].coef.size() * (size_t)words, 0u);
+    for (int o : P.tiles[t].ops) tile_of[o] = t;
+  }
+  for (int j = 0; j < (int)rots.size(); j++) {
+    uint32_t x = P.ops[rots[j]].m, z = P.ops[rots[j]].kind == L_RY ? P.ops[rots[j]].f : 0u;
+    for (int i = rots[j] + 1; i < (int)P.ops.size(); i++) {
+      const LinOp& g = P.ops[i];
+      if (g.kind == L_CZ) {
+        const uint32_t add = (parity32(g.f & x) ? g.f2 : 0u) ^ (parity32(g.f2 & x) ? g.f : 0u);
+        z ^= add;
+      } else if (g.kind == L_H) {
+        if (parity32(g.f & x) ^ parity32(z & g.m)) {
+          x ^= g.m;
+          z ^= g.f;
+        }
+      } else if (P.coef[i] >= 0) {
+        const uint32_t gz = g.kind == L_RX ? 0u : g.f;
+        if (parity32(x & gz) ^ parity32(z & g.m))
+          P.tiles[tile_of[i]].flips[(size_t)P.coef[i] * words + j / 32] |= 1u << (j & 31);
+      }
+    }
+    P.rot_x.push_back(x);
+  }
+}
+
 }  // namespace
 
 LinProgram lin_program(const std::vector<SweepOp>& gates, int n, int k, int L, int mf, int mr, bool adj, bool exact) {
@@ -236,33 +279,29 @@ LinProgram lin_program(const std::vector<SweepOp>& gates, int n, int k, int L, i
     if (adj) t.rev = reg_passes(P.ops, t, W, mr, kRevPassSlots);
     // the gate-tensor table: one row per angle, one per register pass with
     // unscaled gates
-    auto row = [&](int type) {
-      t.rec_ops.push_back(type);
-      return (int)t.rec_ptr.size() - 1;
-    };
     for (int o : t.ops) {
       const LinOp& g = P.ops[o];
       if (g.kind != L_RY && g.kind != L_RX && g.kind != L_PHASE) continue;
-      P.coef[o] = row(g.kind == L_PHASE ? C_PHASE : C_ROT);
-      t.rec_ops.push_back(4 * g.op + g.ang);
-      t.rec_ptr.push_back((int)t.rec_ops.size());
+      P.coef[o] = (int)t.coef.size();
+      t.coef.push_back(angle_record(gates, g));
     }
     for (std::vector<LinReg>* rs : {&t.fwd, &t.rev})
       for (LinReg& r : *rs) {
         int nh = 0, nd = 0;
+        const int first = (int)t.norm.size();
         for (int o : r.ops) {
           nh += P.ops[o].kind == L_H ? 1 : 0;
           nd += P.ops[o].m ? 1 : 0;
+          if (P.ops[o].kind == L_RY || P.ops[o].kind == L_RX)
+            t.norm.push_back(2 * P.coef[o] + (P.ops[o].kind == L_RX ? 1 : 0));
         }
         if (!nd) continue;
-        r.norm = row((exact ? C_NORM_EXACT : C_NORM) + (nh << 8));
-        for (int o : r.ops)
-          if (P.ops[o].kind == L_RY || P.ops[o].kind == L_RX)
-            t.rec_ops.push_back(2 * P.coef[o] + (P.ops[o].kind == L_RX ? 1 : 0));
-        t.rec_ptr.push_back((int)t.rec_ops.size());
+        r.norm = (int)t.coef.size();
+        t.coef.push_back({(int)t.norm.size() - first, 0.f, first, (exact ? C_NORM_EXACT : C_NORM) + (nh << 8)});
       }
     P.tiles.push_back(t);
   } while (!todo.empty());
+  if (!exact) frame_tables(gates, P);
   return P;
 }
 

@@ -98,15 +98,16 @@ struct LinTile {
   uint32_t pivots = 0;
   std::vector<int> ops;
   std::vector<LinReg> fwd, rev;
-  // gate-tensor table: row r is built from rec_ops[rec_ptr[r] .. rec_ptr[r + 1]):
-  // the row's type, then its angle (4 * gate + angle), or for the scale of a
-  // register pass the rows of its rotations (2 * row + 1 for RX)
-  std::vector<int> rec_ptr{0}, rec_ops;
+  std::vector<uint32_t> flips;  // programs with a frame: SweepArgs::rot_flips of the table's rows
+  std::vector<CoefRec> coef;    // gate-tensor table
+  std::vector<int> norm;        // SweepArgs::norm of its scale rows
 };
 
 struct LinProgram {
   int n = 0;
-  bool exact = false;        // keep the global phase (state and amplitude outputs)
+  bool exact = false;        // keep the global phase (state and amplitude outputs): no frame
+  std::vector<CoefRec> rot;  // with a frame: SweepArgs::rot and rot_x
+  std::vector<uint32_t> rot_x;
   std::vector<LinOp> ops;
   std::vector<int> coef;     // table row of every op in its tile pass, or -1
   std::vector<LinTile> tiles;

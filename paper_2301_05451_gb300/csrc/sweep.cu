@@ -198,6 +198,11 @@ struct SweepExec final : tdq_exec {
   RegPass* d_passes = nullptr;
   uint32_t* d_lin = nullptr;  // whole-state specialised programs: SweepArgs::lin
   int quarter = 0;
+  CoefRec* d_coef = nullptr;  // their gate-tensor table (SweepArgs::coef, norm)
+  int* d_norm = nullptr;
+  CoefRec* d_rot = nullptr;   // their rows' frame tables (SweepArgs::rot and on)
+  uint32_t *d_rot_x = nullptr, *d_rot_flips = nullptr;
+  int nrot = 0;
   float* d_odiag = nullptr;  // observable diagonal per group [ng][2^n] (whole state; tiled when small)
   DOp* d_dops = nullptr;
   int* d_rec_ptr = nullptr;
@@ -223,6 +228,11 @@ struct SweepExec final : tdq_exec {
     cudaFree(d_passes);
     cudaFree(d_odiag);
     cudaFree(d_lin);
+    cudaFree(d_rot);
+    cudaFree(d_rot_x);
+    cudaFree(d_rot_flips);
+    cudaFree(d_coef);
+    cudaFree(d_norm);
     cudaFree(d_dops);
     cudaFree(d_rec_ptr);
     cudaFree(d_rec_ops);
@@ -251,6 +261,12 @@ struct SweepExec final : tdq_exec {
     a.odiag = d_odiag;
     a.lin = d_lin;
     a.quarter = quarter;
+    a.rot = d_rot;
+    a.rot_x = d_rot_x;
+    a.rot_flips = d_rot_flips;
+    a.coef = d_coef;
+    a.norm = d_norm;
+    a.nrot = nrot;
     a.init = init;
     a.init_stride = init_stride;
     last_launches = 0;
@@ -505,6 +521,9 @@ static void terms_to_frame(const LinMap& map, std::vector<TermDev>& terms) {
   }
 }
 
+// Tiled sweeps keep the observable's diagonals as tables up to this size.
+constexpr double kDiagTableBytes = 64.0 * 1024 * 1024;
+
 // Part of a multi-circuit launch: the circuit's tables only (its program is
 // compiled with the other circuits'), for a CTA of `threads` threads.
 struct MultiHook {
@@ -624,12 +643,18 @@ static tdq_status compile_sweep_impl(const tdq_circuit* c, const tdq_compile_opt
   // (short per-gate code, re-run by more groups: the instruction footprint
   // decides their speed); tiled and generic programs to 4 / 3
   const bool k2spec = !o->interpret;
-  const int fb = o->fwd_reg_bits ? o->fwd_reg_bits : (k2spec ? kSpecFwdRegBits : kFwdRegBits);
-  const int rb = o->rev_reg_bits ? o->rev_reg_bits : (k2spec ? kSpecRevRegBits : kRevRegBits);
+  const int fb = o->fwd_reg_bits ? o->fwd_reg_bits : (k2spec ? spec_reg_bits(c->n) : kFwdRegBits);
+  const int rb = o->rev_reg_bits ? o->rev_reg_bits : (k2spec ? spec_reg_bits(c->n) : kRevRegBits);
   // tiled programs: the generic kernels are compiled for kFwdRegBits /
   // kRevRegBits; specialised ones take their own defaults
   const int fb1 = o->fwd_reg_bits ? o->fwd_reg_bits : (o->interpret ? kFwdRegBits : kTiledSpecFwdRegBits);
-  const int rb1 = o->rev_reg_bits ? o->rev_reg_bits : (o->interpret ? kRevRegBits : kTiledSpecRevRegBits);
+  int rb1 = o->rev_reg_bits ? o->rev_reg_bits : (o->interpret ? kRevRegBits : kTiledSpecRevRegBits);
+  if (!o->rev_reg_bits && !o->interpret) {  // few tiles per SM: see kTiledFewTiles
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, e->dev);
+    const int k = std::min(c->n, o->tile_qubits > 0 ? o->tile_qubits : 12);
+    if (std::ldexp((double)e->B * e->copies, c->n - k) <= (double)kTiledFewTiles * sms) rb1 = 3;
+  }
   e->cfg_fb = fb;
   e->cfg_rb = rb;
   const int smem_max_n = o->max_smem_qubits > 0 ? o->max_smem_qubits : (adj ? 13 : 14);
@@ -650,9 +675,9 @@ static tdq_status compile_sweep_impl(const tdq_circuit* c, const tdq_compile_opt
     size_t sb = 0;
     if (spec) {
       lin = lin_program(ops, c->n, c->n, 0, fb, rb, adj, exact);
-      e->nrec = (int)lin.tiles[0].rec_ptr.size() - 1;
+      e->nrec = (int)lin.tiles[0].coef.size();
       const size_t gb = adj ? k2_grad_bytes(true, e->P, e->threads) : 0;
-      sb = dim * sizeof(c2) * (adj ? 2 : 1) + sizeof(float4) * e->nrec + ((gb + 7) & ~(size_t)7) + 32 * sizeof(double) + 16;
+      sb = dim * sizeof(c2) * (adj ? 2 : 1) + coef_bytes(e->nrec, (int)lin.rot.size()) + ((gb + 7) & ~(size_t)7) + 32 * sizeof(double) + 16;
       if (sb > 227 * 1024) spec = false;
       else e->smem_bytes = sb;
     }
@@ -695,7 +720,8 @@ static tdq_status compile_sweep_impl(const tdq_circuit* c, const tdq_compile_opt
   // D_g[y] = sum_{t in g} c_t (-1)^{popc(y & mask_t)}: whole states always;
   // tiled sweeps while the tables stay small enough to live in L2 (at most 64
   // MiB), read by the last tile pass instead of evaluating every term
-  if (e->output == TDQ_OUT_EXPVAL && (e->smem_path || std::ldexp((double)e->ng * 4.0, c->n) <= 64.0 * 1024 * 1024)) {
+  if (e->output == TDQ_OUT_EXPVAL && (e->smem_path || std::ldexp(4.0 * e->ng, c->n) <= kDiagTableBytes)) {
+    e->tiled.diag = true;
     std::vector<float> od((size_t)e->ng * dim);
     for (int g = 0; g < e->ng; g++)
       for (size_t x = 0; x < dim; x++) {
@@ -711,13 +737,17 @@ static tdq_status compile_sweep_impl(const tdq_circuit* c, const tdq_compile_opt
     e->kclass = 2;
     // compulsory HBM bytes per row: parameters, inputs, outputs, gradients
     e->bytes_row = 4.0 * e->P + 4.0 * e->F + out_bytes_row(e->output, c->n, e->A, e->ng) + (adj ? 4.0 * e->P : 0);
-    if ((s = upload(&e->d_rec_ptr, spec ? lin.tiles[0].rec_ptr : prog.rec_ptr)) != TDQ_OK) return bail(s);
-    if ((s = upload(&e->d_rec_ops, spec ? lin.tiles[0].rec_ops : prog.rec_ops)) != TDQ_OK) return bail(s);
     if (spec) {
       std::vector<uint32_t> map = lin.map.col;
       map.push_back(lin.map.to_y(0));
       if ((s = upload(&e->d_lin, map)) != TDQ_OK) return bail(s);
       e->quarter = exact ? lin.map.quarter : 0;
+      e->nrot = (int)lin.rot.size();
+      if ((s = upload(&e->d_coef, lin.tiles[0].coef)) != TDQ_OK) return bail(s);
+      if ((s = upload(&e->d_norm, lin.tiles[0].norm)) != TDQ_OK) return bail(s);
+      if ((s = upload(&e->d_rot, lin.rot)) != TDQ_OK) return bail(s);
+      if ((s = upload(&e->d_rot_x, lin.rot_x)) != TDQ_OK) return bail(s);
+      if ((s = upload(&e->d_rot_flips, lin.tiles[0].flips)) != TDQ_OK) return bail(s);
       if (hook) {  // compiled later with the other circuits of the launch
         *out = e;
         return ok();
@@ -728,6 +758,8 @@ static tdq_status compile_sweep_impl(const tdq_circuit* c, const tdq_compile_opt
     } else {
       if ((s = upload(&e->d_passes, prog.passes)) != TDQ_OK) return bail(s);
       if ((s = upload(&e->d_dops, prog.dops)) != TDQ_OK) return bail(s);
+      if ((s = upload(&e->d_rec_ptr, prog.rec_ptr)) != TDQ_OK) return bail(s);
+      if ((s = upload(&e->d_rec_ops, prog.rec_ops)) != TDQ_OK) return bail(s);
     }
 #define TDQ_SETSM(MF, MB, GG) ce = cudaFuncSetAttribute(k2_sweep_smem<MF, MB, GG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e->smem_bytes)
     if (e->spec_kernel) {
@@ -912,8 +944,8 @@ extern "C" tdq_status tdq_sweep_source(const tdq_circuit* c, int grad, int tile_
   std::string src;
   if (tile_qubits == 0) {
     if (c->n > 14) return fail(TDQ_ERR_UNSUPPORTED, "tdq_sweep_source: more than 14 qubits in one CTA");
-    src = k2_specialised_source(k2_program(c, adj, kSpecFwdRegBits, kSpecRevRegBits, c->n_groups > 0), adj,
-                                k2_threads(c->n, std::min(kSpecFwdRegBits, c->n)), c->n_params, "tdq_k2_specialised");
+    src = k2_specialised_source(k2_program(c, adj, spec_reg_bits(c->n), spec_reg_bits(c->n), c->n_groups > 0), adj,
+                                k2_threads(c->n, std::min(spec_reg_bits(c->n), c->n)), c->n_params, "tdq_k2_specialised");
   } else {
     if (c->n > 30) return fail(TDQ_ERR_UNSUPPORTED, "tdq_sweep_source: more than 30 qubits");
     std::vector<int> psg, psa;
@@ -924,9 +956,9 @@ extern "C" tdq_status tdq_sweep_source(const tdq_circuit* c, int grad, int tile_
     tdq_status s = tiled_lin_plan(t, c, ops, 1, adj, tile_qubits, kTiledSpecFwdRegBits, kTiledSpecRevRegBits,
                                   c->n_groups == 0, lin);
     if (s != TDQ_OK) return s;
-    std::vector<int> nacc;
+    t.diag = c->n_groups > 0 && std::ldexp(4.0 * c->n_groups, c->n) <= kDiagTableBytes;
     src = k1_specialised_source(t, lin, std::max(32, std::min(256, 1 << (t.k - kTiledSpecFwdRegBits))),
-                                std::max(32, std::min(256, 1 << (t.k - kTiledSpecRevRegBits))), &nacc);
+                                std::max(32, std::min(256, 1 << (t.k - kTiledSpecRevRegBits))));
   }
   *len = src.size() + 1;
   if (buf) {
@@ -1139,6 +1171,12 @@ static tdq_status multi_build(const tdq_circuit* const* cs, const int* batch, in
     a.ps_copies = x->copies; a.ps_gate = x->d_ps_gate; a.ps_ang = x->d_ps_ang; a.ps_F = x->d_ps_F;
     a.odiag = x->d_odiag;
     a.lin = x->d_lin;
+    a.rot = x->d_rot;
+    a.rot_x = x->d_rot_x;
+    a.rot_flips = x->d_rot_flips;
+    a.coef = x->d_coef;
+    a.norm = x->d_norm;
+    a.nrot = x->nrot;
     m.rec_ptr = x->d_rec_ptr;
     m.rec_ops = x->d_rec_ops;
     m.nrec = x->nrec;
@@ -1275,8 +1313,8 @@ extern "C" tdq_status tdq_compile_multi(const tdq_circuit* const* circuits, cons
   if (rows > (1 << 30)) return fail(TDQ_ERR_ARG, "tdq_compile_multi: too many rows");
   MultiExec* best = nullptr;
   if (!o->autotune) {
-    const int fb = o->fwd_reg_bits ? o->fwd_reg_bits : kSpecFwdRegBits;
-    const int rb = o->rev_reg_bits ? o->rev_reg_bits : kSpecRevRegBits;
+    const int fb = o->fwd_reg_bits ? o->fwd_reg_bits : spec_reg_bits(widest);
+    const int rb = o->rev_reg_bits ? o->rev_reg_bits : spec_reg_bits(widest);
     const int threads = std::max(64, std::min(256, (1 << widest) >> std::min(fb, widest)));
     tdq_status s = multi_build(circuits, batch, n_circuits, o, threads, fb, rb, &best);
     if (s != TDQ_OK) return s;

@@ -158,6 +158,17 @@ __device__ __forceinline__ float diag_weight(const TermDev* terms, int t0, int t
   return d;
 }
 
+// One row of a specialised program's gate-tensor table (build_coefs).
+// Rotations and phases: where the angle comes from, and 4 * gate + angle for
+// the shift rule.  Scales: `src` rows listed from norm[code] on (2 * row + 1
+// for an RX), `type >> 8` factors 1 / sqrt 2.
+struct CoefRec {
+  int32_t src;  // >= 0 parameter column, -1 fixed, <= -2 input (-2 - j)
+  float fixed;
+  int32_t code;
+  int32_t type;
+};
+
 struct SweepArgs {
   const SweepOp* ops;
   int G, n;
@@ -191,6 +202,20 @@ struct SweepArgs {
   // quarter: the state carries i^-quarter
   const uint32_t* lin;
   int quarter;
+  // rotations whose half angle is past 45 degrees leave a Pauli product to the
+  // row's frame (build_coefs): the angles of all rotations of the program, the
+  // part of each one's product that moves the index at the program's end, and
+  // per table row the rotations that flip its sign ((nrot + 31) / 32 words);
+  // nrot = 0: no frame
+  const CoefRec* rot;
+  const uint32_t* rot_x;
+  const uint32_t* rot_flips;
+  int nrot;
+  uint32_t* row_frame;  // tiled state outputs: the index part of every row's frame
+  // specialised programs: rows of the gate-tensor table, and the table rows
+  // multiplied by the scale rows
+  const CoefRec* coef;
+  const int* norm;
 };
 
 // Rows of the gate-tensor table of a specialised program (build_coef).

@@ -127,10 +127,12 @@ class PassWriter {
   }
 
   void move(const char* arr, const char* reg, bool store) {
+    // (a tile's state buffer in use starts at element `buf`)
+    const char* sb = t_.k < P_.n && std::string(arr) == "psi" ? "[sb ^ buf ^ " : "[sb ^ ";
     for (int j = 0; j < N_; j++) {
       const uint32_t so = swz_host(member(j));
-      if (store) s_ << "    " << arr << "[sb ^ " << so << "u] = " << reg << j << ";\n";
-      else s_ << "    c2 " << reg << j << " = " << arr << "[sb ^ " << so << "u];\n";
+      if (store) s_ << "    " << arr << sb << so << "u] = " << reg << j << ";\n";
+      else s_ << "    c2 " << reg << j << " = " << arr << sb << so << "u];\n";
     }
   }
 
@@ -234,8 +236,9 @@ class PassWriter {
         }
       }
     }
-    // unscaled rotations of the u form leave their sign to the group factor;
-    // their words need the frame at that point, so it is walked here first
+    // exact programs' rotations of the second form leave their sign to the
+    // group factor; their words need the frame at that point, so it is walked
+    // here first
     std::vector<Frame> fr;
     for (const std::vector<int>& it : items_) {
       const LinOp& g = P_.ops[it[0]];
@@ -255,6 +258,7 @@ class PassWriter {
         drop_hit(fr, mj, nullptr);
         continue;
       }
+      if (!P_.exact) continue;  // one form only
       Sign sg = frame_sign(fr, mj);
       if (g.kind == L_RY) sg.flip(group_sign(g.f, g.b));
       if (!sg.zero() && (P_.exact || !sg.constant())) {
@@ -404,25 +408,27 @@ class PassWriter {
         s_ << "    dot_" << (ry ? "y" : "x") << "(p" << j << ", p" << k << ", l" << j << ", l" << k << ", gp, gn);\n";
       });
       s_ << "    lin_share(" << dst << ", sx(sc * sc * (" << (ry ? "(gp.x + gp.y) - (gn.x + gn.y)" : "gp - gn") << "), " << sg.str()
-         << "));\n";
+         << " ^ __float_as_uint(q.w)));\n";
     }
     if (rev_) {
       Sign inv;
       inv.c = true;
       sg.flip(inv);
     }
-    s_ << "    const float v = sx(q.x, " << sg.str() << ");\n    if (__float_as_uint(q.w) == 0u) {\n";
+    s_ << "    const float v = sx(q.x, " << sg.str() << ");\n" << (P_.exact ? "    if (__float_as_uint(q.w) == 0u) {\n" : "");
     if (ry) s_ << "    const float2 t = bc2(v), nt = bc2(-v);\n";
     for (const char* a : regs_)
       pairs(mj, ry ? fr : mj & -mj, [&](int j, int k) {
         s_ << "    " << (ry ? "ry_t(" : "rx_t(") << a << j << ", " << a << k << (ry ? ", t, nt);\n" : ", v);\n");
       });
-    s_ << "    } else {\n";
-    for (const char* a : regs_)
-      pairs(mj, ry ? fr : mj & -mj, [&](int j, int k) {
-        s_ << "    " << (ry ? "ry_u(" : "rx_u(") << a << j << ", " << a << k << ", v);\n";
-      });
-    s_ << "    }\n";
+    if (P_.exact) {
+      s_ << "    } else {\n";
+      for (const char* a : regs_)
+        pairs(mj, ry ? fr : mj & -mj, [&](int j, int k) {
+          s_ << "    " << (ry ? "ry_u(" : "rx_u(") << a << j << ", " << a << k << ", v);\n";
+        });
+      s_ << "    }\n";
+    }
     if (rev_ && r_.norm >= 0) s_ << "    sc *= q.y;\n";
     s_ << "    }\n";
   }
@@ -462,7 +468,7 @@ class PassWriter {
         const int cm = combo(basis, reg_parity(g.f));
         s_ << "    lin_share(" << share(withg[i]) << ", sx(" << (r_.norm >= 0 ? "sc * sc * (" : "(");
         for (int c = 0; c < nc; c++) s_ << (cpar(cm & c) ? " - " : c ? " + " : "") << "v" << c;
-        s_ << "), " << group_sign(g.f, g.b).str() << "));\n";
+        s_ << "), " << group_sign(g.f, g.b).str() << " ^ sig[" << P_.coef[withg[i]] << "]));\n";
       }
       s_ << "    }\n";
     }
@@ -640,7 +646,8 @@ static void k2_prog_struct(std::ostringstream& s, std::ostringstream& decl, int*
   }
   s << "  }\n";
   s << "  template <int MB>\n  __device__ __forceinline__ void reverse(c2* psi, c2* lam, const float4* mats, int, "
-       "double*, float* gpart) const {\n";
+       "double*, float* gpart) const {\n  const uint32_t* sig = reinterpret_cast<const uint32_t*>(mats + "
+    << t.coef.size() << ");\n  (void)sig;\n";
   if (grad)
     for (int pi = (int)t.rev.size() - 1; pi >= 0; pi--) {
       s << "  // reverse pass " << pi << "\n";
@@ -742,12 +749,10 @@ static void emit_in_first(std::ostringstream& s, const LinTile& t, int n) {
   s << "    return r == 0u;\n  }\n";
 }
 
-std::string k1_specialised_source(const TiledSweep& t, const LinProgram& prog, int nthreads, int nthreads_r,
-                                  std::vector<int>* nacc) {
+std::string k1_specialised_source(const TiledSweep& t, const LinProgram& prog, int nthreads, int nthreads_r) {
   std::ostringstream s, decl;
   int uid = 0;
   const int np = (int)prog.tiles.size();
-  nacc->assign(np, 0);
   for (int p = 0; p < np; p++) {
     const LinTile& tile = prog.tiles[p];
     // gradient accumulators of the pass: one per angle with a slot
@@ -759,22 +764,27 @@ std::string k1_specialised_source(const TiledSweep& t, const LinProgram& prog, i
           acc[o] = (int)slots.size();
           slots.push_back(prog.ops[o].slot);
         }
-    (*nacc)[p] = (int)slots.size();
     const int na = std::max(1, (int)slots.size());
     s << "__constant__ int tdq_slots_" << p << "[" << na << "] = {";
     for (int i = 0; i < na; i++) s << (i ? ", " : "") << (i < (int)slots.size() ? slots[i] : 0);
     s << "};\n";
     s << "struct TilePass" << p << " {\n  static constexpr bool kSpecialised = true, kFirst = "
-      << (p == 0 ? "true" : "false") << ", kSecond = " << (p == 1 ? "true" : "false") << ";\n";
+      << (p == 0 ? "true" : "false") << ", kSecond = " << (p == 1 ? "true" : "false") << ", kDiag = "
+      << (t.diag ? "true" : "false") << ";\n  static constexpr int kK = " << t.k << ", kN = " << t.n
+      << ", kBuffers = " << (t.dbl ? 2 : 1) << ", kGroups = " << t.ng << ";\n";
     emit_in_first(s, prog.tiles[0], t.n);
     emit_every(s, tile, t.L);
-    s << "  __device__ __forceinline__ static void forward(const TiledDev&, const TileShared& s, uint32_t base) {\n"
+    s << "  __device__ __forceinline__ static void forward(const TiledDev&, const TileShared& s, uint32_t base, "
+         "uint32_t buf) {\n"
       << "  c2* psi = s.psi;\n  const float4* mats = reinterpret_cast<const float4*>(s.mats);\n";
     for (const LinReg& r : tile.fwd) emit_fwd_pass(s, prog, tile, r, t.L, nthreads);
     s << "  }\n";
-    s << "  __device__ __forceinline__ static void reverse(const TiledDev&, const TileShared& s, uint32_t base) {\n"
+    s << "  __device__ __forceinline__ static void reverse(const TiledDev&, const TileShared& s, uint32_t base, "
+         "uint32_t buf) {\n"
       << "  c2* psi = s.psi;\n  c2* lam = s.lam;\n  const float4* mats = reinterpret_cast<const float4*>(s.mats);\n"
-      << "  float* gpart = reinterpret_cast<float*>(s.gpart);\n";
+      << "  float* gpart = reinterpret_cast<float*>(s.gpart);\n"
+      << "  const uint32_t* sig = reinterpret_cast<const uint32_t*>(mats + " << tile.coef.size()
+      << ");\n  (void)sig;\n";
     // (the fused last pass runs its reverse program with the forward kernel's threads)
     for (int q = (int)tile.rev.size() - 1; q >= 0; q--)
       emit_rev_pass(s, decl, &uid, prog, tile, tile.rev[q], t.L, p == np - 1 ? nthreads : nthreads_r, na,

@@ -23,6 +23,7 @@ __global__ void __launch_bounds__(256) k1_reverse(SweepArgs a, TiledDev t) { k1_
 
 // Copy out the chunk's values, F for the shift rule, gradients, amplitudes.
 __global__ void k1_finalize(SweepArgs a, TiledDev t, int nrows, int grad_adj) {
+  chain_wait();
   const int lr = blockIdx.x;
   if (lr >= nrows) return;
   const int row = t.row0 + lr;
@@ -69,7 +70,8 @@ __global__ void __launch_bounds__(256) k1_state_out(SweepArgs a, TiledDev t, int
     const int row = t.row0 + lr;
     if (row % a.ps_copies) continue;
     const int64_t b = row / a.ps_copies, x = i - (int64_t)lr * dim;
-    const uint32_t y = tab[0][x & 255] ^ tab[1][(x >> 8) & 255] ^ tab[2][(x >> 16) & 255] ^ tab[3][(x >> 24) & 255];
+    const uint32_t y = tab[0][x & 255] ^ tab[1][(x >> 8) & 255] ^ tab[2][(x >> 16) & 255] ^ tab[3][(x >> 24) & 255] ^
+                       (a.row_frame ? a.row_frame[lr] : 0u);
     const c2 v = t.psi[(size_t)lr * dim + y];
     if (a.output == TDQ_OUT_STATE) {
       a.values[(b * dim + x) * 2] = v.x;
@@ -98,7 +100,16 @@ void tiled_free(TiledSweep& t) {
   cudaFree(t.d_rec_ptr);
   cudaFree(t.d_rec_ops);
   cudaFree(t.d_lin);
-  t.d_lin = nullptr;
+  cudaFree(t.d_rot);
+  cudaFree(t.d_rot_x);
+  cudaFree(t.d_rot_flips);
+  cudaFree(t.d_coef);
+  cudaFree(t.d_norm);
+  t.d_coef = nullptr;
+  t.d_norm = nullptr;
+  cudaFree(t.d_row_frame);
+  t.d_lin = t.d_rot_x = t.d_rot_flips = t.d_row_frame = nullptr;
+  t.d_rot = nullptr;
   t.d_ps_gate_pass = nullptr;
   t.d_rpass = nullptr;
   t.d_dops = nullptr;
@@ -273,7 +284,7 @@ tdq_status tiled_lin_plan(TiledSweep& t, const tdq_circuit* c, const std::vector
   int r0 = 0;
   for (const LinTile& tile : prog.tiles) {
     t.passes.push_back({tile.pivots, 0, 0});
-    const int nr = (int)tile.rec_ptr.size() - 1;
+    const int nr = (int)tile.coef.size();
     t.rec_begin.push_back(r0);
     t.rec_end.push_back(r0 += nr);
     t.max_rec = std::max(t.max_rec, nr);
@@ -302,9 +313,6 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
         h.offs.push_back((int)o);
       }
       for (int p = 0; p < 32; p++) h.locs.push_back(-1);
-      const int e0 = (int)h.prog.rec_ops.size();
-      for (size_t r = 1; r < tile.rec_ptr.size(); r++) h.prog.rec_ptr.push_back(e0 + tile.rec_ptr[r]);
-      h.prog.rec_ops.insert(h.prog.rec_ops.end(), tile.rec_ops.begin(), tile.rec_ops.end());
     }
   }
   const bool interpret = lin == nullptr;
@@ -327,6 +335,23 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
     map.push_back(lin->map.to_y(0));
     if ((s = up((void**)&t.d_lin, map.data(), sizeof(uint32_t) * map.size())) != TDQ_OK) return s;
     t.quarter = lin->exact ? lin->map.quarter : 0;
+    t.nrot = (int)lin->rot.size();
+    std::vector<uint32_t> flips;
+    for (const LinTile& tile : lin->tiles) flips.insert(flips.end(), tile.flips.begin(), tile.flips.end());
+    if ((s = up((void**)&t.d_rot, lin->rot.data(), sizeof(CoefRec) * lin->rot.size())) != TDQ_OK) return s;
+    if ((s = up((void**)&t.d_rot_x, lin->rot_x.data(), sizeof(uint32_t) * lin->rot_x.size())) != TDQ_OK) return s;
+    std::vector<CoefRec> coef;
+    std::vector<int> norm;
+    for (const LinTile& tile : lin->tiles) {
+      for (CoefRec q : tile.coef) {
+        if (q.type != C_ROT && q.type != C_PHASE) q.code += (int)norm.size();
+        coef.push_back(q);
+      }
+      norm.insert(norm.end(), tile.norm.begin(), tile.norm.end());
+    }
+    if ((s = up((void**)&t.d_coef, coef.data(), sizeof(CoefRec) * coef.size())) != TDQ_OK) return s;
+    if ((s = up((void**)&t.d_norm, norm.data(), sizeof(int) * norm.size())) != TDQ_OK) return s;
+    if ((s = up((void**)&t.d_rot_flips, flips.data(), sizeof(uint32_t) * flips.size())) != TDQ_OK) return s;
   }
   if ((s = up((void**)&t.d_ops, pops.data(), sizeof(SweepOp) * pops.size())) != TDQ_OK) return s;
   if ((s = up((void**)&t.d_off, offs.data(), sizeof(int) * offs.size())) != TDQ_OK) return s;
@@ -348,6 +373,8 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
     return fail(TDQ_ERR_OOM, "tiled sweep: state buffer");
   if (adj && cudaMalloc(&t.d_lam, ((size_t)1 << n) * sizeof(c2) * t.chunk_rows) != cudaSuccess)
     return fail(TDQ_ERR_OOM, "tiled sweep: adjoint buffer");
+  if (t.nrot && cudaMalloc(&t.d_row_frame, sizeof(uint32_t) * t.chunk_rows) != cudaSuccess)
+    return fail(TDQ_ERR_OOM, "tiled sweep: frame buffer");
   if (cudaMalloc(&t.d_gacc, sizeof(double) * std::max(1, t.P) * t.chunk_rows) != cudaSuccess)
     return fail(TDQ_ERR_OOM, "tiled sweep: gradient buffer");
   if (cudaMalloc(&t.d_vals, sizeof(double) * std::max(1, t.ng) * t.chunk_rows) != cudaSuccess)
@@ -361,13 +388,12 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
   t.spec_gbytes.clear();
   const int np = (int)t.passes.size();
   int gmax = 0, ndops_sm = 0;
-  std::string src;
+  std::vector<int> nacc(np, 0);  // gradient accumulators of every pass
   if (!interpret) {
-    // every tile pass as straight-line code; one compilation for all passes
-    std::vector<int> nacc;
-    src = k1_specialised_source(t, *lin, t.nthreads, t.nthreads_r, &nacc);
     const int nw = std::max(t.nthreads, t.nthreads_r) / 32;
     for (int p = 0; p < np; p++) {
+      if (adj)
+        for (int o : lin->tiles[p].ops) nacc[p] += lin->ops[o].slot >= 0 ? 1 : 0;
       t.spec_gbytes.push_back(4 * nw * std::max(1, nacc[p]));
       gmax = std::max(gmax, t.spec_gbytes.back());
     }
@@ -380,7 +406,7 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
   // kernels hold psi and lambda in one buffer each: two CTAs of 256 threads
   // per SM then interleave one CTA's tile loads with the other's compute,
   // which measured faster than one double-buffered CTA of 512 threads.
-  const int mbytes = t.max_rec * (int)(interpret ? sizeof(OpMat) : sizeof(float4));
+  const int mbytes = interpret ? t.max_rec * (int)sizeof(OpMat) : coef_bytes(t.max_rec, t.nrot);
   auto sizes = [&](int nb) {
     t.smem_f.assign(np, 0);
     for (int p = 0; p < np; p++)
@@ -395,6 +421,8 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
   size_t smax = sizes(t.dbl ? 2 : 1);
   if (smax > 227 * 1024) return fail(TDQ_ERR_UNSUPPORTED, "tiled sweep: tile program too large");
   if (!interpret) {
+    // every tile pass as straight-line code; one compilation for all passes
+    const std::string src = k1_specialised_source(t, *lin, t.nthreads, t.nthreads_r);
     for (int p = 0; p < np; p++) {
       const void* kf = nullptr;
       const void* kr = nullptr;
@@ -519,12 +547,36 @@ static void set_pass(const TiledSweep& t, TiledDev& d, int p) {
   }
 }
 
+// A launch that may be dispatched while the kernel before it in the stream is
+// finishing (chained; the kernel waits in chain_wait).
+static cudaError_t launch_chained(const void* k, dim3 g, dim3 b, void** args, size_t smem, cudaStream_t st,
+                                  bool chained) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = g;
+  cfg.blockDim = b;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelExC(&cfg, k, args);
+}
+
 tdq_status tiled_execute(TiledSweep& t, const SweepArgs& a0, int grad, cudaStream_t st,
                          int* launches) {
   SweepArgs a = a0;
   if (a.ps_copies > 1) a.ps_gate = t.d_ps_gate_pass;
   a.lin = t.d_lin;
   a.quarter = t.quarter;
+  a.rot = t.d_rot;
+  a.rot_x = t.d_rot_x;
+  a.rot_flips = t.d_rot_flips;
+  a.coef = t.d_coef;
+  a.norm = t.d_norm;
+  a.nrot = t.nrot;
+  a.row_frame = t.d_row_frame;
   const bool adj = grad == TDQ_GRAD_ADJOINT;
   const int np = (int)t.passes.size();
   const int ntiles = 1 << (t.n - t.k);
@@ -575,7 +627,8 @@ tdq_status tiled_execute(TiledSweep& t, const SweepArgs& a0, int grad, cudaStrea
       if (!t.kf.empty()) {
         int st_flag = (l && !adj) ? store_last : 1;
         void* args[] = {&a, &d, &st_flag};
-        if (cudaLaunchKernel(t.kf[p], grid, dim3(nthr), args, t.smem_f[p], st) != cudaSuccess)
+        // the first pass follows the caller's work and the clears above: unchained
+        if (launch_chained(t.kf[p], grid, dim3(nthr), args, t.smem_f[p], st, p > 0) != cudaSuccess)
           return fail(TDQ_ERR_CUDA, "tiled sweep: launch of a specialised pass");
         if (rec) cudaEventRecord(t.ev[2 * p + 1], st);
         (*launches)++;
@@ -600,13 +653,12 @@ tdq_status tiled_execute(TiledSweep& t, const SweepArgs& a0, int grad, cudaStrea
         d.op_end = t.passes[p].op_end;
         set_pass(t, d, p);
         const dim3 grid = grid_for(t.slots_r, d, p);
-        d.dbl = 0;  // reverse kernels: one buffer per state (see tiled_compile)
         const int u = np + (np - 2 - p);  // launch unit of this reverse pass
         const bool rec = !t.ev.empty() && row0 == 0;
         if (rec) cudaEventRecord(t.ev[2 * u], st);
         if (!t.kr.empty()) {
           void* args[] = {&a, &d};
-          if (cudaLaunchKernel(t.kr[p], grid, dim3(t.nthreads_r), args, t.smem_r, st) != cudaSuccess)
+          if (launch_chained(t.kr[p], grid, dim3(t.nthreads_r), args, t.smem_r, st, true) != cudaSuccess)
             return fail(TDQ_ERR_CUDA, "tiled sweep: launch of a specialised pass");
         } else {
           k1_reverse<<<grid, t.nthreads_r, t.smem_r, st>>>(a, d);
@@ -615,7 +667,12 @@ tdq_status tiled_execute(TiledSweep& t, const SweepArgs& a0, int grad, cudaStrea
         (*launches)++;
       }
     }
-    k1_finalize<<<nr, 128, 0, st>>>(a, d, nr, adj ? 1 : 0);
+    {
+      int nr_ = nr, g = adj ? 1 : 0;
+      void* args[] = {&a, &d, &nr_, &g};
+      if (launch_chained((const void*)k1_finalize, dim3(nr), dim3(128), args, 0, st, !t.kf.empty()) != cudaSuccess)
+        return fail(TDQ_ERR_CUDA, "tiled sweep: launch of the read-out");
+    }
     (*launches)++;
     if (a.output == TDQ_OUT_STATE || a.output == TDQ_OUT_PROBS) {
       const int64_t tot = (int64_t)nr << t.n;

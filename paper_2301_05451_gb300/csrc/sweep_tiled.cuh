@@ -78,10 +78,16 @@ struct TiledSweep {
   std::vector<int> spec_gbytes;
   uint32_t* d_lin = nullptr;             // specialised programs: place of a basis index (SweepArgs::lin)
   int quarter = 0;
+  CoefRec* d_coef = nullptr;             // their gate-tensor tables (SweepArgs::coef, norm)
+  int* d_norm = nullptr;
+  CoefRec* d_rot = nullptr;              // their rows' frame tables (SweepArgs::rot and on)
+  uint32_t *d_rot_x = nullptr, *d_rot_flips = nullptr, *d_row_frame = nullptr;
+  int nrot = 0;
   int nthreads = 256, nthreads_r = 256;  // forward / reverse kernels
   std::vector<size_t> smem_f;            // per forward kernel
   size_t smem_r = 0;
-  int dbl = 1;                           // double-buffered tile loads
+  int dbl = 1;                           // double-buffered tile loads (forward kernels)
+  bool diag = false;                     // the observable's diagonals are tables (SweepArgs::odiag)
   int fb = 4, rb = 3;                    // register bits of forward / reverse passes
   std::vector<int> slots_f;              // resident CTAs of each forward kernel on the GPU
   int slots_r = 1;                       // ... of the reverse kernels

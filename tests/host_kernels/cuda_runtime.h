@@ -60,6 +60,11 @@ T __shfl_xor_sync(unsigned, T v, int o) {
   b.arrive_and_wait();
   return r;
 }
+inline uint32_t __ballot_sync(unsigned, bool v) {
+  uint32_t r = v ? 1u << (threadIdx.x & 31) : 0u;
+  for (int o = 16; o > 0; o >>= 1) r |= __shfl_xor_sync(0u, r, o);
+  return r;
+}
 template <class T, class U>
 T atomicAdd(T* p, U v) {
   std::lock_guard<std::mutex> l(atomic_mu);

@@ -91,14 +91,21 @@ int main() {
   a.terms = terms.data(); a.group_ptr = gptr.data(); a.T = nt; a.n_groups = ng;
   a.output = ng ? TDQ_OUT_EXPVAL : TDQ_OUT_STATE;
   a.values = values.data(); a.grads = grads.data(); a.P = P; a.status = &status; a.ps_copies = 1;
+  std::vector<float> odiag((size_t)ng * dim);
+  for (int g = 0; g < ng; g++)
+    for (size_t y = 0; y < dim; y++)
+      odiag[g * dim + y] = diag_weight(terms.data(), gptr[g], gptr[g + 1], (uint32_t)y);
+  a.odiag = odiag.data();
+  a.rot = prog.rot.data(); a.rot_x = prog.rot_x.data(); a.nrot = (int)prog.rot.size();
   a.lin = lin.data(); a.quarter = ng ? 0 : prog.map.quarter;
 #ifdef WHOLE
   const LinTile& t = prog.tiles[0];
-  const int nrec = (int)t.rec_ptr.size() - 1, threads = std::max(32, std::min(256, (1 << n) >> std::min(fb, n)));
+  const int nrec = (int)t.coef.size(), threads = std::max(32, std::min(256, (1 << n) >> std::min(fb, n)));
   const size_t gb = adj ? k2_grad_bytes(true, P, threads) : 0;
-  const size_t sb = dim * sizeof(c2) * (adj ? 2 : 1) + sizeof(float4) * nrec + ((gb + 7) & ~(size_t)7) + 32 * sizeof(double) + 16;
+  const size_t sb = dim * sizeof(c2) * (adj ? 2 : 1) + coef_bytes(nrec, a.nrot) + ((gb + 7) & ~(size_t)7) + 32 * sizeof(double) + 16;
+  a.rot_flips = t.flips.data(); a.coef = t.coef.data(); a.norm = t.norm.data();
   launch(rows, threads, smem_raw, sb,
-         [&] { tdq_k2_specialised(a, nullptr, 0, t.rec_ptr.data(), t.rec_ops.data(), nrec); });
+         [&] { tdq_k2_specialised(a, nullptr, 0, nullptr, nullptr, nrec); });
 #else
   const int np = (int)prog.tiles.size(), nthr = std::max(32, std::min(256, 1 << (k - std::min(fb, k)))),
             nthr_r = std::max(32, std::min(256, 1 << (k - std::min(rb, k))));
@@ -114,7 +121,7 @@ int main() {
   int max_rec = 0, gmax = 0;
   std::vector<int> nacc(np, 0);
   for (int p = 0; p < np; p++) {
-    max_rec = std::max(max_rec, (int)prog.tiles[p].rec_ptr.size() - 1);
+    max_rec = std::max(max_rec, (int)prog.tiles[p].coef.size());
     for (int o : prog.tiles[p].ops) nacc[p] += adj && prog.ops[o].slot >= 0;
     gmax = std::max(gmax, 4 * (std::max(nthr, nthr_r) / 32) * std::max(1, nacc[p]));
   }
@@ -130,15 +137,16 @@ int main() {
     }
     std::vector<int8_t> loc8(32, -1);
     d.off = off.data(); d.loc = loc8.data(); d.smask = t.pivots;
-    d.rec_ptr = t.rec_ptr.data(); d.rec_ops = t.rec_ops.data(); d.rec0 = 0; d.nrec = (int)t.rec_ptr.size() - 1;
+    d.rec0 = 0; d.nrec = (int)t.coef.size();
     d.gbytes = 4 * (std::max(nthr, nthr_r) / 32) * std::max(1, nacc[p]);
+    a.rot_flips = t.flips.data(); a.coef = t.coef.data(); a.norm = t.norm.data();
     const int units = rows * d.ntiles, ctas = std::min(units, 3);  // uneven shares, rows cut across CTAs
     d.tiles_per_cta = (units + ctas - 1) / ctas;
     const unsigned grid = (units + d.tiles_per_cta - 1) / d.tiles_per_cta;
-    d.dbl = rev ? 0 : 1;
+    d.dbl = 1;
     const bool last = p == np - 1;
-    const size_t sm = rev ? k1_smem_bytes(k, L, 1, 1, 16 * max_rec, 0, ng, gmax)
-                          : k1_smem_bytes(k, L, p == 0 ? 1 : 2, adj && last ? 1 : 0, 16 * max_rec, 0, ng, gmax);
+    const size_t sm = rev ? k1_smem_bytes(k, L, 1, 1, coef_bytes(max_rec, a.nrot), 0, ng, gmax)
+                          : k1_smem_bytes(k, L, p == 0 ? 1 : 2, adj && last ? 1 : 0, coef_bytes(max_rec, a.nrot), 0, ng, gmax);
     if (rev) launch(grid, nthr_r, raw, sm, [&] { kr[p](a, d); });
     else launch(grid, nthr, raw, sm, [&] { kf[p](a, d, last && !adj ? ng == 0 : 1); });
   };
