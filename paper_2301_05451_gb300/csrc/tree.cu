@@ -58,6 +58,7 @@ constexpr int kMaxHyperBits = 16;
 struct StepDev {
   int64_t a_off, b_off, c_off;
   uint32_t pre;   // subtree steps: outputs of the earlier steps of the same level
+  uint32_t preb;  // ... and outputs of their reverse steps (entries of both operands)
   int8_t nm, nn, nk, rc, nh;
   int8_t cm[32];  // C bit position of m bit i (LSB first)
   int8_t cn[32];  // C bit position of n bit i
@@ -263,48 +264,46 @@ __device__ void step_generic(const StepDev& s, c2* arena, int tid, int nt) {
   for (uint32_t o = tid; o < tot; o += nt) step_out<kRot>(s, arena, o);
 }
 
-// Reverse of one step for one batch entry: from C's cotangent (at boff + the
-// value offsets) the cotangents of both operands, which each step writes once
-// (every tensor has one consumer):  Abar[m][k] = sum_n Cbar[m][n] B[n][k],
-// Bbar[n][k] = sum_m Cbar[m][n] A[m][k]  (holomorphic: no conjugation).
-__device__ void step_adjoint(const StepDev& s, c2* arena, int64_t boff, int tid, int nt) {
-  const c2* A = arena + s.a_off;
-  const c2* B = arena + s.b_off;
+// One output o of a step's reverse for one batch entry: from C's cotangent (at
+// boff + the value offsets) the cotangents of both operands (first all of A's
+// entries, then B's), which each step writes once (every tensor has one
+// consumer):  Abar[m][k] = sum_n Cbar[m][n] B[n][k], Bbar[n][k] = sum_m
+// Cbar[m][n] A[m][k]  (holomorphic: no conjugation).  The summed bits run in
+// Gray-code order: one bit of C's place changes per term.
+__device__ __forceinline__ uint32_t adjoint_outputs(const StepDev& s) {
+  return (1u << (s.nh + s.nm + s.nk)) + (1u << (s.nh + s.nn + s.nk));
+}
+__device__ __forceinline__ void adjoint_out(const StepDev& s, c2* arena, int64_t boff, uint32_t o) {
+  const uint32_t na = 1u << (s.nh + s.nm + s.nk);
+  const bool to_a = o < na;
+  if (!to_a) o -= na;
+  const int nr = to_a ? s.nm : s.nn, nx = to_a ? s.nn : s.nm;  // bits of this operand's rows, of the other's
+  const int8_t* pr = to_a ? s.cm : s.cn;
+  const int8_t* px = to_a ? s.cn : s.cm;
+  const uint32_t K = 1u << s.nk, h = o >> (nr + s.nk), r = (o >> s.nk) & ((1u << nr) - 1u), k = o & (K - 1u);
   const c2* Cb = arena + boff + s.c_off;
-  c2* Ab = arena + boff + s.a_off;
-  c2* Bb = arena + boff + s.b_off;
-  const uint32_t K = 1u << s.nk, M = 1u << s.nm, N = 1u << s.nn, H = 1u << s.nh;
-  for (uint32_t o = tid; o < H * M * K; o += nt) {
-    const uint32_t h = o >> (s.nm + s.nk), m = (o >> s.nk) & (M - 1u), k = o & (K - 1u);
-    const uint32_t cm = scatter_bits(h, s.ch, s.nh) | scatter_bits(m, s.cm, s.nm);
-    const c2* Bh = B + (size_t)(h << s.nn) * K;
-    float re = 0.f, im = 0.f;
-    for (uint32_t n = 0; n < N; n++) {
-      const c2 x = Cb[cm | scatter_bits(n, s.cn, s.nn)], y = Bh[(size_t)n * K + k];
-      re = fmaf(x.x, y.x, fmaf(-x.y, y.y, re));
-      im = fmaf(x.x, y.y, fmaf(x.y, y.x, im));
-    }
-    Ab[o] = {re, im};
+  const c2* X = arena + (to_a ? s.b_off : s.a_off) + (size_t)(h << nx) * K + k;
+  uint32_t c = scatter_bits(h, s.ch, s.nh) | scatter_bits(r, pr, nr);
+  float re = 0.f, im = 0.f;
+  for (uint32_t i = 0;;) {
+    const c2 x = Cb[c], y = X[(size_t)(i ^ (i >> 1)) * K];
+    re = fmaf(x.x, y.x, fmaf(-x.y, y.y, re));
+    im = fmaf(x.x, y.y, fmaf(x.y, y.x, im));
+    if (++i == (1u << nx)) break;
+    c ^= 1u << px[__ffs(i) - 1];
   }
-  for (uint32_t o = tid; o < H * N * K; o += nt) {
-    const uint32_t h = o >> (s.nn + s.nk), n = (o >> s.nk) & (N - 1u), k = o & (K - 1u);
-    const uint32_t cn = scatter_bits(h, s.ch, s.nh) | scatter_bits(n, s.cn, s.nn);
-    const c2* Ah = A + (size_t)(h << s.nm) * K;
-    float re = 0.f, im = 0.f;
-    for (uint32_t m = 0; m < M; m++) {
-      const c2 x = Cb[scatter_bits(m, s.cm, s.nm) | cn], y = Ah[(size_t)m * K + k];
-      re = fmaf(x.x, y.x, fmaf(-x.y, y.y, re));
-      im = fmaf(x.x, y.y, fmaf(x.y, y.x, im));
-    }
-    Bb[o] = {re, im};
-  }
+  (arena + boff + (to_a ? s.a_off : s.b_off))[o] = {re, im};
+}
+__device__ void step_adjoint(const StepDev& s, c2* arena, int64_t boff, int tid, int nt) {
+  const uint32_t tot = adjoint_outputs(s);
+  for (uint32_t o = tid; o < tot; o += nt) adjoint_out(s, arena, boff, o);
 }
 
 // dF/d(parameter) of one batch entry: Re sum_e Lbar[e] dL[e]/d(angle) over every
 // gate leaf, added to gacc[b][column] (FP64).
 __device__ void leaf_gradients(const LeafDev* leaves, int nleaves, const c2* arena, int64_t boff,
                                const float* params, int64_t pstride, const float* inputs, int F, int64_t b,
-                               uint32_t sigma, double* gacc_row, int tid, int nt) {
+                               uint32_t sigma, double* gacc_row, int tid, int nt) {  // (global or shared sums)
   for (int w = tid; w < nleaves * 3; w += nt) {
     const int li = w / 3, j = w % 3;
     const LeafDev L = leaves[li];
@@ -377,7 +376,9 @@ __global__ void __launch_bounds__(512) k_tree_subtrees(TreeArgs a, const SubDev*
   const int64_t b = e / a.chunk;
   const uint32_t sigma = a.slice0 + (uint32_t)(e % a.chunk);
   const int ns = sd.step_end - sd.step_begin;
+  int* lv = reinterpret_cast<int*>(st + ns);
   for (int i = threadIdx.x; i < ns; i += blockDim.x) st[i] = ssteps[sd.step_begin + i];
+  for (int i = threadIdx.x; i <= sd.nlev; i += blockDim.x) lv[i] = slev[sd.lev_begin + i];
   int bad = 0;
   build_leaves(sleaves + sd.leaf_begin, sd.leaf_end - sd.leaf_begin, arena, a.params, a.pstride, a.inputs, a.F, b,
                sigma, &bad, threadIdx.x, blockDim.x);
@@ -387,7 +388,7 @@ __global__ void __launch_bounds__(512) k_tree_subtrees(TreeArgs a, const SubDev*
   // come from earlier levels, and the arena keeps them apart), so the level's
   // outputs are shared out over the CTA as one range, one barrier per level
   for (int l = 0; l < sd.nlev; l++) {
-    const int s0 = slev[sd.lev_begin + l], s1 = slev[sd.lev_begin + l + 1];
+    const int s0 = lv[l], s1 = lv[l + 1];
     const uint32_t total = st[s1 - 1].pre + step_outputs(st[s1 - 1]);
     int i = s0;
     for (uint32_t o = threadIdx.x; o < total; o += blockDim.x) {
@@ -407,37 +408,69 @@ __global__ void __launch_bounds__(512) k_tree_subtrees(TreeArgs a, const SubDev*
 // Value and gradient of a whole small network in one CTA: leaves, forward
 // steps, the root, then the reverse tree and the leaf gradients, every
 // tensor and cotangent in shared memory (values at value offsets, cotangents
-// at boff + value offsets).
-__global__ void __launch_bounds__(128) k_tree_fused_adj(TreeArgs a, const LeafDev* leaves, int nleaves,
-                                                        const StepDev* steps, int nsteps, int root_local,
-                                                        int smem_elems) {
+// at boff + value offsets).  Both directions run level by level: the steps of
+// a level are independent, its outputs are shared out over the CTA as one
+// range, one barrier per level.  direct: the launch holds the row's only
+// slice, so the CTA writes the row's value and gradient itself (its sums in
+// shared memory, FP64) instead of leaving them to four small launches.
+// What bounds it is latency (a chain of levels of a few dozen outputs each):
+// 5 x 10 light cone, 92 steps, 32 rows, value and gradient 176 us at 128
+// threads and a barrier per step, 39 us so.
+__global__ void __launch_bounds__(512) k_tree_fused_adj(TreeArgs a, const LeafDev* leaves, int nleaves,
+                                                        const StepDev* steps, int nsteps, const int* lev, int nlev,
+                                                        int root_local, int smem_elems, int direct, double* values,
+                                                        float* grads) {
   chain_start();
   extern __shared__ __align__(16) unsigned char raw[];
   c2* arena = reinterpret_cast<c2*>(raw);
   StepDev* st = reinterpret_cast<StepDev*>(arena + smem_elems);
+  double* gsum = reinterpret_cast<double*>(st + nsteps);
+  const int gw = max(a.P, 1);  // the gradient row's width
+  int* lv = reinterpret_cast<int*>(gsum + (direct ? gw : 0));
   const int e = blockIdx.x;
   const int64_t b = e / a.chunk;
   const uint32_t sigma = a.slice0 + (uint32_t)(e % a.chunk);
   for (int i = threadIdx.x; i < nsteps; i += blockDim.x) st[i] = steps[i];
+  for (int i = threadIdx.x; i <= nlev; i += blockDim.x) lv[i] = lev[i];
+  if (direct)
+    for (int i = threadIdx.x; i < gw; i += blockDim.x) gsum[i] = 0.0;
   int bad = 0;
   build_leaves(leaves, nleaves, arena, a.params, a.pstride, a.inputs, a.F, b, sigma, &bad, threadIdx.x, blockDim.x);
   if (bad) atomicOr(a.status, 1 << TDQ_ERR_NONFINITE);
   __syncthreads();
-  for (int i = 0; i < nsteps; i++) {
-    step_generic<true>(st[i], arena, threadIdx.x, blockDim.x);  // shared-memory arena
+  for (int l = 0; l < nlev; l++) {
+    const int s1 = lv[l + 1];
+    const uint32_t total = st[s1 - 1].pre + step_outputs(st[s1 - 1]);
+    int i = lv[l];
+    for (uint32_t o = threadIdx.x; o < total; o += blockDim.x) {
+      while (o >= st[i].pre + step_outputs(st[i])) i++;
+      step_out<true>(st[i], arena, o - st[i].pre);
+    }
     __syncthreads();
   }
   if (threadIdx.x == 0) {
-    a.roots[e] = arena[root_local];
+    const c2 root = arena[root_local];
+    if (direct) values[b] = a.coeff * (double)root.x;
+    else a.roots[e] = root;
     arena[a.boff + root_local] = {(float)((a.gw ? a.gw[b] : 1.0) * a.coeff), 0.f};
   }
   __syncthreads();
-  for (int i = nsteps - 1; i >= 0; i--) {
-    step_adjoint(st[i], arena, a.boff, threadIdx.x, blockDim.x);
+  for (int l = nlev - 1; l >= 0; l--) {
+    const int s1 = lv[l + 1];
+    const uint32_t total = st[s1 - 1].preb + adjoint_outputs(st[s1 - 1]);
+    int i = lv[l];
+    for (uint32_t o = threadIdx.x; o < total; o += blockDim.x) {
+      while (o >= st[i].preb + adjoint_outputs(st[i])) i++;
+      adjoint_out(st[i], arena, a.boff, o - st[i].preb);
+    }
     __syncthreads();
   }
-  leaf_gradients(leaves, nleaves, arena, a.boff, a.params, a.pstride, a.inputs, a.F, b, sigma, a.gacc + b * a.P,
-                 threadIdx.x, blockDim.x);
+  leaf_gradients(leaves, nleaves, arena, a.boff, a.params, a.pstride, a.inputs, a.F, b, sigma,
+                 direct ? gsum : a.gacc + b * a.P, threadIdx.x, blockDim.x);
+  if (direct) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < gw; i += blockDim.x) grads[b * gw + i] = (float)gsum[i];
+  }
 }
 
 // Plain reverse tree: the root's cotangent, one launch per step, leaf gradients.
@@ -649,6 +682,27 @@ __global__ void k_tree_out(const double* acc, int B, int output, double coeff, d
   }
 }
 
+// The last kernel of a values-only execution whose slices all ride in one
+// batch: roots, their FP64 sum in slice order and the output in one launch
+// (three before).
+__global__ void k_tree_finish(TreeArgs a, int output, double* values) {
+  chain_start();
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= a.B) return;
+  double re = 0.0, im = 0.0;
+  for (int s = 0; s < a.chunk; s++) {
+    const size_t e = (size_t)b * a.chunk + s;
+    const c2 v = a.root_off >= 0 ? a.work[e * a.arena_elems + a.root_off] : a.roots[e];
+    re += (double)v.x;
+    im += (double)v.y;
+  }
+  if (output == TDQ_OUT_EXPVAL) values[b] = a.coeff * re;
+  else {
+    values[2 * b] = re;
+    values[2 * b + 1] = im;
+  }
+}
+
 }  // namespace
 
 // Launch with programmatic stream serialisation: the kernel may be
@@ -670,6 +724,10 @@ static cudaError_t launch_chained(void (*k)(KArgs...), dim3 g, dim3 b, size_t sm
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);
 }
+
+// Shared memory of the fused value-and-gradient kernel at most (200 KiB of
+// tensors and steps, the level bounds, a gradient row where it fits).
+constexpr size_t kFusedAdjSmem = 216 * 1024;
 
 struct TreeExec final : tdq_exec {
   int dev = 0, B = 0, P = 0, F = 0, output = 0, plain = 0;
@@ -705,7 +763,8 @@ struct TreeExec final : tdq_exec {
   int64_t boff = 0;
   LeafDev* d_fleaves = nullptr;  // fused reverse: leaves / steps with shared-arena offsets
   StepDev* d_fsteps = nullptr;
-  int nfleaves = 0, nfsteps = 0, froot = 0, fsmem_elems = 0;
+  int nfleaves = 0, nfsteps = 0, froot = 0, fsmem_elems = 0, nflev = 0;
+  int* d_flev = nullptr;         // level bounds of the steps
   size_t fsmem = 0;
   LeafDev* d_gleaves = nullptr;  // plain reverse: leaves with workspace offsets
   double* d_gacc = nullptr;
@@ -738,6 +797,7 @@ struct TreeExec final : tdq_exec {
     for (cudaStream_t x : side) cudaStreamDestroy(x);
     cudaFree(d_fleaves);
     cudaFree(d_fsteps);
+    cudaFree(d_flev);
     cudaFree(d_gleaves);
     cudaFree(d_rsteps);
     cudaFree(d_gacc);
@@ -857,8 +917,10 @@ struct TreeExec final : tdq_exec {
     a.gacc = d_gacc;
     a.P = P;
     a.gleaves = d_gleaves;
-    if (adj) TDQ_CUDA_TRY(cudaMemsetAsync(d_gacc, 0, sizeof(double) * (size_t)B * std::max(1, P), st));
     const int64_t s_lo = slice_lo, s_hi = slice_hi < 0 ? n_slices : slice_hi;
+    const size_t gsum_bytes = sizeof(double) * (size_t)std::max(1, P);
+    const bool direct = adj == 1 && s_hi - s_lo == 1 && fsmem + gsum_bytes <= kFusedAdjSmem;
+    if (adj && !direct) TDQ_CUDA_TRY(cudaMemsetAsync(d_gacc, 0, sizeof(double) * (size_t)B * std::max(1, P), st));
     if (s_lo >= s_hi)  // an empty slice range: the partial sums are zero
       TDQ_CUDA_TRY(cudaMemsetAsync(d_acc, 0, sizeof(double) * 2 * (size_t)B, st));
     for (int64_t s0 = s_lo; s0 < s_hi; s0 += chunk) {
@@ -866,10 +928,13 @@ struct TreeExec final : tdq_exec {
       a.slice0 = (uint32_t)s0;
       const int nb = B * a.chunk;
       if (adj == 1) {  // value and gradient of the whole network per CTA
-        (void)launch_chained(k_tree_fused_adj, dim3(nb), dim3(128), fsmem, st, a, d_fleaves, nfleaves, d_fsteps,
-                             nfsteps, froot, fsmem_elems);
+        const int ft = nb < 2 * sm_count ? 512 : (nb < 4 * sm_count ? 256 : 128);  // as the subtree launch below
+        (void)launch_chained(k_tree_fused_adj, dim3(nb), dim3(ft), fsmem + (direct ? gsum_bytes : 0), st, a, d_fleaves,
+                             nfleaves, d_fsteps, nfsteps, d_flev, nflev, froot, fsmem_elems, direct ? 1 : 0, values,
+                             grads);
         last_launches++;
         TDQ_CUDA_TRY(cudaGetLastError());
+        if (direct) return ok();
         (void)launch_chained(k_slice_sum, dim3((B + 127) / 128), dim3(128), 0, st, d_roots, B, a.chunk, d_acc,
                              s0 == s_lo);
         last_launches++;
@@ -911,6 +976,12 @@ struct TreeExec final : tdq_exec {
           TDQ_CUDA_TRY(cudaEventRecord(join_ev[k], side[k]));
           TDQ_CUDA_TRY(cudaStreamWaitEvent(st, join_ev[k], 0));
         }
+      }
+      if (!adj && a.chunk == s_hi - s_lo) {
+        (void)launch_chained(k_tree_finish, dim3((B + 127) / 128), dim3(128), 0, st, a, output, values);
+        last_launches++;
+        TDQ_CUDA_TRY(cudaGetLastError());
+        return ok();
       }
       if (root_off >= 0) {
         (void)launch_chained(k_tree_roots, dim3((nb + 255) / 256), dim3(256), 0, st, a);
@@ -1458,9 +1529,10 @@ extern "C" tdq_status tdq_plan_compile(const tdq_plan* p, const tdq_compile_opts
     sd.root_global = consumer[roots[ri]] >= 0 ? goff[roots[ri]] : -1;
     subs.push_back(sd);
     max_smem = std::max(max_smem, sizeof(c2) * (size_t)sd.smem_elems +
-                                      sizeof(StepDev) * (size_t)(sd.step_end - sd.step_begin));
+                                      sizeof(StepDev) * (size_t)(sd.step_end - sd.step_begin) +
+                                      sizeof(int) * (size_t)(sd.nlev + 1));
   }
-  if (max_smem > 200 * 1024)
+  if (max_smem > 202 * 1024)
     return fail(TDQ_ERR_UNSUPPORTED, "tdq_plan_compile: a subtree's shared arena exceeds 200 KiB");
 
   TreeExec* e = new (std::nothrow) TreeExec();
@@ -1705,16 +1777,35 @@ extern "C" tdq_status tdq_plan_compile(const tdq_plan* p, const tdq_compile_opts
     std::vector<LeafDev> fl;
     std::vector<StepDev> fs;
     for (int t = 0; t < nl; t++) fl.push_back(make_leaf(t, vo[t]));
-    for (int s2 = 0; s2 < nst; s2++) fs.push_back(make_step(s2, vo));
+    // level by level (0: the leaves; a step one above its higher operand)
+    std::vector<int> flev{0}, height(ntens, 0);
+    int top = 0;
+    for (int s2 = 0; s2 < nst; s2++)
+      top = std::max(top, height[nl + s2] = 1 + std::max(height[plan.steps[s2].a], height[plan.steps[s2].b]));
+    for (int l = 1; l <= top; l++) {
+      uint32_t pre = 0, preb = 0;
+      for (int s2 = 0; s2 < nst; s2++) {
+        if (height[nl + s2] != l) continue;
+        StepDev d = make_step(s2, vo);
+        d.pre = pre;
+        d.preb = preb;
+        pre += 1u << (d.nh + d.nm + d.nn);
+        preb += (1u << (d.nh + d.nm + d.nk)) + (1u << (d.nh + d.nn + d.nk));
+        fs.push_back(d);
+      }
+      flev.push_back((int)fs.size());
+    }
+    e->nflev = top;
+    if ((s = up((void**)&e->d_flev, flev.data(), sizeof(int) * flev.size())) != TDQ_OK) return bail(s);
     e->nfleaves = nl;
     e->nfsteps = nst;
     e->froot = (int)vo[ntens - 1];
     e->boff = vt_total;
     e->fsmem_elems = (int)((2 * vt_total + 1) & ~(int64_t)1);
-    e->fsmem = sizeof(c2) * (size_t)e->fsmem_elems + sizeof(StepDev) * (size_t)nst;
+    e->fsmem = sizeof(c2) * (size_t)e->fsmem_elems + sizeof(StepDev) * (size_t)nst + sizeof(int) * (size_t)(nst + 1);
     if ((s = up((void**)&e->d_fleaves, fl.data(), sizeof(LeafDev) * fl.size())) != TDQ_OK) return bail(s);
     if ((s = up((void**)&e->d_fsteps, fs.data(), sizeof(StepDev) * fs.size())) != TDQ_OK) return bail(s);
-    if (cudaFuncSetAttribute(k_tree_fused_adj, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e->fsmem) !=
+    if (cudaFuncSetAttribute(k_tree_fused_adj, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedAdjSmem) !=
         cudaSuccess)
       return bail(fail(TDQ_ERR_CUDA, "tdq_plan_compile: shared memory attribute"));
   }
