@@ -59,10 +59,10 @@ struct StepDev {
   int64_t a_off, b_off, c_off;
   uint32_t pre;   // subtree steps: outputs of the earlier steps of the same level
   uint32_t preb;  // ... and outputs of their reverse steps (entries of both operands)
-  int8_t nm, nn, nk, rc, nh;
-  int8_t cm[32];  // C bit position of m bit i (LSB first)
+  int8_t cm[32];  // C bit position of m bit i (LSB first); 8-byte aligned, see scatter_bits
   int8_t cn[32];  // C bit position of n bit i
   int8_t ch[kMaxHyperBits];  // C bit position of h bit i
+  int8_t nm, nn, nk, rc, nh;
 };
 
 __device__ __forceinline__ float leaf_angle(const LeafDev& L, int j, const float* params, int64_t pstride,
@@ -227,9 +227,19 @@ __device__ __forceinline__ void chain_start() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// The low n bits of x (the others zero) at the positions pos[]: eight positions
+// per read, as a byte-by-byte loop waited for shared memory at every bit.
 __device__ __forceinline__ uint32_t scatter_bits(uint32_t x, const int8_t* pos, int n) {
   uint32_t r = 0;
-  for (int i = 0; i < n; i++) r |= ((x >> i) & 1u) << pos[i];
+  for (int i = 0; i < n; i += 8) {
+    const uint2 p = *reinterpret_cast<const uint2*>(pos + i);
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+      r |= ((x >> j) & 1u) << ((p.x >> (8 * j)) & 31u);
+      r |= ((x >> (j + 4)) & 1u) << ((p.y >> (8 * j)) & 31u);
+    }
+    x >>= 8;
+  }
   return r;
 }
 
@@ -247,6 +257,7 @@ __device__ __forceinline__ void step_out(const StepDev& s, c2* arena, uint32_t o
   const c2* a = arena + s.a_off + (size_t)((h << s.nm) | m) * K;
   const c2* bb = arena + s.b_off + (size_t)((h << s.nn) | n) * K;
   float re = 0.f, im = 0.f;
+#pragma unroll 4  // several operand reads in flight: a level waits for its longest sum
   for (uint32_t k0 = 0; k0 < K; k0++) {
     const uint32_t k = kRot ? ((k0 + o) & (K - 1u)) : k0;
     const c2 x = a[k], y = bb[k];
@@ -257,6 +268,18 @@ __device__ __forceinline__ void step_out(const StepDev& s, c2* arena, uint32_t o
 }
 
 __device__ __forceinline__ uint32_t step_outputs(const StepDev& s) { return 1u << (s.nm + s.nn + s.nh); }
+
+// The step of a level, steps [s0, s1), that output o of the level belongs to
+// (kRev: of its reverse): the last one that starts at or before o.
+template <bool kRev>
+__device__ __forceinline__ int step_of(const StepDev* st, int s0, int s1, uint32_t o) {
+  while (s1 - s0 > 1) {
+    const int mid = (s0 + s1) >> 1;
+    if ((kRev ? st[mid].preb : st[mid].pre) <= o) s0 = mid;
+    else s1 = mid;
+  }
+  return s0;
+}
 
 template <bool kRot = false>
 __device__ void step_generic(const StepDev& s, c2* arena, int tid, int nt) {
@@ -390,10 +413,9 @@ __global__ void __launch_bounds__(512) k_tree_subtrees(TreeArgs a, const SubDev*
   for (int l = 0; l < sd.nlev; l++) {
     const int s0 = lv[l], s1 = lv[l + 1];
     const uint32_t total = st[s1 - 1].pre + step_outputs(st[s1 - 1]);
-    int i = s0;
     for (uint32_t o = threadIdx.x; o < total; o += blockDim.x) {
-      while (o >= st[i].pre + step_outputs(st[i])) i++;
-      step_out<true>(st[i], arena, o - st[i].pre);
+      const StepDev& x = st[step_of<false>(st, s0, s1, o)];
+      step_out<true>(x, arena, o - x.pre);
     }
     __syncthreads();
   }
@@ -441,10 +463,9 @@ __global__ void __launch_bounds__(512) k_tree_fused_adj(TreeArgs a, const LeafDe
   for (int l = 0; l < nlev; l++) {
     const int s1 = lv[l + 1];
     const uint32_t total = st[s1 - 1].pre + step_outputs(st[s1 - 1]);
-    int i = lv[l];
     for (uint32_t o = threadIdx.x; o < total; o += blockDim.x) {
-      while (o >= st[i].pre + step_outputs(st[i])) i++;
-      step_out<true>(st[i], arena, o - st[i].pre);
+      const StepDev& x = st[step_of<false>(st, lv[l], s1, o)];
+      step_out<true>(x, arena, o - x.pre);
     }
     __syncthreads();
   }
@@ -458,10 +479,9 @@ __global__ void __launch_bounds__(512) k_tree_fused_adj(TreeArgs a, const LeafDe
   for (int l = nlev - 1; l >= 0; l--) {
     const int s1 = lv[l + 1];
     const uint32_t total = st[s1 - 1].preb + adjoint_outputs(st[s1 - 1]);
-    int i = lv[l];
     for (uint32_t o = threadIdx.x; o < total; o += blockDim.x) {
-      while (o >= st[i].preb + adjoint_outputs(st[i])) i++;
-      adjoint_out(st[i], arena, a.boff, o - st[i].preb);
+      const StepDev& x = st[step_of<true>(st, lv[l], s1, o)];
+      adjoint_out(x, arena, a.boff, o - x.preb);
     }
     __syncthreads();
   }
@@ -535,55 +555,170 @@ __global__ void __launch_bounds__(256) k_tree_step_warp(TreeArgs a, int s) {
   }
 }
 
-// Few outputs, long k: split k.  Block (c, e) sums k in [c KC, (c + 1) KC)
+// Few outputs, long k: split k.  Block (c, e) sums `loops` chunks of KC k values
 // for every output of batch entry e from operand chunks staged in shared
-// memory, and adds its partial sums to C (zeroed before the launch) with FP32
-// atomics.  With fewer than 256 outputs, 256 / outputs consecutive lanes share
-// one (the kind rule sends 1..4096 outputs here); lanes of one output reduce
-// within their warp, and each warp's sum is added separately.
+// memory.  With fewer than 256 outputs, 256 / outputs consecutive lanes share
+// one (the kind rule sends 1..4096 outputs here); with more, a thread's sums
+// stay in shared memory between the chunks.  A block that holds all of k
+// writes C (no clearing, no atomics); otherwise the blocks add their sums to C
+// (cleared before the launch) with FP32 atomics.  (More chunks per block cost
+// more than the atomics they save: 1024 outputs, k 4096, 8 entries, 33 us with
+// one, 45 with four.)
 constexpr int kSplitSmemC2 = 6144;  // staged complex operands per block (48 KiB)
-__global__ void __launch_bounds__(256) k_tree_step_splitk(TreeArgs a, int s, int kc_log2) {
+__global__ void __launch_bounds__(256) k_tree_step_splitk(TreeArgs a, int s, int kc_log2, int loops, int direct) {
   chain_start();
   extern __shared__ __align__(16) unsigned char sk_raw[];
+  __shared__ c2 part[8];
   c2* As = reinterpret_cast<c2*>(sk_raw);
-  const StepDev st = a.steps[s];
+  const StepDev& st = a.steps[s];
+  const int nm = st.nm, nn = st.nn, nh = st.nh;
   c2* base = a.work + (size_t)blockIdx.y * a.arena_elems;
   const c2* A = base + st.a_off;
   const c2* B = base + st.b_off;
   c2* C = base + st.c_off;
-  const uint32_t K = 1u << st.nk, N = 1u << st.nn, KC = 1u << kc_log2;
-  const uint32_t HM = 1u << (st.nh + st.nm), HN = 1u << (st.nh + st.nn), MN = 1u << (st.nm + st.nn);
-  const uint32_t tot = MN << st.nh, k0 = blockIdx.x * KC;
+  const uint32_t K = 1u << st.nk, KC = 1u << kc_log2;
+  const uint32_t HM = 1u << (nh + nm), HN = 1u << (nh + nn), MN = 1u << (nm + nn), N = 1u << nn;
+  const uint32_t tot = MN << nh;
   c2* Bs = As + HM * KC;
-  // chunk rows: As[hm][kk] = A[hm][k0 + kk], Bs[hn][kk] = B[hn][k0 + kk] (coalesced along k)
-  for (uint32_t i = threadIdx.x; i < HM * KC; i += blockDim.x) As[i] = A[(size_t)(i >> kc_log2) * K + k0 + (i & (KC - 1))];
-  for (uint32_t i = threadIdx.x; i < HN * KC; i += blockDim.x) Bs[i] = B[(size_t)(i >> kc_log2) * K + k0 + (i & (KC - 1))];
-  __syncthreads();
-  // lanes per output: 256 / tot (1..16 for tot >= 16), consecutive lanes of a warp
+  c2* acc = Bs + HN * KC;  // [tot], for tot > 256
+  // lanes per output: 256 / tot (1..256), consecutive lanes
   const uint32_t lpo = tot >= 256 ? 1u : 256u / tot;
   const uint32_t lane_o = threadIdx.x % lpo;
-  for (uint32_t o = threadIdx.x / lpo; o < tot; o += blockDim.x / lpo) {
-    const uint32_t h = o >> (st.nm + st.nn), m = (o & (MN - 1u)) >> st.nn, n = o & (N - 1u);
-    const c2* x = As + ((h << st.nm) | m) * KC;
-    const c2* y = Bs + ((h << st.nn) | n) * KC;
-    float re = 0.f, im = 0.f;
-    for (uint32_t kk = lane_o; kk < KC; kk += lpo) {
-      // rotate the start so that lanes reading different rows hit different banks
-      const uint32_t q = (kk + (n & 31u)) & (KC - 1u);
-      const c2 u = x[q], v = y[q];
-      re = fmaf(u.x, v.x, fmaf(-u.y, v.y, re));
-      im = fmaf(u.x, v.y, fmaf(u.y, v.x, im));
+  float re = 0.f, im = 0.f;
+  for (int l = 0; l < loops; l++) {
+    const uint32_t k0 = (blockIdx.x * (uint32_t)loops + (uint32_t)l) * KC;
+    if (l) __syncthreads();
+    // chunk rows: As[hm][kk] = A[hm][k0 + kk], Bs[hn][kk] = B[hn][k0 + kk] (coalesced along k)
+    for (uint32_t i = threadIdx.x; i < HM * KC; i += 256) As[i] = A[(size_t)(i >> kc_log2) * K + k0 + (i & (KC - 1))];
+    for (uint32_t i = threadIdx.x; i < HN * KC; i += 256) Bs[i] = B[(size_t)(i >> kc_log2) * K + k0 + (i & (KC - 1))];
+    __syncthreads();
+    for (uint32_t o = threadIdx.x / lpo; o < tot; o += 256 / lpo) {
+      const uint32_t h = o >> (nm + nn), m = (o & (MN - 1u)) >> nn, n = o & (N - 1u);
+      const c2* x = As + ((h << nm) | m) * KC;
+      const c2* y = Bs + ((h << nn) | n) * KC;
+      if (tot > 256) {
+        const c2 v = l ? acc[o] : c2{0.f, 0.f};
+        re = v.x;
+        im = v.y;
+      }
+#pragma unroll 4
+      for (uint32_t kk = lane_o; kk < KC; kk += lpo) {
+        // rotate the start so that lanes reading different rows hit different banks
+        const uint32_t q = (kk + (n & 31u)) & (KC - 1u);
+        const c2 u = x[q], v = y[q];
+        re = fmaf(u.x, v.x, fmaf(-u.y, v.y, re));
+        im = fmaf(u.x, v.y, fmaf(u.y, v.x, im));
+      }
+      if (tot > 256) acc[o] = {re, im};
     }
-    const uint32_t red = lpo < 32u ? lpo : 32u;  // lanes of this output within one warp
-    for (uint32_t d = red >> 1; d > 0; d >>= 1) {
-      re += __shfl_xor_sync(0xffffffffu, re, d);
-      im += __shfl_xor_sync(0xffffffffu, im, d);
+  }
+  // lanes of one output within a warp, then (fewer than 8 outputs) its warps
+  const uint32_t red = lpo < 32u ? lpo : 32u;
+  for (uint32_t d = red >> 1; d > 0; d >>= 1) {
+    re += __shfl_xor_sync(0xffffffffu, re, d);
+    im += __shfl_xor_sync(0xffffffffu, im, d);
+  }
+  const uint32_t wpo = lpo / 32u;  // warps per output, 0 if an output has at most a warp
+  if (wpo > 1) {
+    if ((threadIdx.x & 31u) == 0) part[threadIdx.x >> 5] = {re, im};
+    __syncthreads();
+    if (lane_o == 0)
+      for (uint32_t w = 1; w < wpo; w++) {
+        re += part[(threadIdx.x >> 5) + w].x;
+        im += part[(threadIdx.x >> 5) + w].y;
+      }
+  }
+  for (uint32_t o = threadIdx.x / lpo; o < tot; o += 256 / lpo) {
+    if (lane_o) break;
+    const uint32_t h = o >> (nm + nn), m = (o & (MN - 1u)) >> nn, n = o & (N - 1u);
+    const c2 v = tot > 256 ? acc[o] : c2{re, im};
+    c2* c = &C[scatter_bits(h, st.ch, nh) | scatter_bits(m, st.cm, nm) | scatter_bits(n, st.cn, nn)];
+    if (direct) {
+      *c = v;
+    } else {
+      atomicAdd(&c->x, v.x);
+      atomicAdd(&c->y, v.y);
     }
-    if (lane_o % red == 0) {
-      float* c = reinterpret_cast<float*>(
-          &C[scatter_bits(h, st.ch, st.nh) | scatter_bits(m, st.cm, st.nm) | scatter_bits(n, st.cn, st.nn)]);
-      atomicAdd(c, re);
-      atomicAdd(c + 1, im);
+  }
+}
+
+// Middling steps: (256 R R)-output tiles of C[m][n] = sum_k A[m][k] B[n][k], R x R
+// outputs per thread, operand rows staged in shared memory a chunk of k at a
+// time, read along k (coalesced; rows padded by one entry, so that the lanes'
+// rows lie in different banks).  The step's bit places are staged too (as a
+// local copy they lived in local memory).  lsplit > 0: k is split over 2^lsplit
+// blocks, which add their sums to C (cleared before the launch) with FP32
+// atomics: 32 x 32 outputs, k 4096, 8 entries, 20 us (33 in
+// k_tree_step_splitk, an output at a time).  Bound by latency: 128 x 32 outputs, k
+// 128, 4 entries 10 us (17 at a warp per output), 512 x 8, k 32: 8.9 (10.5 at a
+// thread per output); the 7 x 7 amplitude, 13 large steps, 127 -> 79 us.
+constexpr int kTileK = 64;  // k entries staged at a time
+template <int R>
+__global__ void __launch_bounds__(256) k_tree_tile(TreeArgs a, int s, int ltm, int ltn, int lsplit) {
+  chain_start();
+  extern __shared__ __align__(16) unsigned char tl_raw[];
+  __shared__ __align__(8) int8_t pos[80];
+  const StepDev& st = a.steps[s];
+  const int nm = st.nm, nn = st.nn, nk = st.nk, nh = st.nh;
+  if (threadIdx.x < 80) {
+    const int i = threadIdx.x;
+    pos[i] = i < 32 ? st.cm[i] : i < 64 ? st.cn[i - 32] : st.ch[i - 64];
+  }
+  const uint32_t K = 1u << nk, KC = min(K, (uint32_t)kTileK), P = KC + 1u;
+  const int lkc = nk < 6 ? nk : 6;
+  const uint32_t TM = 1u << ltm, TN = 1u << ltn;
+  c2* As = reinterpret_cast<c2*>(tl_raw);
+  c2* Bs = As + TM * P;
+  const uint32_t h = blockIdx.z & ((1u << nh) - 1u), m0 = blockIdx.x << ltm,
+                 n0 = (blockIdx.y >> lsplit) << ltn;
+  const uint32_t ks = K >> lsplit, kb = (blockIdx.y & ((1u << lsplit) - 1u)) * ks;  // this block's k
+  c2* base = a.work + (size_t)(blockIdx.z >> nh) * a.arena_elems;
+  const c2* A = base + st.a_off + ((size_t)((h << nm) + m0) << nk);
+  const c2* B = base + st.b_off + ((size_t)((h << nn) + n0) << nk);
+  c2* C = base + st.c_off;
+  const uint32_t tn = threadIdx.x & ((TN / R) - 1u), tm = threadIdx.x / (TN / R);
+  const bool active = tm < TM / R;
+  float re[R][R] = {}, im[R][R] = {};
+  for (uint32_t k0 = kb; k0 < kb + ks; k0 += KC) {
+    if (k0 > kb) __syncthreads();
+#pragma unroll 4
+    for (uint32_t i = threadIdx.x; i < (TM << lkc); i += 256) As[(i >> lkc) * P + (i & (KC - 1u))] = A[((size_t)(i >> lkc) << nk) + k0 + (i & (KC - 1u))];
+#pragma unroll 4
+    for (uint32_t i = threadIdx.x; i < (TN << lkc); i += 256) Bs[(i >> lkc) * P + (i & (KC - 1u))] = B[((size_t)(i >> lkc) << nk) + k0 + (i & (KC - 1u))];
+    __syncthreads();
+    if (active) {
+#pragma unroll 4
+      for (uint32_t kk = 0; kk < KC; kk++) {
+        c2 x[R], y[R];
+#pragma unroll
+        for (int i = 0; i < R; i++) {
+          x[i] = As[(tm + i * (TM / R)) * P + kk];
+          y[i] = Bs[(tn + i * (TN / R)) * P + kk];
+        }
+#pragma unroll
+        for (int i = 0; i < R; i++)
+#pragma unroll
+          for (int j = 0; j < R; j++) {
+            re[i][j] = fmaf(x[i].x, y[j].x, fmaf(-x[i].y, y[j].y, re[i][j]));
+            im[i][j] = fmaf(x[i].x, y[j].y, fmaf(x[i].y, y[j].x, im[i][j]));
+          }
+      }
+    }
+  }
+  if (!active) return;
+  const uint32_t ch = scatter_bits(h, pos + 64, nh);
+#pragma unroll
+  for (int i = 0; i < R; i++) {
+    const uint32_t cm = ch | scatter_bits(m0 + tm + i * (TM / R), pos, nm);
+#pragma unroll
+    for (int j = 0; j < R; j++) {
+      c2* c = &C[cm | scatter_bits(n0 + tn + j * (TN / R), pos + 32, nn)];
+      if (lsplit) {
+        atomicAdd(&c->x, re[i][j]);
+        atomicAdd(&c->y, im[i][j]);
+      } else {
+        *c = {re[i][j], im[i][j]};
+      }
     }
   }
 }
@@ -725,6 +860,10 @@ static cudaError_t launch_chained(void (*k)(KArgs...), dim3 g, dim3 b, size_t sm
   return cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);
 }
 
+// Tensor-core and 64 x 64-tile steps up to this many complex multiply-adds (over
+// the batch) run in k_tree_tile instead.
+constexpr double kTileMacs = 1 << 22;
+
 // Shared memory of the fused value-and-gradient kernel at most (200 KiB of
 // tensors and steps, the level bounds, a gradient row where it fits).
 constexpr size_t kFusedAdjSmem = 216 * 1024;
@@ -812,6 +951,21 @@ struct TreeExec final : tdq_exec {
     cudaFree(d_status);
   }
 
+  // Whether a step runs in k_tree_tile: thread- and warp-per-output steps,
+  // 64 x 64 SIMT tiles over a short k (2^12 x 2^5 outputs, k 16, 8 entries: 16 us
+  // against 39), and tensor-core steps whose fixed cost outweighs the arithmetic
+  // (128 x 128, k 8, 8 entries: 9 us against 19; 2^10 x 2^7, k 8: 14 against 17;
+  // 2^8 x 2^6, k 128: 22 against 18).  (At least 256 outputs per batch entry; 256 x
+  // 65 rows of staged operands at most, 135 KB.)
+  static bool tile_step(const StepDev& sd, int kind, int nb) {
+    const int out = sd.nm + sd.nn;
+    if (kind == 5) return sd.nm >= 5 && sd.nn >= 5 && ((int64_t)nb << sd.nh) <= 65535;
+    if (out < 8 || ((int64_t)nb << sd.nh) > 65535 || sd.nn > 19) return false;
+    if (kind == 0 || kind == 4 || (kind == 1 && sd.nk <= 5)) return true;
+    const double macs = std::ldexp((double)nb, sd.nh + out + sd.nk);
+    return macs <= kTileMacs;
+  }
+
   // One large step for nb batch entries on stream st (descriptors: host H,
   // device D == a.steps, kinds K; default: the forward steps).
   tdq_status launch_step(const TreeArgs& a, int s, int nb, cudaStream_t st) {
@@ -821,7 +975,24 @@ struct TreeExec final : tdq_exec {
                             const StepDev* D, const std::vector<int>& K) {
     const StepDev& sd = H[s];
     const std::vector<int>& step_kind = K;
-    if (step_kind[s] == 2 || step_kind[s] == 3) {
+    if (tile_step(sd, step_kind[s], nb)) {
+      const int64_t outs = (int64_t)nb << (sd.nh + sd.nm + sd.nn);
+      // 32 x 32 tiles while they fill the SMs, or over a long k, split to fill them
+      const bool split = step_kind[s] == 5;
+      const bool two = sd.nm >= 5 && sd.nn >= 5 && (split || outs >= (1 << 17));
+      int lsplit = 0;
+      while (split && lsplit < sd.nk - 6 && (outs >> 10 << lsplit) < 256) lsplit++;
+      if (lsplit && cudaMemset2DAsync(reinterpret_cast<c2*>(d_work) + sd.c_off, (size_t)arena * sizeof(c2), 0,
+                                      sizeof(c2) << (sd.nh + sd.nm + sd.nn), nb, st) != cudaSuccess)
+        return fail(TDQ_ERR_CUDA, "step " + std::to_string(s) + ": clearing the split-k output");
+      const int lt = two ? 10 : 8;
+      int ltn = std::min((int)sd.nn, lt / 2), ltm = std::min((int)sd.nm, lt - ltn);
+      ltn = std::min((int)sd.nn, lt - ltm);
+      const dim3 g(1u << (sd.nm - ltm), 1u << (sd.nn - ltn + lsplit), (unsigned)nb << sd.nh);
+      const size_t sm = sizeof(c2) * ((1u << ltm) + (1u << ltn)) * ((size_t)std::min(1 << sd.nk, kTileK) + 1);
+      if (two) (void)launch_chained(k_tree_tile<2>, g, dim3(256), sm, st, a, s, ltm, ltn, lsplit);
+      else (void)launch_chained(k_tree_tile<1>, g, dim3(256), sm, st, a, s, ltm, ltn, 0);
+    } else if (step_kind[s] == 2 || step_kind[s] == 3) {
       const bool ax = step_kind[s] == 2;
       const StepDev* dd = D + s;
       CgemmOut map{ax ? dd->cm : dd->cn, ax ? dd->cn : dd->cm, ax ? sd.nm : sd.nn, ax ? sd.nn : sd.nm, 0};
@@ -849,16 +1020,22 @@ struct TreeExec final : tdq_exec {
                    (unsigned)nb << sd.nh);
       (void)launch_chained(k_tree_gemm, dim3(g), dim3(256), 0, st, a, s);
     } else if (step_kind[s] == 5) {
-      // chunk of k: the largest power of two that keeps both operand chunks in 48 KiB
+      // chunk of k: the largest power of two that keeps both operand chunks in
+      // 48 KiB; a block takes all of them while that is at most 4096 k x outputs,
+      // and then writes the result itself
       const int mn = ((1 << sd.nm) + (1 << sd.nn)) << sd.nh;
       int kcl = 0;
       while (kcl < sd.nk && ((int64_t)mn << (kcl + 1)) <= kSplitSmemC2) kcl++;
-      const size_t csize = sizeof(c2) << (sd.nh + sd.nm + sd.nn);
-      if (cudaMemset2DAsync(reinterpret_cast<c2*>(d_work) + sd.c_off, (size_t)arena * sizeof(c2), 0, csize, nb, st) !=
-          cudaSuccess)
+      const int out = sd.nh + sd.nm + sd.nn, chunks = 1 << (sd.nk - kcl);
+      const int loops = out + sd.nk <= 12 ? chunks : 1;
+      const bool direct = loops == chunks;
+      const size_t csize = sizeof(c2) << out;
+      if (!direct && cudaMemset2DAsync(reinterpret_cast<c2*>(d_work) + sd.c_off, (size_t)arena * sizeof(c2), 0, csize,
+                                       nb, st) != cudaSuccess)
         return fail(TDQ_ERR_CUDA, "step " + std::to_string(s) + ": clearing the split-k output");
-      (void)launch_chained(k_tree_step_splitk, dim3(1u << (sd.nk - kcl), nb), dim3(256),
-                           sizeof(c2) * ((size_t)mn << kcl), st, a, s, kcl);
+      (void)launch_chained(k_tree_step_splitk, dim3((unsigned)(chunks / loops), nb), dim3(256),
+                           sizeof(c2) * (((size_t)mn << kcl) + (out > 8 ? (size_t)1 << out : 0)), st, a, s, kcl, loops,
+                           direct ? 1 : 0);
     } else if (step_kind[s] == 4) {
       const int64_t tot = (int64_t)1 << (sd.nh + sd.nm + sd.nn);
       const unsigned blocks = (unsigned)std::min<int64_t>((tot * 32 + 255) / 256, 8192);
@@ -1718,6 +1895,13 @@ extern "C" tdq_status tdq_plan_compile(const tdq_plan* p, const tdq_compile_opts
   if ((s = up((void**)&e->d_slev, slev.data(), sizeof(int) * slev.size())) != TDQ_OK) return bail(s);
   if ((s = up((void**)&e->d_steps, e->steps_h.data(), sizeof(StepDev) * e->steps_h.size())) != TDQ_OK)
     return bail(s);
+  constexpr int kTileSmem = (int)sizeof(c2) * (256 + 1) * (kTileK + 1);
+  if (cudaFuncSetAttribute(k_tree_tile<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmem) != cudaSuccess ||
+      cudaFuncSetAttribute(k_tree_tile<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmem) != cudaSuccess)
+    return bail(fail(TDQ_ERR_CUDA, "tdq_plan_compile: shared memory attribute"));
+  if (cudaFuncSetAttribute(k_tree_step_splitk, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)sizeof(c2) * (8192 + 4096)) != cudaSuccess)
+    return bail(fail(TDQ_ERR_CUDA, "tdq_plan_compile: shared memory attribute"));
   if (cudaFuncSetAttribute(k_tree_subtrees, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem) !=
       cudaSuccess)
     return bail(fail(TDQ_ERR_CUDA, "tdq_plan_compile: shared memory attribute"));
