@@ -203,23 +203,28 @@ __device__ __forceinline__ void k1_issue(c2* buf, c2* g, const TiledDev& t, cons
 }
 
 // The (row, tile) units of this CTA: a contiguous range of the row-major
-// unit index, cut into per-row segments; f(lr, tile0, tile1) runs one.
-template <class F>
-__device__ __forceinline__ void k1_for_segments(const TiledDev& t, F&& f) {
-  const int64_t total = (int64_t)t.nrows * t.ntiles;
-  int64_t u = (int64_t)blockIdx.x * t.tiles_per_cta;
-  const int64_t u1 = min(total, u + t.tiles_per_cta);
+// unit index, cut into per-row segments: tiles [tile0, tile1) of row lr.  (Not
+// a callback: the largest programs' was compiled as a function of its own, and
+// spilled 1.6 KB at its register limit.)
+struct Segments {
+  int64_t u, u1;
+  int lr = 0, tile0 = 0, tile1 = 0;
   bool first = true;
-  while (u < u1) {
-    const int lr = (int)(u / t.ntiles);
-    const int tile0 = (int)(u - (int64_t)lr * t.ntiles);
-    const int tile1 = (int)min((int64_t)t.ntiles, tile0 + (u1 - u));
-    if (!first) __syncthreads();  // the previous row's partial sums are read out
-    f(lr, tile0, tile1);
-    first = false;
-    u += tile1 - tile0;
+  __device__ __forceinline__ explicit Segments(const TiledDev& t) {
+    u = (int64_t)blockIdx.x * t.tiles_per_cta;
+    u1 = min((int64_t)t.nrows * t.ntiles, u + t.tiles_per_cta);
   }
-}
+  __device__ __forceinline__ bool next(const TiledDev& t) {
+    if (u >= u1) return false;
+    if (!first) __syncthreads();  // the previous row's partial sums are read out
+    first = false;
+    lr = (int)(u / t.ntiles);
+    tile0 = (int)(u - (int64_t)lr * t.ntiles);
+    tile1 = (int)min((int64_t)t.ntiles, tile0 + (u1 - u));
+    u += tile1 - tile0;
+    return true;
+  }
+};
 
 // Forward pass.  FIRST: the tile starts as the initial state (|0...0> or the
 // caller's) instead of being read.  LAST: accumulate the observable groups; with GRAD also form lambda = O_w psi
@@ -249,7 +254,8 @@ __device__ __forceinline__ void k1_forward_body(const SweepArgs& a, const TiledD
   // 5 rows, 7 passes of 15 to 50 us, 215 -> 143 us; 16 qubits, 24 rows, 218 -> 168
   chain_dispatch();
   bool waited = false;
-  k1_for_segments(t, [&](int lr, int tile0, int tile1) {
+  for (Segments seg(t); seg.next(t);) {
+    const int lr = seg.lr, tile0 = seg.tile0, tile1 = seg.tile1;
     const int row = t.row0 + lr;
     const int64_t b = row / a.ps_copies;
     const int kk = row % a.ps_copies;
@@ -350,7 +356,7 @@ __device__ __forceinline__ void k1_forward_body(const SweepArgs& a, const TiledD
         atomicAdd(&t.vals[(int64_t)lr * a.n_groups + g], s.vsum[g]);
     }
     if (GRAD && LAST) Prog::flush(a, t, s, lr);
-  });
+  }
 }
 
 // Reverse pass over the tiles of one pass (passes before the last), one
@@ -364,7 +370,8 @@ __device__ __forceinline__ void k1_reverse_body(const SweepArgs& a, const TiledD
   const uint32_t other = (dim - 1u) & ~t.smask;
   chain_dispatch();
   bool waited = false;
-  k1_for_segments(t, [&](int lr, int tile0, int tile1) {
+  for (Segments seg(t); seg.next(t);) {
+    const int lr = seg.lr, tile0 = seg.tile0, tile1 = seg.tile1;
     const int row = t.row0 + lr;
     const int64_t b = row / a.ps_copies;
     int bad = 0;
@@ -402,7 +409,7 @@ __device__ __forceinline__ void k1_reverse_body(const SweepArgs& a, const TiledD
       __syncthreads();
     }
     Prog::flush(a, t, s, lr);
-  });
+  }
 }
 
 }  // namespace tdq

@@ -119,4 +119,10 @@ struct LinProgram {
 // adj, mr (reverse) bits.
 LinProgram lin_program(const std::vector<SweepOp>& ops, int n, int k, int L, int mf, int mr, bool adj, bool exact);
 
+// Tiled program: the number of lowest index bits that every tile holds is
+// chosen here (4 .. 2, returned in *L): fewer leave a tile more directions of
+// its own.
+LinProgram lin_tiled_program(const std::vector<SweepOp>& ops, int n, int k, int mf, int mr, bool adj, bool exact,
+                             int* L);
+
 }  // namespace tdq

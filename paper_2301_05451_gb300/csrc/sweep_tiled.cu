@@ -271,13 +271,12 @@ tdq_status tiled_lin_plan(TiledSweep& t, const tdq_circuit* c, const std::vector
   const int kq = tile_qubits > 0 ? tile_qubits : 12;
   if (kq < 5 || kq > 13) return fail(TDQ_ERR_ARG, "tile_qubits must be in 5..13");
   t.k = std::min(t.n, kq);
-  t.L = std::min(4, t.k);
   t.adj = adj;
   t.rows = rows;
   t.P = c->n_params;
   t.ng = c->n_groups;
   if (t.ng > 1024) return fail(TDQ_ERR_UNSUPPORTED, "tiled sweep: more than 1024 output groups");
-  prog = lin_program(ops, t.n, t.k, t.L, fb, rb, adj, exact);
+  prog = lin_tiled_program(ops, t.n, t.k, fb, rb, adj, exact, &t.L);
   t.passes.clear();
   t.max_rec = 0;
   t.max_dops = 0;

@@ -71,8 +71,10 @@ int main() {
   }
   std::vector<float> params((size_t)rows * P);
   for (float& p : params) p = get<float>();
-  const int k = tile ? std::min(n, tile) : n, L = tile ? std::min(4, k) : 0;
-  LinProgram prog = lin_program(ops, n, k, L, fb, rb, adj, ng == 0);
+  const int k = tile ? std::min(n, tile) : n;
+  int L = 0;
+  LinProgram prog = tile ? lin_tiled_program(ops, n, k, fb, rb, adj, ng == 0, &L)
+                         : lin_program(ops, n, n, 0, fb, rb, adj, ng == 0);
   for (TermDev& t : terms) {
     uint32_t m = 0;
     for (int q = 0; q < n; q++)
