@@ -47,25 +47,17 @@ __global__ void __launch_bounds__(kK2GenericThreads) k2_sweep_smem(SweepArgs a, 
 // held or a free slot remains; a gate left out blocks its qubits for the rest
 // of the scan (every later gate on them must follow it).  The next pass scans
 // the gates left out, in order.  Each pass lists its gates in a valid order.
-// max_slots > 0 caps the gradient slots of a pass (a gate whose angles would
-// exceed it waits for the next pass, like a gate whose bit does not fit): a
-// reverse pass keeps one accumulator per slot in registers beside its
-// amplitudes, and large sets of them spilled registers.
 static void reg_pass_schedule(const std::vector<SweepOp>& ops, int b, int e, const int8_t* loc, int k,
-                              int mreg, std::vector<std::pair<std::vector<int>, std::vector<int>>>& out,
-                              int max_slots = 0) {
+                              int mreg, std::vector<std::pair<std::vector<int>, std::vector<int>>>& out) {
   const int M = std::min(mreg, k);
   std::vector<int> todo;
   for (int o = b; o < e; o++) todo.push_back(o);
   while (!todo.empty()) {
     std::vector<int> bits, taken, left;
     uint64_t blocked = 0;  // global bit positions
-    int nslots = 0;
     for (int o : todo) {
       const SweepOp& op = ops[o];
       const uint64_t qm = (1ull << op.p0) | (op.p1 >= 0 ? 1ull << op.p1 : 0ull);
-      int ns = 0;
-      for (int j = 0; j < op.nang && j < 3; j++) ns += op.slot[j] >= 0 ? 1 : 0;
       int need = -1;
       switch (op.kind) {
         case K_RZ: case K_Z: case K_CZ: case K_RZZ: break;
@@ -73,14 +65,11 @@ static void reg_pass_schedule(const std::vector<SweepOp>& ops, int b, int e, con
         default: need = loc[op.p0]; break;
       }
       bool ok = (blocked & qm) == 0;
-      // a pass always takes its first gate, whatever its slots
-      if (ok && max_slots > 0 && !taken.empty() && nslots + ns > max_slots) ok = false;
       if (ok && need >= 0 && std::find(bits.begin(), bits.end(), need) == bits.end()) {
         if ((int)bits.size() < M) bits.push_back(need);
         else ok = false;
       }
       if (ok) {
-        nslots += ns;
         taken.push_back(o);
       } else {
         blocked |= qm;
@@ -98,7 +87,7 @@ static void reg_pass_schedule(const std::vector<SweepOp>& ops, int b, int e, con
 void build_program(const std::vector<SweepOp>& ops, int b, int e, const int8_t* loc, int k, bool fuse,
                    int rec0, int mreg, Program& P) {
   std::vector<std::pair<std::vector<int>, std::vector<int>>> ranges;
-  reg_pass_schedule(ops, b, e, loc, k, mreg, ranges, fuse ? 0 : kRevPassSlots);
+  reg_pass_schedule(ops, b, e, loc, k, mreg, ranges);
   const int M = std::min(mreg, k);
   for (const auto& rg : ranges) {
     const std::vector<int>& lb = rg.second;
@@ -772,7 +761,7 @@ static tdq_status compile_sweep_impl(const tdq_circuit* c, const tdq_compile_opt
   }
   if (!e->smem_path) {
     s = tiled_compile(e->tiled, c, ops, ps_gate, e->B * e->copies, adj, o->tile_qubits, spec ? &lin : nullptr, fb1, rb1,
-                      &e->bytes_row);
+                      o->output == TDQ_OUT_STATE || o->output == TDQ_OUT_PROBS, &e->bytes_row);
     if (s != TDQ_OK) return bail(s);
     // outputs: the state read back from HBM and written out as values
     if (e->output == TDQ_OUT_STATE || e->output == TDQ_OUT_PROBS)

@@ -3,6 +3,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <map>
 #include <string>
 #include <vector>
 
@@ -51,35 +52,147 @@ __global__ void k1_finalize(SweepArgs a, TiledDev t, int nrows, int grad_adj) {
     for (int j = threadIdx.x; j < a.P; j += blockDim.x) a.grads[b * a.P + j] = (float)t.gacc[(int64_t)lr * a.P + j];
 }
 
+// (double)f and (double)f * f without the FP64 pipe, which runs at less than a
+// 64th of the FP32 rate and is what a read-out of states waits for (four FP64
+// instructions per probability: 160 us for 2^24 of them).  Exact; only
+// subnormal and non-finite floats take the conversion.
+__device__ __forceinline__ double exact_double(float f) {
+  const uint32_t u = __float_as_uint(f), e = (u >> 23) & 255u;
+  if ((e == 0u && (u << 1)) || e == 255u) return (double)f;
+  const uint32_t hi = (u & 0x80000000u) | (e ? ((u & 0x7fffffffu) >> 3) + (896u << 20) : 0u);
+  return __hiloint2double((int)hi, (int)(u << 29));
+}
+__device__ __forceinline__ double exact_square(float f) {
+  const uint32_t u = __float_as_uint(f), e = (u >> 23) & 255u;
+  if (e - 1u >= 254u) return (u << 1) ? (double)f * (double)f : 0.0;
+  // (2^7 m)^2 with the 24-bit m: in [2^60, 2^62); normalised to bit 62
+  const uint32_t m = ((u & 0x7fffffu) | 0x800000u) << 7;
+  const uint32_t ph = __umulhi(m, m), pl = m * m, top = ph >> 29;  // (bit 61)
+  const uint32_t h = top ? ph : __funnelshift_l(pl, ph, 1), l = top ? pl : pl << 1;
+  // mantissa bits 61..9 of (h, l); 2 e - 254 + 1023 - 1 (the leading one adds 1), + 1 for the top half
+  return __hiloint2double((int)(((2u * e + 768u + top) << 20) + (h >> 9)), (int)__funnelshift_r(l, h, 9));
+}
+
 // The chunk's final states as the output: the whole state (TDQ_OUT_STATE) or
-// the probabilities (TDQ_OUT_PROBS) of every row, grid-stride over (row, x).
-// Basis index x sits at place y(x), linear over its bits: tables of y over
-// the bits 0..7, 8..15, 16..23 and 24..29 give it with four reads.
-__global__ void __launch_bounds__(256) k1_state_out(SweepArgs a, TiledDev t, int nrows) {
-  __shared__ uint32_t tab[4][256];
-  for (int q = 0; q < 4; q++) {
-    uint32_t y = 0;
-    for (int i = 0; i < 8; i++)
-      if (((threadIdx.x >> i) & 1u) && 8 * q + i < t.n) y ^= a.lin ? a.lin[8 * q + i] : 1u << (8 * q + i);
-    tab[q][threadIdx.x] = y ^ (q == 0 && a.lin ? a.lin[t.n] : 0u);
+// the probabilities (TDQ_OUT_PROBS) of every row.  Basis index x sits at place
+// y(x), a linear map: element by element one of the two sides would be
+// scattered, 32 bytes moved for 8 used.  A block moves one coset at a time of
+// a space that holds both 2^5 consecutive x and the x of 2^5 consecutive y
+// (OutMap): read in runs of y, turned in shared memory, written in runs of x.
+// The maps are linear: a thread's elements tid + 256 i differ by constants.
+// 20 qubits, 16 rows, 128 MiB read, 128 MiB of probabilities written:
+// 77 us, 160 element by element with FP64 conversions.
+constexpr int kOutPer = (1 << kOutBits) / 256;  // elements per thread
+__global__ void __launch_bounds__(256) k1_state_out(SweepArgs a, TiledDev t, int nrows, const OutMap* __restrict__ m) {
+  __shared__ c2 buf[1 << kOutBits];
+  __shared__ uint32_t at_yx[2];  // this tile's first y and x
+  const int size = 1 << m->bits, tid = threadIdx.x;
+  const bool on = tid < size;
+  const uint32_t ox = m->x[tid], oy = m->y[tid], at = m->at[tid];
+  uint32_t cx[kOutPer], cy[kOutPer], ca[kOutPer];
+#pragma unroll
+  for (int i = 0; i < kOutPer; i++) {
+    cx[i] = m->x[256 * i];
+    cy[i] = m->y[256 * i];
+    ca[i] = swz(m->at[256 * i]);
   }
-  __syncthreads();
-  const int64_t dim = (int64_t)1 << t.n, tot = dim * nrows;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < tot; i += (int64_t)gridDim.x * blockDim.x) {
-    const int lr = (int)(i >> t.n);
+  const int per = max(1, size / 256);
+  const int64_t dim = (int64_t)1 << t.n, per_row = dim >> m->bits, tot = per_row * nrows;
+  const uint32_t other = (uint32_t)(dim - 1) & ~m->pivots;
+  for (int64_t tile = blockIdx.x; tile < tot; tile += gridDim.x) {
+    const int lr = (int)(tile / per_row);
     const int row = t.row0 + lr;
+    const int64_t b = row / a.ps_copies;
     if (row % a.ps_copies) continue;
-    const int64_t b = row / a.ps_copies, x = i - (int64_t)lr * dim;
-    const uint32_t y = tab[0][x & 255] ^ tab[1][(x >> 8) & 255] ^ tab[2][(x >> 16) & 255] ^ tab[3][(x >> 24) & 255] ^
-                       (a.row_frame ? a.row_frame[lr] : 0u);
-    const c2 v = t.psi[(size_t)lr * dim + y];
-    if (a.output == TDQ_OUT_STATE) {
-      a.values[(b * dim + x) * 2] = v.x;
-      a.values[(b * dim + x) * 2 + 1] = v.y;
-    } else {
-      a.values[b * dim + x] = (double)v.x * v.x + (double)v.y * v.y;
+    if (tid < 32) {  // y of the tile's first x: a bit of x per lane
+      const uint32_t x0 = deposit((uint32_t)(tile - (int64_t)lr * per_row), other);
+      uint32_t y = tid < t.n && ((x0 >> tid) & 1u) ? (a.lin ? a.lin[tid] : 1u << tid) : 0u;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) y ^= __shfl_xor_sync(0xffffffffu, y, o);
+      if (tid == 0) {
+        at_yx[0] = y ^ (a.lin ? a.lin[t.n] : 0u) ^ (a.row_frame ? a.row_frame[lr] : 0u);
+        at_yx[1] = x0;
+      }
+    }
+    __syncthreads();
+    const uint32_t y0 = at_yx[0] ^ oy, x0 = at_yx[1] ^ ox;
+    const c2* psi = t.psi + (size_t)lr * dim;
+    c2 v[kOutPer];
+    if (on) {
+#pragma unroll
+      for (int i = 0; i < kOutPer; i++)
+        if (i < per) v[i] = psi[y0 ^ cy[i]];
+#pragma unroll
+      for (int i = 0; i < kOutPer; i++)
+        if (i < per) buf[swz(tid) ^ swz(256 * i)] = v[i];
+    }
+    __syncthreads();
+    if (on) {
+#pragma unroll
+      for (int i = 0; i < kOutPer; i++)
+        if (i < per) v[i] = buf[swz(at) ^ ca[i]];
+      double* out = a.values + (a.output == TDQ_OUT_STATE ? 2 : 1) * b * dim;
+#pragma unroll
+      for (int i = 0; i < kOutPer; i++) {
+        if (i >= per) continue;
+        const size_t x = x0 ^ cx[i];
+        if (a.output == TDQ_OUT_STATE) {
+          out[2 * x] = exact_double(v[i].x);
+          out[2 * x + 1] = exact_double(v[i].y);
+        } else {
+          out[x] = exact_square(v[i].x) + exact_square(v[i].y);
+        }
+      }
     }
   }
+}
+
+// The map of k1_state_out for x = A y (+ a constant).
+OutMap out_map(const LinMap& map) {
+  OutMap m{};
+  const int n = map.n, r = std::min(5, n);
+  std::vector<uint32_t> ax(n, 0);  // ax[i]: the x that y's bit i flips
+  for (int q = 0; q < n; q++)
+    for (int i = 0; i < n; i++) ax[i] |= ((map.row[q] >> i) & 1u) << q;
+  // the space in the order of x (consecutive x first) and in the order of y
+  LinSpace S;
+  std::vector<uint32_t> bx, by;
+  auto grow = [](LinSpace& sp, std::vector<uint32_t>& list, uint32_t v, int dim) {
+    if ((int)sp.v.size() < dim && sp.reduce(v)) {
+      sp.add(v);
+      list.push_back(v);
+    }
+  };
+  const int bits = std::min(n, kOutBits);
+  for (int i = 0; i < r; i++) grow(S, bx, 1u << i, bits);
+  for (int i = 0; i < r; i++) grow(S, bx, ax[i], bits);
+  for (int i = r; i < n; i++) grow(S, bx, ax[i], bits);
+  m.bits = bits;
+  m.pivots = S.pivots();
+  LinSpace Y;
+  for (int i = 0; i < n; i++)
+    if (!S.reduce(ax[i])) grow(Y, by, ax[i], bits);
+  for (uint32_t v : bx) grow(Y, by, v, bits);
+  auto y_of = [&](uint32_t x) {
+    uint32_t y = 0;
+    for (int q = 0; q < n; q++)
+      if ((x >> q) & 1u) y ^= map.col[q];
+    return y;
+  };
+  std::map<uint32_t, int> place;  // x offset -> position in the order of y
+  for (int l = 0; l < (1 << bits); l++) {
+    uint32_t x = 0, xy = 0;
+    for (int i = 0; i < bits; i++) {
+      if (!((l >> i) & 1)) continue;
+      x ^= bx[i];
+      xy ^= by[i];
+    }
+    m.x[l] = x;
+    m.y[l] = y_of(xy);
+    place[xy] = l;
+  }
+  for (int l = 0; l < (1 << bits); l++) m.at[l] = (uint16_t)place.at(m.x[l]);
+  return m;
 }
 
 }  // namespace
@@ -105,6 +218,8 @@ void tiled_free(TiledSweep& t) {
   cudaFree(t.d_rot_flips);
   cudaFree(t.d_coef);
   cudaFree(t.d_norm);
+  cudaFree(t.d_out);
+  t.d_out = nullptr;
   t.d_coef = nullptr;
   t.d_norm = nullptr;
   cudaFree(t.d_row_frame);
@@ -296,7 +411,7 @@ tdq_status tiled_lin_plan(TiledSweep& t, const tdq_circuit* c, const std::vector
 
 tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<SweepOp>& ops,
                          const std::vector<int>& ps_gate, int rows, bool adj, int tile_qubits, const LinProgram* lin,
-                         int fb, int rb, double* bytes_row) {
+                         int fb, int rb, bool whole_output, double* bytes_row) {
   TiledHost h;
   if (!lin) {
     tdq_status s0 = tiled_plan(t, c, ops, ps_gate, rows, adj, tile_qubits, fb, rb, h);
@@ -361,6 +476,12 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
   if ((s = up((void**)&t.d_dops, prog.dops.data(), sizeof(DOp) * prog.dops.size())) != TDQ_OK) return s;
   if ((s = up((void**)&t.d_rec_ptr, prog.rec_ptr.data(), sizeof(int) * prog.rec_ptr.size())) != TDQ_OK) return s;
   if ((s = up((void**)&t.d_rec_ops, prog.rec_ops.data(), sizeof(int) * prog.rec_ops.size())) != TDQ_OK) return s;
+  if (whole_output) {
+    LinMap id;
+    lin_ops({}, n, &id);
+    const OutMap m = out_map(lin ? lin->map : id);
+    if ((s = up((void**)&t.d_out, &m, sizeof(m))) != TDQ_OK) return s;
+  }
   // resident rows: bounded by a workspace budget of 3/4 of free memory, 64 GiB at most
   size_t freeb = 0, totb = 0;
   cudaMemGetInfo(&freeb, &totb);
@@ -453,6 +574,7 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    t.sms = std::max(1, nsm);
     auto slots = [&](const void* fn, int threads, size_t smem) {
       int nb = 0;
       if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, threads, smem) != cudaSuccess || nb < 1) {
@@ -675,7 +797,7 @@ tdq_status tiled_execute(TiledSweep& t, const SweepArgs& a0, int grad, cudaStrea
     (*launches)++;
     if (a.output == TDQ_OUT_STATE || a.output == TDQ_OUT_PROBS) {
       const int64_t tot = (int64_t)nr << t.n;
-      k1_state_out<<<(unsigned)std::min<int64_t>((tot + 255) / 256, 2432), 256, 0, st>>>(a, d, nr);
+      k1_state_out<<<(unsigned)std::min<int64_t>(tot >> std::min(t.n, kOutBits), 8 * t.sms), 256, 0, st>>>(a, d, nr, t.d_out);
       (*launches)++;
     }
     cudaError_t e = cudaGetLastError();

@@ -47,6 +47,16 @@ struct TiledPass {
   int op_begin, op_end;
 };
 
+// The read-out of whole states (k1_state_out): a space of `bits` dimensions in
+// the order of x and of y; entry l of the first is entry at[l] of the second.
+constexpr int kOutBits = 11;
+struct OutMap {
+  int bits;
+  uint32_t pivots;
+  uint32_t x[1 << kOutBits], y[1 << kOutBits];
+  uint16_t at[1 << kOutBits];
+};
+
 struct TiledSweep {
   int n = 0, k = 0, L = 0;
   int rows = 0;        // rows (batch x shift copies) per execute
@@ -78,6 +88,8 @@ struct TiledSweep {
   std::vector<int> spec_gbytes;
   uint32_t* d_lin = nullptr;             // specialised programs: place of a basis index (SweepArgs::lin)
   int quarter = 0;
+  OutMap* d_out = nullptr;               // read-out of whole states
+  int sms = 1;
   CoefRec* d_coef = nullptr;             // their gate-tensor tables (SweepArgs::coef, norm)
   int* d_norm = nullptr;
   CoefRec* d_rot = nullptr;              // their rows' frame tables (SweepArgs::rot and on)
@@ -139,9 +151,10 @@ tdq_status tiled_lin_plan(TiledSweep& t, const tdq_circuit* c, const std::vector
                           int tile_qubits, int fb, int rb, bool exact, LinProgram& prog);
 
 // lin: the program of tiled_lin_plan, or NULL for the generic kernels
+// whole_output: states or probabilities will be read out
 tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<SweepOp>& ops,
                          const std::vector<int>& ps_gate, int rows, bool adj, int tile_qubits, const LinProgram* lin,
-                         int fb, int rb, double* bytes_row);
+                         int fb, int rb, bool whole_output, double* bytes_row);
 tdq_status tiled_execute(TiledSweep& t, const SweepArgs& a, int grad, cudaStream_t st,
                          int* launches);
 
