@@ -74,6 +74,14 @@ static_assert(sizeof(DOp) == 16, "DOp layout");
 // residues mod 4 reads 16 different slots.
 __device__ __forceinline__ uint32_t swz(uint32_t x) { return x ^ ((x >> 4) & 15u) ^ ((x >> 8) & 15u); }
 
+// The same for tiles moved in pairs of neighbours (16 bytes): the pair index is
+// XORed, local bit p > 0 moves slot bit 1 + (p - 1) mod 3.  A half-warp whose
+// lanes differ in bit 0 and three bits of different residues reads 16 different
+// slots; a quarter-warp reading pairs, 8.
+__host__ __device__ __forceinline__ uint32_t swz_pair(uint32_t x) {
+  return x ^ ((((x >> 4) ^ (x >> 7) ^ (x >> 10)) & 7u) << 1);
+}
+
 // Gate tensor of op o for one row: forward matrix (diagonal gates keep their
 // two phases in m00 / m11), and for U3 dU3/dtheta.
 struct OpMat {
@@ -574,12 +582,20 @@ __device__ __forceinline__ void cp_async8(c2* dst_smem, const c2* src_gmem) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst_smem);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src_gmem) : "memory");
 }
+__device__ __forceinline__ void cp_async16(c2* dst_smem, const c2* src_gmem) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst_smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src_gmem) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 // Wait until at most N of this thread's committed groups are still in flight.
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 #else
 inline void cp_async8(c2* dst_smem, const c2* src_gmem) { *dst_smem = *src_gmem; }
+inline void cp_async16(c2* dst_smem, const c2* src_gmem) {
+  dst_smem[0] = src_gmem[0];
+  dst_smem[1] = src_gmem[1];
+}
 inline void cp_async_commit() {}
 template <int N>
 inline void cp_async_wait() {}

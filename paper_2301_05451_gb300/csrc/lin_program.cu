@@ -129,10 +129,13 @@ void take(const std::vector<LinOp>& ops, std::vector<int>& todo, int dim, LinSpa
 
 // Register passes over the tile's ops.  A pass's group index bits are sent to
 // the local bits outside U's pivots so that 16 consecutive groups read 16
-// different shared-memory slots (see swz: local bit p moves slot bit p mod 4
-// for p < 12), as far as the free bits allow.
+// different shared-memory slots (see swz and swz_pair: local bit p moves slot
+// bit p mod 4, or 0 and 1 + (p - 1) mod 3, for p < 12), as far as the free bits
+// allow.  In pairs, local bit 0 is a pivot only of the vector 1: the members
+// are then read two at a time.
 std::vector<LinReg> reg_passes(const std::vector<LinOp>& ops, const LinTile& t, const LinSpace& V, int mreg,
-                               int max_slots) {
+                               int max_slots, bool pairs) {
+  auto slot_bit = [&](int l) { return !pairs ? l & 3 : l ? 1 + (l - 1) % 3 : 0; };
   std::vector<LinReg> out;
   const int M = std::min(mreg, t.k);
   auto local = [&](uint32_t m) {  // coordinates of m in the tile's basis
@@ -159,19 +162,16 @@ std::vector<LinReg> reg_passes(const std::vector<LinOp>& ops, const LinTile& t, 
     // greedily: move a pivot to another set bit of its vector when that frees
     // a slot bit no free local bit reaches
     auto reach = [&](uint32_t p) {
-      int c = 0;
-      for (int b = 0; b < 4; b++) {
-        bool any = false;
-        for (int l = b; l < std::min(t.k, 12); l += 4) any = any || !((p >> l) & 1u);
-        c += any ? 1 : 0;
-      }
-      return c;
+      uint32_t any = pairs ? 1u : 0u;  // (bit 0: read in pairs where it is a pivot)
+      for (int l = 0; l < std::min(t.k, 12); l++)
+        if (!((p >> l) & 1u)) any |= 1u << slot_bit(l);
+      return __builtin_popcount(any);
     };
     best = reach(piv);
     for (int round = 0; round < M && best < 4; round++)
       for (int i = 0; i < M && best < 4; i++)
         for (int l = 0; l < t.k; l++) {
-          if (!((U.v[i] >> l) & 1u) || l == U.pivot[i]) continue;
+          if (!((U.v[i] >> l) & 1u) || l == U.pivot[i] || (pairs && l == 0)) continue;
           const uint32_t p2 = (piv & ~(1u << U.pivot[i])) | (1u << l);
           if (reach(p2) <= best) continue;
           for (int j = 0; j < M; j++)
@@ -189,8 +189,8 @@ std::vector<LinReg> reg_passes(const std::vector<LinOp>& ops, const LinTile& t, 
     std::vector<char> used(free_pos.size(), 0);
     uint32_t slots = 0;
     for (size_t i = 0; i < free_pos.size() && r.grp_pos.size() < 4; i++)
-      if (free_pos[i] < 12 && !((slots >> (free_pos[i] & 3)) & 1u)) {
-        slots |= 1u << (free_pos[i] & 3);
+      if (free_pos[i] < 12 && !((slots >> slot_bit(free_pos[i])) & 1u)) {
+        slots |= 1u << slot_bit(free_pos[i]);
         used[i] = 1;
         r.grp_pos.push_back(free_pos[i]);
       }
@@ -250,6 +250,7 @@ LinProgram lin_program(const std::vector<SweepOp>& gates, int n, int k, int L, i
   LinProgram P;
   P.n = n;
   P.exact = exact;
+  P.pairs = L > 0;
   P.ops = lin_ops(gates, n, &P.map);
   P.coef.assign(P.ops.size(), -1);
   std::vector<int> todo;
@@ -275,8 +276,8 @@ LinProgram lin_program(const std::vector<SweepOp>& gates, int n, int k, int L, i
     }
     t.v = W.v;
     t.pivots = W.pivots();
-    t.fwd = reg_passes(P.ops, t, W, mf, 0);
-    if (adj) t.rev = reg_passes(P.ops, t, W, mr, kRevPassSlots);
+    t.fwd = reg_passes(P.ops, t, W, mf, 0, P.pairs);
+    if (adj) t.rev = reg_passes(P.ops, t, W, mr, kRevPassSlots, P.pairs);
     // the gate-tensor table: one row per angle, one per register pass with
     // unscaled gates
     for (int o : t.ops) {

@@ -105,6 +105,7 @@ struct LinTile {
 
 struct LinProgram {
   int n = 0;
+  bool pairs = false;        // tiles move in pairs of neighbours (swz_pair), whole states in swz order
   bool exact = false;        // keep the global phase (state and amplitude outputs): no frame
   std::vector<CoefRec> rot;  // with a frame: SweepArgs::rot and rot_x
   std::vector<uint32_t> rot_x;

@@ -21,7 +21,10 @@ namespace tdq {
 
 namespace {
 
-uint32_t swz_host(uint32_t x) { return x ^ ((x >> 4) & 15u) ^ ((x >> 8) & 15u); }
+// (swz and swz_pair)
+uint32_t swz_host(uint32_t x, bool pairs) {
+  return pairs ? x ^ ((((x >> 4) ^ (x >> 7) ^ (x >> 10)) & 7u) << 1) : x ^ ((x >> 4) & 15u) ^ ((x >> 8) & 15u);
+}
 
 // A sign known at compile time up to group-dependent words: the XOR of the
 // words w<i> (top bit) and a constant.
@@ -74,7 +77,8 @@ class PassWriter {
              const std::vector<const char*>& regs, Share share) {
     const int groups = 1 << (t_.k - r_.M);
     s_ << "  for (int grp = threadIdx.x; grp < " << groups << "; grp += " << nthreads << ") {\n";
-    s_ << "    const uint32_t gb = " << spread() << ";\n    const uint32_t sb = swz(gb);\n    const uint32_t y0 = " << y0
+    s_ << "    const uint32_t gb = " << spread() << ";\n    const uint32_t sb = " << (P_.pairs ? "swz_pair" : "swz")
+       << "(gb);\n    const uint32_t y0 = " << y0
        << ";\n    (void)y0;\n";
     regs_ = regs;
     for (size_t i = 0; i < arrays.size(); i++) move(arrays[i], regs[i], false);
@@ -129,8 +133,24 @@ class PassWriter {
   void move(const char* arr, const char* reg, bool store) {
     // (a tile's state buffer in use starts at element `buf`)
     const char* sb = t_.k < P_.n && std::string(arr) == "psi" ? "[sb ^ buf ^ " : "[sb ^ ";
+    // members that differ in local bit 0 are neighbours: 16 bytes at a time
+    int pair = -1;
+    for (int i = 0; i < r_.M; i++)
+      if (P_.pairs && r_.u[i] == 1u) pair = i;
     for (int j = 0; j < N_; j++) {
-      const uint32_t so = swz_host(member(j));
+      const uint32_t so = swz_host(member(j), P_.pairs);
+      if (pair >= 0) {
+        if ((j >> pair) & 1) continue;
+        const int j2 = j | (1 << pair);
+        if (store)
+          s_ << "    *reinterpret_cast<float4*>(&" << arr << sb << so << "u]) = make_float4(" << reg << j << ".x, " << reg
+             << j << ".y, " << reg << j2 << ".x, " << reg << j2 << ".y);\n";
+        else
+          s_ << "    const float4 " << reg << "q" << j << " = *reinterpret_cast<const float4*>(&" << arr << sb << so
+             << "u]);\n    c2 " << reg << j << " = {" << reg << "q" << j << ".x, " << reg << "q" << j << ".y}, " << reg << j2
+             << " = {" << reg << "q" << j << ".z, " << reg << "q" << j << ".w};\n";
+        continue;
+      }
       if (store) s_ << "    " << arr << sb << so << "u] = " << reg << j << ";\n";
       else s_ << "    c2 " << reg << j << " = " << arr << sb << so << "u];\n";
     }
@@ -718,21 +738,26 @@ std::vector<std::string> k2_multi_modules(const std::vector<K2Part>& parts, bool
   return mods;
 }
 
-// every(f): f(shared-memory slot, global index) for this thread's elements of
-// a tile.  A thread's local indices are tid + NT i: the part of both indices
-// that tid gives is computed once per tile, the rest are constants.
+// pairs(f): f(shared-memory slot, global index) for this thread's pairs of
+// neighbours of a tile (both even; see swz_pair), every(f) for its elements.
+// A thread's local indices are 2 (tid + NT i): the part of both indices that
+// tid gives is computed once per tile, the rest are constants.
 static void emit_every(std::ostringstream& s, const LinTile& t, int L) {
-  s << "  template <int NT, class F>\n  __device__ __forceinline__ static void every(const TiledDev&, const TileShared& s, "
+  s << "  template <int NT, class F>\n  __device__ __forceinline__ static void pairs(const TiledDev&, const TileShared& s, "
        "uint32_t base, F&& f) {\n"
     << "    constexpr uint32_t v[" << t.k << "] = {";
   for (int i = 0; i < t.k; i++) s << (i ? ", " : "") << t.v[i] << "u";
-  s << "};\n    if (NT > " << (1 << t.k) << " && threadIdx.x >= " << (1 << t.k) << ") return;\n"
-    << "    const uint32_t y = base ^ (threadIdx.x & " << (1u << L) - 1u << "u) ^ (uint32_t)s.off[threadIdx.x >> " << L
-    << "], z = swz(threadIdx.x);\n"
-    << "#pragma unroll\n    for (uint32_t i = 0; i < " << (1 << t.k) << "u; i += NT) {\n"
+  s << "};\n    const uint32_t j = 2u * threadIdx.x;\n    if (2 * NT > " << (1 << t.k) << " && j >= " << (1 << t.k)
+    << "u) return;\n"
+    << "    const uint32_t y = base ^ (j & " << (1u << L) - 1u << "u) ^ (uint32_t)s.off[j >> " << L
+    << "], z = swz_pair(j);\n"
+    << "#pragma unroll\n    for (uint32_t i = 0; i < " << (1 << t.k) << "u; i += 2 * NT) {\n"
     << "      uint32_t x = 0;\n#pragma unroll\n      for (int q = 0; q < " << t.k
     << "; q++) x ^= ((i >> q) & 1u) ? v[q] : 0u;\n"
-    << "      f(z ^ swz(i), y ^ x);\n    }\n  }\n";
+    << "      f(z ^ swz_pair(i), y ^ x);\n    }\n  }\n"
+    << "  template <int NT, class F>\n  __device__ __forceinline__ static void every(const TiledDev& t, const TileShared& s, "
+       "uint32_t base, F&& f) {\n    pairs<NT>(t, s, base, [&](uint32_t j, uint32_t x) {\n      f(j, x);\n"
+       "      f(j | 1u, x | 1u);\n    });\n  }\n";
 }
 
 // in_first(x): whether index x lies in the first pass's space (the remainder
