@@ -469,9 +469,11 @@ tdq_status tdq_exec_set_slice_range(tdq_exec* e, int64_t first, int64_t count);
 tdq_status tdq_exec_timings(tdq_exec* e, float* ms, int max, int* n);
 
 /* Algorithmic work of each launch unit that tdq_exec_timings times, for a
- * tiled state sweep (the state in HBM): flops[u] (FP32 operations by the
- * counting rule of tdq_exec_work), bytes[u] (its HBM traffic model: the
- * state read and written once per pass, psi and lambda in reverse passes)
+ * tiled state sweep (the state in HBM): flops[u] (FP32 operations: dense
+ * gates by the counting rule of tdq_exec_work for the generic kernels, the
+ * operations that the specialised kernels run, from |0...0>), bytes[u] (its
+ * HBM traffic model: the state read and written once per pass, psi and lambda
+ * in reverse passes; of the first pass, its one nonzero tile where specialised)
  * and kind[u] (0 forward tile pass, 1 last pass with the observable and its
  * reverse sweep fused, 2 reverse tile pass), for the rows of the first row
  * chunk; units in launch order.  Any array may be NULL; all NULL queries *n.

@@ -598,52 +598,64 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
     t.slots_r = nsm;
     if (adj && np > 1) t.slots_r = slots(!t.kr.empty() ? t.kr[0] : (const void*)k1_reverse, t.nthreads_r, t.smem_r);
   }
-  // HBM traffic model per row: every pass reads and writes the state (the
-  // first pass only writes it, a value-only last pass only reads it); with the
-  // reverse sweep each earlier pass reads and writes psi and lambda again.
+  // HBM traffic model per row and launch unit: every pass reads and writes the
+  // state (the first pass only writes it, a value-only last pass only reads
+  // it); with the reverse sweep each earlier pass reads and writes psi and
+  // lambda again.  From |0...0> the specialised passes' first one holds its one
+  // nonzero tile, which is all that the second reads and the reverse of the
+  // second leaves.
   const double sb = (double)((size_t)1 << n) * sizeof(c2);
-  double by = 0;
-  for (int p = 0; p < np; p++) {
-    const bool f = p == 0, l = p == np - 1;
-    by += (f ? 0 : sb) + ((l && !adj && c->n_groups > 0) ? 0 : sb);
-    if (adj && l) by += sb;  // lambda written by the fused last pass
-    if (adj && !l) by += 4 * sb;
-  }
-  *bytes_row = by;
-  // the same model per launch unit, with the algorithmic FLOPs of each pass
-  // (forward passes, then the reverse passes from the second last down)
+  const double part = lin && np > 1 ? std::ldexp(1.0, t.k - n) : 1.0;
+  auto in = [&](int p) { return p == 0 ? 0.0 : p == 1 ? part * sb : sb; };
+  auto out = [&](int p) { return p == 0 ? part * sb : sb; };
+  auto left = [&](int p) { return lin ? in(p) : sb; };  // of psi and lambda each, by the reverse of pass p
+  // the FLOPs of each unit (forward passes, then the reverse passes from the
+  // second last down): dense gates, or the operations of the specialised
+  // passes per amplitude -- rotation 4, H and a pass's scale 2, its phases one
+  // product 6; a dot 4 -- psi and lambda both in reverse
   const double dim = std::ldexp(1.0, n);
   const double obs = c->n_groups > 0 ? (3.0 + 2.0 * (double)c->terms.size()) * dim : 0.0;
-  std::vector<double> fw(np, 0.0), dots(np, 0.0);
+  std::vector<double> fw(np, 0.0), dots(np, 0.0), bw(np, 0.0);
   for (int p = 0; p < np; p++) {
     for (int o = t.passes[p].op_begin; o < t.passes[p].op_end; o++) {
       fw[p] += gate_fwd_flops(pops[o].kind, dim);
       dots[p] += gate_dot_flops(pops[o].kind, dim);
     }
-    if (lin)
-      for (int o : lin->tiles[p].ops) {
+    bw[p] = 2 * fw[p] + dots[p];
+    if (!lin) continue;
+    auto count = [&](const LinReg& r, bool rev) {
+      double c = r.norm >= 0 ? 2 : 0, dot = 0;
+      bool phase = false;
+      for (int o : r.ops) {
         const LinOp& g = lin->ops[o];
-        if (g.p) continue;  // a factor of a U3, counted with its RY
-        const int kind = g.kind == L_SIGN ? K_Z : g.kind == L_CZ ? K_CZ : g.kind == L_H ? K_H : ops[g.op].kind;
-        fw[p] += gate_fwd_flops(kind, dim);
-        dots[p] += gate_dot_flops(kind, dim);
+        c += g.kind == L_RY || g.kind == L_RX ? 4 : g.kind == L_H ? 2 : 0;
+        phase |= g.kind == L_PHASE;
+        dot += g.slot >= 0 && g.kind != L_PHASE ? 4 : 0;
       }
+      c += phase ? 6 : 0;
+      return (rev ? 2 * c + dot + (phase ? 4 : 0) : c) * dim * (p == 0 ? part : 1.0);
+    };
+    for (const LinReg& r : lin->tiles[p].fwd) fw[p] += count(r, false);
+    if (adj)
+      for (const LinReg& r : lin->tiles[p].rev) bw[p] += count(r, true);
   }
   t.unit_flops.clear();
   t.unit_bytes.clear();
   t.unit_kind.clear();
   for (int p = 0; p < np; p++) {
-    const bool f = p == 0, l = p == np - 1;
+    const bool l = p == np - 1;
     t.unit_kind.push_back(l && adj ? 1 : 0);
-    t.unit_flops.push_back(fw[p] + (l ? obs : 0.0) + (l && adj ? 2 * fw[p] + dots[p] + obs : 0.0));
-    t.unit_bytes.push_back((f ? 0 : sb) + ((l && !adj && c->n_groups > 0) ? 0 : sb) + (adj && l ? sb : 0));
+    t.unit_flops.push_back(fw[p] + (l ? obs : 0.0) + (l && adj ? bw[p] + obs : 0.0));
+    t.unit_bytes.push_back(in(p) + (!l ? out(p) : adj ? 2 * left(p) : c->n_groups > 0 ? 0.0 : out(p)));
   }
   if (adj)
     for (int p = np - 2; p >= 0; p--) {
       t.unit_kind.push_back(2);
-      t.unit_flops.push_back(2 * fw[p] + dots[p]);
-      t.unit_bytes.push_back(4 * sb);
+      t.unit_flops.push_back(bw[p]);
+      t.unit_bytes.push_back(2 * (out(p) + left(p)));
     }
+  *bytes_row = 0;
+  for (double by : t.unit_bytes) *bytes_row += by;
   return TDQ_OK;
 }
 
