@@ -946,8 +946,9 @@ extern "C" tdq_status tdq_sweep_source(const tdq_circuit* c, int grad, int tile_
                                   c->n_groups == 0, lin);
     if (s != TDQ_OK) return s;
     t.diag = c->n_groups > 0 && std::ldexp(4.0 * c->n_groups, c->n) <= kDiagTableBytes;
-    src = k1_specialised_source(t, lin, std::max(32, std::min(256, 1 << (t.k - kTiledSpecFwdRegBits))),
-                                std::max(32, std::min(256, 1 << (t.k - kTiledSpecRevRegBits))));
+    t.nthreads = std::max(32, std::min(256, 1 << (t.k - kTiledSpecFwdRegBits)));
+    t.threads_f.assign(lin.tiles.size(), t.nthreads);
+    src = k1_specialised_source(t, lin, std::max(32, std::min(256, 1 << (t.k - kTiledSpecRevRegBits))));
   }
   *len = src.size() + 1;
   if (buf) {

@@ -774,12 +774,13 @@ static void emit_in_first(std::ostringstream& s, const LinTile& t, int n) {
   s << "    return r == 0u;\n  }\n";
 }
 
-std::string k1_specialised_source(const TiledSweep& t, const LinProgram& prog, int nthreads, int nthreads_r) {
+std::string k1_specialised_source(const TiledSweep& t, const LinProgram& prog, int nthreads_r) {
   std::ostringstream s, decl;
   int uid = 0;
   const int np = (int)prog.tiles.size();
   for (int p = 0; p < np; p++) {
     const LinTile& tile = prog.tiles[p];
+    const int nthreads = t.threads_f[p];
     // gradient accumulators of the pass: one per angle with a slot
     std::map<int, int> acc;
     std::vector<int> slots;
@@ -796,7 +797,7 @@ std::string k1_specialised_source(const TiledSweep& t, const LinProgram& prog, i
     s << "struct TilePass" << p << " {\n  static constexpr bool kSpecialised = true, kFirst = "
       << (p == 0 ? "true" : "false") << ", kSecond = " << (p == 1 ? "true" : "false") << ", kDiag = "
       << (t.diag ? "true" : "false") << ";\n  static constexpr int kK = " << t.k << ", kN = " << t.n
-      << ", kBuffers = " << (t.dbl ? 2 : 1) << ", kGroups = " << t.ng << ";\n";
+      << ", kBuffers = " << (t.dbl && nthreads == t.nthreads ? 2 : 1) << ", kGroups = " << t.ng << ";\n";
     emit_in_first(s, prog.tiles[0], t.n);
     emit_every(s, tile, t.L);
     s << "  __device__ __forceinline__ static void forward(const TiledDev&, const TileShared& s, uint32_t base, "
@@ -826,9 +827,10 @@ std::string k1_specialised_source(const TiledSweep& t, const LinProgram& prog, i
   s << "}  // namespace tdq\n";
   std::ostringstream out;
   out << "#include \"k1_body.cuh\"\nnamespace tdq {\n" << decl.str() << s.str();
-  const int minb = nthreads >= 256 ? 2 : 1;
   for (int p = 0; p < np; p++) {
     const bool f = p == 0, l = p == np - 1;
+    const int nthreads = t.threads_f[p];
+    const int minb = nthreads < t.nthreads ? (l && t.adj ? 3 : 4) : nthreads >= 256 ? 2 : 1;
     out << "extern \"C\" __global__ void __launch_bounds__(" << nthreads << ", " << minb << ") tdq_k1f_" << p
       << "(tdq::SweepArgs a, tdq::TiledDev t, int store) {\n  tdq::k1_forward_body<" << nthreads << ", "
       << (f ? "true" : "false") << ", " << (l ? "true" : "false") << ", " << ((l && t.adj) ? "true" : "false")

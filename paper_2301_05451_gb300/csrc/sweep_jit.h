@@ -40,7 +40,7 @@ constexpr const char* kModuleMark = "// ==== tdq module ";
 // Source of the K1 kernels of every tile pass p of t (program prog):
 // tdq_k1f_<p> (forward; the last one also runs its reverse sweep with
 // gradients) and tdq_k1r_<p> (reverse, passes before the last).
-std::string k1_specialised_source(const TiledSweep& t, const LinProgram& prog, int nthreads, int nthreads_r);
+std::string k1_specialised_source(const TiledSweep& t, const LinProgram& prog, int nthreads_r);
 
 // Compiles `src` for the current device and returns the kernel `name` (a
 // handle usable with cudaLaunchKernel / cudaFuncSetAttribute).  Compiled

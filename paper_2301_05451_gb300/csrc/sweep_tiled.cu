@@ -409,6 +409,22 @@ tdq_status tiled_lin_plan(TiledSweep& t, const tdq_circuit* c, const std::vector
   return TDQ_OK;
 }
 
+// Whether a forward kernel over 12-bit tiles runs in CTAs of 128 threads with
+// one tile buffer, four per SM (fused with its reverse sweep three), or in two of
+// 256 threads with two buffers.  A tile's load, its register passes (a
+// barrier each) and its store follow one another, and more CTAs overlap them
+// better than a second buffer does: 20-qubit ladder, 481 rows, values 8.81 ->
+// 8.00 ms (two CTAs with one buffer 8.95, seven of 64 threads 9.37), fused last
+// pass of 64 rows 732 -> 635 us.  A round of four (three) such CTAs takes 1.85 (1.45)
+// rounds of two, so the last round's fill decides: 16 qubits, 24 rows, fused pass,
+// 2.5 tiles per SM, one round for two 82 -> 47 us; 17 qubits, 16 rows, 3.4 per SM,
+// two rounds either way, 106 us in CTAs of 256 and 125 in CTAs of 128.  (Reverse
+// kernels stay at two of 256: 1.56 ms against 1.98 at three of 128.)
+static bool narrow_pass(double tiles, int sms, bool fused) {
+  const double wide = std::ceil(tiles / (2.0 * sms));
+  return fused ? 1.45 * std::ceil(tiles / (3.0 * sms)) < wide : 1.85 * std::ceil(tiles / (4.0 * sms)) < wide;
+}
+
 tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<SweepOp>& ops,
                          const std::vector<int>& ps_gate, int rows, bool adj, int tile_qubits, const LinProgram* lin,
                          int fb, int rb, bool whole_output, double* bytes_row) {
@@ -507,6 +523,14 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
   t.kr.clear();
   t.spec_gbytes.clear();
   const int np = (int)t.passes.size();
+  int dev = 0, nsm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  t.sms = std::max(1, nsm);
+  t.threads_f.assign(np, t.nthreads);
+  if (!interpret && t.k == 12 && t.nthreads == 256)
+    for (int p = 0; p < np; p++)
+      if (narrow_pass(std::ldexp((double)t.chunk_rows, p ? n - t.k : 0), t.sms, adj && p == np - 1)) t.threads_f[p] = 128;
   int gmax = 0, ndops_sm = 0;
   std::vector<int> nacc(np, 0);  // gradient accumulators of every pass
   if (!interpret) {
@@ -522,7 +546,8 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
     ndops_sm = t.max_dops;
   }
   // shared memory per kernel: forward kernels a double-buffered state (psi;
-  // the last pass also lambda; one buffer where two do not fit).  Reverse
+  // the last pass also lambda; one buffer where two do not fit, or in CTAs of
+  // 128 threads, see narrow_pass).  Reverse
   // kernels hold psi and lambda in one buffer each: two CTAs of 256 threads
   // per SM then interleave one CTA's tile loads with the other's compute,
   // which measured faster than one double-buffered CTA of 512 threads.
@@ -530,7 +555,7 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
   auto sizes = [&](int nb) {
     t.smem_f.assign(np, 0);
     for (int p = 0; p < np; p++)
-      t.smem_f[p] = k1_smem_bytes(t.k, t.L, p == 0 ? 1 : nb, (adj && p == np - 1) ? 1 : 0, mbytes, ndops_sm,
+      t.smem_f[p] = k1_smem_bytes(t.k, t.L, p == 0 || t.threads_f[p] < t.nthreads ? 1 : nb, (adj && p == np - 1) ? 1 : 0, mbytes, ndops_sm,
                                   t.ng, gmax);
     t.smem_r = adj ? k1_smem_bytes(t.k, t.L, 1, 1, mbytes, ndops_sm, t.ng, gmax) : 0;
     size_t m = t.smem_r;
@@ -542,7 +567,7 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
   if (smax > 227 * 1024) return fail(TDQ_ERR_UNSUPPORTED, "tiled sweep: tile program too large");
   if (!interpret) {
     // every tile pass as straight-line code; one compilation for all passes
-    const std::string src = k1_specialised_source(t, *lin, t.nthreads, t.nthreads_r);
+    const std::string src = k1_specialised_source(t, *lin, t.nthreads_r);
     for (int p = 0; p < np; p++) {
       const void* kf = nullptr;
       const void* kr = nullptr;
@@ -571,17 +596,13 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
   }
   // resident CTAs per kernel (occupancy of the kernel at its launch shape)
   {
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    t.sms = std::max(1, nsm);
     auto slots = [&](const void* fn, int threads, size_t smem) {
       int nb = 0;
       if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, threads, smem) != cudaSuccess || nb < 1) {
         cudaGetLastError();
         nb = 1;
       }
-      return std::max(1, nsm) * nb;
+      return t.sms * nb;
     };
     t.slots_f.assign(np, 0);
     for (int p = 0; p < np; p++) {
@@ -593,9 +614,9 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
                        : (!adj) ? (const void*)k1_forward<false, true, false>
                        : f ? (const void*)k1_forward<true, true, true>
                            : (const void*)k1_forward<false, true, true>;
-      t.slots_f[p] = slots(fn, t.nthreads, t.smem_f[p]);
+      t.slots_f[p] = slots(fn, t.threads_f[p], t.smem_f[p]);
     }
-    t.slots_r = nsm;
+    t.slots_r = t.sms;
     if (adj && np > 1) t.slots_r = slots(!t.kr.empty() ? t.kr[0] : (const void*)k1_reverse, t.nthreads_r, t.smem_r);
   }
   // HBM traffic model per row and launch unit: every pass reads and writes the
@@ -744,7 +765,7 @@ tdq_status tiled_execute(TiledSweep& t, const SweepArgs& a0, int grad, cudaStrea
     d.row0 = row0;
     d.nrows = nr;
     d.dbl = t.dbl;
-    const int nthr = t.nthreads;
+    const int nthr = t.nthreads;  // (generic kernels)
     const int store_last = (a.output != TDQ_OUT_EXPVAL) ? 1 : 0;  // amplitudes, states: read from HBM
     for (int p = 0; p < np; p++) {
       d.off = t.d_off + (size_t)p * (1 << (t.k - t.L));
@@ -761,7 +782,7 @@ tdq_status tiled_execute(TiledSweep& t, const SweepArgs& a0, int grad, cudaStrea
         int st_flag = (l && !adj) ? store_last : 1;
         void* args[] = {&a, &d, &st_flag};
         // the first pass follows the caller's work and the clears above: unchained
-        if (launch_chained(t.kf[p], grid, dim3(nthr), args, t.smem_f[p], st, p > 0) != cudaSuccess)
+        if (launch_chained(t.kf[p], grid, dim3(t.threads_f[p]), args, t.smem_f[p], st, p > 0) != cudaSuccess)
           return fail(TDQ_ERR_CUDA, "tiled sweep: launch of a specialised pass");
         if (rec) cudaEventRecord(t.ev[2 * p + 1], st);
         (*launches)++;

@@ -98,6 +98,7 @@ struct TiledSweep {
   int nthreads = 256, nthreads_r = 256;  // forward / reverse kernels
   std::vector<size_t> smem_f;            // per forward kernel
   size_t smem_r = 0;
+  std::vector<int> threads_f;            // of each forward kernel (narrow_pass)
   int dbl = 1;                           // double-buffered tile loads (forward kernels)
   bool diag = false;                     // the observable's diagonals are tables (SweepArgs::odiag)
   int fb = 4, rb = 3;                    // register bits of forward / reverse passes
