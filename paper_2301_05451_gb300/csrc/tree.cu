@@ -652,7 +652,16 @@ __global__ void __launch_bounds__(256) k_tree_step_splitk(TreeArgs a, int s, int
 // k_tree_step_splitk, an output at a time).  Bound by latency: 128 x 32 outputs, k
 // 128, 4 entries 10 us (17 at a warp per output), 512 x 8, k 32: 8.9 (10.5 at a
 // thread per output); the 7 x 7 amplitude, 13 large steps, 127 -> 79 us.
-constexpr int kTileK = 64;  // k entries staged at a time
+constexpr int kTileK = 64;   // k entries staged at a time
+// Sums are taken in FP32 pieces of kTileSum entries, added with compensation: a
+// long k then rounds less than in the lane-split sums that the tile replaces.
+constexpr int kTileSum = 4;
+// s += v, with the rounding errors so far in c
+__device__ __forceinline__ void kahan(float& s, float& c, float v) {
+  const float y = v - c, t = s + y;
+  c = (t - s) - y;
+  s = t;
+}
 template <int R>
 __global__ void __launch_bounds__(256) k_tree_tile(TreeArgs a, int s, int ltm, int ltn, int lsplit) {
   chain_start();
@@ -678,7 +687,7 @@ __global__ void __launch_bounds__(256) k_tree_tile(TreeArgs a, int s, int ltm, i
   c2* C = base + st.c_off;
   const uint32_t tn = threadIdx.x & ((TN / R) - 1u), tm = threadIdx.x / (TN / R);
   const bool active = tm < TM / R;
-  float re[R][R] = {}, im[R][R] = {};
+  float re[R][R] = {}, im[R][R] = {}, re_c[R][R] = {}, im_c[R][R] = {};
   for (uint32_t k0 = kb; k0 < kb + ks; k0 += KC) {
     if (k0 > kb) __syncthreads();
 #pragma unroll 4
@@ -686,24 +695,34 @@ __global__ void __launch_bounds__(256) k_tree_tile(TreeArgs a, int s, int ltm, i
 #pragma unroll 4
     for (uint32_t i = threadIdx.x; i < (TN << lkc); i += 256) Bs[(i >> lkc) * P + (i & (KC - 1u))] = B[((size_t)(i >> lkc) << nk) + k0 + (i & (KC - 1u))];
     __syncthreads();
-    if (active) {
-#pragma unroll 4
-      for (uint32_t kk = 0; kk < KC; kk++) {
-        c2 x[R], y[R];
+    if (active)
+      for (uint32_t k1 = 0; k1 < KC; k1 += kTileSum) {
+        float pr[R][R] = {}, pi[R][R] = {};
 #pragma unroll
-        for (int i = 0; i < R; i++) {
-          x[i] = As[(tm + i * (TM / R)) * P + kk];
-          y[i] = Bs[(tn + i * (TN / R)) * P + kk];
+        for (uint32_t kk = k1; kk < k1 + kTileSum; kk++) {
+          if (kk >= KC) break;
+          c2 x[R], y[R];
+#pragma unroll
+          for (int i = 0; i < R; i++) {
+            x[i] = As[(tm + i * (TM / R)) * P + kk];
+            y[i] = Bs[(tn + i * (TN / R)) * P + kk];
+          }
+#pragma unroll
+          for (int i = 0; i < R; i++)
+#pragma unroll
+            for (int j = 0; j < R; j++) {
+              pr[i][j] = fmaf(x[i].x, y[j].x, fmaf(-x[i].y, y[j].y, pr[i][j]));
+              pi[i][j] = fmaf(x[i].x, y[j].y, fmaf(x[i].y, y[j].x, pi[i][j]));
+            }
         }
 #pragma unroll
         for (int i = 0; i < R; i++)
 #pragma unroll
           for (int j = 0; j < R; j++) {
-            re[i][j] = fmaf(x[i].x, y[j].x, fmaf(-x[i].y, y[j].y, re[i][j]));
-            im[i][j] = fmaf(x[i].x, y[j].y, fmaf(x[i].y, y[j].x, im[i][j]));
+            kahan(re[i][j], re_c[i][j], pr[i][j]);
+            kahan(im[i][j], im_c[i][j], pi[i][j]);
           }
       }
-    }
   }
   if (!active) return;
   const uint32_t ch = scatter_bits(h, pos + 64, nh);
@@ -953,12 +972,13 @@ struct TreeExec final : tdq_exec {
 
   // Whether a step runs in k_tree_tile: thread- and warp-per-output steps,
   // 64 x 64 SIMT tiles over a short k (2^12 x 2^5 outputs, k 16, 8 entries: 16 us
-  // against 39), and tensor-core steps whose fixed cost outweighs the arithmetic
-  // (128 x 128, k 8, 8 entries: 9 us against 19; 2^10 x 2^7, k 8: 14 against 17;
-  // 2^8 x 2^6, k 128: 22 against 18).  (At least 256 outputs per batch entry; 256 x
+  // against 39), and tensor-core steps over a short k, whose fixed cost outweighs
+  // the arithmetic (128 x 128, k 8, 8 entries: 9 us against 19; 2^10 x 2^7, k 8: 14
+  // against 17; but 2^8 x 2^6, k 128: 22 against 18).  (At least 256 outputs per batch entry; 256 x
   // 65 rows of staged operands at most, 135 KB.)
   static bool tile_step(const StepDev& sd, int kind, int nb) {
     const int out = sd.nm + sd.nn;
+    if ((kind == 2 || kind == 3) && sd.nk > 5) return false;
     if (kind == 5) return sd.nm >= 5 && sd.nn >= 5 && ((int64_t)nb << sd.nh) <= 65535;
     if (out < 8 || ((int64_t)nb << sd.nh) > 65535 || sd.nn > 19) return false;
     if (kind == 0 || kind == 4 || (kind == 1 && sd.nk <= 5)) return true;
