@@ -419,8 +419,15 @@ tdq_status tiled_lin_plan(TiledSweep& t, const tdq_circuit* c, const std::vector
 // rounds of two, so the last round's fill decides: 16 qubits, 24 rows, fused pass,
 // 2.5 tiles per SM, one round for two 82 -> 47 us; 17 qubits, 16 rows, 3.4 per SM,
 // two rounds either way, 106 us in CTAs of 256 and 125 in CTAs of 128.  (Reverse
-// kernels stay at two of 256: 1.56 ms against 1.98 at three of 128.)
-static bool narrow_pass(double tiles, int sms, bool fused) {
+// kernels stay at two of 256: 1.56 ms against 1.98 at three of 128.)  A pass of few
+// register passes over parts of 128-byte lines waits for memory alone, and more
+// tiles at once spread it thinner: 20 qubits, 16 rows, three register passes over
+// 32-byte runs 94 us in CTAs of 256 and 111 in CTAs of 128; but four, 481 rows, 2.72 ms
+// and 2.53, and two over whole lines 1.64 and 1.31.
+static bool narrow_pass(const LinTile& tile, double tiles, int sms, bool fused) {
+  bool lines = true;
+  for (int i = 0; i < 4; i++) lines = lines && tile.v[i] == 1u << i;
+  if (!lines && tile.fwd.size() < 4) return false;
   const double wide = std::ceil(tiles / (2.0 * sms));
   return fused ? 1.45 * std::ceil(tiles / (3.0 * sms)) < wide : 1.85 * std::ceil(tiles / (4.0 * sms)) < wide;
 }
@@ -530,7 +537,8 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
   t.threads_f.assign(np, t.nthreads);
   if (!interpret && t.k == 12 && t.nthreads == 256)
     for (int p = 0; p < np; p++)
-      if (narrow_pass(std::ldexp((double)t.chunk_rows, p ? n - t.k : 0), t.sms, adj && p == np - 1)) t.threads_f[p] = 128;
+      if (narrow_pass(lin->tiles[p], std::ldexp((double)t.chunk_rows, p ? n - t.k : 0), t.sms, adj && p == np - 1))
+        t.threads_f[p] = 128;
   int gmax = 0, ndops_sm = 0;
   std::vector<int> nacc(np, 0);  // gradient accumulators of every pass
   if (!interpret) {
