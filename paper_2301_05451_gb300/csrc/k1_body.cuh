@@ -40,6 +40,14 @@ struct TiledDev {
   int nrows;           // rows of the chunk: units are (row, tile), row-major
   int gbytes;          // shared-memory bytes of the gradient partial sums
   int dbl;             // 1: two tile buffers in the forward kernels (loads overlap compute)
+  // Parameter shift with shared prefixes (ps_rows: NULL without): copy k is the
+  // unshifted copy up to pass ps_first[k].  A pass runs the ps_active copies
+  // ps_rows of every batch entry; the unshifted copy, read by those that start
+  // here, changes between its row and a second buffer (alt, per entry).
+  const int* ps_rows;
+  const int* ps_first;
+  c2* alt;
+  int ps_active, pass;
 };
 
 // Spread the bits of t over the positions of mask (lowest first).
@@ -271,7 +279,10 @@ __device__ __forceinline__ void k1_forward_body(const SweepArgs& a, const TiledD
   chain_dispatch();
   bool waited = false;
   for (Segments seg(t); seg.next(t);) {
-    const int lr = seg.lr, tile0 = seg.tile0, tile1 = seg.tile1;
+    const int tile0 = seg.tile0, tile1 = seg.tile1;
+    int lr = seg.lr;
+    if (Prog::kSpecialised && !GRAD && t.ps_rows)
+      lr = lr / t.ps_active * a.ps_copies + t.ps_rows[lr % t.ps_active];
     const int row = t.row0 + lr;
     const int64_t b = row / a.ps_copies;
     const int kk = row % a.ps_copies;
@@ -282,6 +293,12 @@ __device__ __forceinline__ void k1_forward_body(const SweepArgs& a, const TiledD
     if (bad) atomicOr(a.status, 1 << TDQ_ERR_NONFINITE);
     c2* gpsi = t.psi + (size_t)lr * dim;
     c2* glam = GRAD ? t.lam + (size_t)lr * dim : nullptr;
+    c2 *gin = gpsi, *gout = gpsi;
+    if (Prog::kSpecialised && !GRAD && t.ps_rows) {
+      c2 *even = t.psi + (size_t)(lr - kk) * dim, *odd = t.alt + (size_t)b * dim;
+      if (kk == 0 || t.ps_first[kk] == t.pass) gin = (t.pass & 1) ? odd : even;
+      if (kk == 0) gout = (t.pass & 1) ? even : odd;
+    }
     // index part of the row's frame: the observable of y is read at y ^ mu
     uint32_t mu = 0u;
     if constexpr (Prog::kSpecialised && LAST) {
@@ -289,7 +306,7 @@ __device__ __forceinline__ void k1_forward_body(const SweepArgs& a, const TiledD
       if (a.row_frame && threadIdx.x == 0) a.row_frame[lr] = mu;
     }
     if (!FIRST && nbuf == 2 && tile0 < tile1) {
-      k1_issue<NT, Prog>(s.psi, gpsi, t, s, deposit((uint32_t)tile0, other), !a.init);
+      k1_issue<NT, Prog>(s.psi, gin, t, s, deposit((uint32_t)tile0, other), !a.init);
       cp_async_commit();
     }
     for (int tile = tile0, it = 0; tile < tile1; tile++, it++) {
@@ -330,14 +347,14 @@ __device__ __forceinline__ void k1_forward_body(const SweepArgs& a, const TiledD
         }
       } else if (nbuf == 2) {
         if (tile + 1 < tile1) {  // the buffer of the previous tile is free (barrier at the loop end)
-          k1_issue<NT, Prog>((it & 1) ? s.psi : s.psi2, gpsi, t, s, deposit((uint32_t)(tile + 1), other), !a.init);
+          k1_issue<NT, Prog>((it & 1) ? s.psi : s.psi2, gin, t, s, deposit((uint32_t)(tile + 1), other), !a.init);
           cp_async_commit();
           cp_async_wait<1>();
         } else {
           cp_async_wait<0>();
         }
       } else {  // one buffer: load, then compute
-        k1_issue<NT, Prog>(s.psi, gpsi, t, s, base, !a.init);
+        k1_issue<NT, Prog>(s.psi, gin, t, s, base, !a.init);
         cp_async_commit();
         cp_async_wait<0>();
       }
@@ -372,7 +389,7 @@ __device__ __forceinline__ void k1_forward_body(const SweepArgs& a, const TiledD
           }
         }
       }
-      if (!(LAST && GRAD) && store) k1_store<NT, Prog>(s.psi + buf, gpsi, t, s, base);
+      if (!(LAST && GRAD) && store) k1_store<NT, Prog>(s.psi + buf, gout, t, s, base);
       __syncthreads();
     }
     if (LAST && a.output == TDQ_OUT_EXPVAL) {

@@ -760,7 +760,7 @@ static tdq_status compile_sweep_impl(const tdq_circuit* c, const tdq_compile_opt
     if (ce != cudaSuccess) return bail(fail(TDQ_ERR_CUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(ce)));
   }
   if (!e->smem_path) {
-    s = tiled_compile(e->tiled, c, ops, ps_gate, e->B * e->copies, adj, o->tile_qubits, spec ? &lin : nullptr, fb1, rb1,
+    s = tiled_compile(e->tiled, c, ops, ps_gate, ps_ang, e->copies, e->B * e->copies, adj, o->tile_qubits, spec ? &lin : nullptr, fb1, rb1,
                       o->output == TDQ_OUT_STATE || o->output == TDQ_OUT_PROBS, &e->bytes_row);
     if (s != TDQ_OK) return bail(s);
     // outputs: the state read back from HBM and written out as values

@@ -208,6 +208,9 @@ void tiled_free(TiledSweep& t) {
   cudaFree(t.d_gacc);
   cudaFree(t.d_vals);
   cudaFree(t.d_ps_gate_pass);
+  cudaFree(t.d_ps_rows);
+  cudaFree(t.d_ps_first);
+  cudaFree(t.d_alt);
   cudaFree(t.d_rpass);
   cudaFree(t.d_dops);
   cudaFree(t.d_rec_ptr);
@@ -225,7 +228,8 @@ void tiled_free(TiledSweep& t) {
   cudaFree(t.d_row_frame);
   t.d_lin = t.d_rot_x = t.d_rot_flips = t.d_row_frame = nullptr;
   t.d_rot = nullptr;
-  t.d_ps_gate_pass = nullptr;
+  t.d_ps_gate_pass = t.d_ps_rows = t.d_ps_first = nullptr;
+  t.d_alt = nullptr;
   t.d_rpass = nullptr;
   t.d_dops = nullptr;
   t.d_rec_ptr = t.d_rec_ops = nullptr;
@@ -433,8 +437,8 @@ static bool narrow_pass(const LinTile& tile, double tiles, int sms, bool fused) 
 }
 
 tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<SweepOp>& ops,
-                         const std::vector<int>& ps_gate, int rows, bool adj, int tile_qubits, const LinProgram* lin,
-                         int fb, int rb, bool whole_output, double* bytes_row) {
+                         const std::vector<int>& ps_gate, const std::vector<int>& ps_ang, int copies, int rows, bool adj,
+                         int tile_qubits, const LinProgram* lin, int fb, int rb, bool whole_output, double* bytes_row) {
   TiledHost h;
   if (!lin) {
     tdq_status s0 = tiled_plan(t, c, ops, ps_gate, rows, adj, tile_qubits, fb, rb, h);
@@ -522,6 +526,34 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
     return fail(TDQ_ERR_OOM, "tiled sweep: gradient buffer");
   if (cudaMalloc(&t.d_vals, sizeof(double) * std::max(1, t.ng) * t.chunk_rows) != cudaSuccess)
     return fail(TDQ_ERR_OOM, "tiled sweep: value buffer");
+  // Parameter shift: a copy's state is the unshifted copy's until the tile pass
+  // that holds its angle (rotations that a pass has not reached yet commute with
+  // what ran before them), so it starts there.  20-qubit ladder, 481 copies,
+  // 361 of them in the second pass and 441 in the third: 7.99 -> 6.88 ms, the same bits.
+  // Kept to executions whose rows are all resident; one more state per batch entry.
+  t.copies = copies;
+  t.ps_active.clear();
+  if (lin && copies > 1 && t.chunk_rows == rows && lin->tiles.size() > 1 && c->n_groups > 0 &&
+      cudaMalloc(&t.d_alt, ((size_t)1 << n) * sizeof(c2) * (rows / copies)) == cudaSuccess) {
+    std::vector<int> first(copies, 0), list;
+    for (int k = 1; k < copies; k++) {
+      const int gate = ps_gate[(k - 1) / 2], ang = ps_ang[(k - 1) / 2];
+      for (int p = (int)lin->tiles.size() - 1; p >= 0; p--)
+        for (int o : lin->tiles[p].ops)
+          if (lin->ops[o].op == gate && lin->ops[o].ang == ang && lin->ops[o].kind <= L_PHASE && lin->ops[o].kind != L_H)
+            first[k] = p;
+    }
+    for (int p = 0; p < (int)lin->tiles.size(); p++) {
+      const size_t at = list.size();
+      for (int k = 0; k < copies; k++)
+        if (first[k] <= p) list.push_back(k);
+      t.ps_active.push_back((int)(list.size() - at));
+    }
+    if ((s = up((void**)&t.d_ps_rows, list.data(), sizeof(int) * list.size())) != TDQ_OK) return s;
+    if ((s = up((void**)&t.d_ps_first, first.data(), sizeof(int) * first.size())) != TDQ_OK) return s;
+  } else {
+    cudaGetLastError();  // (no room: every copy runs every pass)
+  }
   // threads: one forward group (2^4 amplitudes) per thread; reverse kernels
   // up to 256 threads (two CTAs per SM)
   t.nthreads = std::max(32, std::min(256, 1 << (t.k - fb)));
@@ -675,7 +707,9 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
     const bool l = p == np - 1;
     t.unit_kind.push_back(l && adj ? 1 : 0);
     t.unit_flops.push_back(fw[p] + (l ? obs : 0.0) + (l && adj ? bw[p] + obs : 0.0));
-    t.unit_bytes.push_back(in(p) + (!l ? out(p) : adj ? 2 * left(p) : c->n_groups > 0 ? 0.0 : out(p)));
+    const double share = t.ps_active.empty() ? 1.0 : (double)t.ps_active[p] / copies;
+    t.unit_flops.back() *= share;
+    t.unit_bytes.push_back(share * (in(p) + (!l ? out(p) : adj ? 2 * left(p) : c->n_groups > 0 ? 0.0 : out(p))));
   }
   if (adj)
     for (int p = np - 2; p >= 0; p--) {
@@ -755,7 +789,7 @@ tdq_status tiled_execute(TiledSweep& t, const SweepArgs& a0, int grad, cudaStrea
     const bool lone = !a.init && !t.kf.empty() && (np > 1 || a.output == TDQ_OUT_EXPVAL);
     auto grid_for = [&](int slots, TiledDev& dd, int p) {
       dd.ntiles = p == 0 && lone ? 1 : ntiles;
-      const int64_t total = (int64_t)nr * dd.ntiles;
+      const int64_t total = (int64_t)dd.nrows * dd.ntiles;
       const int64_t n0 = std::max<int64_t>(1, std::min<int64_t>(total, slots));
       const int64_t upc = (total + n0 - 1) / n0;
       dd.tiles_per_cta = (int)upc;
@@ -783,6 +817,14 @@ tdq_status tiled_execute(TiledSweep& t, const SweepArgs& a0, int grad, cudaStrea
       d.op_end = t.passes[p].op_end;
       set_pass(t, d, p);
       const bool f = p == 0, l = p == np - 1;
+      if (!t.ps_active.empty()) {
+        d.ps_rows = p ? d.ps_rows + d.ps_active : t.d_ps_rows;
+        d.ps_first = t.d_ps_first;
+        d.alt = t.d_alt;
+        d.ps_active = t.ps_active[p];
+        d.pass = p;
+        d.nrows = nr / t.copies * d.ps_active;
+      }
       const dim3 grid = grid_for(t.slots_f[p], d, p);
       const bool rec = !t.ev.empty() && row0 == 0;
       if (rec) cudaEventRecord(t.ev[2 * p], st);

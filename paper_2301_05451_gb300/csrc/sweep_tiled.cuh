@@ -98,6 +98,11 @@ struct TiledSweep {
   int nthreads = 256, nthreads_r = 256;  // forward / reverse kernels
   std::vector<size_t> smem_f;            // per forward kernel
   size_t smem_r = 0;
+  // shared prefixes of parameter-shift copies (TiledDev::ps_rows)
+  int copies = 1;
+  std::vector<int> ps_active;            // copies run by every pass (empty: all, no sharing)
+  int *d_ps_rows = nullptr, *d_ps_first = nullptr;
+  c2* d_alt = nullptr;
   std::vector<int> threads_f;            // of each forward kernel (narrow_pass)
   int dbl = 1;                           // double-buffered tile loads (forward kernels)
   bool diag = false;                     // the observable's diagonals are tables (SweepArgs::odiag)
@@ -154,7 +159,8 @@ tdq_status tiled_lin_plan(TiledSweep& t, const tdq_circuit* c, const std::vector
 // lin: the program of tiled_lin_plan, or NULL for the generic kernels
 // whole_output: states or probabilities will be read out
 tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<SweepOp>& ops,
-                         const std::vector<int>& ps_gate, int rows, bool adj, int tile_qubits, const LinProgram* lin,
+                         const std::vector<int>& ps_gate, const std::vector<int>& ps_ang, int copies, int rows, bool adj,
+                         int tile_qubits, const LinProgram* lin,
                          int fb, int rb, bool whole_output, double* bytes_row);
 tdq_status tiled_execute(TiledSweep& t, const SweepArgs& a, int grad, cudaStream_t st,
                          int* launches);

@@ -97,3 +97,22 @@ def test_tiled_passes_at_each_cta_shape(api, orc, B, grad):
     if grad == "adjoint":
         ref = orc.param_grads_param_shift(spec, params[B - 1].astype(np.float64))
         np.testing.assert_allclose(g[B - 1].cpu().numpy(), ref, atol=1e-4)
+
+
+@pytest.mark.parametrize("B,n,tile", [(1, 7, 5), (3, 9, 5), (2, 11, 8)])
+def test_shifted_copies_start_at_their_pass(api, orc, B, n, tile):
+    """Parameter shift over two to a dozen tile passes, every copy taken over from
+    the unshifted one at the pass that holds its angle (U3's three angles in
+    passes of their own), against the oracle's shift rule."""
+    import torch
+    spec, params, _ = W.random_circuit(n, 12 * n, 800 + n, batch=B)
+    E = api.Exec(api.Circuit(spec), B, grad="param_shift", max_smem_qubits=1, tile_qubits=tile)
+    p = torch.as_tensor(params).cuda()
+    for _ in range(2):
+        v, g = E.run(p)
+    torch.cuda.synchronize()
+    E.status()
+    np.testing.assert_allclose(v.cpu().numpy(), orc.expvals(spec, W.resolve_angles(spec, params)), atol=1e-5)
+    for b in range(B):
+        ref = orc.param_grads_param_shift(spec, params[b].astype(np.float64))
+        np.testing.assert_allclose(g[b].cpu().numpy(), ref, atol=1e-4)
