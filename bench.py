@@ -638,7 +638,6 @@ def main():
         hbm_peak = peaks.get("hbm_gbs", 6800.0)
         ach_f = flops_row * B / dur_s / 1e12
         ach_b = bytes_row * B / dur_s / 1e9
-        ach_f_step, ach_b_step = ach_f / alu_peak, ach_b / hbm_peak
         kern = "k1 tiled passes (whole step)" if args.interpret else "tdq_k1f_* / tdq_k1r_* (whole step)"
         alu = {"bound": "alu", "achieved": ach_f, "peak": alu_peak, "unit": "TFLOP/s", "frac": ach_f / alu_peak,
                "peak_note": "FP32 SIMT %d SMs x 128 lanes x 2 flop x %.0f MHz (%s max clock)" % (sm_count, mhz, src)}
@@ -673,7 +672,9 @@ def main():
                         arithmetic_intensity_flop_per_byte=fl / max(by, 1.0),
                         ridge_flop_per_byte=alu_peak * 1e3 / hbm_peak, other=second,
                         per_kind_ms_per_step={names[k]: share[k] for k in share},
-                        whole_step={"alu_frac": ach_f_step, "hbm_frac": ach_b_step})
+                        # (the timed launches' own work; with rows in several chunks, of the first)
+                        whole_step={"alu_frac": sum(w[0] for w in work) / dur_s / 1e12 / alu_peak,
+                                    "hbm_frac": sum(w[1] for w in work) / dur_s / 1e9 / hbm_peak})
 
     plain = None
     if rank == 0 and tree is None and multi is None and wl["grad"] == "adjoint" and not args.no_plain:
