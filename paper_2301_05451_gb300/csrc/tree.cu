@@ -662,8 +662,10 @@ __device__ __forceinline__ void kahan(float& s, float& c, float v) {
   c = (t - s) - y;
   s = t;
 }
-template <int R>
-__global__ void __launch_bounds__(256) k_tree_tile(TreeArgs a, int s, int ltm, int ltn, int lsplit) {
+// KS: groups of 256 threads in the block, each with a KS-th of every staged chunk;
+// the last groups' sums go through shared memory to the first.
+template <int R, int KS>
+__global__ void __launch_bounds__(256 * KS) k_tree_tile(TreeArgs a, int s, int ltm, int ltn, int lsplit) {
   chain_start();
   extern __shared__ __align__(16) unsigned char tl_raw[];
   __shared__ __align__(8) int8_t pos[80];
@@ -685,18 +687,19 @@ __global__ void __launch_bounds__(256) k_tree_tile(TreeArgs a, int s, int ltm, i
   const c2* A = base + st.a_off + ((size_t)((h << nm) + m0) << nk);
   const c2* B = base + st.b_off + ((size_t)((h << nn) + n0) << nk);
   c2* C = base + st.c_off;
-  const uint32_t tn = threadIdx.x & ((TN / R) - 1u), tm = threadIdx.x / (TN / R);
+  const uint32_t tid = threadIdx.x & 255u, part = threadIdx.x >> 8;
+  const uint32_t tn = tid & ((TN / R) - 1u), tm = tid / (TN / R);
   const bool active = tm < TM / R;
   float re[R][R] = {}, im[R][R] = {}, re_c[R][R] = {}, im_c[R][R] = {};
   for (uint32_t k0 = kb; k0 < kb + ks; k0 += KC) {
     if (k0 > kb) __syncthreads();
 #pragma unroll 4
-    for (uint32_t i = threadIdx.x; i < (TM << lkc); i += 256) As[(i >> lkc) * P + (i & (KC - 1u))] = A[((size_t)(i >> lkc) << nk) + k0 + (i & (KC - 1u))];
+    for (uint32_t i = threadIdx.x; i < (TM << lkc); i += 256 * KS) As[(i >> lkc) * P + (i & (KC - 1u))] = A[((size_t)(i >> lkc) << nk) + k0 + (i & (KC - 1u))];
 #pragma unroll 4
-    for (uint32_t i = threadIdx.x; i < (TN << lkc); i += 256) Bs[(i >> lkc) * P + (i & (KC - 1u))] = B[((size_t)(i >> lkc) << nk) + k0 + (i & (KC - 1u))];
+    for (uint32_t i = threadIdx.x; i < (TN << lkc); i += 256 * KS) Bs[(i >> lkc) * P + (i & (KC - 1u))] = B[((size_t)(i >> lkc) << nk) + k0 + (i & (KC - 1u))];
     __syncthreads();
     if (active)
-      for (uint32_t k1 = 0; k1 < KC; k1 += kTileSum) {
+      for (uint32_t k1 = part * (KC / KS); k1 < (part + 1) * (KC / KS); k1 += kTileSum) {
         float pr[R][R] = {}, pi[R][R] = {};
 #pragma unroll
         for (uint32_t kk = k1; kk < k1 + kTileSum; kk++) {
@@ -723,6 +726,17 @@ __global__ void __launch_bounds__(256) k_tree_tile(TreeArgs a, int s, int ltm, i
             kahan(im[i][j], im_c[i][j], pi[i][j]);
           }
       }
+  }
+  if constexpr (KS > 1) {  // (R = 1: one output per thread of a group)
+    __syncthreads();
+    if (part) As[(part - 1) * 256 + tid] = {re[0][0], im[0][0]};
+    __syncthreads();
+    if (part) return;
+    for (int p = 0; p < KS - 1; p++) {
+      const c2 v = As[p * 256 + tid];
+      kahan(re[0][0], re_c[0][0], v.x);
+      kahan(im[0][0], im_c[0][0], v.y);
+    }
   }
   if (!active) return;
   const uint32_t ch = scatter_bits(h, pos + 64, nh);
@@ -1010,8 +1024,12 @@ struct TreeExec final : tdq_exec {
       ltn = std::min((int)sd.nn, lt - ltm);
       const dim3 g(1u << (sd.nm - ltm), 1u << (sd.nn - ltn + lsplit), (unsigned)nb << sd.nh);
       const size_t sm = sizeof(c2) * ((1u << ltm) + (1u << ltn)) * ((size_t)std::min(1 << sd.nk, kTileK) + 1);
-      if (two) (void)launch_chained(k_tree_tile<2>, g, dim3(256), sm, st, a, s, ltm, ltn, lsplit);
-      else (void)launch_chained(k_tree_tile<1>, g, dim3(256), sm, st, a, s, ltm, ltn, 0);
+      // a long k in few blocks: four groups of threads per output tile (32 x 128
+      // outputs, k 128, 4 entries: 12.8 -> 8.2 us)
+      const bool wide = !two && sd.nk >= 6 && (int64_t)g.x * g.y * g.z <= 2 * sm_count;
+      if (two) (void)launch_chained(k_tree_tile<2, 1>, g, dim3(256), sm, st, a, s, ltm, ltn, lsplit);
+      else if (wide) (void)launch_chained(k_tree_tile<1, 4>, g, dim3(1024), sm, st, a, s, ltm, ltn, 0);
+      else (void)launch_chained(k_tree_tile<1, 1>, g, dim3(256), sm, st, a, s, ltm, ltn, 0);
     } else if (step_kind[s] == 2 || step_kind[s] == 3) {
       const bool ax = step_kind[s] == 2;
       const StepDev* dd = D + s;
@@ -1916,8 +1934,9 @@ extern "C" tdq_status tdq_plan_compile(const tdq_plan* p, const tdq_compile_opts
   if ((s = up((void**)&e->d_steps, e->steps_h.data(), sizeof(StepDev) * e->steps_h.size())) != TDQ_OK)
     return bail(s);
   constexpr int kTileSmem = (int)sizeof(c2) * (256 + 1) * (kTileK + 1);
-  if (cudaFuncSetAttribute(k_tree_tile<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmem) != cudaSuccess ||
-      cudaFuncSetAttribute(k_tree_tile<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmem) != cudaSuccess)
+  if (cudaFuncSetAttribute(k_tree_tile<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmem) != cudaSuccess ||
+      cudaFuncSetAttribute(k_tree_tile<1, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmem) != cudaSuccess ||
+      cudaFuncSetAttribute(k_tree_tile<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmem) != cudaSuccess)
     return bail(fail(TDQ_ERR_CUDA, "tdq_plan_compile: shared memory attribute"));
   if (cudaFuncSetAttribute(k_tree_step_splitk, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)sizeof(c2) * (8192 + 4096)) != cudaSuccess)

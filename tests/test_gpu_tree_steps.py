@@ -89,7 +89,7 @@ def _path(N, n, left, opened, nk, nn):
 # k split over blocks with and without a sum of blocks
 SHAPES = [(8, 5, 3, 3, 3), (8, 4, 4, 7, 2), (9, 9, 0, 6, 1), (8, 2, 6, 6, 5), (9, 1, 7, 8, 2), (7, 5, 5, 6, 1),
           (6, 5, 5, 5, 130), (7, 7, 6, 7, 1), (9, 8, 6, 7, 9), (10, 7, 7, 10, 1), (8, 5, 5, 8, 1), (8, 6, 5, 8, 160),
-          (10, 5, 6, 9, 3), (8, 4, 4, 8, 2), (9, 0, 3, 9, 4), (8, 2, 2, 8, 3), (9, 6, 5, 5, 33)]
+          (10, 5, 6, 9, 3), (8, 4, 4, 8, 2), (9, 0, 3, 9, 4), (8, 2, 2, 8, 3), (9, 6, 5, 5, 33), (8, 4, 4, 6, 400)]
 
 
 @pytest.mark.parametrize("plain", [False, True])
