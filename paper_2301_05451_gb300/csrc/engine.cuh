@@ -22,7 +22,7 @@ constexpr int kRevRegBits = 3;
 // Whole-state programs specialised to a circuit: narrow passes while a few
 // hundred groups are all a pass has (their straight-line code is shorter, and
 // fetching it is what a small state waits for: 9 qubits, 1001 rows, values,
-// 32 us at 2 bits, 36 at 3; 6 qubits, value and gradient, 17.9 against 19.7),
+// 32 us at 2 bits, 36 at 3; 6 qubits, value and gradient, 15.3 against 16.9),
 // 3 bits from 11 qubits (12 qubits, 256 rows, value and gradient: 86 us at 3/3
 // bits, 100 at 2/2, 85 at 4/4, which has twice the code).
 __host__ __device__ constexpr int spec_reg_bits(int n) { return n >= 11 ? 3 : 2; }
@@ -688,15 +688,16 @@ __device__ __forceinline__ OpMat build_recipe(const SweepArgs& a, const SweepOp*
 // sqrt(2) per gate, and every gate has one form.  Programs that return
 // amplitudes (exact) need the frame's phase too; they keep a second form
 // instead, (u a0 - a1, u a1 + a0) with u = cos / sin and factor sin.
-// What bounds the tiled kernels is issue slots and latency at 16 warps per SM
-// (ncu, 20-qubit ladder: issue 52 % forward, 45 % reverse, FMA pipe 31-36 %,
-// DRAM 41 % of its rate).  Against one fused 2 x 2 product per qubit forward
+// What bounds the tiled kernels is no one pipe, at 16 warps per SM (ncu, 20-qubit
+// ladder: issue about half, FMA pipe 34 to 52 %, shared-memory data pipe 34 to 52
+// %, DRAM 6 to 40 %).  Against one fused 2 x 2 product per qubit forward
 // and one op per gate in reverse, with CNOTs as register moves: 20-qubit
 // ladder, 64 rows, value and gradient 12.74 -> 6.17 ms (tile passes 8 -> 6),
 // 5.5 with one form per rotation (a second one behind a branch had a third of
-// the code); its 481 shifted circuits 26.3 -> 13.0 -> 11.3 ms; 16 qubits of
-// random gates, 24 rows, 611 -> 223 us; state vectors of 20 qubits, 16 rows,
-// 1024 -> 644 -> 590 us.
+// the code), 4.3 with the tiles' low bits chosen, 16-byte moves and narrower
+// forward CTAs; its 481 shifted circuits 26.3 -> 13.0 -> 11.3 -> 8.0 ms; 16 qubits
+// of random gates, 24 rows, 611 -> 223 -> 139 us; state vectors of 20 qubits, 16
+// rows, 1024 -> 644 -> 590 -> 451 us.
 
 __device__ __forceinline__ float sx(float v, uint32_t sign) { return __uint_as_float(__float_as_uint(v) ^ sign); }
 

@@ -254,7 +254,8 @@ struct Segments {
 // caller's) instead of being read.  LAST: accumulate the observable groups; with GRAD also form lambda = O_w psi
 // and run this pass's reverse sweep at once (psi and lambda then written).
 // Tiles after the first of a row segment are read while the previous one is
-// being computed (two shared-memory buffers).
+// being computed (two shared-memory buffers; specialised CTAs of 128 threads have
+// one and leave the overlap to the three others of their SM, see narrow_pass).
 // NT: threads per CTA (specialised programs).
 //
 // From |0...0> the state after the first pass is zero outside the pass's tile
@@ -264,7 +265,7 @@ struct Segments {
 // of reading it, and its reverse sweep keeps psi and lambda only on V0, all
 // that the first pass's reverse sweep visits (its gradient shares are
 // products with psi, zero elsewhere).  On the 20-qubit ladder (64 rows) the
-// first pass went from 116 to 27 us forward and from 2.9 ms to 82 us in reverse.
+// first pass went from 116 to 16 us forward and from 2.9 ms to 59 us in reverse.
 template <int NT, bool FIRST, bool LAST, bool GRAD, class Prog>
 __device__ __forceinline__ void k1_forward_body(const SweepArgs& a, const TiledDev& t, int store) {
   extern __shared__ __align__(16) unsigned char raw[];

@@ -629,8 +629,7 @@ static tdq_status compile_sweep_impl(const tdq_circuit* c, const tdq_compile_opt
   if (o->interpret && (o->fwd_reg_bits || o->rev_reg_bits))
     return bail(fail(TDQ_ERR_ARG, "tdq_compile_sweep: register bits apply to specialised programs only"));
   // register bits: specialised whole-state programs default to narrow passes
-  // (short per-gate code, re-run by more groups: the instruction footprint
-  // decides their speed); tiled and generic programs to 4 / 3
+  // (spec_reg_bits); tiled ones to 4 / 4, generic programs to 4 / 3
   const bool k2spec = !o->interpret;
   const int fb = o->fwd_reg_bits ? o->fwd_reg_bits : (k2spec ? spec_reg_bits(c->n) : kFwdRegBits);
   const int rb = o->rev_reg_bits ? o->rev_reg_bits : (k2spec ? spec_reg_bits(c->n) : kRevRegBits);

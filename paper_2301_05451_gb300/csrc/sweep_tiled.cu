@@ -587,8 +587,8 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
   }
   // shared memory per kernel: forward kernels a double-buffered state (psi;
   // the last pass also lambda; one buffer where two do not fit, or in CTAs of
-  // 128 threads, see narrow_pass).  Reverse
-  // kernels hold psi and lambda in one buffer each: two CTAs of 256 threads
+  // 128 threads, see narrow_pass).  Reverse kernels hold psi and lambda in one
+  // buffer each: two CTAs of 256 threads
   // per SM then interleave one CTA's tile loads with the other's compute,
   // which measured faster than one double-buffered CTA of 512 threads.
   const int mbytes = interpret ? t.max_rec * (int)sizeof(OpMat) : coef_bytes(t.max_rec, t.nrot);
