@@ -25,8 +25,6 @@
 
 namespace tdq {
 
-enum LinKind : uint8_t { L_RY, L_RX, L_H, L_PHASE, L_SIGN, L_CZ };
-
 struct LinOp {
   LinKind kind;
   uint32_t m;      // pairing mask (RY, RX, H), else 0

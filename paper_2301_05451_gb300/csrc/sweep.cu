@@ -192,6 +192,8 @@ struct SweepExec final : tdq_exec {
   CoefRec* d_rot = nullptr;   // their rows' frame tables (SweepArgs::rot and on)
   uint32_t *d_rot_x = nullptr, *d_rot_flips = nullptr;
   int nrot = 0;
+  FineOp* d_fine = nullptr;   // the values' own program (SweepArgs::fine), or NULL
+  int nfine = 0;
   float* d_odiag = nullptr;  // observable diagonal per group [ng][2^n] (whole state; tiled when small)
   DOp* d_dops = nullptr;
   int* d_rec_ptr = nullptr;
@@ -222,6 +224,7 @@ struct SweepExec final : tdq_exec {
     cudaFree(d_rot_flips);
     cudaFree(d_coef);
     cudaFree(d_norm);
+    cudaFree(d_fine);
     cudaFree(d_dops);
     cudaFree(d_rec_ptr);
     cudaFree(d_rec_ops);
@@ -258,9 +261,12 @@ struct SweepExec final : tdq_exec {
     a.nrot = nrot;
     a.init = init;
     a.init_stride = init_stride;
+    a.fine = d_fine;
+    a.nfine = nfine;
+    a.fine_rows = d_fine ? B : 0;
     last_launches = 0;
     if (smem_path) {
-      const unsigned grid = (unsigned)((int64_t)B * copies);
+      const unsigned grid = (unsigned)((int64_t)B * copies + a.fine_rows);
       const bool adj = grad == TDQ_GRAD_ADJOINT;
       if (spec_kernel) {
         int nd0 = 0;
@@ -496,6 +502,42 @@ static LinProgram k2_program(const tdq_circuit* c, bool adj, int fb, int rb, boo
   std::vector<int> psg, psa;
   const std::vector<int> tail = peel ? clifford_tail(c) : std::vector<int>();
   return lin_program(sweep_ops(c, &psg, &psa, &tail), c->n, c->n, 0, fb, rb, adj, !peel);
+}
+
+// Whether the values of the whole-state program P come from CTAs of their own,
+// k2_fine_row: while every CTA of the launch has an SM to itself, and the gates,
+// 0.28 us each (a rotation and the phase behind it as one), are through before
+// the gradient sweep's register passes, 0.39 us each.  6 qubits, 3 and 12 layers,
+// 1 to 16 rows, value and gradient: 11.6 and 38.2 us, 11.5 and 37.7 without;
+// where the rule says no, 16 -> 22 us (6 qubits, 60 random gates), 12 -> 16.5 (7
+// qubits, two pairs per thread), values alone 7.1 -> 9.4 (6 qubits).
+constexpr int kFineQubits = 6;
+static bool fine_values(const LinProgram& P, int output, int grad, int batch, int dev) {
+  if (P.n > kFineQubits || output != TDQ_OUT_EXPVAL || grad != TDQ_GRAD_ADJOINT) return false;
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  int gates = 0;
+  for (size_t i = 0; i < P.ops.size(); i++)
+    gates += P.ops[i].kind == L_PHASE && i && P.ops[i - 1].m && P.ops[i - 1].f == P.ops[i].f ? 0 : 1;
+  return gates > 0 && 2 * (int64_t)batch <= sms && 0.28 * gates <= 0.39 * (double)(P.tiles[0].fwd.size() + P.tiles[0].rev.size());
+}
+
+static std::vector<FineOp> fine_program(const LinProgram& P, const std::vector<SweepOp>& gates) {
+  std::vector<FineOp> out;
+  for (const LinOp& g : P.ops) {
+    FineOp f{};
+    f.kind = g.kind;
+    f.m = g.m;
+    f.f = g.f;
+    f.f2 = g.f2;
+    f.b = g.b | (g.b2 << 1);
+    if (g.op >= 0) {
+      f.src = gates[g.op].src[g.ang];
+      f.fixed = gates[g.op].fixed[g.ang];
+    }
+    out.push_back(f);
+  }
+  return out;
 }
 
 // Observable terms and amplitude requests in the frame of a linear program:
@@ -740,7 +782,14 @@ static tdq_status compile_sweep_impl(const tdq_circuit* c, const tdq_compile_opt
         *out = e;
         return ok();
       }
-      const std::string src = k2_specialised_source(lin, adj, e->threads, e->P, "tdq_k2_specialised");
+      const bool fine = fine_values(lin, o->output, o->grad, e->B, e->dev);
+      if (fine) {
+        const std::vector<FineOp> fp = fine_program(lin, ops);
+        if ((s = upload(&e->d_fine, fp)) != TDQ_OK) return bail(s);
+        e->nfine = (int)fp.size();
+        e->smem_bytes = std::max(e->smem_bytes, k2_fine_bytes(c->n));
+      }
+      const std::string src = k2_specialised_source(lin, adj, e->threads, e->P, "tdq_k2_specialised", fine);
       if ((s = jit_kernel(src, "tdq_k2_specialised", &e->spec_kernel)) != TDQ_OK) return bail(s);
       ce = cudaFuncSetAttribute(e->spec_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e->smem_bytes);
     } else {
@@ -872,9 +921,10 @@ static tdq_status sweep_autotune(const tdq_circuit* c, const tdq_compile_opts* o
           std::vector<int> psg, psa;
           const std::vector<int> tail = o->output == TDQ_OUT_EXPVAL ? clifford_tail(c) : std::vector<int>();
           const bool exact = o->output == TDQ_OUT_STATE || o->output == TDQ_OUT_AMPLITUDE;
-          const std::string src = k2_specialised_source(
-              lin_program(sweep_ops(c, &psg, &psa, &tail), c->n, c->n, 0, k.bits, k.bits, adj, exact), adj, k.threads,
-              c->n_params, "tdq_k2_specialised");
+          const LinProgram lin =
+              lin_program(sweep_ops(c, &psg, &psa, &tail), c->n, c->n, 0, k.bits, k.bits, adj, exact);
+          const std::string src = k2_specialised_source(lin, adj, k.threads, c->n_params, "tdq_k2_specialised",
+                                                        fine_values(lin, o->output, o->grad, o->batch, o->device));
           const void* kern = nullptr;
           jit_kernel(src, "tdq_k2_specialised", &kern);  // failures surface again in the build below
         } catch (...) {  // (the build below reports it)

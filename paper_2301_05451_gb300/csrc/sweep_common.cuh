@@ -169,6 +169,19 @@ struct CoefRec {
   int32_t type;
 };
 
+// Ops of a program in a linear frame (lin_program.h).
+enum LinKind : uint8_t { L_RY, L_RX, L_H, L_PHASE, L_SIGN, L_CZ };
+
+// One gate of the values' own program (k2_fine_row), in program order.
+struct FineOp {
+  int32_t kind;
+  uint32_t m, f, f2;  // pairing mask; parities that give the logical bits
+  int32_t b;          // constants added to them (bit 0: f's, bit 1: f2's)
+  int32_t src;        // angle, as CoefRec
+  float fixed;
+  int32_t pad;
+};
+
 struct SweepArgs {
   const SweepOp* ops;
   int G, n;
@@ -216,6 +229,10 @@ struct SweepArgs {
   // multiplied by the scale rows
   const CoefRec* coef;
   const int* norm;
+  // whole states: the launch's first fine_rows CTAs take the values of the rows
+  // from k2_fine_row's program (0: every row's CTA writes its own)
+  const FineOp* fine;
+  int nfine, fine_rows;
 };
 
 // Rows of the gate-tensor table of a specialised program (build_coef).

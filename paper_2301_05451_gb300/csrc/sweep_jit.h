@@ -16,7 +16,9 @@ namespace tdq {
 // Source of a K2 kernel named `name` for the whole-state program `prog` (one
 // tile; grad: with its reverse passes).  nthreads threads per CTA, nparams
 // gradient columns.
-std::string k2_specialised_source(const LinProgram& prog, bool grad, int nthreads, int nparams, const char* name);
+// fine: with the values' own CTAs (SweepArgs::fine_rows).
+std::string k2_specialised_source(const LinProgram& prog, bool grad, int nthreads, int nparams, const char* name,
+                                  bool fine = false);
 
 // One circuit of a multi-circuit whole-state kernel.
 struct K2Part {
