@@ -99,17 +99,19 @@ namespace {
 // Takes ops of `todo` (program order) whose masks fit a space of at most dim
 // vectors grown from `space`; an op may pass earlier ones left behind that it
 // commutes with.  mask(o): the op's mask in the space's coordinates.
-// max_slots > 0 caps the gradient slots taken (the first op always fits).
+// max_slots, max_rows > 0 cap the gradient slots and the angles taken (the first
+// op always fits).
 template <class Mask>
-void take(const std::vector<LinOp>& ops, std::vector<int>& todo, int dim, LinSpace& space, int max_slots, Mask mask,
-          std::vector<int>* taken) {
+void take(const std::vector<LinOp>& ops, std::vector<int>& todo, int dim, LinSpace& space, int max_slots, int max_rows,
+          Mask mask, std::vector<int>* taken) {
   std::vector<int> left;
-  int ns = 0;
+  int ns = 0, nr = 0;
   for (int o : todo) {
     bool ok = true;
     for (size_t i = 0; i < left.size() && ok; i++) ok = lin_commute(ops[o], ops[left[i]]);
-    const int s = ops[o].slot >= 0 ? 1 : 0;
+    const int s = ops[o].slot >= 0 ? 1 : 0, r = ops[o].op >= 0 ? 1 : 0;
     if (ok && max_slots > 0 && !taken->empty() && ns + s > max_slots) ok = false;
+    if (ok && max_rows > 0 && !taken->empty() && nr + r > max_rows) ok = false;
     if (ok && ops[o].m) {
       const uint32_t m = mask(ops[o].m);
       if (space.reduce(m)) {
@@ -120,6 +122,7 @@ void take(const std::vector<LinOp>& ops, std::vector<int>& todo, int dim, LinSpa
     if (ok) {
       taken->push_back(o);
       ns += s;
+      nr += r;
     } else {
       left.push_back(o);
     }
@@ -149,7 +152,7 @@ std::vector<LinReg> reg_passes(const std::vector<LinOp>& ops, const LinTile& t, 
     LinReg r;
     r.M = M;
     LinSpace U;
-    take(ops, todo, M, U, max_slots, local, &r.ops);
+    take(ops, todo, M, U, max_slots, 0, local, &r.ops);
     for (int l = 0; l < t.k && (int)U.v.size() < M; l++)
       if (U.reduce(1u << l)) U.add(1u << l);
     // order by pivot; the pivots are free to choose: prefer those that leave
@@ -260,9 +263,12 @@ LinProgram lin_program(const std::vector<SweepOp>& gates, int n, int k, int L, i
     t.k = k;
     LinSpace V;
     for (int i = 0; i < L; i++) V.add(1u << i);
-    // a tile pass keeps at most kTileSlots gradient accumulators in shared memory
-    constexpr int kTileSlots = 512;
-    take(P.ops, todo, k, V, kTileSlots, [](uint32_t m) { return m; }, &t.ops);
+    // A tile pass keeps at most kTileSlots gradient accumulators, 32 bytes each,
+    // and the tables of kTileRows angles, 16 to 20 bytes each, beside its states in
+    // shared memory.  A whole state is one tile whatever its angles: where its
+    // tables do not fit, it is not run as one.
+    constexpr int kTileSlots = 512, kTileRows = 2048;
+    take(P.ops, todo, k, V, L > 0 && adj ? kTileSlots : 0, L > 0 ? kTileRows : 0, [](uint32_t m) { return m; }, &t.ops);
     for (int p = 0; p < n && (int)V.v.size() < k; p++)
       if (V.reduce(1u << p)) V.add(1u << p);
     // local bits in the order of their pivots (the L lowest first)

@@ -113,9 +113,9 @@ struct LinProgram {
   LinMap map;
 };
 
-// Program of n index bits in tiles of k bits (k = n: the whole state), the L
-// lowest in every tile; register passes of at most mf (forward) and, with
-// adj, mr (reverse) bits.
+// Program of n index bits in tiles of k bits, the L lowest in every tile (L = 0,
+// k = n: the whole state, one tile); register passes of at most mf (forward)
+// and, with adj, mr (reverse) bits.
 LinProgram lin_program(const std::vector<SweepOp>& ops, int n, int k, int L, int mf, int mr, bool adj, bool exact);
 
 // Tiled program: the number of lowest index bits that every tile holds is

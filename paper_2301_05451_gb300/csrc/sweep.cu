@@ -705,6 +705,7 @@ static tdq_status compile_sweep_impl(const tdq_circuit* c, const tdq_compile_opt
     size_t sb = 0;
     if (spec) {
       lin = lin_program(ops, c->n, c->n, 0, fb, rb, adj, exact);
+      if (lin.tiles.size() != 1) return bail(fail(TDQ_ERR_STATE, "tdq_compile_sweep: a whole state in several tiles"));
       e->nrec = (int)lin.tiles[0].coef.size();
       const size_t gb = adj ? k2_grad_bytes(true, e->P, e->threads) : 0;
       sb = dim * sizeof(c2) * (adj ? 2 : 1) + coef_bytes(e->nrec, (int)lin.rot.size()) + ((gb + 7) & ~(size_t)7) + 32 * sizeof(double) + 16;
