@@ -488,7 +488,10 @@ class PassWriter {
         const int cm = combo(basis, reg_parity(g.f));
         s_ << "    lin_share(" << share(withg[i]) << ", sx(" << (r_.norm >= 0 ? "sc * sc * (" : "(");
         for (int c = 0; c < nc; c++) s_ << (cpar(cm & c) ? " - " : c ? " + " : "") << "v" << c;
-        s_ << "), " << group_sign(g.f, g.b).str() << " ^ sig[" << P_.coef[withg[i]] << "]));\n";
+        // (the angle's sign in the row's frame; without rotations there is no frame)
+        s_ << "), " << group_sign(g.f, g.b).str();
+        if (!P_.rot.empty()) s_ << " ^ sig[" << P_.coef[withg[i]] << "]";
+        s_ << "));\n";
       }
       s_ << "    }\n";
     }

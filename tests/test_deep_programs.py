@@ -25,6 +25,28 @@ def _ladder(n, layers):
     return spec
 
 
+def _iqp(n, layers):
+    """No RX, RY, U3: H, RZ, RZZ, CZ and CNOT; parameters numbered last to first."""
+    spec = W.CircuitSpec(n)
+    P = layers * (2 * n - 1)
+    for q in range(n):
+        spec.add("H", [q])
+    for _ in range(layers):
+        for q in range(n):
+            spec.add("RZ", [q], ("p", P - 1))
+            P -= 1
+        for q in range(n - 1):
+            spec.add("RZZ", [q, q + 1], ("p", P - 1))
+            P -= 1
+        for q in range(0, n - 1, 2):
+            spec.add("CZ" if q & 2 else "CNOT", [q, q + 1])
+        for q in range(n):
+            spec.add("H", [q])
+    for q in range(n):
+        spec.z([q], 1.0, q)
+    return spec
+
+
 def _params(spec, rows, lo=0.0, hi=2 * math.pi):
     return np.random.default_rng(spec.n_params).uniform(lo, hi, (rows, spec.n_params)).astype(np.float32)
 
@@ -36,10 +58,13 @@ def _host_case(name):
         if name.endswith("state"):
             spec.terms, spec.n_groups = [], 0
         return spec, _params(spec, 1), 0, not name.endswith("state")
+    if name.startswith("iqp"):
+        spec = _iqp(*(int(v) for v in name[3:].split("_")[0].split("x")))
+        return spec, _params(spec, 2), 5 if "tiled" in name else 0, True
     raise AssertionError(name)
 
 
-HOST = ["ladder3x86", "ladder3x86_state"]
+HOST = ["ladder3x86", "ladder3x86_state", "iqp6x3", "iqp7x2_tiled"]
 
 
 @pytest.mark.parametrize("name", HOST)
@@ -118,3 +143,12 @@ def test_multi_circuit_launch_with_many_angles(api):
         np.testing.assert_allclose(got.cpu().numpy(), orc.expvals(s, W.resolve_angles(s, p)), atol=1e-4)
         cols = [0, s.n_params - 1]
         np.testing.assert_allclose(gr[0].cpu().numpy()[cols], _grads(s, W.resolve_angles(s, p)[0], cols), atol=2.5e-4)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,kw", [(6, {}), (9, {}), (7, dict(max_smem_qubits=1, tile_qubits=5)), (14, {})])
+def test_phase_gradients_without_rotations(api, n, kw):
+    """Circuits of H, RZ, RZZ, CZ and CNOT alone have no sign table."""
+    spec = _iqp(n, 3)
+    params = _params(spec, 2)
+    _check(api, spec, params, list(range(spec.n_params)), 2e-5, 5e-5, ("adjoint", "param_shift"), **kw)
