@@ -99,19 +99,24 @@ namespace {
 // Takes ops of `todo` (program order) whose masks fit a space of at most dim
 // vectors grown from `space`; an op may pass earlier ones left behind that it
 // commutes with.  mask(o): the op's mask in the space's coordinates.
-// max_slots, max_rows > 0 cap the gradient slots and the angles taken (the first
-// op always fits).
+// The first op always fits; what else may be taken:
+struct TakeCaps {  // (0: any number)
+  int slots;     // gradient slots
+  int rows;      // angles
+  int unscaled;  // gates that leave their factor to the pass's scale
+};
 template <class Mask>
-void take(const std::vector<LinOp>& ops, std::vector<int>& todo, int dim, LinSpace& space, int max_slots, int max_rows,
-          Mask mask, std::vector<int>* taken) {
+void take(const std::vector<LinOp>& ops, std::vector<int>& todo, int dim, LinSpace& space, TakeCaps caps, Mask mask,
+          std::vector<int>* taken) {
   std::vector<int> left;
-  int ns = 0, nr = 0;
+  int ns = 0, nr = 0, nu = 0;
   for (int o : todo) {
     bool ok = true;
     for (size_t i = 0; i < left.size() && ok; i++) ok = lin_commute(ops[o], ops[left[i]]);
-    const int s = ops[o].slot >= 0 ? 1 : 0, r = ops[o].op >= 0 ? 1 : 0;
-    if (ok && max_slots > 0 && !taken->empty() && ns + s > max_slots) ok = false;
-    if (ok && max_rows > 0 && !taken->empty() && nr + r > max_rows) ok = false;
+    const int s = ops[o].slot >= 0 ? 1 : 0, r = ops[o].op >= 0 ? 1 : 0, u = ops[o].m ? 1 : 0;
+    if (!taken->empty() && ((caps.slots && ns + s > caps.slots) || (caps.rows && nr + r > caps.rows) ||
+                            (caps.unscaled && nu + u > caps.unscaled)))
+      ok = false;
     if (ok && ops[o].m) {
       const uint32_t m = mask(ops[o].m);
       if (space.reduce(m)) {
@@ -123,12 +128,20 @@ void take(const std::vector<LinOp>& ops, std::vector<int>& todo, int dim, LinSpa
       taken->push_back(o);
       ns += s;
       nr += r;
+      nu += u;
     } else {
       left.push_back(o);
     }
   }
   todo.swap(left);
 }
+
+// Gates that a register pass leaves unscaled at most: each grows the amplitudes by
+// up to sqrt 2, so by 2^24 in a pass, and the scale that takes it back is at least
+// 2^-24 (its square, for the shares of a reverse pass, 2^-48).  Chains of hundreds
+// of gates on one or two qubits would overflow; a pass of a wider circuit is full
+// long before.
+constexpr int kUnscaled = 48;
 
 // Register passes over the tile's ops.  A pass's group index bits are sent to
 // the local bits outside U's pivots so that 16 consecutive groups read 16
@@ -152,7 +165,7 @@ std::vector<LinReg> reg_passes(const std::vector<LinOp>& ops, const LinTile& t, 
     LinReg r;
     r.M = M;
     LinSpace U;
-    take(ops, todo, M, U, max_slots, 0, local, &r.ops);
+    take(ops, todo, M, U, {max_slots, 0, kUnscaled}, local, &r.ops);
     for (int l = 0; l < t.k && (int)U.v.size() < M; l++)
       if (U.reduce(1u << l)) U.add(1u << l);
     // order by pivot; the pivots are free to choose: prefer those that leave
@@ -268,7 +281,8 @@ LinProgram lin_program(const std::vector<SweepOp>& gates, int n, int k, int L, i
     // shared memory.  A whole state is one tile whatever its angles: where its
     // tables do not fit, it is not run as one.
     constexpr int kTileSlots = 512, kTileRows = 2048;
-    take(P.ops, todo, k, V, L > 0 && adj ? kTileSlots : 0, L > 0 ? kTileRows : 0, [](uint32_t m) { return m; }, &t.ops);
+    take(P.ops, todo, k, V, {L > 0 && adj ? kTileSlots : 0, L > 0 ? kTileRows : 0, 0}, [](uint32_t m) { return m; },
+         &t.ops);
     for (int p = 0; p < n && (int)V.v.size() < k; p++)
       if (V.reduce(1u << p)) V.add(1u << p);
     // local bits in the order of their pivots (the L lowest first)

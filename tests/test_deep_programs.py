@@ -47,6 +47,32 @@ def _iqp(n, layers):
     return spec
 
 
+def _deep(kind, n, gates):
+    """Hundreds of gates that mix amplitudes on one or two qubits, more than
+    one register pass may leave unscaled."""
+    spec = W.CircuitSpec(n)
+    for i in range(gates):
+        q = i % n
+        if kind == "hz":
+            spec.add("H", [q])
+            spec.add("RZ", [q], ("p", spec.n_params))
+        elif kind == "hcz":  # (few gradient slots: long reverse passes too)
+            spec.add("H", [q])
+            spec.add("CZ", [0, 1])
+            if i % 40 == 0:
+                spec.add("RY", [q], ("p", spec.n_params))
+        elif kind == "fixed":
+            spec.add(("RX", "RY")[i // n & 1], [q], ("c", 1.3) if i % 8 else ("p", spec.n_params))
+        else:
+            spec.add(("RX", "RY")[i // n & 1], [q], ("p", spec.n_params))
+        if n == 2 and i % 4 == 3 and kind != "hcz":
+            spec.add("CZ", [0, 1])
+    for q in range(n):
+        spec.add("RX", [q], ("p", spec.n_params))
+        spec.z([q], 1.0, q)
+    return spec
+
+
 def _params(spec, rows, lo=0.0, hi=2 * math.pi):
     return np.random.default_rng(spec.n_params).uniform(lo, hi, (rows, spec.n_params)).astype(np.float32)
 
@@ -58,13 +84,19 @@ def _host_case(name):
         if name.endswith("state"):
             spec.terms, spec.n_groups = [], 0
         return spec, _params(spec, 1), 0, not name.endswith("state")
+    if name.startswith("deep"):
+        kind, size = name[5:].split("_")
+        spec = _deep(kind, *(int(v) for v in size.split("x")))
+        if kind == "rot":
+            return spec, _params(spec, 1, 1.0, 2.0), 0, True
+        return spec, _params(spec, 1), 0, True
     if name.startswith("iqp"):
         spec = _iqp(*(int(v) for v in name[3:].split("_")[0].split("x")))
         return spec, _params(spec, 2), 5 if "tiled" in name else 0, True
     raise AssertionError(name)
 
 
-HOST = ["ladder3x86", "ladder3x86_state", "iqp6x3", "iqp7x2_tiled"]
+HOST = ["ladder3x86", "ladder3x86_state", "iqp6x3", "iqp7x2_tiled", "deep_rot_2x480", "deep_hz_1x300", "deep_hcz_2x400"]
 
 
 @pytest.mark.parametrize("name", HOST)
@@ -152,3 +184,22 @@ def test_phase_gradients_without_rotations(api, n, kw):
     spec = _iqp(n, 3)
     params = _params(spec, 2)
     _check(api, spec, params, list(range(spec.n_params)), 2e-5, 5e-5, ("adjoint", "param_shift"), **kw)
+
+
+# (FP32 rounding as above: 2e-5 and 5e-5 up to 200 gates, in proportion past that)
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind,n,gates", [("rot", 2, 480), ("rot", 1, 1000), ("hz", 1, 300), ("hcz", 2, 600),
+                                          ("fixed", 1, 600), ("fixed", 2, 600)])
+@pytest.mark.parametrize("kw", [{}, dict(max_smem_qubits=1, tile_qubits=5)])
+def test_long_chains_of_unscaled_gates(api, kind, n, gates, kw):
+    if kw:  # the same chain on two qubits of six
+        spec = W.CircuitSpec(6)
+        small = _deep(kind, n, gates)
+        spec.gates, spec.n_params = list(small.gates), small.n_params
+        for q in range(6):
+            spec.z([q], 1.0, q)
+    else:
+        spec = _deep(kind, n, gates)
+    params = _params(spec, 2, 1.0, 2.0) if kind == "rot" else _params(spec, 2)
+    cols = sorted({0, spec.n_params // 2, spec.n_params - 1})
+    _check(api, spec, params, cols, 1e-7 * len(spec.gates), 2.5e-7 * len(spec.gates), ("none", "adjoint"), **kw)
