@@ -188,9 +188,9 @@ def test_phase_gradients_without_rotations(api, n, kw):
 
 # (FP32 rounding as above: 2e-5 and 5e-5 up to 200 gates, in proportion past that)
 @pytest.mark.gpu
-@pytest.mark.parametrize("kind,n,gates", [("rot", 2, 480), ("rot", 1, 1000), ("hz", 1, 300), ("hcz", 2, 600),
-                                          ("fixed", 1, 600), ("fixed", 2, 600)])
-@pytest.mark.parametrize("kw", [{}, dict(max_smem_qubits=1, tile_qubits=5)])
+@pytest.mark.parametrize("kind,n,gates,kw", [("rot", 2, 480, {}), ("rot", 1, 1000, {}), ("hz", 1, 300, {}), ("hcz", 2, 600, {}),
+                                             ("fixed", 2, 600, {}), ("hz", 1, 120, dict(max_smem_qubits=1, tile_qubits=5)),
+                                             ("rot", 2, 160, dict(max_smem_qubits=1, tile_qubits=5))])
 def test_long_chains_of_unscaled_gates(api, kind, n, gates, kw):
     if kw:  # the same chain on two qubits of six
         spec = W.CircuitSpec(6)
