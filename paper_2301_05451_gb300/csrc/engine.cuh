@@ -703,9 +703,10 @@ __device__ __forceinline__ float sx(float v, uint32_t sign) { return __uint_as_f
 
 __host__ __device__ constexpr int cpar(int v) { return ((v >> 3) ^ (v >> 2) ^ (v >> 1) ^ v) & 1; }
 
-// sin x and cos x as unevaluated sums hi + lo of two floats, correct to about
-// 2^-28: the coefficients' errors are the same for every amplitude, so they,
-// not the rounding of single amplitudes, decide the error of an expectation.
+// sin x and cos x as unevaluated sums hi + lo of two floats, off by 2^-28.4 RMS and
+// 2^-25.4 at most (near odd multiples of pi/4, where the cubic terms' rounding
+// counts): a coefficient's error is the same for every amplitude, so it does not
+// average out as the rounding of single amplitudes does.
 // x is reduced by multiples of pi/2 (Cody and Waite: the constant in pieces of
 // 8 and 11 bits and a rest, so that the products are exact); the remainder's
 // Taylor series (to r^9 / r^10, |r| <= pi/4) has its leading terms as two

@@ -326,6 +326,41 @@ LinProgram lin_program(const std::vector<SweepOp>& gates, int n, int k, int L, i
   return P;
 }
 
+std::string lin_key(const LinProgram& P) {
+  std::string k;
+  auto put = [&](int64_t v) { k.append(reinterpret_cast<const char*>(&v), sizeof(v)); };
+  auto list = [&](const auto& v) {
+    put((int64_t)v.size());
+    if (!v.empty()) k.append(reinterpret_cast<const char*>(v.data()), v.size() * sizeof(v[0]));
+  };
+  for (int64_t v : {(int64_t)P.n, (int64_t)P.pairs, (int64_t)P.exact, (int64_t)P.rot.empty(), (int64_t)P.ops.size()}) put(v);
+  for (const LinOp& o : P.ops) {
+    put((int64_t)o.kind | (int64_t)o.b << 8 | (int64_t)o.b2 << 16 | (int64_t)o.p << 24 | (int64_t)o.m << 32);
+    put((int64_t)o.f | (int64_t)o.f2 << 32);
+    put(o.slot);
+  }
+  list(P.coef);
+  put((int64_t)P.tiles.size());
+  for (const LinTile& t : P.tiles) {
+    put(t.k);
+    put(t.pivots);
+    put((int64_t)t.coef.size());
+    list(t.v);
+    list(t.ops);
+    for (const std::vector<LinReg>* rs : {&t.fwd, &t.rev}) {
+      put((int64_t)rs->size());
+      for (const LinReg& r : *rs) {
+        put(r.M);
+        put(r.norm);
+        for (int i = 0; i < r.M; i++) put(r.u[i]);
+        list(r.grp_pos);
+        list(r.ops);
+      }
+    }
+  }
+  return k;
+}
+
 // A tile is read in runs of 2^L amplitudes.  Runs of 128 bytes (L = 4) need the
 // fewest cache lines per read, but bits held for them are taken from the
 // gates; 32-byte runs (L = 2) still fill the sectors that memory moves, and a

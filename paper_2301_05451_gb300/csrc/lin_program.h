@@ -19,6 +19,7 @@
 #pragma once
 
 #include <cstdint>
+#include <string>
 #include <vector>
 
 #include "engine.cuh"
@@ -112,6 +113,9 @@ struct LinProgram {
   std::vector<LinTile> tiles;
   LinMap map;
 };
+
+// All that a program's generated code depends on, as bytes: equal for equal code.
+std::string lin_key(const LinProgram& P);
 
 // Program of n index bits in tiles of k bits, the L lowest in every tile (L = 0,
 // k = n: the whole state, one tile); register passes of at most mf (forward)

@@ -13,6 +13,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <string>
 #include <thread>
@@ -790,8 +791,8 @@ static tdq_status compile_sweep_impl(const tdq_circuit* c, const tdq_compile_opt
         e->nfine = (int)fp.size();
         e->smem_bytes = std::max(e->smem_bytes, k2_fine_bytes(c->n));
       }
-      const std::string src = k2_specialised_source(lin, adj, e->threads, e->P, "tdq_k2_specialised", fine);
-      if ((s = jit_kernel(src, "tdq_k2_specialised", &e->spec_kernel)) != TDQ_OK) return bail(s);
+      const JitCode code = k2_code(lin, adj, e->threads, e->P, "tdq_k2_specialised", fine);
+      if ((s = jit_kernel(code, "tdq_k2_specialised", &e->spec_kernel)) != TDQ_OK) return bail(s);
       ce = cudaFuncSetAttribute(e->spec_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e->smem_bytes);
     } else {
       if ((s = upload(&e->d_passes, prog.passes)) != TDQ_OK) return bail(s);
@@ -924,10 +925,10 @@ static tdq_status sweep_autotune(const tdq_circuit* c, const tdq_compile_opts* o
           const bool exact = o->output == TDQ_OUT_STATE || o->output == TDQ_OUT_AMPLITUDE;
           const LinProgram lin =
               lin_program(sweep_ops(c, &psg, &psa, &tail), c->n, c->n, 0, k.bits, k.bits, adj, exact);
-          const std::string src = k2_specialised_source(lin, adj, k.threads, c->n_params, "tdq_k2_specialised",
-                                                        fine_values(lin, o->output, o->grad, o->batch, o->device));
+          const JitCode code = k2_code(lin, adj, k.threads, c->n_params, "tdq_k2_specialised",
+                                       fine_values(lin, o->output, o->grad, o->batch, o->device));
           const void* kern = nullptr;
-          jit_kernel(src, "tdq_k2_specialised", &kern);  // failures surface again in the build below
+          jit_kernel(code, "tdq_k2_specialised", &kern);  // failures surface again in the build below
         } catch (...) {  // (the build below reports it)
         }
       });
@@ -1150,15 +1151,20 @@ static int multi_maxrreg(int threads) { return std::min(255, 65536 / threads); }
 // Modules of the persistent kernel over the circuits cs (threads per CTA,
 // register bits fb / rb); the same text for the export, the build and the
 // autotuner, so that they share one compilation.
-static std::vector<std::string> multi_modules(const tdq_circuit* const* cs, int nc, bool adj, int threads, int fb,
-                                              int rb) {
-  std::vector<LinProgram> progs(nc);
-  std::vector<K2Part> parts;
+static JitCode multi_modules(const tdq_circuit* const* cs, int nc, bool adj, int threads, int fb, int rb) {
+  const auto progs = std::make_shared<std::vector<LinProgram>>();
+  std::vector<int> params;
+  std::string key = "multi " + std::to_string(adj) + ' ' + std::to_string(threads);
   for (int c = 0; c < nc; c++) {
-    progs[c] = k2_program(cs[c], adj, fb, rb, true);
-    parts.push_back({&progs[c], cs[c]->n_params});
+    progs->push_back(k2_program(cs[c], adj, fb, rb, true));
+    params.push_back(cs[c]->n_params);
+    key += ' ' + std::to_string(params.back()) + lin_key(progs->back());
   }
-  return k2_multi_modules(parts, adj, threads, "tdq_k2_multi");
+  return {key, [=] {
+            std::vector<K2Part> parts;
+            for (int c = 0; c < nc; c++) parts.push_back({&(*progs)[c], params[c]});
+            return k2_multi_modules(parts, adj, threads, "tdq_k2_multi");
+          }};
 }
 
 // One configuration of a multi-circuit launch: every circuit's tables and
@@ -1433,7 +1439,8 @@ extern "C" tdq_status tdq_multi_source(const tdq_circuit* const* circuits, int n
     if (circuits[c]->n > (adj ? 13 : 14)) return fail(TDQ_ERR_UNSUPPORTED, "tdq_multi_source: circuit too large");
   }
   std::string src;
-  const std::vector<std::string> mods = multi_modules(circuits, n_circuits, adj, threads, fwd_reg_bits, rev_reg_bits);
+  const std::vector<std::string> mods =
+      multi_modules(circuits, n_circuits, adj, threads, fwd_reg_bits, rev_reg_bits).modules();
   for (size_t i = 0; i < mods.size(); i++) src += std::string(kModuleMark) + std::to_string(i) + "\n" + mods[i];
   *len = src.size() + 1;
   if (buf) {

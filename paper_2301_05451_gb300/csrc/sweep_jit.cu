@@ -7,11 +7,12 @@
 
 #include <algorithm>
 #include <atomic>
+#include <charconv>
 #include <cstdlib>
 #include <map>
 #include <mutex>
-#include <sstream>
 #include <thread>
+#include <type_traits>
 
 namespace tdq {
 
@@ -20,6 +21,29 @@ namespace tdq {
 #include "jit_headers.inc"
 
 namespace {
+
+// Generated text (half the time of a string stream).
+class Text {
+ public:
+  Text& operator<<(const char* v) {
+    b_.append(v);
+    return *this;
+  }
+  Text& operator<<(const std::string& v) {
+    b_.append(v);
+    return *this;
+  }
+  template <class T, class = std::enable_if_t<std::is_integral<T>::value>>
+  Text& operator<<(T v) {
+    char d[24];
+    b_.append(d, std::to_chars(d, d + sizeof(d), v).ptr);
+    return *this;
+  }
+  const std::string& str() const { return b_; }
+
+ private:
+  std::string b_;
+};
 
 // (swz and swz_pair)
 uint32_t swz_host(uint32_t x, bool pairs) {
@@ -59,7 +83,7 @@ struct Sign {
 // off-diagonal sign, a phase block absorbs them.
 class PassWriter {
  public:
-  PassWriter(std::ostringstream& s, const LinProgram& P, const LinTile& t, const LinReg& r, bool rev)
+  PassWriter(Text& s, const LinProgram& P, const LinTile& t, const LinReg& r, bool rev)
       : s_(s), P_(P), t_(t), r_(r), rev_(rev), N_(1 << r.M) {
     for (int pos : r.grp_pos) varying_ |= t.v[pos];
     const uint32_t all = P.n >= 32 ? ~0u : (1u << P.n) - 1u;
@@ -108,7 +132,7 @@ class PassWriter {
 
   // local index of the group's first member: group bit i at local bit grp_pos[i]
   std::string spread() const {
-    std::ostringstream e;
+    Text e;
     const int n = (int)r_.grp_pos.size();
     if (n == 0) return "0u * (uint32_t)grp";
     for (int i = 0; i < n;) {
@@ -562,7 +586,7 @@ class PassWriter {
     return nm;
   }
 
-  std::ostringstream& s_;
+  Text& s_;
   const LinProgram& P_;
   const LinTile& t_;
   const LinReg& r_;
@@ -586,7 +610,7 @@ std::string group_index(const LinProgram& P, const LinTile& t, int L) {
   return "base ^ (gb & " + low + "u) ^ (uint32_t)s.off[gb >> " + std::to_string(L) + "]";
 }
 
-void emit_fwd_pass(std::ostringstream& s, const LinProgram& P, const LinTile& t, const LinReg& r, int L, int nthreads) {
+void emit_fwd_pass(Text& s, const LinProgram& P, const LinTile& t, const LinReg& r, int L, int nthreads) {
   s << "  {\n";
   PassWriter(s, P, t, r, false).write(nthreads, group_index(P, t, L), {"psi"}, {"a"}, [](int) { return std::string(); });
   s << "  }\n  __syncthreads();\n";
@@ -597,7 +621,7 @@ void emit_fwd_pass(std::ostringstream& s, const LinProgram& P, const LinTile& t,
 // over the warp for up to 32 accumulators at once (grad_share_multi; their
 // index tables are declared into `decl`).
 template <class F>
-void emit_rev_pass(std::ostringstream& s, std::ostringstream& decl, int* uid, const LinProgram& P, const LinTile& t,
+void emit_rev_pass(Text& s, Text& decl, int* uid, const LinProgram& P, const LinTile& t,
                    const LinReg& r, int L, int nthreads, int stride, F acc_index) {
   // The pass's gradient shares, summed per accumulator index in registers
   // gs<chunk>[position] (a chunk holds at most 32 distinct indices; shares of
@@ -657,7 +681,7 @@ void emit_rev_pass(std::ostringstream& s, std::ostringstream& decl, int* uid, co
 
 // The program struct `sname` of one circuit; constant tables go to decl,
 // numbered from *uid.
-static void k2_prog_struct(std::ostringstream& s, std::ostringstream& decl, int* uid, const LinProgram& P, int nparams,
+static void k2_prog_struct(Text& s, Text& decl, int* uid, const LinProgram& P, int nparams,
                            int nthreads, bool grad, const std::string& sname) {
   const LinTile& t = P.tiles[0];
   s << "struct " << sname << " {\n"
@@ -681,11 +705,11 @@ static void k2_prog_struct(std::ostringstream& s, std::ostringstream& decl, int*
 
 std::string k2_specialised_source(const LinProgram& prog, bool grad, int nthreads, int nparams, const char* name,
                                   bool fine) {
-  std::ostringstream s, decl;
+  Text s, decl;
   int uid = 0;
   k2_prog_struct(s, decl, &uid, prog, nparams, nthreads, grad, "SpecProg");
   s << "}  // namespace tdq\n";
-  std::ostringstream out;
+  Text out;
   out << "#include \"k2_body.cuh\"\nnamespace tdq {\n" << decl.str() << s.str();
   const int minb = nthreads >= 256 ? 2 : 1;
   out << "extern \"C\" __global__ void __launch_bounds__(" << nthreads << ", " << minb << ") " << name
@@ -702,9 +726,9 @@ std::vector<std::string> k2_multi_modules(const std::vector<K2Part>& parts, bool
   std::vector<std::string> mods(1);
   int uid = 0;  // constant tables numbered across modules: their names stay unique at link time
   for (size_t c = 0; c < parts.size(); c++) {
-    std::ostringstream s, decl;
+    Text s, decl;
     k2_prog_struct(s, decl, &uid, *parts[c].prog, parts[c].P, nthreads, grad, "SpecProg_" + std::to_string(c));
-    std::ostringstream out;
+    Text out;
     out << "#include \"k2_body.cuh\"\nnamespace tdq {\n" << decl.str() << s.str() << "}  // namespace tdq\n";
     // the circuit's row body: a function of its own, linked to the launch module
     out << "__device__ __noinline__ void tdq_multi_row_" << c
@@ -713,7 +737,7 @@ std::vector<std::string> k2_multi_modules(const std::vector<K2Part>& parts, bool
         << c << "{nullptr}, nullptr, 0, m.rec_ptr, m.rec_ops, m.nrec, r);\n}\n";
     mods.push_back(out.str());
   }
-  std::ostringstream out;
+  Text out;
   out << "#include \"sweep_common.cuh\"\n";
   for (size_t c = 0; c < parts.size(); c++)
     out << "__device__ void tdq_multi_row_" << c << "(const tdq::SweepArgs& a, const tdq::MultiCirc& m, int r);\n";
@@ -748,7 +772,7 @@ std::vector<std::string> k2_multi_modules(const std::vector<K2Part>& parts, bool
 // neighbours of a tile (both even; see swz_pair), every(f) for its elements.
 // A thread's local indices are 2 (tid + NT i): the part of both indices that
 // tid gives is computed once per tile, the rest are constants.
-static void emit_every(std::ostringstream& s, const LinTile& t, int L) {
+static void emit_every(Text& s, const LinTile& t, int L) {
   s << "  template <int NT, class F>\n  __device__ __forceinline__ static void pairs(const TiledDev&, const TileShared& s, "
        "uint32_t base, F&& f) {\n"
     << "    constexpr uint32_t v[" << t.k << "] = {";
@@ -768,7 +792,7 @@ static void emit_every(std::ostringstream& s, const LinTile& t, int L) {
 
 // in_first(x): whether index x lies in the first pass's space (the remainder
 // of x by the space's basis is zero).
-static void emit_in_first(std::ostringstream& s, const LinTile& t, int n) {
+static void emit_in_first(Text& s, const LinTile& t, int n) {
   const uint32_t out = (n >= 32 ? ~0u : (1u << n) - 1u) & ~t.pivots;
   s << "  __device__ __forceinline__ static bool in_first(uint32_t x) {\n    uint32_t r = x & " << out << "u;\n";
   for (uint32_t v : t.v) {
@@ -780,11 +804,12 @@ static void emit_in_first(std::ostringstream& s, const LinTile& t, int n) {
   s << "    return r == 0u;\n  }\n";
 }
 
-std::string k1_specialised_source(const TiledSweep& t, const LinProgram& prog, int nthreads_r) {
-  std::ostringstream s, decl;
+std::string k1_specialised_source(const TiledSweep& t, const LinProgram& prog, int nthreads_r, int only) {
+  Text s, decl;
   int uid = 0;
   const int np = (int)prog.tiles.size();
   for (int p = 0; p < np; p++) {
+    if (only >= 0 && p != only) continue;
     const LinTile& tile = prog.tiles[p];
     const int nthreads = t.threads_f[p];
     // gradient accumulators of the pass: one per angle with a slot
@@ -831,9 +856,10 @@ std::string k1_specialised_source(const TiledSweep& t, const LinProgram& prog, i
       << "    atomicAdd(&t.gacc[(int64_t)lr * a.P + tdq_slots_" << p << "[i]], v);\n  }\n  }\n};\n";
   }
   s << "}  // namespace tdq\n";
-  std::ostringstream out;
+  Text out;
   out << "#include \"k1_body.cuh\"\nnamespace tdq {\n" << decl.str() << s.str();
   for (int p = 0; p < np; p++) {
+    if (only >= 0 && p != only) continue;
     const bool f = p == 0, l = p == np - 1;
     const int nthreads = t.threads_f[p];
     const int minb = nthreads < t.nthreads ? (l && t.adj ? 3 : 4) : nthreads >= 256 ? 2 : 1;
@@ -854,7 +880,7 @@ namespace {
 
 struct JitCache {
   std::mutex mu;
-  std::map<std::string, cudaLibrary_t> libs;  // by source
+  std::map<std::string, cudaLibrary_t> libs;  // by key
 };
 
 JitCache& cache() {
@@ -872,7 +898,30 @@ std::string nvrtc_log(nvrtcProgram p) {
 
 }  // namespace
 
-tdq_status jit_kernel(const std::string& src, const char* name, const void** kernel) {
+JitCode k2_code(const LinProgram& prog, bool grad, int nthreads, int nparams, const char* name, bool fine) {
+  std::string key = "k2";
+  for (int v : {(int)grad, nthreads, nparams, (int)fine}) key += ' ' + std::to_string(v);
+  return {key + name + lin_key(prog), [=, &prog] {
+            return std::vector<std::string>{k2_specialised_source(prog, grad, nthreads, nparams, name, fine)};
+          }};
+}
+
+JitCode k1_code(const TiledSweep& t, const LinProgram& prog, int nthreads_r, int pass) {
+  std::string key = "k1";
+  for (int v : {t.n, t.k, t.L, (int)t.adj, (int)t.diag, t.ng, t.dbl, t.nthreads, t.threads_f[pass], nthreads_r, pass})
+    key += ' ' + std::to_string(v);
+  return {key + lin_key(prog), [=, &t, &prog] {
+            return std::vector<std::string>{k1_specialised_source(t, prog, nthreads_r, pass)};
+          }};
+}
+
+bool jit_cached(const JitCode& code) {
+  JitCache& C = cache();
+  std::lock_guard<std::mutex> lk(C.mu);
+  return C.libs.count(code.key) > 0;
+}
+
+tdq_status jit_kernel(const JitCode& code, const char* name, const void** kernel) {
   *kernel = nullptr;
   int dev = 0;
   TDQ_CUDA_TRY(cudaGetDevice(&dev));
@@ -882,16 +931,17 @@ tdq_status jit_kernel(const std::string& src, const char* name, const void** ker
   if (maj != 10 || min != 3)
     return fail(TDQ_ERR_UNSUPPORTED, "specialised sweep: built for sm_103a, device is sm_" +
                                          std::to_string(maj) + std::to_string(min));
-  // one compilation per source, all its kernels; NVRTC runs outside the lock
+  // one compilation per key, all its kernels; NVRTC runs outside the lock
   // so that different sources compile concurrently
   JitCache& C = cache();
   cudaLibrary_t lib = nullptr;
   {
     std::lock_guard<std::mutex> lk(C.mu);
-    auto it = C.libs.find(src);
+    auto it = C.libs.find(code.key);
     if (it != C.libs.end()) lib = it->second;
   }
   if (!lib) {
+    const std::string src = code.modules()[0];
     nvrtcProgram p;
     if (nvrtcCreateProgram(&p, src.c_str(), "tdq_specialised.cu", kJitHeaderCount, kJitHeaderSrc,
                            kJitHeaderNames) != NVRTC_SUCCESS)
@@ -912,8 +962,8 @@ tdq_status jit_kernel(const std::string& src, const char* name, const void** ker
     nvrtcDestroyProgram(&p);
     TDQ_CUDA_TRY(cudaLibraryLoadData(&lib, cubin.data(), nullptr, nullptr, 0, nullptr, nullptr, 0));
     std::lock_guard<std::mutex> lk(C.mu);
-    auto ins = C.libs.emplace(src, lib);
-    if (!ins.second) {  // another thread compiled the same source meanwhile
+    auto ins = C.libs.emplace(code.key, lib);
+    if (!ins.second) {  // another thread compiled the same code meanwhile
       cudaLibraryUnload(lib);
       lib = ins.first->second;
     }
@@ -950,7 +1000,7 @@ static tdq_status jit_module(const std::string& src, int maxrreg, std::string* c
   return TDQ_OK;
 }
 
-tdq_status jit_link_kernel(const std::vector<std::string>& mods, const char* name, int maxrreg, const void** kernel) {
+tdq_status jit_link_kernel(const JitCode& code, const char* name, int maxrreg, const void** kernel) {
   *kernel = nullptr;
   int dev = 0;
   TDQ_CUDA_TRY(cudaGetDevice(&dev));
@@ -960,11 +1010,7 @@ tdq_status jit_link_kernel(const std::vector<std::string>& mods, const char* nam
   if (maj != 10 || min != 3)
     return fail(TDQ_ERR_UNSUPPORTED, "specialised sweep: built for sm_103a, device is sm_" + std::to_string(maj) +
                                          std::to_string(min));
-  std::string key = std::to_string(maxrreg) + '\0';
-  for (const std::string& m : mods) {
-    key += m;
-    key.push_back('\0');
-  }
+  const std::string key = std::to_string(maxrreg) + ' ' + code.key;
   JitCache& C = cache();
   cudaLibrary_t lib = nullptr;
   {
@@ -973,6 +1019,7 @@ tdq_status jit_link_kernel(const std::vector<std::string>& mods, const char* nam
     if (it != C.libs.end()) lib = it->second;
   }
   if (!lib) {
+    const std::vector<std::string> mods = code.modules();
     // every module on its own host thread, then one link
     std::vector<std::string> cubins(mods.size()), errs(mods.size());
     std::vector<tdq_status> st(mods.size(), TDQ_OK);

@@ -4,6 +4,7 @@
 // compiled at run time for the device in use.
 #pragma once
 
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -41,18 +42,32 @@ constexpr const char* kModuleMark = "// ==== tdq module ";
 
 // Source of the K1 kernels of every tile pass p of t (program prog):
 // tdq_k1f_<p> (forward; the last one also runs its reverse sweep with
-// gradients) and tdq_k1r_<p> (reverse, passes before the last).
-std::string k1_specialised_source(const TiledSweep& t, const LinProgram& prog, int nthreads_r);
+// gradients) and tdq_k1r_<p> (reverse, passes before the last).  only >= 0:
+// that pass's kernels alone.
+std::string k1_specialised_source(const TiledSweep& t, const LinProgram& prog, int nthreads_r, int only = -1);
 
-// Compiles `src` for the current device and returns the kernel `name` (a
-// handle usable with cudaLaunchKernel / cudaFuncSetAttribute).  Compiled
-// kernels are cached by source for the life of the process.
-tdq_status jit_kernel(const std::string& src, const char* name, const void** kernel);
+// Code to compile: bytes that differ wherever its text does, and the text, written
+// out only if no kernel of that key is in the cache (writing it takes longer than
+// the rest of a compile that finds its kernels there: 2 ms for the 20-qubit ladder).
+struct JitCode {
+  std::string key;
+  std::function<std::vector<std::string>()> modules;
+};
+JitCode k2_code(const LinProgram& prog, bool grad, int nthreads, int nparams, const char* name, bool fine);
+JitCode k1_code(const TiledSweep& t, const LinProgram& prog, int nthreads_r, int pass);
+
+// Whether the code is compiled already.
+bool jit_cached(const JitCode& code);
+
+// Compiles the code (one module) for the current device and returns the kernel
+// `name` (a handle usable with cudaLaunchKernel / cudaFuncSetAttribute).  Compiled
+// kernels are cached by key for the life of the process.
+tdq_status jit_kernel(const JitCode& code, const char* name, const void** kernel);
 
 // Compiles the modules concurrently (NVRTC, relocatable device code, one host
 // thread each, every function within maxrreg registers -- the kernel's launch
 // bounds, which separately compiled callees cannot see), links them
-// (nvJitLink) and returns the kernel `name`; cached by the modules' text.
-tdq_status jit_link_kernel(const std::vector<std::string>& mods, const char* name, int maxrreg, const void** kernel);
+// (nvJitLink) and returns the kernel `name`; cached by key.
+tdq_status jit_link_kernel(const JitCode& code, const char* name, int maxrreg, const void** kernel);
 
 }  // namespace tdq

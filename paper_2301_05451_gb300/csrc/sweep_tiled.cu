@@ -2,9 +2,11 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <map>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "k1_body.cuh"
@@ -606,18 +608,43 @@ tdq_status tiled_compile(TiledSweep& t, const tdq_circuit* c, const std::vector<
   size_t smax = sizes(t.dbl ? 2 : 1);
   if (smax > 227 * 1024) return fail(TDQ_ERR_UNSUPPORTED, "tiled sweep: tile program too large");
   if (!interpret) {
-    // every tile pass as straight-line code; one compilation for all passes
-    const std::string src = k1_specialised_source(t, *lin, t.nthreads_r);
+    // every tile pass as straight-line code, a module per pass; those not in the
+    // cache are compiled on a host thread each (failures surface again below)
+    std::vector<JitCode> code(np);
+    std::vector<int> todo;
+    for (int p = 0; p < np; p++) {
+      code[p] = k1_code(t, *lin, t.nthreads_r, p);
+      if (!jit_cached(code[p])) todo.push_back(p);
+    }
+    std::atomic<size_t> next{0};
+    std::vector<std::thread> pool;
+    auto work = [&] {
+      try {
+        if (cudaSetDevice(dev) != cudaSuccess) return;
+        for (size_t i = next++; i < todo.size(); i = next++) {
+          const void* k = nullptr;
+          jit_kernel(code[todo[i]], ("tdq_k1f_" + std::to_string(todo[i])).c_str(), &k);
+        }
+      } catch (...) {
+      }
+    };
+    const size_t nt = std::min<size_t>(todo.size(), std::thread::hardware_concurrency());
+    pool.reserve(nt);
+    try {
+      for (size_t w = 0; w < nt && nt > 1; w++) pool.emplace_back(work);
+    } catch (...) {  // (as many threads as there are)
+    }
+    for (std::thread& th : pool) th.join();
     for (int p = 0; p < np; p++) {
       const void* kf = nullptr;
       const void* kr = nullptr;
       const std::string nf = "tdq_k1f_" + std::to_string(p), nr = "tdq_k1r_" + std::to_string(p);
-      tdq_status s2 = jit_kernel(src, nf.c_str(), &kf);
+      tdq_status s2 = jit_kernel(code[p], nf.c_str(), &kf);
       if (s2 != TDQ_OK) return s2;
       if (cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t.smem_f[p]) != cudaSuccess)
         return fail(TDQ_ERR_CUDA, "tiled sweep: cudaFuncSetAttribute");
       if (adj && p + 1 < np) {
-        if ((s2 = jit_kernel(src, nr.c_str(), &kr)) != TDQ_OK) return s2;
+        if ((s2 = jit_kernel(code[p], nr.c_str(), &kr)) != TDQ_OK) return s2;
         if (cudaFuncSetAttribute(kr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t.smem_r) != cudaSuccess)
           return fail(TDQ_ERR_CUDA, "tiled sweep: cudaFuncSetAttribute");
       }

@@ -655,6 +655,7 @@ __global__ void __launch_bounds__(256) k_tree_step_splitk(TreeArgs a, int s, int
 constexpr int kTileK = 64;   // k entries staged at a time
 // Sums are taken in FP32 pieces of kTileSum entries, added with compensation: a
 // long k then rounds less than in the lane-split sums that the tile replaces.
+// (Where k is split over blocks, their sums meet in FP32 atomics without it.)
 constexpr int kTileSum = 4;
 // s += v, with the rounding errors so far in c
 __device__ __forceinline__ void kahan(float& s, float& c, float v) {
@@ -1027,9 +1028,12 @@ struct TreeExec final : tdq_exec {
   // 65 rows of staged operands at most, 135 KB.)
   static bool tile_step(const StepDev& sd, int kind, int nb) {
     const int out = sd.nm + sd.nn;
-    // (from four batch entries -- rows times slices -- up, where the figures are
-    // from; with fewer the kinds stay as they are, which the cost model's features
-    // describe: its pick then beats the FLOP count's by 4.5 %, with tiles by 0.2 %)
+    // (From four batch entries -- rows times slices -- up.  With fewer the tiles
+    // are faster too: 74 unsliced plans of 20 to 50 qubits, 1, 2 and 3 rows, 11, 13
+    // and 14 % in geometric mean, none slower by more than 2 %.  But the cost model
+    // is trained on and ranks executions of one entry, and tiles make their steps so
+    // alike that its pick is no faster than the fewest FLOPs': 0.99 to 1.01 of it
+    // over 8 trainings, also with a feature for the tiles, against 1.04 to 1.06.)
     if (kind != 5 && nb < 4) return false;
     if ((kind == 2 || kind == 3) && sd.nk > 5) return false;
     if (kind == 5) return sd.nm >= 5 && sd.nn >= 5 && ((int64_t)nb << sd.nh) <= 65535;
