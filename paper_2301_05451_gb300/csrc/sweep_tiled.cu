@@ -4,9 +4,9 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
-#include <map>
 #include <string>
 #include <thread>
+#include <utility>
 #include <vector>
 
 #include "k1_body.cuh"
@@ -181,19 +181,32 @@ OutMap out_map(const LinMap& map) {
       if ((x >> q) & 1u) y ^= map.col[q];
     return y;
   };
-  std::map<uint32_t, int> place;  // x offset -> position in the order of y
-  for (int l = 0; l < (1 << bits); l++) {
-    uint32_t x = 0, xy = 0;
-    for (int i = 0; i < bits; i++) {
-      if (!((l >> i) & 1)) continue;
-      x ^= bx[i];
-      xy ^= by[i];
-    }
-    m.x[l] = x;
-    m.y[l] = y_of(xy);
-    place[xy] = l;
+  // everything is linear: entry l from the entries of its bits; `at` of a basis
+  // vector are its coordinates in the other basis
+  std::vector<std::pair<uint32_t, int>> rows;  // reduced vectors of `by`, and which they are sums of
+  for (int i = 0; i < bits; i++) {
+    std::pair<uint32_t, int> v{by[i], 1 << i};
+    for (const auto& r : rows)
+      if (v.first & r.first & (0u - r.first)) v = {v.first ^ r.first, v.second ^ r.second};
+    const uint32_t low = v.first & (0u - v.first);
+    for (auto& r : rows)
+      if (r.first & low) r = {r.first ^ v.first, r.second ^ v.second};
+    rows.push_back(v);
   }
-  for (int l = 0; l < (1 << bits); l++) m.at[l] = (uint16_t)place.at(m.x[l]);
+  for (int i = 0; i < bits; i++) {
+    int at = 0;
+    for (const auto& r : rows)
+      if (bx[i] & r.first & (0u - r.first)) at ^= r.second;
+    m.x[1 << i] = bx[i];
+    m.y[1 << i] = y_of(by[i]);
+    m.at[1 << i] = (uint16_t)at;
+  }
+  for (int l = 1; l < (1 << bits); l++) {
+    const int low = l & -l;
+    m.x[l] = m.x[l ^ low] ^ m.x[low];
+    m.y[l] = m.y[l ^ low] ^ m.y[low];
+    m.at[l] = (uint16_t)(m.at[l ^ low] ^ m.at[low]);
+  }
   return m;
 }
 
