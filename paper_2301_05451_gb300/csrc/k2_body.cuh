@@ -258,7 +258,7 @@ __host__ __device__ __forceinline__ size_t k2_fine_bytes(int n) {
 }
 
 // layout: psi[dim] (x.h, x.l, y.h, y.l) | ops[kFineOps] | coefficients[kFineOps] | red[32]
-__device__ __noinline__ void k2_fine_row(const SweepArgs& a, int64_t b) {
+static __device__ __noinline__ void k2_fine_row(const SweepArgs& a, int64_t b) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const uint32_t dim = 1u << a.n, tid = threadIdx.x, nt = blockDim.x;
   float4* psi = reinterpret_cast<float4*>(smem_raw);
