@@ -328,27 +328,29 @@ LinProgram lin_program(const std::vector<SweepOp>& gates, int n, int k, int L, i
 
 std::string lin_key(const LinProgram& P) {
   std::string k;
-  auto put = [&](int64_t v) { k.append(reinterpret_cast<const char*>(&v), sizeof(v)); };
+  auto put = [&](uint64_t v) { k.append(reinterpret_cast<const char*>(&v), sizeof(v)); };
   auto list = [&](const auto& v) {
-    put((int64_t)v.size());
+    put(v.size());
     if (!v.empty()) k.append(reinterpret_cast<const char*>(v.data()), v.size() * sizeof(v[0]));
   };
-  for (int64_t v : {(int64_t)P.n, (int64_t)P.pairs, (int64_t)P.exact, (int64_t)P.rot.empty(), (int64_t)P.ops.size()}) put(v);
+  put(P.n);
+  put((P.pairs ? 1u : 0u) | (P.exact ? 2u : 0u) | (P.rot.empty() ? 4u : 0u));
+  put(P.ops.size());
   for (const LinOp& o : P.ops) {
-    put((int64_t)o.kind | (int64_t)o.b << 8 | (int64_t)o.b2 << 16 | (int64_t)o.p << 24 | (int64_t)o.m << 32);
-    put((int64_t)o.f | (int64_t)o.f2 << 32);
+    put(o.kind | o.b << 8 | o.b2 << 16 | (o.p ? 1 : 0) << 24 | (uint64_t)o.m << 32);
+    put(o.f | (uint64_t)o.f2 << 32);
     put(o.slot);
   }
   list(P.coef);
-  put((int64_t)P.tiles.size());
+  put(P.tiles.size());
   for (const LinTile& t : P.tiles) {
     put(t.k);
     put(t.pivots);
-    put((int64_t)t.coef.size());
+    put(t.coef.size());
     list(t.v);
     list(t.ops);
     for (const std::vector<LinReg>* rs : {&t.fwd, &t.rev}) {
-      put((int64_t)rs->size());
+      put(rs->size());
       for (const LinReg& r : *rs) {
         put(r.M);
         put(r.norm);

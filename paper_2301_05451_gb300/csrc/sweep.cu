@@ -1149,7 +1149,7 @@ struct MultiExec final : tdq_exec {
 static int multi_maxrreg(int threads) { return std::min(255, 65536 / threads); }
 
 // Modules of the persistent kernel over the circuits cs (threads per CTA,
-// register bits fb / rb); the same text for the export, the build and the
+// register bits fb / rb); the same for the export, the build and the
 // autotuner, so that they share one compilation.
 static JitCode multi_modules(const tdq_circuit* const* cs, int nc, bool adj, int threads, int fb, int rb) {
   const auto progs = std::make_shared<std::vector<LinProgram>>();
