@@ -183,6 +183,10 @@ __device__ __forceinline__ void k2_body(const SweepArgs& a, Prog prog, const DOp
 // gradients in float.  What bounds it is the chain of gates: a barrier, shared
 // memory there and back and some 100 dependent instructions, 0.28 us each.
 constexpr int kFineOps = 64;   // gates staged at a time
+// CTAs between the rows' and the values' that leave at once: on the SM beside it, a
+// value's CTA slows the row's while both fetch cold code (6 qubits, one row, L2
+// flushed: 21.2 us; 19.1 with a gap; 18.1 without the values' CTA).
+constexpr int kFineGap = 8;
 
 struct df {  // h + l, |l| at most half an ulp of h
   float h, l;

@@ -267,7 +267,7 @@ struct SweepExec final : tdq_exec {
     a.fine_rows = d_fine ? B : 0;
     last_launches = 0;
     if (smem_path) {
-      const unsigned grid = (unsigned)((int64_t)B * copies + a.fine_rows);
+      const unsigned grid = (unsigned)((int64_t)B * copies + (d_fine ? kFineGap + B : 0));
       const bool adj = grad == TDQ_GRAD_ADJOINT;
       if (spec_kernel) {
         int nd0 = 0;
@@ -509,7 +509,7 @@ static LinProgram k2_program(const tdq_circuit* c, bool adj, int fb, int rb, boo
 // k2_fine_row: while every CTA of the launch has an SM to itself, and the gates,
 // 0.28 us each (a rotation and the phase behind it as one), are through before
 // the gradient sweep's register passes, 0.39 us each.  6 qubits, 3 and 12 layers,
-// 1 to 16 rows, value and gradient: 11.6 and 38.2 us, 11.5 and 37.7 without;
+// 1 to 16 rows, value and gradient: 11.5 and 37.7 us with them and without;
 // where the rule says no, 16 -> 22 us (6 qubits, 60 random gates), 12 -> 16.5 (7
 // qubits, two pairs per thread), values alone 7.1 -> 9.4 (6 qubits).
 constexpr int kFineQubits = 6;
@@ -520,7 +520,7 @@ static bool fine_values(const LinProgram& P, int output, int grad, int batch, in
   int gates = 0;
   for (size_t i = 0; i < P.ops.size(); i++)
     gates += P.ops[i].kind == L_PHASE && i && P.ops[i - 1].m && P.ops[i - 1].f == P.ops[i].f ? 0 : 1;
-  return gates > 0 && 2 * (int64_t)batch <= sms && 0.28 * gates <= 0.39 * (double)(P.tiles[0].fwd.size() + P.tiles[0].rev.size());
+  return gates > 0 && 2 * (int64_t)batch + kFineGap <= sms && 0.28 * gates <= 0.39 * (double)(P.tiles[0].fwd.size() + P.tiles[0].rev.size());
 }
 
 static std::vector<FineOp> fine_program(const LinProgram& P, const std::vector<SweepOp>& gates) {

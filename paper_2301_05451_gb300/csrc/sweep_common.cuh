@@ -229,8 +229,9 @@ struct SweepArgs {
   // multiplied by the scale rows
   const CoefRec* coef;
   const int* norm;
-  // whole states: the launch's first fine_rows CTAs take the values of the rows
-  // from k2_fine_row's program (0: every row's CTA writes its own)
+  // whole states: behind the rows' CTAs and kFineGap empty ones, a CTA per row
+  // takes the values from k2_fine_row's program (fine_rows = 0: every row's own
+  // CTA writes them)
   const FineOp* fine;
   int nfine, fine_rows;
 };

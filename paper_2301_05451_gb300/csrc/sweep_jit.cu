@@ -714,10 +714,12 @@ std::string k2_specialised_source(const LinProgram& prog, bool grad, int nthread
   const int minb = nthreads >= 256 ? 2 : 1;
   out << "extern \"C\" __global__ void __launch_bounds__(" << nthreads << ", " << minb << ") " << name
     << "(tdq::SweepArgs a, const tdq::DOp* gdops, int ndops, const int* rec_ptr, const int* rec_ops, int nrec) {\n"
-    << (fine ? "  if ((int)blockIdx.x < a.fine_rows) {\n    tdq::k2_fine_row(a, blockIdx.x);\n    return;\n  }\n" : "")
+    << (fine ? "  if (a.fine_rows && (int)blockIdx.x >= a.fine_rows) {\n"
+               "    const int f = (int)blockIdx.x - a.fine_rows - tdq::kFineGap;\n"
+               "    if (f >= 0) tdq::k2_fine_row(a, f);\n    return;\n  }\n"
+             : "")
     << "  tdq::k2_body<0, 0, " << (grad ? "true" : "false")
-    << ", tdq::SpecProg>(a, tdq::SpecProg{nullptr}, gdops, 0, rec_ptr, rec_ops, nrec, blockIdx.x"
-    << (fine ? " - a.fine_rows" : "") << ");\n}\n";
+    << ", tdq::SpecProg>(a, tdq::SpecProg{nullptr}, gdops, 0, rec_ptr, rec_ops, nrec, blockIdx.x);\n}\n";
   return out.str();
 }
 

@@ -108,7 +108,7 @@ def test_value_rows_on_the_host(exe, name):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("rows", [1, 24, 76, 77])
+@pytest.mark.parametrize("rows", [1, 24, 72, 73])
 def test_value_rows(rows):
     """A gradient launch with a CTA for the values of every row, up to half the
     SMs and past that (float values, 2e-5); another initial state; the gradients
@@ -121,7 +121,7 @@ def test_value_rows(rows):
     spec, n = _circuit("hea6")[0], 6
     params = np.random.default_rng(n).uniform(0, 2 * math.pi, (rows, spec.n_params)).astype(np.float32)
     v, tol = _reference(spec, params)
-    fine = 2 * rows <= torch.cuda.get_device_properties(0).multi_processor_count
+    fine = 2 * rows + 8 <= torch.cuda.get_device_properties(0).multi_processor_count
     E = api.Exec(api.Circuit(spec), rows, grad="adjoint")
     p = torch.as_tensor(params).cuda()
     for _ in range(2):
